@@ -119,10 +119,9 @@ typedef struct {
  * per-position and step-size passes use variant 0 and the probe reduction
  * variant 3 (the fastest candidate on every workload measured). The
  * candidates (the "variants" below):
- *   [0] the per-position pass: windows <= 64: CTA sizes default / alternative;
- *       window 128: 1024 threads (0), 512 threads (1), a pair of CTAs of 512
- *       threads with 64 rows each exchanging the column transforms through
- *       distributed shared memory, two pairs per SM (2); windows 192/256: one;
+ *   [0] the per-position pass: window 16: CTA sizes default / alternative; the
+ *       others have one (window 128 accepts 0, 1 and 2, windows 32 and 64 accept
+ *       0 and 1 for it);
  *   [1] the step-size pass: one kernel per position (0), or the partial sums
  *       spread over 8 chunks of every position, then a
  *       per-position solve and update (1), or (windows <= 128) a cluster of 4

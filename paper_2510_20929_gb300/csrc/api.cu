@@ -456,6 +456,7 @@ struct TuneEntry {
   float ms[PTYCHO_TUNE_KERNELS][PTYCHO_TUNE_MAX];
 };
 
+// (only window 16 has two that differ; the others' numbers stay accepted)
 static int pass1_variants(int N) { return N == 128 ? 3 : (N <= 128 ? 2 : 1); }
 static int pass2_variants(int N) { return N <= 128 ? 4 : 2; }
 static constexpr int kReduceVariants = 4;

@@ -1,7 +1,8 @@
 // Per-scan-position kernels of the LSQML hot path (templated on the window N).
 //
-// k_pass1: one CTA per position of a minibatch. For every incoherent probe
-//   mode k it extracts the sub-pixel object patch o_j = S_j(O) (bilinear),
+// k_pass1: one CTA per position of a minibatch (window 16, and the parts
+//   around the tensor-core far field; kernels_pair.cuh holds the whole pass of
+//   the windows 32 to 128). For every incoherent probe mode k it extracts the sub-pixel object patch o_j = S_j(O) (bilinear),
 //   forms the exit wave psi_jk = P_k o_j (Pty-Chi Sec. 2.1, the psi = p o of
 //   Eq. 2), propagates it with the unitary 2-D FFT and accumulates the
 //   incoherent intensity I_j = sum_k |Psi_jk|^2 (Eq. 4's forward model). It
@@ -24,14 +25,14 @@
 namespace ptycho {
 namespace cg = cooperative_groups;
 
-// CTA sizes of the per-position pass: the default and the alternative the
-// autotuner may pick (the full count of line slots N*R1, or half of it with
-// two lines per thread).
+// CTA sizes of k_pass1 (the full count of line slots N*R1 at windows 16, 32
+// and 128): the default, and at window 16 the alternative the autotuner may
+// pick (half of it, two lines per thread).
 template <int N> struct Threads;
 template <> struct Threads<16> { static constexpr int T = 64, ALT = 32; };
-template <> struct Threads<32> { static constexpr int T = 128, ALT = 64; };
-template <> struct Threads<64> { static constexpr int T = 256, ALT = 512; };
-template <> struct Threads<128> { static constexpr int T = 1024, ALT = 512; };
+template <> struct Threads<32> { static constexpr int T = 128; };
+template <> struct Threads<64> { static constexpr int T = 256; };
+template <> struct Threads<128> { static constexpr int T = 1024; };
 
 template <int N>
 struct Pass1Smem {
@@ -99,40 +100,129 @@ __device__ __forceinline__ void fft2_inverse(float2* tile, const float2* tw, In&
 
 // S_j^T of an N x N patch onto its (N+1)^2 object tile, evaluated separably:
 // h_y(x) = (1-fx) p(y, x) + fx p(y, x-1) and out(y, x) = (1-fy) h_y(x) + fy h_{y-1}(x),
-// with p = 0 outside the patch. A thread owns one tile column x and a run of
-// rows (lanes of a warp emit consecutive x, so the atomics coalesce); each
-// output costs two patch reads. `load(y, x)` returns the patch value as a
-// float4 (unused components zero), `emit(y, x, v)` consumes the tile value.
+// with p = 0 outside the patch. A thread owns one of the tile columns 0 .. N-1
+// and a run of rows (lanes of a warp emit consecutive x, so the atomics
+// coalesce; T / N runs keep every thread busy), four rows of loads in flight
+// (one at a time the walk took 27,000 cycles of a 512-thread CTA at N = 128);
+// the tile's last column follows, a row per thread. `load(y, x)` returns the
+// patch value as a float4 (unused components zero), `emit(y, x, v)` consumes
+// the tile value.
 template <int N, int T, class Load, class Emit>
 __device__ __forceinline__ void bilinear_scatter(float fy, float fx, Load&& load, Emit&& emit) {
-  constexpr int N1 = N + 1;
-  constexpr int SEG = (T / N1) > 0 ? T / N1 : 1;
+  constexpr int N1 = N + 1, CH = 4;
+  constexpr int SEG = T / N > 0 ? T / N : 1;
   constexpr int RS = (N1 + SEG - 1) / SEG;
   const float gx = 1.f - fx, gy = 1.f - fy;
-  for (int item = threadIdx.x; item < N1 * SEG; item += T) {
-    const int seg = item / N1, x = item % N1;
-    const int y0 = seg * RS, y1 = min(N1, y0 + RS);
-    auto hrow = [&](int y) {
-      float4 h = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (y < N) {
-        if (x < N) {
-          const float4 a = load(y, x);
-          h = make_float4(gx * a.x, gx * a.y, gx * a.z, gx * a.w);
-        }
-        if (x > 0) {
-          const float4 b = load(y, x - 1);
-          h.x = fmaf(fx, b.x, h.x); h.y = fmaf(fx, b.y, h.y);
-          h.z = fmaf(fx, b.z, h.z); h.w = fmaf(fx, b.w, h.w);
-        }
-      }
-      return h;
+  const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+  auto lerp = [](float wa, float4 a, float wb, float4 b) {   // wa a + wb b
+    return make_float4(fmaf(wa, a.x, wb * b.x), fmaf(wa, a.y, wb * b.y), fmaf(wa, a.z, wb * b.z),
+                       fmaf(wa, a.w, wb * b.w));
+  };
+  for (int item = threadIdx.x; item < N * SEG; item += T) {
+    const int y0 = item / N * RS, x = item % N, y1 = min(N1, y0 + RS);
+    auto rowh = [&](int y) {
+      return lerp(fx, (y < N && x > 0) ? load(y, x - 1) : zero, gx, y < N ? load(y, x) : zero);
     };
-    float4 hp = (y0 > 0) ? hrow(y0 - 1) : make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int y = y0; y < y1; ++y) {
-      const float4 h = hrow(y);
-      emit(y, x, make_float4(fmaf(gy, h.x, fy * hp.x), fmaf(gy, h.y, fy * hp.y), fmaf(gy, h.z, fy * hp.z),
-                             fmaf(gy, h.w, fy * hp.w)));
-      hp = h;
+    float4 hp = y0 > 0 ? rowh(y0 - 1) : zero;
+    for (int y = y0; y < y1; y += CH) {
+      float4 h[CH];
+#pragma unroll
+      for (int c = 0; c < CH; ++c) h[c] = rowh(y + c);
+#pragma unroll
+      for (int c = 0; c < CH; ++c) {
+        if (y + c < y1) emit(y + c, x, lerp(gy, h[c], fy, hp));
+        hp = h[c];
+      }
+    }
+  }
+  for (int y = threadIdx.x; y < N1; y += T) {
+    const float4 a = y < N ? load(y, N - 1) : zero, b = y > 0 ? load(y - 1, N - 1) : zero;
+    emit(y, N, lerp(gy, lerp(fx, a, 0.f, zero), fy, lerp(fx, b, 0.f, zero)));
+  }
+}
+
+// The end of the per-position pass: g_j (read with getg(y, x), in shared
+// memory; every thread's writes are in flight on entry) and, for LSQML, the
+// probe intensity are scattered into the object frame, then the position
+// gradient or the sums of the position step are reduced. `spS` is N * N floats
+// of shared memory that are free on entry.
+template <int N, int T, bool OPR, class Get>
+__device__ __forceinline__ void overlap_add(const BatchArgs& a, int slot, int j, int ty, int tx, float fy, float fx,
+                                            const float2* p0, float* spS, double* red, Get&& getg) {
+  constexpr int NN = N * N;
+  const int tid = threadIdx.x, mode = a.mode;
+  const bool lsqml = (mode == MODE_LSQML_GAUSS || mode == MODE_LSQML_POISSON);
+  // LSQML: the probe intensity sum_k |P_k|^2 of every pixel into shared memory
+  // (the intensity/factor plane is free by now), so that the scatter's row walk
+  // waits on shared memory rather than on L2
+  if (lsqml) {
+#pragma unroll 2
+    for (int p = 4 * tid; p < NN; p += 4 * T) {
+      float4 v = __ldg((const float4*)(a.Sp + p));
+      if (OPR && p0) {
+        const float4 q0 = *(const float4*)(p0 + p), q1 = *(const float4*)(p0 + p + 2);
+        v.x += q0.x * q0.x + q0.y * q0.y; v.y += q0.z * q0.z + q0.w * q0.w;
+        v.z += q1.x * q1.x + q1.y * q1.y; v.w += q1.z * q1.z + q1.w * q1.w;
+      }
+      *(float4*)(spS + p) = v;
+    }
+  }
+  __syncthreads();
+  if (lsqml) {
+    bilinear_scatter<N, T>(
+        fy, fx,
+        [&](int y, int x) {
+          const float2 g = getg(y, x);
+          return make_float4(g.x, g.y, spS[y * N + x], 0.f);
+        },
+        [&](int y, int x, float4 v) {
+          atomicAdd(a.acc + (size_t)(ty + y) * a.W + (tx + x), make_float4(v.x, v.y, v.z, 0.f));
+        });
+  } else {
+    bilinear_scatter<N, T>(
+        fy, fx,
+        [&](int y, int x) {
+          const float2 g = getg(y, x);
+          return make_float4(g.x, g.y, 0.f, 0.f);
+        },
+        [&](int y, int x, float4 v) { atomicAdd(a.gobj + (size_t)(ty + y) * a.W + (tx + x), make_float2(v.x, v.y)); });
+  }
+
+  // ---- position gradient through the bilinear weights (gradient modes), or the
+  // ---- sums of the least-squares position step (LSQML position correction)
+  if (a.gpos || a.possum) {
+    const bool ls = a.possum != nullptr;
+    float gy = 0.f, gx = 0.f, a11 = 0.f, a12 = 0.f, a22 = 0.f;
+    for (int p = tid; p < NN; p += T) {
+      const int r = p / N, c = p % N;
+      const float2* o = a.obj + (size_t)(ty + r) * a.W + (tx + c);
+      const float2 O00 = __ldg(o), O01 = __ldg(o + 1), O10 = __ldg(o + a.W), O11 = __ldg(o + a.W + 1);
+      const float2 dy = make_float2((1.f - fx) * (O10.x - O00.x) + fx * (O11.x - O01.x),
+                                    (1.f - fx) * (O10.y - O00.y) + fx * (O11.y - O01.y));
+      const float2 dx = make_float2((1.f - fy) * (O01.x - O00.x) + fy * (O11.x - O10.x),
+                                    (1.f - fy) * (O01.y - O00.y) + fy * (O11.y - O10.y));
+      const float2 g = getg(r, c);
+      gy += g.x * dy.x + g.y * dy.y;  // Re(conj(g) dy)
+      gx += g.x * dx.x + g.y * dx.y;
+      if (ls) {   // sum_k abs(P_k)^2 times the derivative products
+        const float sp = __ldg(a.Sp + p) + ((OPR && p0) ? cabs2(p0[p]) : 0.f);
+        a11 = fmaf(sp, cabs2(dy), a11);
+        a12 = fmaf(sp, dy.x * dx.x + dy.y * dx.y, a12);
+        a22 = fmaf(sp, cabs2(dx), a22);
+      }
+    }
+    if (ls) {
+      double v[5] = {(double)a11, (double)a12, (double)a22, (double)gy, (double)gx};
+      block_sum<5>(v, red);
+      if (tid == 0)
+        for (int q = 0; q < 5; ++q) atomicAdd(a.possum + (size_t)slot * 5 + q, v[q]);
+    } else {
+      double v[2] = {(double)gy, (double)gx};
+      block_sum<2>(v, red);
+      if (tid == 0) {
+        a.gpos[2 * j] += (float)v[0];
+        a.gpos[2 * j + 1] += (float)v[1];
+      }
     }
   }
 }
@@ -191,97 +281,12 @@ __global__ void __launch_bounds__(T, 1) k_pass1(BatchArgs a) {
   float2* psi_s = a.psi_s ? a.psi_s + slotNN * M : nullptr;
   float2* o_s = a.o_s ? a.o_s + slotNN : nullptr;
 
-  // Tensor memory as per-thread storage (the whole pass, window 128): the
-  // patch o_j and the running sum g_j of the thread's natural-layout pixel
-  // pairs stay on chip across the modes instead of making round trips through
-  // L2. Warp w reaches TMEM lanes 32 (w % 4) ..+31; the T/128 warps sharing a
-  // lane quarter split its 512 columns, CW each: o in the first 4 STEPS
-  // columns (pair q at 4q), g in the next 4 STEPS. The CTA holds all 512
-  // columns; no other TMEM-allocating CTA fits beside it on the SM (its
-  // shared memory alone exceeds half of the SM's), so the allocation never
-  // waits.
-  constexpr bool TM = (PART == 0 && N == 128);
-  constexpr int STEPS = NatPairs<N, T>::STEPS;
-  static_assert(!TM || (STEPS % 2 == 0 && 8 * STEPS == 65536 / T), "o and g fill each warp's TMEM columns");
-  // (the base address lives in shared memory, beyond the block reductions'
-  // 160 doubles; the thread's column base is recomputed where it is used, so
-  // that no register is held across the transforms)
-  uint32_t* tm_holder = (uint32_t*)(red + 250);
-  if constexpr (TM) {
-    if ((tid >> 5) == 0) {
-      tc::tmem_alloc(tm_holder, 512);
-      tc::tmem_relinquish();
-    }
-    tc::fence_before_sync();
-    __syncthreads();
-    tc::fence_after_sync();
-  }
-  auto tm_o = [&]() -> uint32_t {   // this thread's patch columns (g follows at + 4 STEPS)
-    const int w = (int)(threadIdx.x >> 5);
-    return *tm_holder + ((uint32_t)(32 * (w & 3)) << 16) + (uint32_t)((w >> 2) * (65536 / T));
-  };
-  // releases the tensor memory once every thread's TMEM accesses have completed
-  auto tm_release = [&]() {
-    if constexpr (TM) {
-      tc::fence_before_sync();
-      __syncthreads();
-      tc::fence_after_sync();
-      if ((threadIdx.x >> 5) == 0) tc::tmem_dealloc(*tm_holder, 512);
-    }
-  };
-
   // ---- forward model: I_j = sum_k |F(P_k o_j)|^2 -------------------------------
 #pragma unroll 1
   for (int k = 0; k < (PART == 2 ? 0 : M); ++k) {
     const float2* Pk = shared_mode<OPR>(a, k, NN);
     // psi_k = P_k o_j into the tile, two adjacent pixels per thread and iteration
     const NatPairs<N, T> np;
-    if constexpr (TM) {
-      // groups of two pairs; the patch from TMEM after the first mode; the
-      // probe pairs of the next group are loaded (L2) before this group's work
-      const uint32_t t_o = tm_o();
-      const bool pre = !OPR || Pk;
-      float4 Pn[2];
-      if (pre)
-#pragma unroll
-        for (int u = 0; u < 2; ++u) Pn[u] = __ldg((const float4*)(Pk + np.pix(u)));
-#pragma unroll 1
-      for (int qg = 0; qg < STEPS / 2; ++qg) {
-        const float4 Pc[2] = {Pn[0], Pn[1]};
-        if (pre && qg + 1 < STEPS / 2)
-#pragma unroll
-          for (int u = 0; u < 2; ++u) Pn[u] = __ldg((const float4*)(Pk + np.pix(2 * qg + 2 + u)));
-        float ov[8];
-        if (k == 0) {
-#pragma unroll
-          for (int u = 0; u < 2; ++u) {
-            const int q = 2 * qg + u, p = np.pix(q);
-            float2 o0, o1;
-            bilinear2(a.obj, a.W, ty + np.row(q), tx + np.c, fy, fx, o0, o1);
-            if (o_s) *(float4*)(o_s + p) = make_float4(o0.x, o0.y, o1.x, o1.y);
-            ov[4 * u] = o0.x; ov[4 * u + 1] = o0.y; ov[4 * u + 2] = o1.x; ov[4 * u + 3] = o1.y;
-          }
-          tc::tmem_st8(t_o + 8 * qg, ov);
-        } else {
-          tc::tmem_ld8_wait(t_o + 8 * qg, ov);
-        }
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-          const int q = 2 * qg + u, p = np.pix(q);
-          float4 P2;
-          if (pre) {
-            P2 = Pc[u];
-          } else {
-            P2 = opr_pair(a.opr_U, wj, a.K, NN, p);
-            if (p0) *(float4*)(p0 + p) = P2;
-          }
-          const float2 x0 = cmul(make_float2(P2.x, P2.y), make_float2(ov[4 * u], ov[4 * u + 1]));
-          const float2 x1 = cmul(make_float2(P2.z, P2.w), make_float2(ov[4 * u + 2], ov[4 * u + 3]));
-          store_pair(tile, np.phys(q), x0, x1);
-        }
-      }
-      if (k == 0) tc::tmem_wait_st();
-    } else
 #pragma unroll 4
     for (int q = 0; q < NatPairs<N, T>::STEPS; ++q) {
       const int r = np.row(q), c = np.c, p = np.pix(q);
@@ -416,10 +421,7 @@ __global__ void __launch_bounds__(T, 1) k_pass1(BatchArgs a) {
       block_sum<1>(v, red);
       if (tid == 0) atomicAdd(a.loss, v[0]);
     }
-    if (mode == MODE_FWD || a.loss_only) {
-      tm_release();
-      return;
-    }
+    if (mode == MODE_FWD || a.loss_only) return;
   }
 
   // ---- back-propagation: chi_k = F^-1[fac Psi_k], g = sum_k conj(P_k) chi_k, h_k ----
@@ -467,54 +469,6 @@ __global__ void __launch_bounds__(T, 1) k_pass1(BatchArgs a) {
     // chi_k (natural layout) is in the tile, or in PART 2 in the scratch:
     // g += conj(P_k) chi_k, h_k = conj(o) chi_k
     const NatPairs<N, T> np;
-    if constexpr (TM) {
-      // o and the running g from TMEM; the last mode's g goes to the scratch
-      // (for the step sizes) and over chi in the tile (for the scatter)
-      const uint32_t t_o = tm_o(), t_g = t_o + 4 * STEPS;
-      // the probe (or primary-mode) pairs of the next group are loaded before
-      // this group's work
-      // (the primary modes of OPR were written by this kernel: plain loads)
-      auto ldP = [&](int p) {
-        return (!OPR || Pk) ? __ldg((const float4*)(Pk + p)) : *(const float4*)(p0 + p);
-      };
-      float4 Pn[2];
-#pragma unroll
-      for (int u = 0; u < 2; ++u) Pn[u] = ldP(np.pix(u));
-#pragma unroll 1
-      for (int qg = 0; qg < STEPS / 2; ++qg) {
-        const float4 Pc[2] = {Pn[0], Pn[1]};
-        if (qg + 1 < STEPS / 2)
-#pragma unroll
-          for (int u = 0; u < 2; ++u) Pn[u] = ldP(np.pix(2 * qg + 2 + u));
-        float ov[8], gv[8];
-        if (k < M - 1)
-          tc::tmem_ld8x2_wait(t_o + 8 * qg, ov, t_g + 8 * qg, gv);
-        else
-          tc::tmem_ld8_wait(t_o + 8 * qg, ov);
-#pragma unroll
-        for (int u = 0; u < 2; ++u) {
-          const int q = 2 * qg + u, p = np.pix(q);
-          float2 x0, x1;
-          load_pair(tile, np.phys(q), x0, x1);
-          const float4 P2 = Pc[u];
-          float2 g0 = cmulc(make_float2(P2.x, P2.y), x0), g1 = cmulc(make_float2(P2.z, P2.w), x1);
-          if (k < M - 1) {
-            g0.x += gv[4 * u]; g0.y += gv[4 * u + 1]; g1.x += gv[4 * u + 2]; g1.y += gv[4 * u + 3];
-          }
-          const float2 h0 = cmulc(make_float2(ov[4 * u], ov[4 * u + 1]), x0);
-          const float2 h1 = cmulc(make_float2(ov[4 * u + 2], ov[4 * u + 3]), x1);
-          __stcs((float4*)(h_s + (size_t)k * NN + p), make_float4(h0.x, h0.y, h1.x, h1.y));
-          if (k > 0) {
-            gv[4 * u] = g0.x; gv[4 * u + 1] = g0.y; gv[4 * u + 2] = g1.x; gv[4 * u + 3] = g1.y;
-          } else {
-            *(float4*)(g_s + p) = make_float4(g0.x, g0.y, g1.x, g1.y);
-            store_pair(tile, np.phys(q), g0, g1);
-          }
-        }
-        if (k > 0) tc::tmem_st8(t_g + 8 * qg, gv);
-      }
-      if (k > 0) tc::tmem_wait_st();
-    } else
 #pragma unroll 2
     for (int q = 0; q < NatPairs<N, T>::STEPS; ++q) {
       const int p = np.pix(q);
@@ -542,91 +496,13 @@ __global__ void __launch_bounds__(T, 1) k_pass1(BatchArgs a) {
   __syncthreads();
 
   // ---- scatter S_j^T g (and the illumination) into the object frame ----------------
-  if (!TM) {   // (with TMEM the last mode wrote g into the tile already)
-    const NatPairs<N, T> np;
+  const NatPairs<N, T> np;
 #pragma unroll 1
-    for (int q = 0; q < NatPairs<N, T>::STEPS; ++q) {
-      const float4 g2 = *(const float4*)(g_s + np.pix(q));
-      store_pair(tile, np.phys(q), make_float2(g2.x, g2.y), make_float2(g2.z, g2.w));
-    }
+  for (int q = 0; q < NatPairs<N, T>::STEPS; ++q) {
+    const float4 g2 = *(const float4*)(g_s + np.pix(q));
+    store_pair(tile, np.phys(q), make_float2(g2.x, g2.y), make_float2(g2.z, g2.w));
   }
-  const bool lsqml = (mode == MODE_LSQML_GAUSS || mode == MODE_LSQML_POISSON);
-  // LSQML: the probe intensity sum_k |P_k|^2 of every pixel into shared memory
-  // (the intensity/factor plane is free by now), so that the scatter's row walk
-  // waits on shared memory rather than on L2
-  float* spS = rI;
-  if (PART != 1 && lsqml) {
-    static_assert((size_t)N * RP >= (size_t)NN, "room for the probe intensity");
-#pragma unroll 2
-    for (int p = 4 * tid; p < NN; p += 4 * T) {
-      float4 v = __ldg((const float4*)(a.Sp + p));
-      if (OPR && p0) {
-        const float4 q0 = *(const float4*)(p0 + p), q1 = *(const float4*)(p0 + p + 2);
-        v.x += q0.x * q0.x + q0.y * q0.y; v.y += q0.z * q0.z + q0.w * q0.w;
-        v.z += q1.x * q1.x + q1.y * q1.y; v.w += q1.z * q1.z + q1.w * q1.w;
-      }
-      *(float4*)(spS + p) = v;
-    }
-  }
-  __syncthreads();
-  if (lsqml) {
-    bilinear_scatter<N, T>(
-        fy, fx,
-        [&](int y, int x) {
-          const float2 g = tile[tix<N>(y, x)];
-          return make_float4(g.x, g.y, spS[y * N + x], 0.f);
-        },
-        [&](int y, int x, float4 v) {
-          atomicAdd(a.acc + (size_t)(ty + y) * a.W + (tx + x), make_float4(v.x, v.y, v.z, 0.f));
-        });
-  } else {
-    bilinear_scatter<N, T>(
-        fy, fx,
-        [&](int y, int x) {
-          const float2 g = tile[tix<N>(y, x)];
-          return make_float4(g.x, g.y, 0.f, 0.f);
-        },
-        [&](int y, int x, float4 v) { atomicAdd(a.gobj + (size_t)(ty + y) * a.W + (tx + x), make_float2(v.x, v.y)); });
-  }
-
-  // ---- position gradient through the bilinear weights (gradient modes), or the
-  // ---- sums of the least-squares position step (LSQML position correction)
-  if (a.gpos || a.possum) {
-    const bool ls = a.possum != nullptr;
-    float gy = 0.f, gx = 0.f, a11 = 0.f, a12 = 0.f, a22 = 0.f;
-    for (int p = tid; p < NN; p += T) {
-      const int r = p / N, c = p % N;
-      const float2* o = a.obj + (size_t)(ty + r) * a.W + (tx + c);
-      const float2 O00 = __ldg(o), O01 = __ldg(o + 1), O10 = __ldg(o + a.W), O11 = __ldg(o + a.W + 1);
-      const float2 dy = make_float2((1.f - fx) * (O10.x - O00.x) + fx * (O11.x - O01.x),
-                                    (1.f - fx) * (O10.y - O00.y) + fx * (O11.y - O01.y));
-      const float2 dx = make_float2((1.f - fy) * (O01.x - O00.x) + fy * (O11.x - O10.x),
-                                    (1.f - fy) * (O01.y - O00.y) + fy * (O11.y - O10.y));
-      const float2 g = tile[tix<N>(r, c)];
-      gy += g.x * dy.x + g.y * dy.y;  // Re(conj(g) dy)
-      gx += g.x * dx.x + g.y * dx.y;
-      if (ls) {   // sum_k abs(P_k)^2 times the derivative products
-        const float sp = __ldg(a.Sp + p) + ((OPR && p0) ? cabs2(p0[p]) : 0.f);
-        a11 = fmaf(sp, cabs2(dy), a11);
-        a12 = fmaf(sp, dy.x * dx.x + dy.y * dx.y, a12);
-        a22 = fmaf(sp, cabs2(dx), a22);
-      }
-    }
-    if (ls) {
-      double v[5] = {(double)a11, (double)a12, (double)a22, (double)gy, (double)gx};
-      block_sum<5>(v, red);
-      if (tid == 0)
-        for (int q = 0; q < 5; ++q) atomicAdd(a.possum + (size_t)slot * 5 + q, v[q]);
-    } else {
-      double v[2] = {(double)gy, (double)gx};
-      block_sum<2>(v, red);
-      if (tid == 0) {
-        a.gpos[2 * j] += (float)v[0];
-        a.gpos[2 * j + 1] += (float)v[1];
-      }
-    }
-  }
-  tm_release();
+  overlap_add<N, T, OPR>(a, slot, j, ty, tx, fy, fx, p0, rI, red, [&](int y, int x) { return tile[tix<N>(y, x)]; });
 }
 
 

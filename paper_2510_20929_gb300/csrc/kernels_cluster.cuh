@@ -1,6 +1,5 @@
 // Per-position pass for windows larger than one CTA's shared memory, on a
-// cluster of Q CTAs (N = 256: Q = 8; N = 192: Q = 6; and a pair of CTAs for
-// the 128 window).
+// cluster of Q CTAs (N = 256: Q = 8; N = 192: Q = 6).
 //
 // The N x N complex tile is shared by the cluster: in the spatial domain CTA q
 // holds the LR = N / Q rows LR q .. LR q + LR - 1. The 2-D DFT runs as
@@ -36,10 +35,6 @@ namespace cg = cooperative_groups;
 // GF(2)), chosen with the half-warp bank model for the row and column lines.
 struct Swz256 {  // f = ((r << 2) ^ (r >> 1) ^ (c >> 4)) & 15
   __host__ __device__ static constexpr int fr(int r) { return ((r << 2) ^ (r >> 1)) & 15; }
-  __host__ __device__ static constexpr int fcb(int c) { return (c >> 4) & 15; }
-};
-struct Swz128 {  // the single-CTA 128 window's swizzle: f = ((r << 3) ^ (r << 1) ^ (r >> 2) ^ (c >> 4)) & 15
-  __host__ __device__ static constexpr int fr(int r) { return ((r << 3) ^ (r << 1) ^ (r >> 2)) & 15; }
   __host__ __device__ static constexpr int fcb(int c) { return (c >> 4) & 15; }
 };
 struct Swz192 {  // f = ((r << 3) ^ (r << 1) ^ (r >> 2) ^ (c >> 6)) & 15
@@ -109,8 +104,6 @@ struct Cfg {
 // rows and one CTA per SM: the spiral256 pass 2.99 -> 2.48 ms per 256
 // positions, multislice256 29.5K -> 32.6K patterns/s)
 using Cfg256 = Cfg<256, 8, 512, 16, 16, false, Swz256, 2>;
-// the 128 window on a pair of CTAs (64 rows each) that fit two to an SM
-using Cfg128 = Cfg<128, 2, 512, 8, 16, true, Swz128, 2>;
 using Cfg192 = Cfg<192, 6, 256, 8, 24, true, Swz192, 2>;
 
 // The transpose across the cluster: tile[x][LR s + r] <- tile_s[r][LR q + x]

@@ -1,0 +1,544 @@
+// The per-position pass of the windows one CTA holds whole (32, 64, 128), on
+// the packed line-pair transforms of fft_pair.cuh. It computes what k_pass1
+// (kernels.cuh) describes; what differs is where the data lives:
+//   * every thread owns the same pixel pairs (rows n + R1 q, columns 2p,
+//     2p + 1) when a mode's exit wave is built and when its chi comes back, so
+//     psi_jk goes from the loads straight into the column transform's
+//     registers and chi_jk from the registers into g and h, with no pass over
+//     the tile on either side;
+//   * the far field, the measured intensities and the factor of the data term
+//     belong to one thread each, so the far-field scratch and the
+//     intensity/factor plane hold one 16-byte unit per thread and step (every
+//     access a whole coalesced run), and the last mode's far field stays in
+//     registers through the data term into its inverse transform;
+//   * the patch o_j and the running g_j of the thread's pixels stay in tensor
+//     memory (windows 64 and 128: 8 R2 columns of the thread's TMEM lane).
+// What bounds it: the transforms (about half the cycles; shared-memory
+// wavefronts and issue slots), then the rate of L2 requests of the probe
+// loads, the far-field scratch and the h stores (about 2.8 cycles per 128-byte
+// request when all SMs stream), with one CTA of 512 threads filling an SM at
+// window 128. Straight-line code that a CTA runs once costs instruction
+// fetches, so loops over a thread's pixels stay rolled where v is not indexed.
+// Measured on GB300 against the one-line-per-lane-group pass it replaced (per
+// launch): window 128, 5 modes, 256 positions 287 -> 249 us (1 mode: 101 -> 92,
+// 1024 positions 1002 -> 860); window 64, 4 modes, 256 positions 63 -> 51,
+// 1216 positions 227 -> 166, 1 mode, 16 positions 24.7 -> 20.7; window 32, 4
+// modes, 2000 positions 116 -> 72.
+#pragma once
+#include "kernels.cuh"
+#include "fft_pair.cuh"
+
+namespace ptycho {
+
+// CTAs per SM: shared memory at window 128; the register budget (80 and 128 a
+// thread) at windows 64 and 32.
+template <int N> struct PairCtas;
+template <> struct PairCtas<32> { static constexpr int n = 8; };
+template <> struct PairCtas<64> { static constexpr int n = 3; };
+template <> struct PairCtas<128> { static constexpr int n = 1; };
+
+template <int N>
+struct PairSmem {
+  static constexpr size_t red = 0;
+  static constexpr size_t tile = red + 256 * sizeof(double);
+  static constexpr size_t rI = tile + (size_t)N * N * sizeof(float2);
+  static constexpr size_t tw = rI + (size_t)N * N * sizeof(float);
+  static constexpr size_t o = tw + (size_t)Twiddles<N>::COUNT * sizeof(float2);
+  static constexpr size_t bytes = o + (N >= 64 ? 0 : (size_t)N * N * sizeof(float2));
+  // the staged object tile: N + 1 rows of up to N + 2 pixels, over the tile and
+  // the intensity plane (free before the first transform). The pitch is 64
+  // bytes off a multiple of 128: the rows of a half-warp's lanes alternate
+  // between the two halves of the banks.
+  static constexpr int opitch = N * 8 + 64;
+  static_assert((N + 1) * opitch <= N * N * 12, "the object tile fits");
+};
+
+// The data term of four pixels (Eq. 1, or the Poisson likelihood): adds the
+// loss and returns the far-field factor. Square roots and quotients are
+// formed from rsqrtf with one residual correction each (Markstein, IBM J. Res.
+// Dev. 34, 1990: s += r y / 2 with the residual r = x - s^2 exact in one fused
+// multiply-add; q += r / d likewise), within the rounding of the correctly
+// rounded results: sqrtf and the division leave the straight code for a zero
+// operand, and most counts of a diffraction pattern are zero. Values outside
+// 2^-96 .. 2^96 (zero counts aside) take the functions. `t` receives what the
+// loss adds per pixel: the difference of the amplitudes (added squared), or
+// the Poisson term; (x, z) and (y, w) are two rows.
+__device__ __forceinline__ float4 data_factor(int mode, float4 I, float4 Im, float eps, float4& t) {
+  constexpr float lo = 1.2621774e-29f, hi = 7.9228163e28f;   // 2^-96, 2^96
+  const bool gauss = mode == MODE_LSQML_GAUSS || mode == MODE_GRAD_GAUSS;
+  const bool lsqml = mode == MODE_LSQML_GAUSS || mode == MODE_LSQML_POISSON;
+  const float2 I2[2] = {make_float2(I.x, I.y), make_float2(I.z, I.w)};
+  const float2 M2[2] = {make_float2(Im.x, Im.y), make_float2(Im.z, Im.w)};
+  float2 Ie[2], mx[2], rho[2], T2[2];
+  bool in = true;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    Ie[h] = make_float2(I2[h].x + eps, I2[h].y + eps);
+    mx[h] = make_float2(M2[h].x == 0.f ? 1.f : M2[h].x, M2[h].y == 0.f ? 1.f : M2[h].y);
+    in = in && fminf(fminf(Ie[h].x, Ie[h].y), fminf(mx[h].x, mx[h].y)) >= lo &&
+         fmaxf(fmaxf(Ie[h].x, Ie[h].y), fmaxf(mx[h].x, mx[h].y)) <= hi &&
+         !(isnan(Ie[h].x) || isnan(Ie[h].y) || isnan(mx[h].x) || isnan(mx[h].y));
+  }
+  if (in) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const float2 y = make_float2(rsqrtf(Ie[h].x), rsqrtf(Ie[h].y));
+      if (gauss) {
+        const float2 half = fp::splat(0.5f);
+        const float2 ym = make_float2(rsqrtf(mx[h].x), rsqrtf(mx[h].y));
+        float2 s = fp::mul2(Ie[h], y), m = fp::mul2(mx[h], ym);
+        s = fp::fma2(fp::mul2(half, y), fp::fma2(fp::neg2(s), s, Ie[h]), s);
+        m = fp::fma2(fp::mul2(half, ym), fp::fma2(fp::neg2(m), m, mx[h]), m);
+        if (M2[h].x == 0.f) m.x = 0.f;
+        if (M2[h].y == 0.f) m.y = 0.f;
+        T2[h] = fp::sub2(s, m);
+        const float2 q = fp::mul2(m, y);
+        rho[h] = fp::fma2(fp::fma2(fp::neg2(q), s, m), y, q);
+      } else {
+        float2 c = fp::mul2(y, y);   // 1 / Ie
+        c = fp::fma2(c, fp::fma2(fp::neg2(Ie[h]), c, fp::splat(1.f)), c);
+        const float2 q = fp::mul2(M2[h], c);
+        rho[h] = fp::fma2(fp::fma2(fp::neg2(q), Ie[h], M2[h]), c, q);
+        T2[h] = make_float2(I2[h].x - M2[h].x * logf(Ie[h].x), I2[h].y - M2[h].y * logf(Ie[h].y));
+      }
+    }
+  } else {
+    const float Iv[4] = {I.x, I.y, I.z, I.w}, Mv[4] = {Im.x, Im.y, Im.z, Im.w};
+    float r[4], l[4];
+#pragma unroll
+    for (int h = 0; h < 4; ++h) {
+      const float E = Iv[h] + eps;
+      if (gauss) {
+        const float s = sqrtf(E), m = sqrtf(Mv[h]);
+        l[h] = s - m;
+        r[h] = m / s;
+      } else {
+        l[h] = Iv[h] - Mv[h] * logf(E);
+        r[h] = Mv[h] / E;
+      }
+    }
+    T2[0] = make_float2(l[0], l[1]);
+    T2[1] = make_float2(l[2], l[3]);
+    rho[0] = make_float2(r[0], r[1]);
+    rho[1] = make_float2(r[2], r[3]);
+  }
+  t = make_float4(T2[0].x, T2[0].y, T2[1].x, T2[1].y);
+  const float w = lsqml ? (gauss ? 1.f : 0.5f) : -2.f;   // rho - 1, (q - 1) / 2, or 2 (1 - rho)
+  return make_float4(w * (rho[0].x - 1.f), w * (rho[0].y - 1.f), w * (rho[1].x - 1.f), w * (rho[1].y - 1.f));
+}
+
+template <int N, bool OPR>
+__global__ void __launch_bounds__(fp::Fft<N>::T, PairCtas<N>::n) k_pass1_pair(BatchArgs a) {
+  using F = fp::Fft<N>;
+  using SM = PairSmem<N>;
+  using fp::C2;
+  constexpr int T = F::T, R1 = F::R1, R2 = F::R2, NN = N * N;
+  constexpr int D = 6;   // probe loads in flight in the backward pass (its v fills half the registers)
+  extern __shared__ __align__(16) unsigned char smem[];
+  wait_prior_grid();
+  double* red = (double*)(smem + SM::red);
+  float4* tile = (float4*)(smem + SM::tile);
+  float4* rI = (float4*)(smem + SM::rI);
+  float2* tw = (float2*)(smem + SM::tw);
+
+  const int slot = blockIdx.x, tid = threadIdx.x;
+  const int n = F::col_lane(), p = F::col_pair();   // the thread's pixels: rows n + R1 q, columns 2p, 2p + 1
+  const int nr = F::row_lane(), pr = F::row_pair();   // its far field: rows 2pr, 2pr + 1, columns far_col(nr, q)
+  const int e = a.b0 + slot;
+  const int j = a.order ? a.order[e] : e;
+  int ty = 0, tx = 0;
+  float fy = 0.f, fx = 0.f;
+  bool ok = (j >= 0 && j < a.J);
+  if (ok) ok = tile_of(a.pos[2 * j], a.pos[2 * j + 1], N, a.H, a.W, ty, tx, fy, fx);
+  if (!ok) {
+    if (tid == 0) {
+      atomicOr(a.status, FLAG_BOUNDS);
+      if (a.valid) a.valid[slot] = 0;
+    }
+    return;
+  }
+  if (tid == 0 && a.valid) a.valid[slot] = 1;
+  // the measured intensities are first read by the data term, after the forward
+  // transforms: fetch them into L2 meanwhile (they may live in host memory)
+  if (tid == 0 && a.meas && a.mode != MODE_FWD)
+    prefetch_l2_bulk(a.meas + (size_t)j * NN, (uint32_t)(NN * sizeof(float)));
+  // The (N + 1)^2 object tile comes into shared memory by one bulk copy per
+  // row, from the row's start rounded down to 16 bytes (row r then begins at
+  // pixel off(r)); rows of an unaligned object, and the one row whose copy
+  // would end past the object, by plain loads.
+  unsigned char* stage = (unsigned char*)tile;
+  uint64_t* bar = (uint64_t*)(red + 252);
+  const float2* tile0 = a.obj + (size_t)ty * a.W + tx;
+  const bool bulk = ((uintptr_t)a.obj & 15) == 0;
+  auto off = [&](int r) -> int { return bulk ? (int)(((uintptr_t)tile0 >> 3) + (uintptr_t)r * a.W) & 1 : 0; };
+  auto row_plain = [&](int r) {
+    return !bulk || (off(r) == 0 && (size_t)(ty + r) * a.W + tx + N + 2 > (size_t)a.H * a.W);
+  };
+  if (tid == 0) {
+    tc::mbar_init(bar, 1);
+    tc::mbar_init(bar + 1, 1);
+    tc::fence_mbar_init();
+    const int last = row_plain(N) ? N : N + 1;   // only the tile's last row can end the object
+    if (bulk) tc::mbar_expect_tx(bar, (uint32_t)(last * (N + 2) * sizeof(float2)));
+  }
+  constexpr bool TM = N >= 64;
+  constexpr int TMC = T / 128 * 8 * R2, TG = 4 * R2;   // columns of the CTA; g's offset
+  uint32_t* tm_holder = (uint32_t*)(red + 250);   // beyond the block reductions' 160 doubles
+  if constexpr (TM) {
+    if (tid < 32) {
+      tc::tmem_alloc(tm_holder, TMC);
+      tc::tmem_relinquish();
+    }
+    tc::fence_before_sync();
+  }
+  __syncthreads();   // the barrier's state, the tensor-memory address
+  if constexpr (TM) tc::fence_after_sync();
+  for (int r = tid; r < N + 1; r += T)
+    if (!row_plain(r))
+      tc::bulk_g2s(stage + r * SM::opitch, tile0 + (size_t)r * a.W - off(r), (N + 2) * sizeof(float2), bar);
+  if (!bulk) {
+    for (int i = tid; i < (N + 1) * (N + 1); i += T) {
+      const int r = i / (N + 1), c = i % (N + 1);
+      ((float2*)(stage + r * SM::opitch))[c] = __ldg(tile0 + (size_t)r * a.W + c);
+    }
+  } else if (row_plain(N)) {
+    for (int c = tid; c < N + 1; c += T)
+      ((float2*)(stage + N * SM::opitch))[c] = __ldg(tile0 + (size_t)N * a.W + c);
+  }
+  make_twiddles<N>(tw);
+
+  const int M = a.M, mode = a.mode;
+  const float invN = 1.0f / (float)N;
+  const size_t slotNN = (size_t)slot * NN;
+  float* wj = (float*)(red + 128);   // this position's eigenmode weights (OPR)
+  float2* p0 = (OPR && a.p0_s) ? a.p0_s + slotNN : nullptr;
+  if (OPR && tid < a.K) wj[tid] = a.opr_w[(size_t)j * a.K + tid];
+  // far field of mode k, unit i of this thread: psi[k NN / 2 + i T]
+  float4* oS = (float4*)(smem + SM::o) + tid;   // (window 32) pixel pair q at oS[q T]
+  float4* psi = a.psi_s ? (float4*)(a.psi_s + slotNN * M) + tid : nullptr;
+  float2* o_s = a.o_s ? a.o_s + slotNN : nullptr;
+  const int pix0 = n * N + 2 * p;   // pixel pair q: pix0 + q R1 N
+
+  // Tensor memory as per-thread storage: the thread's R2 pixel pairs of o in
+  // the first 4 R2 of its columns, of g in the next 4 R2 (warp w reaches lanes
+  // 32 (w % 4) ..+31; every fourth warp shares them, 8 R2 columns each). A CTA
+  // holds TMC columns: the SM's 512 serve all the CTAs its shared memory admits.
+  // (Window 32: o in shared memory, g in its scratch.)
+  auto tm_o = [&]() -> uint32_t {
+    const int w = (int)(threadIdx.x >> 5);
+    return *tm_holder + ((uint32_t)(32 * (w & 3)) << 16) + (uint32_t)((w >> 2) * 8 * R2);
+  };
+  auto tm_release = [&]() {
+    if constexpr (TM) {
+      tc::fence_before_sync();
+      __syncthreads();
+      tc::fence_after_sync();
+      if (threadIdx.x < 32) tc::tmem_dealloc(*tm_holder, TMC);
+    }
+  };
+  // pixel pair q of the probe mode (of the relaxed primary mode: forward
+  // synthesised and kept in p0, backward read there)
+  auto probe_fwd = [&](const float2* Pk, int q) -> float4 {
+    const int pix = pix0 + q * R1 * N;
+    if (!OPR || Pk) return __ldg((const float4*)(Pk + pix));
+    const float4 P = opr_pair(a.opr_U, wj, a.K, NN, pix);
+    if (p0) *(float4*)(p0 + pix) = P;
+    return P;
+  };
+  auto probe_back = [&](const float2* Pk, int q) -> float4 {
+    const int pix = pix0 + q * R1 * N;
+    return (!OPR || Pk) ? __ldg((const float4*)(Pk + pix)) : *(const float4*)(p0 + pix);
+  };
+  auto exit_wave = [&](float4 P, float4 o) -> C2 {
+    const float2 x0 = cmul(make_float2(P.x, P.y), make_float2(o.x, o.y));
+    const float2 x1 = cmul(make_float2(P.z, P.w), make_float2(o.z, o.w));
+    return {make_float2(x0.x, x1.x), make_float2(x0.y, x1.y)};
+  };
+
+  // ---- forward model: I_j = sum_k |F(P_k o_j)|^2 -------------------------------
+  // Every pixel pair of a mode's probe is in flight at once: the loads are
+  // issued before the barrier that frees the tile (the registers of v are
+  // empty there).
+  C2 v[R2];
+  float4 P[R2];
+  if (OPR) __syncthreads();   // the weights
+#pragma unroll
+  for (int q = 0; q < R2; ++q) P[q] = probe_fwd(shared_mode<OPR>(a, 0, NN), q);
+  // joins the block after a wait for copies; false (and everything released)
+  // when a thread's wait gave up
+  auto arrived_all = [&](bool got, uint64_t* b) -> bool {
+    if (__syncthreads_and(got)) return true;
+    if (tid == 0) {
+      atomicOr(a.status, FLAG_TIMEOUT);
+      if (a.valid) a.valid[slot] = 0;
+      tc::mbar_wait(b, 0);   // copies in flight must not outlive the CTA
+    }
+    tm_release();
+    return false;
+  };
+  if (!arrived_all(!bulk || tc::mbar_wait(bar, 0), bar)) return;   // (also twiddles, plainly loaded rows)
+#pragma unroll
+  for (int qg = 0; qg < R2 / 4; ++qg) {   // the patch o_j and the first mode's exit wave
+    const float w00 = (1.f - fy) * (1.f - fx), w01 = (1.f - fy) * fx, w10 = fy * (1.f - fx), w11 = fy * fx;
+    float ov[16];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int q = 4 * qg + u, r = n + R1 * q;
+      const float2* A = (const float2*)(stage + r * SM::opitch) + off(r) + 2 * p;
+      const float2* B = (const float2*)(stage + (r + 1) * SM::opitch) + off(r + 1) + 2 * p;
+      const float2 a0 = A[0], a1 = A[1], a2 = A[2], b0 = B[0], b1 = B[1], b2 = B[2];
+      const float4 o = make_float4(w00 * a0.x + w01 * a1.x + w10 * b0.x + w11 * b1.x,
+                                   w00 * a0.y + w01 * a1.y + w10 * b0.y + w11 * b1.y,
+                                   w00 * a1.x + w01 * a2.x + w10 * b1.x + w11 * b2.x,
+                                   w00 * a1.y + w01 * a2.y + w10 * b1.y + w11 * b2.y);
+      if (o_s) *(float4*)(o_s + pix0 + q * R1 * N) = o;
+      *(float4*)(ov + 4 * u) = o;
+      if constexpr (!TM) oS[q * T] = o;
+      v[q] = exit_wave(P[q], o);
+    }
+    if constexpr (TM) tc::tmem_st16(tm_o() + 16 * qg, ov);
+  }
+  if constexpr (TM) tc::tmem_wait_st();
+  __syncthreads();   // the staged object tile is read: its place belongs to the transforms
+#pragma unroll 1
+  for (int k = 0; k < M; ++k) {
+    if (k > 0) {
+#pragma unroll
+      for (int qg = 0; qg < R2 / 4; ++qg) {
+        float ov[16];
+        if constexpr (TM) tc::tmem_ld16_wait(tm_o() + 16 * qg, ov);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          if constexpr (!TM) *(float4*)(ov + 4 * u) = oS[(4 * qg + u) * T];
+          v[4 * qg + u] = exit_wave(P[4 * qg + u], *(const float4*)(ov + 4 * u));
+        }
+      }
+    }
+    F::fwd_cols(v, tile, p, n, tw);
+    __syncthreads();
+    F::fwd_rows(v, tile, pr, nr, tw);
+#pragma unroll
+    for (int q = 0; q < R2; ++q) v[q] = fp::pscale(v[q], fp::splat(invN));
+#pragma unroll
+    for (int q = 0; q < R2; q += 2) {
+      float2 i0 = fp::fma2(v[q].re, v[q].re, fp::mul2(v[q].im, v[q].im));
+      float2 i1 = fp::fma2(v[q + 1].re, v[q + 1].re, fp::mul2(v[q + 1].im, v[q + 1].im));
+      float4* ri = rI + (q / 2) * T + tid;
+      if (k > 0) {
+        const float4 s = *ri;
+        i0 = fp::add2(make_float2(s.x, s.y), i0);
+        i1 = fp::add2(make_float2(s.z, s.w), i1);
+      }
+      *ri = make_float4(i0.x, i0.y, i1.x, i1.y);
+    }
+    if (k == M - 1) break;   // the last mode's far field stays in v
+    if (psi)
+#pragma unroll
+      for (int q = 0; q < R2; ++q)
+        psi[(size_t)k * (NN / 2) + q * T] = make_float4(v[q].re.x, v[q].re.y, v[q].im.x, v[q].im.y);
+#pragma unroll
+    for (int q = 0; q < R2; ++q) P[q] = probe_fwd(shared_mode<OPR>(a, k + 1, NN), q);
+    __syncthreads();   // the tile is free for the next mode
+  }
+
+  // ---- data term: loss and the far-field factor, on the thread's own pixels ------
+  // (a rolled loop over the units of the intensity plane: unrolled over v it
+  // would be most of the kernel's code, and ran at the speed of instruction
+  // fetches)
+  {
+    const float eps = a.eps;
+    float2 ls = make_float2(0.f, 0.f);   // rows 2pr and 2pr + 1
+    bool bad = false;
+    const bool sq = mode == MODE_LSQML_GAUSS || mode == MODE_GRAD_GAUSS;
+    auto add_loss = [&](float4 t) {
+      if (sq)
+        ls = fp::fma2(make_float2(t.z, t.w), make_float2(t.z, t.w),
+                      fp::fma2(make_float2(t.x, t.y), make_float2(t.x, t.y), ls));
+      else
+        ls = fp::add2(fp::add2(ls, make_float2(t.x, t.y)), make_float2(t.z, t.w));
+    };
+    // The pattern into the tile, one bulk copy per row (loaded straight to its
+    // threads, 32 bytes of a row per request, it took 6,000 cycles). The pitch
+    // spreads the row pairs of a warp over the banks.
+    constexpr int MP = N + 4;
+    float* mS = (float*)tile;
+    const float* meas = a.meas + (size_t)j * NN;
+    if (mode != MODE_FWD) {
+      const bool mbulk = ((uintptr_t)a.meas & 15) == 0;
+      tc::fence_async_smem();
+      __syncthreads();   // the tile is free
+      if (mbulk) {
+        if (tid == 0) tc::mbar_expect_tx(bar + 1, (uint32_t)(NN * sizeof(float)));
+        for (int r = tid; r < N; r += T) tc::bulk_g2s(mS + r * MP, meas + r * N, N * sizeof(float), bar + 1);
+      } else {
+        for (int i = tid; i < NN; i += T) mS[i / N * MP + i % N] = __ldg(meas + i);
+      }
+      if (!arrived_all(!mbulk || tc::mbar_wait(bar + 1, 0), bar + 1)) return;
+    }
+    // unit i of the intensity plane: registers 2i and 2i + 1 of v, columns c0 and c1
+    auto cols = [&](int i, int& c0, int& c1) {
+      c0 = F::far_col(nr, 2 * i);
+      c1 = F::far_col(nr, 2 * i + 1);
+    };
+#pragma unroll 1
+    for (int i = 0; i < R2 / 2; ++i) {
+      const float4 I = rI[i * T + tid];
+      int c0, c1;
+      cols(i, c0, c1);
+      if (a.ipred) {
+        float* d = a.ipred + (size_t)j * NN + (size_t)(2 * pr) * N;
+        if constexpr (F::S > 1) {   // c1 = c0 + 1, c0 even (the array is only 4-byte aligned)
+          d[c0] = I.x; d[c1] = I.z; d[N + c0] = I.y; d[N + c1] = I.w;
+        } else {
+          d[c0] = I.x; d[N + c0] = I.y; d[c1] = I.z; d[N + c1] = I.w;
+        }
+      }
+      if (mode == MODE_FWD) continue;
+      float* m = mS + 2 * pr * MP;
+      const float4 Im = make_float4(m[c0], m[MP + c0], m[c1], m[MP + c1]);
+      float4 f;
+      if (mode == MODE_VJP) {
+        bad |= !isfinite(Im.x) || !isfinite(Im.y) || !isfinite(Im.z) || !isfinite(Im.w);
+        f = make_float4(2.f * Im.x, 2.f * Im.y, 2.f * Im.z, 2.f * Im.w);
+      } else {
+        auto off = [](float x) { return !(x >= 0.f) || !isfinite(x); };
+        bad |= off(Im.x) || off(Im.y) || off(Im.z) || off(Im.w);
+        float4 t;
+        f = data_factor(mode, I, Im, eps, t);
+        add_loss(t);
+        if constexpr (N == 64) {   // kept for the upper rows' sum below
+          m[c0] = t.x; m[MP + c0] = t.y; m[c1] = t.z; m[MP + c1] = t.w;
+        }
+      }
+      rI[i * T + tid] = make_float4(f.x * invN, f.y * invN, f.z * invN, f.w * invN);
+    }
+    if (bad) atomicOr(a.status, FLAG_NONFINITE);
+    if (a.loss && mode != MODE_FWD && mode != MODE_VJP) {
+      // FP32 per row and lane (window 64: rows r and r + 32 in one sum), a
+      // tree over the lanes and over G rows, FP64 from there: the loss keeps
+      // one order of summation, whatever the packing
+      bool mine = true;
+      if constexpr (N == 64) {
+        float2* lo = (float2*)red;
+        mine = tid >= T / 2;
+        if (!mine) lo[tid] = ls;
+        __syncthreads();
+        if (mine) {
+          ls = lo[tid - T / 2];
+#pragma unroll 1
+          for (int i = 0; i < R2 / 2; ++i) {
+            int c0, c1;
+            cols(i, c0, c1);
+            const float* m = mS + 2 * pr * MP;
+            add_loss(make_float4(m[c0], m[MP + c0], m[c1], m[MP + c1]));
+          }
+        }
+        __syncthreads();
+      }
+      constexpr int G = F::G;
+#pragma unroll
+      for (int o = 16; o >= 1; o /= 2)
+        if (o != G / 2) {
+          ls.x += __shfl_down_sync(0xffffffffu, ls.x, o);
+          ls.y += __shfl_down_sync(0xffffffffu, ls.y, o);
+        }
+      const int lane = tid & 31, slots = 2 * (T / 32);   // lanes 0 and G / 2 hold G rows each
+      if ((lane & ~(G / 2)) == 0) red[(tid >> 5) * 2 + (lane != 0)] = mine ? (double)(ls.x + ls.y) : 0.0;
+      __syncthreads();
+      if (tid < 32) {
+        double s = lane < slots ? red[lane] : 0.0;
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+        if (tid == 0) atomicAdd(a.loss, s);
+      }
+    }
+    if (mode == MODE_FWD || a.loss_only) {
+      tm_release();
+      return;
+    }
+  }
+
+  // ---- back-propagation: chi_k = F^-1[fac Psi_k], g = sum_k conj(P_k) chi_k, h_k ----
+  // The modes run last to first: the far fields written last are read first,
+  // while they are still in L2.
+  float2* g_s = a.g_s + slotNN;
+  float2* h_s = a.h_s + slotNN * M;
+#pragma unroll 1
+  for (int k = M - 1; k >= 0; --k) {
+    const float2* Pk = shared_mode<OPR>(a, k, NN);
+    if (k < M - 1) {
+#pragma unroll
+      for (int q = 0; q < R2; ++q) {
+        const float4 x = psi[(size_t)k * (NN / 2) + q * T];
+        v[q] = {make_float2(x.x, x.y), make_float2(x.z, x.w)};
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < R2; q += 2) {
+      const float4 f = rI[(q / 2) * T + tid];
+      v[q] = fp::pscale(v[q], make_float2(f.x, f.y));
+      v[q + 1] = fp::pscale(v[q + 1], make_float2(f.z, f.w));
+    }
+    __syncthreads();   // the tile is free
+    F::inv_rows(v, tile, pr, nr, tw);
+    __syncthreads();
+    F::inv_cols(v, tile, p, n, tw);
+    if (k == 0) F::col_sync();   // the line's units are read: g may overwrite them
+    float4 Pr[D];   // the probe pairs, D loads ahead
+#pragma unroll
+    for (int q = 0; q < D; ++q) Pr[q] = probe_back(Pk, q);
+#pragma unroll
+    for (int qg = 0; qg < R2 / 2; ++qg) {
+      float ov[8], gv[8];
+      if constexpr (TM) {
+        if (k < M - 1)
+          tc::tmem_ld8x2_wait(tm_o() + 8 * qg, ov, tm_o() + TG + 8 * qg, gv);
+        else
+          tc::tmem_ld8_wait(tm_o() + 8 * qg, ov);
+      } else {
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+          *(float4*)(ov + 4 * u) = oS[(2 * qg + u) * T];
+          if (k < M - 1) *(float4*)(gv + 4 * u) = *(const float4*)(g_s + pix0 + (2 * qg + u) * R1 * N);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        const int q = 2 * qg + u, pix = pix0 + q * R1 * N;
+        const float4 P2 = Pr[q % D];
+        if (q + D < R2) Pr[q % D] = probe_back(Pk, q + D);
+        const float2 x0 = make_float2(v[q].re.x, v[q].im.x), x1 = make_float2(v[q].re.y, v[q].im.y);
+        float2 g0 = cmulc(make_float2(P2.x, P2.y), x0), g1 = cmulc(make_float2(P2.z, P2.w), x1);
+        if (k < M - 1) {
+          g0.x += gv[4 * u]; g0.y += gv[4 * u + 1]; g1.x += gv[4 * u + 2]; g1.y += gv[4 * u + 3];
+        }
+        const float2 h0 = cmulc(make_float2(ov[4 * u], ov[4 * u + 1]), x0);
+        const float2 h1 = cmulc(make_float2(ov[4 * u + 2], ov[4 * u + 3]), x1);
+        __stcs((float4*)(h_s + (size_t)k * NN + pix), make_float4(h0.x, h0.y, h1.x, h1.y));
+        const float4 g4 = make_float4(g0.x, g0.y, g1.x, g1.y);
+        if (!TM || k == 0) *(float4*)(g_s + pix) = g4;
+        if (k == 0) tile[F::colu(n + R1 * q, p)] = g4;   // (re, im) pairs, for the scatter
+        *(float4*)(gv + 4 * u) = g4;
+      }
+      if constexpr (TM)
+        if (k > 0) tc::tmem_st8(tm_o() + TG + 8 * qg, gv);
+    }
+    if (TM && k > 0) tc::tmem_wait_st();
+  }
+  __syncthreads();
+  const float2* gt = (const float2*)tile;
+  overlap_add<N, T, OPR>(a, slot, j, ty, tx, fy, fx, p0, (float*)rI, red,
+                         [&](int y, int x) { return gt[2 * F::colu(y, x >> 1) + (x & 1)]; });
+  tm_release();
+}
+
+template <int N, bool OPR>
+cudaError_t launch_pass1_pair(const BatchArgs& a, cudaStream_t s) {
+  constexpr size_t sm = PairSmem<N>::bytes;
+  static unsigned long long done = 0;
+  cudaError_t e = smem_optin(k_pass1_pair<N, OPR>, sm, &done);
+  if (e != cudaSuccess) return e;
+  if (a.nb <= 0) return cudaSuccess;
+  return launch_pdl(k_pass1_pair<N, OPR>, dim3(a.nb), dim3(fp::Fft<N>::T), sm, s, a);
+}
+
+}  // namespace ptycho

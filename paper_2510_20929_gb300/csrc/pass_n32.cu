@@ -1,8 +1,11 @@
 // Per-position kernels instantiated for the 32 x 32 window.
-#include "kernels.cuh"
+#include "kernels_pair.cuh"
 #include "launch.h"
 
 namespace ptycho {
-template cudaError_t launch_pass1<32>(const BatchArgs&, cudaStream_t, int);
+template <>
+cudaError_t launch_pass1<32>(const BatchArgs& a, cudaStream_t s, int) {
+  return a.opr_U ? launch_pass1_pair<32, true>(a, s) : launch_pass1_pair<32, false>(a, s);
+}
 template cudaError_t launch_pass2<32>(const Pass2Args&, cudaStream_t, int);
 }  // namespace ptycho

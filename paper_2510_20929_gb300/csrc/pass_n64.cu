@@ -1,8 +1,11 @@
 // Per-position kernels instantiated for the 64 x 64 window.
-#include "kernels.cuh"
+#include "kernels_pair.cuh"
 #include "launch.h"
 
 namespace ptycho {
-template cudaError_t launch_pass1<64>(const BatchArgs&, cudaStream_t, int);
+template <>
+cudaError_t launch_pass1<64>(const BatchArgs& a, cudaStream_t s, int) {
+  return a.opr_U ? launch_pass1_pair<64, true>(a, s) : launch_pass1_pair<64, false>(a, s);
+}
 template cudaError_t launch_pass2<64>(const Pass2Args&, cudaStream_t, int);
 }  // namespace ptycho
