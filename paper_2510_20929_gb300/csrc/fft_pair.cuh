@@ -155,6 +155,26 @@ template <int DIR> struct PDft<16, DIR> {
   }
 };
 
+// The twiddles of fft.cuh (W^(n k), k = 1..R2-1: four from the table, the rest
+// as products) for lane indices n and n + 1, packed.
+template <int R2>
+__device__ __forceinline__ void pair_twiddles(C2 (&t)[R2], const float2* tw, int n) {
+  constexpr int L4 = R2 - 1 < 4 ? R2 - 1 : 4;
+#pragma unroll
+  for (int k = 1; k <= L4; ++k) {
+    const float2 a = tw[n * (R2 + 1) + k], b = tw[(n + 1) * (R2 + 1) + k];
+    t[k] = {make_float2(a.x, b.x), make_float2(a.y, b.y)};
+  }
+  auto mul = [](C2 a, C2 b) -> C2 {
+    return {fma2(a.re, b.re, neg2(mul2(a.im, b.im))), fma2(a.re, b.im, mul2(a.im, b.re))};
+  };
+#pragma unroll
+  for (int k = 5; k < R2; ++k) {
+    const int a = k & ~3, b = k & 3;
+    t[k] = b == 0 ? mul(t[a - 4], t[4]) : mul(t[a], t[b]);
+  }
+}
+
 // Line split (that of fft.cuh) and the unit maps' XOR terms. By columns a
 // quarter warp covers 8 consecutive line pairs of one lane index n; by rows 8
 // line pairs (R1 = 4), or 4 line pairs of two n that differ in bit 0 (R1 = 8).
@@ -222,24 +242,6 @@ struct Fft {
   __device__ __forceinline__ static void twiddles(float2 (&t)[R2], const float2* tw, int n) {
     Fft2<N>::twiddles(t, tw, n);
   }
-  // the same for lane indices n and n + 1, packed
-  __device__ __forceinline__ static void twiddles2(C2 (&t)[R2], const float2* tw, int n) {
-    constexpr int L4 = R2 - 1 < 4 ? R2 - 1 : 4;
-#pragma unroll
-    for (int k = 1; k <= L4; ++k) {
-      const float2 a = tw[n * (R2 + 1) + k], b = tw[(n + 1) * (R2 + 1) + k];
-      t[k] = {make_float2(a.x, b.x), make_float2(a.y, b.y)};
-    }
-    auto mul = [](C2 a, C2 b) -> C2 {
-      return {fma2(a.re, b.re, neg2(mul2(a.im, b.im))), fma2(a.re, b.im, mul2(a.im, b.re))};
-    };
-#pragma unroll
-    for (int k = 5; k < R2; ++k) {
-      const int a = k & ~3, b = k & 3;
-      t[k] = b == 0 ? mul(t[a - 4], t[4]) : mul(t[a], t[b]);
-    }
-  }
-
   // Forward, first pass: columns. In: v[n2] = pixels (n + R1 n2, 2p), (.., 2p + 1).
   // Leaves the half-transformed tile in row units.
   __device__ __forceinline__ static void fwd_cols(C2 (&v)[R2], float4* tile, int p, int n, const float2* tw) {
@@ -314,7 +316,7 @@ struct Fft {
     for (int k2 = 0; k2 < R2; ++k2) v[k2] = get(tile, at(rb, colu(0, R1 / 2 * k2)));
     {
       C2 t[R2];
-      twiddles2(t, tw, 2 * m);
+      pair_twiddles<R2>(t, tw, 2 * m);
 #pragma unroll
       for (int k = 1; k < R2; ++k) v[k] = pmulc(v[k], t[k]);
     }

@@ -98,20 +98,20 @@ __device__ __forceinline__ void fft2_inverse(float2* tile, const float2* tw, In&
   }
 }
 
-// S_j^T of an N x N patch onto its (N+1)^2 object tile, evaluated separably:
+// S_j^T of a patch of LR x N pixels (the whole patch, or a band of its rows)
+// onto its (LR+1) x (N+1) object tile, evaluated separably:
 // h_y(x) = (1-fx) p(y, x) + fx p(y, x-1) and out(y, x) = (1-fy) h_y(x) + fy h_{y-1}(x),
-// with p = 0 outside the patch. A thread owns one of the tile columns 0 .. N-1
-// and a run of rows (lanes of a warp emit consecutive x, so the atomics
-// coalesce; T / N runs keep every thread busy), four rows of loads in flight
-// (one at a time the walk took 27,000 cycles of a 512-thread CTA at N = 128);
-// the tile's last column follows, a row per thread. `load(y, x)` returns the
-// patch value as a float4 (unused components zero), `emit(y, x, v)` consumes
-// the tile value.
-template <int N, int T, class Load, class Emit>
+// with p = 0 outside. A thread owns one of the tile columns 0 .. N-1 and a run
+// of rows (lanes of a warp emit consecutive x, so the atomics coalesce; the
+// runs keep every thread busy), four rows of loads in flight (one at a time
+// the walk took 27,000 cycles of a 512-thread CTA at N = 128); the tile's last
+// column follows, a row per thread. `load(y, x)` returns the patch value as a
+// float4 (unused components zero), `emit(y, x, v)` consumes the tile value.
+template <int N, int LR, int T, class Load, class Emit>
 __device__ __forceinline__ void bilinear_scatter(float fy, float fx, Load&& load, Emit&& emit) {
-  constexpr int N1 = N + 1, CH = 4;
-  constexpr int SEG = T / N > 0 ? T / N : 1;
-  constexpr int RS = (N1 + SEG - 1) / SEG;
+  constexpr int L1 = LR + 1, CH = 4;
+  constexpr int SEG = T / N > 0 ? T / N : (N % T != 0 && 2 * N % T == 0) ? 2 : 1;
+  constexpr int RS = (L1 + SEG - 1) / SEG;
   const float gx = 1.f - fx, gy = 1.f - fy;
   const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
   auto lerp = [](float wa, float4 a, float wb, float4 b) {   // wa a + wb b
@@ -119,9 +119,9 @@ __device__ __forceinline__ void bilinear_scatter(float fy, float fx, Load&& load
                        fmaf(wa, a.w, wb * b.w));
   };
   for (int item = threadIdx.x; item < N * SEG; item += T) {
-    const int y0 = item / N * RS, x = item % N, y1 = min(N1, y0 + RS);
+    const int y0 = item / N * RS, x = item % N, y1 = min(L1, y0 + RS);
     auto rowh = [&](int y) {
-      return lerp(fx, (y < N && x > 0) ? load(y, x - 1) : zero, gx, y < N ? load(y, x) : zero);
+      return lerp(fx, (y < LR && x > 0) ? load(y, x - 1) : zero, gx, y < LR ? load(y, x) : zero);
     };
     float4 hp = y0 > 0 ? rowh(y0 - 1) : zero;
     for (int y = y0; y < y1; y += CH) {
@@ -135,8 +135,8 @@ __device__ __forceinline__ void bilinear_scatter(float fy, float fx, Load&& load
       }
     }
   }
-  for (int y = threadIdx.x; y < N1; y += T) {
-    const float4 a = y < N ? load(y, N - 1) : zero, b = y > 0 ? load(y - 1, N - 1) : zero;
+  for (int y = threadIdx.x; y < L1; y += T) {
+    const float4 a = y < LR ? load(y, N - 1) : zero, b = y > 0 ? load(y - 1, N - 1) : zero;
     emit(y, N, lerp(gy, lerp(fx, a, 0.f, zero), fy, lerp(fx, b, 0.f, zero)));
   }
 }
@@ -144,23 +144,24 @@ __device__ __forceinline__ void bilinear_scatter(float fy, float fx, Load&& load
 // The end of the per-position pass: g_j (read with getg(y, x), in shared
 // memory; every thread's writes are in flight on entry) and, for LSQML, the
 // probe intensity are scattered into the object frame, then the position
-// gradient or the sums of the position step are reduced. `spS` is N * N floats
-// of shared memory that are free on entry.
-template <int N, int T, bool OPR, class Get>
-__device__ __forceinline__ void overlap_add(const BatchArgs& a, int slot, int j, int ty, int tx, float fy, float fx,
-                                            const float2* p0, float* spS, double* red, Get&& getg) {
-  constexpr int NN = N * N;
-  const int tid = threadIdx.x, mode = a.mode;
+// gradient or the sums of the position step are reduced. The CTA holds rows
+// y0 .. y0 + LR - 1 of the patch (getg's y counts from y0). `spS` is LR * N
+// floats of shared memory that are free on entry.
+template <int N, int LR, int T, bool OPR, class Get>
+__device__ __forceinline__ void overlap_add(const BatchArgs& a, int slot, int j, int y0, int ty, int tx, float fy,
+                                            float fx, const float2* p0, float* spS, double* red, Get&& getg) {
+  constexpr int LNN = LR * N;
+  const int tid = threadIdx.x, mode = a.mode, pb = y0 * N;
   const bool lsqml = (mode == MODE_LSQML_GAUSS || mode == MODE_LSQML_POISSON);
   // LSQML: the probe intensity sum_k |P_k|^2 of every pixel into shared memory
   // (the intensity/factor plane is free by now), so that the scatter's row walk
   // waits on shared memory rather than on L2
   if (lsqml) {
 #pragma unroll 2
-    for (int p = 4 * tid; p < NN; p += 4 * T) {
-      float4 v = __ldg((const float4*)(a.Sp + p));
+    for (int p = 4 * tid; p < LNN; p += 4 * T) {
+      float4 v = __ldg((const float4*)(a.Sp + pb + p));
       if (OPR && p0) {
-        const float4 q0 = *(const float4*)(p0 + p), q1 = *(const float4*)(p0 + p + 2);
+        const float4 q0 = *(const float4*)(p0 + pb + p), q1 = *(const float4*)(p0 + pb + p + 2);
         v.x += q0.x * q0.x + q0.y * q0.y; v.y += q0.z * q0.z + q0.w * q0.w;
         v.z += q1.x * q1.x + q1.y * q1.y; v.w += q1.z * q1.z + q1.w * q1.w;
       }
@@ -169,23 +170,25 @@ __device__ __forceinline__ void overlap_add(const BatchArgs& a, int slot, int j,
   }
   __syncthreads();
   if (lsqml) {
-    bilinear_scatter<N, T>(
+    bilinear_scatter<N, LR, T>(
         fy, fx,
         [&](int y, int x) {
           const float2 g = getg(y, x);
           return make_float4(g.x, g.y, spS[y * N + x], 0.f);
         },
         [&](int y, int x, float4 v) {
-          atomicAdd(a.acc + (size_t)(ty + y) * a.W + (tx + x), make_float4(v.x, v.y, v.z, 0.f));
+          atomicAdd(a.acc + (size_t)(ty + y0 + y) * a.W + (tx + x), make_float4(v.x, v.y, v.z, 0.f));
         });
   } else {
-    bilinear_scatter<N, T>(
+    bilinear_scatter<N, LR, T>(
         fy, fx,
         [&](int y, int x) {
           const float2 g = getg(y, x);
           return make_float4(g.x, g.y, 0.f, 0.f);
         },
-        [&](int y, int x, float4 v) { atomicAdd(a.gobj + (size_t)(ty + y) * a.W + (tx + x), make_float2(v.x, v.y)); });
+        [&](int y, int x, float4 v) {
+          atomicAdd(a.gobj + (size_t)(ty + y0 + y) * a.W + (tx + x), make_float2(v.x, v.y));
+        });
   }
 
   // ---- position gradient through the bilinear weights (gradient modes), or the
@@ -193,9 +196,9 @@ __device__ __forceinline__ void overlap_add(const BatchArgs& a, int slot, int j,
   if (a.gpos || a.possum) {
     const bool ls = a.possum != nullptr;
     float gy = 0.f, gx = 0.f, a11 = 0.f, a12 = 0.f, a22 = 0.f;
-    for (int p = tid; p < NN; p += T) {
+    for (int p = tid; p < LNN; p += T) {
       const int r = p / N, c = p % N;
-      const float2* o = a.obj + (size_t)(ty + r) * a.W + (tx + c);
+      const float2* o = a.obj + (size_t)(ty + y0 + r) * a.W + (tx + c);
       const float2 O00 = __ldg(o), O01 = __ldg(o + 1), O10 = __ldg(o + a.W), O11 = __ldg(o + a.W + 1);
       const float2 dy = make_float2((1.f - fx) * (O10.x - O00.x) + fx * (O11.x - O01.x),
                                     (1.f - fx) * (O10.y - O00.y) + fx * (O11.y - O01.y));
@@ -205,7 +208,7 @@ __device__ __forceinline__ void overlap_add(const BatchArgs& a, int slot, int j,
       gy += g.x * dy.x + g.y * dy.y;  // Re(conj(g) dy)
       gx += g.x * dx.x + g.y * dx.y;
       if (ls) {   // sum_k abs(P_k)^2 times the derivative products
-        const float sp = __ldg(a.Sp + p) + ((OPR && p0) ? cabs2(p0[p]) : 0.f);
+        const float sp = __ldg(a.Sp + pb + p) + ((OPR && p0) ? cabs2(p0[pb + p]) : 0.f);
         a11 = fmaf(sp, cabs2(dy), a11);
         a12 = fmaf(sp, dy.x * dx.x + dy.y * dx.y, a12);
         a22 = fmaf(sp, cabs2(dx), a22);
@@ -220,8 +223,8 @@ __device__ __forceinline__ void overlap_add(const BatchArgs& a, int slot, int j,
       double v[2] = {(double)gy, (double)gx};
       block_sum<2>(v, red);
       if (tid == 0) {
-        a.gpos[2 * j] += (float)v[0];
-        a.gpos[2 * j + 1] += (float)v[1];
+        atomicAdd(a.gpos + 2 * j, (float)v[0]);
+        atomicAdd(a.gpos + 2 * j + 1, (float)v[1]);
       }
     }
   }
@@ -502,7 +505,7 @@ __global__ void __launch_bounds__(T, 1) k_pass1(BatchArgs a) {
     const float4 g2 = *(const float4*)(g_s + np.pix(q));
     store_pair(tile, np.phys(q), make_float2(g2.x, g2.y), make_float2(g2.z, g2.w));
   }
-  overlap_add<N, T, OPR>(a, slot, j, ty, tx, fy, fx, p0, rI, red, [&](int y, int x) { return tile[tix<N>(y, x)]; });
+  overlap_add<N, N, T, OPR>(a, slot, j, 0, ty, tx, fy, fx, p0, rI, red, [&](int y, int x) { return tile[tix<N>(y, x)]; });
 }
 
 

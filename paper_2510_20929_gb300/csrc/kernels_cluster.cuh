@@ -1,5 +1,5 @@
-// Per-position pass for windows larger than one CTA's shared memory, on a
-// cluster of Q CTAs (N = 256: Q = 8; N = 192: Q = 6).
+// 2-D transforms of the multislice passes for windows larger than one CTA's
+// shared memory, on a cluster of Q CTAs (N = 256: Q = 8; N = 192: Q = 6).
 //
 // The N x N complex tile is shared by the cluster: in the spatial domain CTA q
 // holds the LR = N / Q rows LR q .. LR q + LR - 1. The 2-D DFT runs as
@@ -15,12 +15,6 @@
 // same transpose back, row inverses). Each CTA reads (Q-1)/Q of its tile from
 // the other CTAs once per transform (a Q-point DFT across the cluster would
 // read every element from every CTA: Q times that).
-// Everything else (patch gather, back-propagation, scatter, the position
-// gradient) follows the single-CTA k_pass1 on the CTA's own spatial rows; the
-// far-field loops (intensity, data term, the inverse's input) walk the CTA's
-// columns with consecutive threads on consecutive columns (freq_index), so
-// that the measured intensities and the predicted ones are read and written
-// coalesced in their natural [k_y][k_x] order.
 #pragma once
 #include <cooperative_groups.h>
 
@@ -191,290 +185,6 @@ __device__ __forceinline__ void inv2d(cg::cluster_group& cluster, float2* tile, 
   transpose_exchange<C>(cluster, tile, q);
   row_pass<C, false>(tile, twr);
   __syncthreads();
-}
-
-template <class C, bool OPR>
-__global__ void __launch_bounds__(C::T, C::MINB) k_pass1_cluster(BatchArgs a) {
-  constexpr int N = C::N, Q = C::Q, T = C::T, LR = C::LR, NN = C::NN, LNN = C::LNN;
-  constexpr int NAT_STEPS = C::NAT_STEPS;
-  static_assert(LNN % (2 * T) == 0, "data-term loop takes two elements per step");
-  using SM = typename C::Smem;
-  cg::cluster_group cluster = cg::this_cluster();
-  extern __shared__ __align__(16) unsigned char smem[];
-  double* red = (double*)(smem + SM::red);
-  float2* tile = (float2*)(smem + SM::tile);
-  float2* twr = (float2*)(smem + SM::twr);
-  float* rI = (float*)(smem + SM::rI);
-  constexpr int RP = SM::RP;
-
-  const int q = (int)cluster.block_rank();
-  const int slot = blockIdx.x / Q;
-  const int tid = threadIdx.x;
-  const int e = a.b0 + slot;
-  const int j = a.order ? a.order[e] : e;
-  int ty = 0, tx = 0;
-  float fy = 0.f, fx = 0.f;
-  bool ok = (j >= 0 && j < a.J);
-  if (ok) ok = tile_of(a.pos[2 * j], a.pos[2 * j + 1], N, a.H, a.W, ty, tx, fy, fx);
-  if (!ok) {   // the same decision in every CTA of the cluster
-    if (tid == 0 && q == 0) {
-      atomicOr(a.status, FLAG_BOUNDS);
-      if (a.valid) a.valid[slot] = 0;
-    }
-    return;
-  }
-  if (tid == 0 && q == 0 && a.valid) a.valid[slot] = 1;
-  make_line_twiddles<N, C::RR1, C::RR2>(twr);
-
-  const int M = a.M;
-  const float invN = 1.0f / (float)N;
-  const size_t slotNN = (size_t)slot * NN;
-  float* wj = (float*)(red + 128);   // this position's eigenmode weights (OPR)
-  float2* p0 = (OPR && a.p0_s) ? a.p0_s + slotNN : nullptr;
-  if (OPR) {
-    if (tid < a.K) wj[tid] = a.opr_w[(size_t)j * a.K + tid];
-    __syncthreads();
-  }
-  float2* psi_s = a.psi_s ? a.psi_s + slotNN * M : nullptr;
-  float2* o_s = a.o_s ? a.o_s + slotNN : nullptr;
-  const int rowbase = LR * q;   // first spatial row of this CTA
-
-  // ---- forward model --------------------------------------------------------------
-#pragma unroll 1
-  for (int k = 0; k < M; ++k) {
-    const float2* Pk = shared_mode<OPR>(a, k, NN);
-    __syncthreads();
-#pragma unroll 2
-    for (int s = 0; s < NAT_STEPS; ++s) {
-      const int pl = 2 * tid + 2 * T * s, r = pl / N, c = pl % N;
-      const int p = (rowbase + r) * N + c;
-      float2 o0, o1;
-      if (k == 0 || !o_s) {
-        bilinear2(a.obj, a.W, ty + rowbase + r, tx + c, fy, fx, o0, o1);
-        if (k == 0 && o_s) *(float4*)(o_s + p) = make_float4(o0.x, o0.y, o1.x, o1.y);
-      } else {
-        const float4 o2 = *(const float4*)(o_s + p);
-        o0 = make_float2(o2.x, o2.y);
-        o1 = make_float2(o2.z, o2.w);
-      }
-      float4 P2;
-      if (!OPR || Pk) {
-        P2 = __ldg((const float4*)(Pk + p));
-      } else {   // relaxed primary mode of this position
-        P2 = opr_pair(a.opr_U, wj, a.K, NN, p);
-        if (p0) *(float4*)(p0 + p) = P2;
-      }
-      store_pair(tile, C::tix(r, c), cmul(make_float2(P2.x, P2.y), o0), cmul(make_float2(P2.z, P2.w), o1));
-    }
-    __syncthreads();
-    fwd2d<C>(cluster, tile, twr, q);
-    // far field of this CTA's columns: the intensity sum and (gradient and
-    // LSQML modes) the far field itself, in a CTA-private scratch order
-#pragma unroll 4
-    for (int e = tid; e < LNN; e += T) {
-      int x, ky;
-      C::freq_index(e, x, ky);
-      const float2 X = cscale(tile[C::tix(x, ky)], invN);
-      float* ri = rI + x * RP + ky;
-      *ri = (k == 0) ? cabs2(X) : *ri + cabs2(X);
-      if (psi_s) psi_s[(size_t)k * NN + (size_t)q * LNN + e] = X;
-    }
-  }
-
-  // ---- data term (this CTA's far-field columns) ------------------------------------
-  const int mode = a.mode;
-  const float eps = a.eps;
-  const float* meas = a.meas + (size_t)j * NN;
-  float lsum = 0.f;
-  bool bad = false;
-#pragma unroll 1
-  for (int e0 = tid; e0 < LNN; e0 += 2 * T) {
-#pragma unroll
-    for (int u = 0; u < 2; ++u) {
-      const int e = e0 + u * T;
-      int x, ky;
-      C::freq_index(e, x, ky);
-      const int pix = ky * N + LR * q + x;
-      float* ri = rI + x * RP + ky;
-      const float I = *ri;
-      if (a.ipred) a.ipred[(size_t)j * NN + pix] = I;
-      if (mode == MODE_FWD) continue;
-      const float Im = __ldg(meas + pix);
-      float fac;
-      if (mode == MODE_VJP) {
-        bad |= !isfinite(Im);
-        fac = 2.f * Im;
-      } else {
-        bad |= !(Im >= 0.f) || !isfinite(Im);
-        const float Ie = I + eps;
-        if (mode == MODE_LSQML_GAUSS || mode == MODE_GRAD_GAUSS) {
-          const float sIe = sqrtf(Ie), sIm = sqrtf(Im);
-          const float d = sIe - sIm;
-          lsum = fmaf(d, d, lsum);
-          const float rho = sIm / sIe;
-          fac = (mode == MODE_LSQML_GAUSS) ? rho - 1.f : 2.f * (1.f - rho);
-        } else {
-          lsum += I - Im * logf(Ie);
-          const float qq = Im / Ie;
-          fac = (mode == MODE_LSQML_POISSON) ? 0.5f * (qq - 1.f) : 2.f * (1.f - qq);
-        }
-      }
-      *ri = fac * invN;
-    }
-  }
-  if (bad) atomicOr(a.status, FLAG_NONFINITE);
-  if (a.loss && mode != MODE_FWD && mode != MODE_VJP) {
-    double v[1] = {(double)lsum};
-    block_sum<1>(v, red);
-    if (tid == 0) atomicAdd(a.loss, v[0]);
-  }
-  if (mode == MODE_FWD || a.loss_only) {
-    cluster.sync();   // no CTA leaves while another may still read its tile
-    return;
-  }
-
-  // ---- back-propagation -------------------------------------------------------------
-  // modes last to first: the far fields written last are read first (L2)
-  float2* g_s = a.g_s + slotNN;
-  float2* h_s = a.h_s + slotNN * M;
-#pragma unroll 1
-  for (int k = M - 1; k >= 0; --k) {
-    const float2* Pk = shared_mode<OPR>(a, k, NN);
-    __syncthreads();
-#pragma unroll 4
-    for (int e = tid; e < LNN; e += T) {
-      int x, ky;
-      C::freq_index(e, x, ky);
-      tile[C::tix(x, ky)] = cscale(psi_s[(size_t)k * NN + (size_t)q * LNN + e], rI[x * RP + ky]);
-    }
-    __syncthreads();
-    inv2d<C>(cluster, tile, twr, q);
-#pragma unroll 2
-    for (int s = 0; s < NAT_STEPS; ++s) {
-      const int pl = 2 * tid + 2 * T * s, r = pl / N, c = pl % N;
-      const int p = (rowbase + r) * N + c;
-      float2 x0, x1;
-      load_pair(tile, C::tix(r, c), x0, x1);
-      const float4 P2 = (!OPR || Pk) ? __ldg((const float4*)(Pk + p)) : *(const float4*)(p0 + p);
-      const float4 o2 = *(const float4*)(o_s + p);
-      const float2 g0 = cmulc(make_float2(P2.x, P2.y), x0), g1 = cmulc(make_float2(P2.z, P2.w), x1);
-      float4 gv = make_float4(g0.x, g0.y, g1.x, g1.y);
-      if (k < M - 1) {
-        const float4 gp = *(const float4*)(g_s + p);
-        gv = make_float4(gv.x + gp.x, gv.y + gp.y, gv.z + gp.z, gv.w + gp.w);
-      }
-      *(float4*)(g_s + p) = gv;
-      if (k == 0)   // the finished g of this CTA's rows also into its (now free) tile
-        store_pair(tile, C::tix(r, c), make_float2(gv.x, gv.y), make_float2(gv.z, gv.w));
-      const float2 h0 = cmulc(make_float2(o2.x, o2.y), x0), h1 = cmulc(make_float2(o2.z, o2.w), x1);
-      __stcs((float4*)(h_s + (size_t)k * NN + p), make_float4(h0.x, h0.y, h1.x, h1.y));
-    }
-  }
-  const bool lsqml = (mode == MODE_LSQML_GAUSS || mode == MODE_LSQML_POISSON);
-  // LSQML: the probe intensity of this CTA's rows into the free intensity/factor
-  // plane, so that the scatter reads its own rows from shared memory
-  float* spS = rI;
-  if (lsqml) {
-    static_assert(LR * RP >= LNN, "room for the probe intensity");
-    for (int e = 4 * tid; e < LNN; e += 4 * T) {
-      const int p = rowbase * N + e;
-      float4 v = __ldg((const float4*)(a.Sp + p));
-      if (OPR && p0) {
-        const float4 q0 = *(const float4*)(p0 + p), q1 = *(const float4*)(p0 + p + 2);
-        v.x += q0.x * q0.x + q0.y * q0.y; v.y += q0.z * q0.z + q0.w * q0.w;
-        v.z += q1.x * q1.x + q1.y * q1.y; v.w += q1.z * q1.z + q1.w * q1.w;
-      }
-      *(float4*)(spS + e) = v;
-    }
-  }
-  // every CTA's rows of g are written (the scatter reads one row of the neighbour)
-  cluster.sync();
-
-  // ---- scatter S_j^T g (and the illumination), this CTA's rows (+ row N) ----------
-  {
-    const int y0 = rowbase, y1 = rowbase + LR + (q == Q - 1 ? 1 : 0);
-    constexpr int N1 = N + 1;
-    const float gx = 1.f - fx, gy = 1.f - fy;
-    auto loadg = [&](int y, int x) {
-      if (y >= y0 && y < y0 + LR) {   // this CTA's rows: shared memory
-        const float2 g = tile[C::tix(y - y0, x)];
-        return make_float4(g.x, g.y, lsqml ? spS[(y - y0) * N + x] : 0.f, 0.f);
-      }
-      const float2 g = g_s[y * N + x];   // the row above, from the neighbour's rows in L2
-      const float sp = lsqml ? __ldg(a.Sp + y * N + x) + ((OPR && p0) ? cabs2(p0[y * N + x]) : 0.f) : 0.f;
-      return make_float4(g.x, g.y, sp, 0.f);
-    };
-    auto hrow = [&](int y, int x) {
-      float4 h = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (y >= 0 && y < N) {
-        if (x < N) {
-          const float4 v = loadg(y, x);
-          h = make_float4(gx * v.x, gx * v.y, gx * v.z, 0.f);
-        }
-        if (x > 0) {
-          const float4 v = loadg(y, x - 1);
-          h.x = fmaf(fx, v.x, h.x); h.y = fmaf(fx, v.y, h.y); h.z = fmaf(fx, v.z, h.z);
-        }
-      }
-      return h;
-    };
-    constexpr int SEG = T / N1 > 0 ? T / N1 : 1;      // row segments of the CTA's rows
-    const int rows = y1 - y0, rs = (rows + SEG - 1) / SEG;
-    for (int item = tid; item < N1 * SEG; item += T) {
-      const int sg = item / N1, x = item % N1;
-      const int ya = y0 + sg * rs, yb = min(y1, ya + rs);
-      if (ya >= yb) continue;
-      float4 hp = hrow(ya - 1, x);
-      for (int y = ya; y < yb; ++y) {
-        const float4 hc = hrow(y, x);
-        const float4 v = make_float4(fmaf(gy, hc.x, fy * hp.x), fmaf(gy, hc.y, fy * hp.y),
-                                     fmaf(gy, hc.z, fy * hp.z), 0.f);
-        const size_t oi = (size_t)(ty + y) * a.W + (tx + x);
-        if (lsqml) atomicAdd(a.acc + oi, v);
-        else atomicAdd(a.gobj + oi, make_float2(v.x, v.y));
-        hp = hc;
-      }
-    }
-  }
-
-  // ---- position gradient (gradient modes) or the least-squares position-step
-  // ---- sums (LSQML position correction), this CTA's rows ----------------------------
-  if (a.gpos || a.possum) {
-    const bool ls = a.possum != nullptr;
-    float gyv = 0.f, gxv = 0.f, a11 = 0.f, a12 = 0.f, a22 = 0.f;
-    for (int pl = tid; pl < LNN; pl += T) {
-      const int r = rowbase + pl / N, c = pl % N;
-      const float2* o = a.obj + (size_t)(ty + r) * a.W + (tx + c);
-      const float2 O00 = __ldg(o), O01 = __ldg(o + 1), O10 = __ldg(o + a.W), O11 = __ldg(o + a.W + 1);
-      const float2 dy = make_float2((1.f - fx) * (O10.x - O00.x) + fx * (O11.x - O01.x),
-                                    (1.f - fx) * (O10.y - O00.y) + fx * (O11.y - O01.y));
-      const float2 dx = make_float2((1.f - fy) * (O01.x - O00.x) + fy * (O11.x - O10.x),
-                                    (1.f - fy) * (O01.y - O00.y) + fy * (O11.y - O10.y));
-      const float2 g = g_s[r * N + c];
-      gyv += g.x * dy.x + g.y * dy.y;
-      gxv += g.x * dx.x + g.y * dx.y;
-      if (ls) {
-        const int p = r * N + c;
-        const float sp = __ldg(a.Sp + p) + ((OPR && p0) ? cabs2(p0[p]) : 0.f);
-        a11 = fmaf(sp, cabs2(dy), a11);
-        a12 = fmaf(sp, dy.x * dx.x + dy.y * dx.y, a12);
-        a22 = fmaf(sp, cabs2(dx), a22);
-      }
-    }
-    if (ls) {
-      double v[5] = {(double)a11, (double)a12, (double)a22, (double)gyv, (double)gxv};
-      block_sum<5>(v, red);
-      if (tid == 0)
-        for (int q = 0; q < 5; ++q) atomicAdd(a.possum + (size_t)slot * 5 + q, v[q]);
-    } else {
-      double v[2] = {(double)gyv, (double)gxv};
-      block_sum<2>(v, red);
-      if (tid == 0) {
-        atomicAdd(a.gpos + 2 * j, (float)v[0]);
-        atomicAdd(a.gpos + 2 * j + 1, (float)v[1]);
-      }
-    }
-  }
 }
 
 }  // namespace cl

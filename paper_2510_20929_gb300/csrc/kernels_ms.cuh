@@ -346,7 +346,7 @@ __global__ void __launch_bounds__(T, 1) k_pass1_ms(MsArgs a) {
     if (lsqml) {   // S_j^T of the slice's direction numerator and of its illumination
       float4* acc = a.acc + s * HW;
       const float* wsl = s > 0 ? a.w_s + (slotNN * (S - 1) + (size_t)(s - 1) * NN) : a.Sp;
-      bilinear_scatter<N, T>(
+      bilinear_scatter<N, N, T>(
           fy, fx,
           [&](int y, int x) {
             const float2 g = tile[tix<N>(y, x)];
@@ -358,7 +358,7 @@ __global__ void __launch_bounds__(T, 1) k_pass1_ms(MsArgs a) {
     }
     if (a.gobj) {
       float2* gplane = a.gobj + s * HW;
-      bilinear_scatter<N, T>(
+      bilinear_scatter<N, N, T>(
           fy, fx,
           [&](int y, int x) {
             const float2 g = tile[tix<N>(y, x)];

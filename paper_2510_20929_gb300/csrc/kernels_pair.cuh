@@ -1,8 +1,9 @@
-// The per-position pass of the windows one CTA holds whole (32, 64, 128), on
-// the packed line-pair transforms of fft_pair.cuh. It computes what k_pass1
-// (kernels.cuh) describes; what differs is where the data lives:
-//   * every thread owns the same pixel pairs (rows n + R1 q, columns 2p,
-//     2p + 1) when a mode's exit wave is built and when its chi comes back, so
+// The per-position pass on the packed line-pair transforms: windows 32, 64 and
+// 128 in one CTA (fft_pair.cuh), 192 and 256 on a cluster of CTAs with 32 rows
+// each (fft_cluster.cuh). It computes what k_pass1 (kernels.cuh) describes;
+// what differs is where the data lives:
+//   * every thread owns the same pixel pairs (two neighbours of one row, or, on
+//     a cluster, of one column) when a mode's exit wave is built and when its chi comes back, so
 //     psi_jk goes from the loads straight into the column transform's
 //     registers and chi_jk from the registers into g and h, with no pass over
 //     the tile on either side;
@@ -12,45 +13,92 @@
 //     access a whole coalesced run), and the last mode's far field stays in
 //     registers through the data term into its inverse transform;
 //   * the patch o_j and the running g_j of the thread's pixels stay in tensor
-//     memory (windows 64 and 128: 8 R2 columns of the thread's TMEM lane).
+//     memory (windows 64 and up: 8 NP columns of the thread's TMEM lane).
 // What bounds it: the transforms (about half the cycles; shared-memory
 // wavefronts and issue slots), then the rate of L2 requests of the probe
 // loads, the far-field scratch and the h stores (about 2.8 cycles per 128-byte
 // request when all SMs stream), with one CTA of 512 threads filling an SM at
-// window 128. Straight-line code that a CTA runs once costs instruction
+// window 128, and on the cluster windows the waits for the cluster. Straight-line code that a CTA runs once costs instruction
 // fetches, so loops over a thread's pixels stay rolled where v is not indexed.
-// Measured on GB300 against the one-line-per-lane-group pass it replaced (per
-// launch): window 128, 5 modes, 256 positions 287 -> 249 us (1 mode: 101 -> 92,
+// Measured on GB300 against the one-line-per-lane-group passes it replaced (per
+// launch): window 256, 8 modes, 256 positions 2423 -> 1705 us, 1 mode 496 ->
+// 342; window 192, 4 modes 986 -> 673, 1 mode 406 -> 293; window 128, 5 modes, 256 positions 287 -> 249 us (1 mode: 101 -> 92,
 // 1024 positions 1002 -> 860); window 64, 4 modes, 256 positions 63 -> 51,
 // 1216 positions 227 -> 166, 1 mode, 16 positions 24.7 -> 20.7; window 32, 4
 // modes, 2000 positions 116 -> 72.
 #pragma once
+#include <type_traits>
+
 #include "kernels.cuh"
-#include "fft_pair.cuh"
+#include "fft_cluster.cuh"
 
 namespace ptycho {
 
-// CTAs per SM: shared memory at window 128; the register budget (80 and 128 a
-// thread) at windows 64 and 32.
-template <int N> struct PairCtas;
-template <> struct PairCtas<32> { static constexpr int n = 8; };
-template <> struct PairCtas<64> { static constexpr int n = 3; };
-template <> struct PairCtas<128> { static constexpr int n = 1; };
+// One thread's view of a window held by one CTA (ClFft is that of a cluster):
+// pixel pair i = (row(i), col(i)) and the next column; far field of register i
+// at rows far_y(i), far_y(i) + 1 of column far_x(i).
+template <int N_>
+struct OneCta {
+  using F = fp::Fft<N_>;
+  static constexpr int N = N_, R1 = F::R1, NP = F::R2, LR = N, Q = 1, T = F::T, TW = Twiddles<N>::COUNT;
+  static constexpr bool VERT = false;
+  __device__ __forceinline__ static void fill_twiddles(float2* tw) { make_twiddles<N>(tw); }
+  float4* tile;
+  const float2* tw;
+  int p, n, pr, nr;
+  __device__ __forceinline__ OneCta(float4* tile_, const float2* tw_)
+      : tile(tile_), tw(tw_), p(F::col_pair()), n(F::col_lane()), pr(F::row_pair()), nr(F::row_lane()) {}
+  static constexpr int q = 0;
+  __device__ __forceinline__ int row(int i) const { return n + R1 * i; }
+  __device__ __forceinline__ int col(int) const { return 2 * p; }
+  __device__ __forceinline__ int far_y(int) const { return 2 * pr; }
+  __device__ __forceinline__ int far_x(int i) const { return F::far_col(nr, i); }
+  __device__ __forceinline__ static void pixel_sync() { F::col_sync(); }
+  __device__ __forceinline__ void forward(fp::C2 (&v)[NP]) const {
+    F::fwd_cols(v, tile, p, n, tw);
+    __syncthreads();
+    F::fwd_rows(v, tile, pr, nr, tw);
+  }
+  __device__ __forceinline__ void inverse(fp::C2 (&v)[NP]) const {
+    F::inv_rows(v, tile, pr, nr, tw);
+    __syncthreads();
+    F::inv_cols(v, tile, p, n, tw);
+  }
+  // unit that holds pixel pair i once the line's lanes have read theirs, and
+  // the 8-byte slot of local pixel (y, x) in those units
+  __device__ __forceinline__ int pixel_unit(int i) const { return F::colu(row(i), p); }
+  __device__ __forceinline__ static int pixel_slot(int y, int x) { return 2 * F::colu(y, x >> 1) + (x & 1); }
+};
 
-template <int N>
+// Launch shape: CTAs per SM (shared memory at the windows 128 and up; the
+// register budget, 80 and 128 a thread, at 64 and 32). On the cluster windows
+// two CTAs of different clusters share an SM: one computes while the other
+// waits on its cluster. Their 256 TMEM columns each fill it, and their shared
+// memory (over a third of the SM's) keeps a third from fitting, so no CTA of
+// a cluster can wait for tensor memory that another waiting cluster holds.
+template <class G> struct PairCtas;
+template <> struct PairCtas<OneCta<32>> { static constexpr int n = 8; };
+template <> struct PairCtas<OneCta<64>> { static constexpr int n = 3; };
+template <> struct PairCtas<OneCta<128>> { static constexpr int n = 1; };
+template <> struct PairCtas<fp::ClFft<192>> { static constexpr int n = 2; };
+template <> struct PairCtas<fp::ClFft<256>> { static constexpr int n = 2; };
+
+template <class G>
 struct PairSmem {
+  static constexpr int N = G::N, LNN = G::LR * G::N;   // pixels of the CTA
   static constexpr size_t red = 0;
   static constexpr size_t tile = red + 256 * sizeof(double);
-  static constexpr size_t rI = tile + (size_t)N * N * sizeof(float2);
-  static constexpr size_t tw = rI + (size_t)N * N * sizeof(float);
-  static constexpr size_t o = tw + (size_t)Twiddles<N>::COUNT * sizeof(float2);
-  static constexpr size_t bytes = o + (N >= 64 ? 0 : (size_t)N * N * sizeof(float2));
-  // the staged object tile: N + 1 rows of up to N + 2 pixels, over the tile and
+  static constexpr size_t rI = tile + (size_t)LNN * sizeof(float2);
+  static constexpr size_t tw = rI + (size_t)LNN * sizeof(float);
+  static constexpr size_t o = tw + (size_t)G::TW * sizeof(float2);
+  static constexpr size_t bytes = o + (N >= 64 ? 0 : (size_t)LNN * sizeof(float2));
+  // the staged object tile: LR + 1 rows of up to N + 2 pixels, over the tile and
   // the intensity plane (free before the first transform). The pitch is 64
   // bytes off a multiple of 128: the rows of a half-warp's lanes alternate
   // between the two halves of the banks.
   static constexpr int opitch = N * 8 + 64;
-  static_assert((N + 1) * opitch <= N * N * 12, "the object tile fits");
+  static_assert((G::LR + 1) * opitch <= LNN * 12, "the object tile fits");
+  static_assert(G::Q == 1 || 3 * (bytes + 1024) > 228 * 1024, "no third CTA (its tensor memory would not fit)");
 };
 
 // The data term of four pixels (Eq. 1, or the Poisson likelihood): adds the
@@ -127,12 +175,12 @@ __device__ __forceinline__ float4 data_factor(int mode, float4 I, float4 Im, flo
   return make_float4(w * (rho[0].x - 1.f), w * (rho[0].y - 1.f), w * (rho[1].x - 1.f), w * (rho[1].y - 1.f));
 }
 
-template <int N, bool OPR>
-__global__ void __launch_bounds__(fp::Fft<N>::T, PairCtas<N>::n) k_pass1_pair(BatchArgs a) {
-  using F = fp::Fft<N>;
-  using SM = PairSmem<N>;
+template <class G, bool OPR>
+__global__ void __launch_bounds__(G::T, PairCtas<G>::n) k_pass1_pair(BatchArgs a) {
+  using SM = PairSmem<G>;
   using fp::C2;
-  constexpr int T = F::T, R1 = F::R1, R2 = F::R2, NN = N * N;
+  constexpr int N = G::N, T = G::T, NP = G::NP, NN = N * N, LR = G::LR, Q = G::Q, LNN = LR * N;
+  static_assert(NP % 4 == 0 && NP * T * 2 == LNN, "pixel pairs");
   constexpr int D = 6;   // probe loads in flight in the backward pass (its v fills half the registers)
   extern __shared__ __align__(16) unsigned char smem[];
   wait_prior_grid();
@@ -141,48 +189,49 @@ __global__ void __launch_bounds__(fp::Fft<N>::T, PairCtas<N>::n) k_pass1_pair(Ba
   float4* rI = (float4*)(smem + SM::rI);
   float2* tw = (float2*)(smem + SM::tw);
 
-  const int slot = blockIdx.x, tid = threadIdx.x;
-  const int n = F::col_lane(), p = F::col_pair();   // the thread's pixels: rows n + R1 q, columns 2p, 2p + 1
-  const int nr = F::row_lane(), pr = F::row_pair();   // its far field: rows 2pr, 2pr + 1, columns far_col(nr, q)
+  const int slot = blockIdx.x / Q, tid = threadIdx.x;
+  const G geo(tile, tw);
+  const int y0 = LR * geo.q;   // first patch row of this CTA
+  const bool first = tid == 0 && geo.q == 0;
   const int e = a.b0 + slot;
   const int j = a.order ? a.order[e] : e;
   int ty = 0, tx = 0;
   float fy = 0.f, fx = 0.f;
   bool ok = (j >= 0 && j < a.J);
   if (ok) ok = tile_of(a.pos[2 * j], a.pos[2 * j + 1], N, a.H, a.W, ty, tx, fy, fx);
-  if (!ok) {
-    if (tid == 0) {
+  if (!ok) {   // (the same decision in every CTA of a cluster)
+    if (first) {
       atomicOr(a.status, FLAG_BOUNDS);
       if (a.valid) a.valid[slot] = 0;
     }
     return;
   }
-  if (tid == 0 && a.valid) a.valid[slot] = 1;
+  if (first && a.valid) a.valid[slot] = 1;
   // the measured intensities are first read by the data term, after the forward
   // transforms: fetch them into L2 meanwhile (they may live in host memory)
-  if (tid == 0 && a.meas && a.mode != MODE_FWD)
+  if (first && a.meas && a.mode != MODE_FWD)
     prefetch_l2_bulk(a.meas + (size_t)j * NN, (uint32_t)(NN * sizeof(float)));
-  // The (N + 1)^2 object tile comes into shared memory by one bulk copy per
+  // The CTA's rows of the (N + 1)^2 object tile come into shared memory by one bulk copy per
   // row, from the row's start rounded down to 16 bytes (row r then begins at
   // pixel off(r)); rows of an unaligned object, and the one row whose copy
   // would end past the object, by plain loads.
   unsigned char* stage = (unsigned char*)tile;
   uint64_t* bar = (uint64_t*)(red + 252);
-  const float2* tile0 = a.obj + (size_t)ty * a.W + tx;
+  const float2* tile0 = a.obj + (size_t)(ty + y0) * a.W + tx;
   const bool bulk = ((uintptr_t)a.obj & 15) == 0;
   auto off = [&](int r) -> int { return bulk ? (int)(((uintptr_t)tile0 >> 3) + (uintptr_t)r * a.W) & 1 : 0; };
   auto row_plain = [&](int r) {
-    return !bulk || (off(r) == 0 && (size_t)(ty + r) * a.W + tx + N + 2 > (size_t)a.H * a.W);
+    return !bulk || (off(r) == 0 && (size_t)(ty + y0 + r) * a.W + tx + N + 2 > (size_t)a.H * a.W);
   };
   if (tid == 0) {
     tc::mbar_init(bar, 1);
     tc::mbar_init(bar + 1, 1);
     tc::fence_mbar_init();
-    const int last = row_plain(N) ? N : N + 1;   // only the tile's last row can end the object
+    const int last = row_plain(LR) ? LR : LR + 1;   // only the tile's last row can end the object
     if (bulk) tc::mbar_expect_tx(bar, (uint32_t)(last * (N + 2) * sizeof(float2)));
   }
   constexpr bool TM = N >= 64;
-  constexpr int TMC = T / 128 * 8 * R2, TG = 4 * R2;   // columns of the CTA; g's offset
+  constexpr int TMN = T / 128 * 8 * NP, TMC = TMN == 192 ? 256 : TMN, TG = 4 * NP;   // columns of the CTA; g's offset
   uint32_t* tm_holder = (uint32_t*)(red + 250);   // beyond the block reductions' 160 doubles
   if constexpr (TM) {
     if (tid < 32) {
@@ -193,19 +242,19 @@ __global__ void __launch_bounds__(fp::Fft<N>::T, PairCtas<N>::n) k_pass1_pair(Ba
   }
   __syncthreads();   // the barrier's state, the tensor-memory address
   if constexpr (TM) tc::fence_after_sync();
-  for (int r = tid; r < N + 1; r += T)
+  for (int r = tid; r < LR + 1; r += T)
     if (!row_plain(r))
       tc::bulk_g2s(stage + r * SM::opitch, tile0 + (size_t)r * a.W - off(r), (N + 2) * sizeof(float2), bar);
   if (!bulk) {
-    for (int i = tid; i < (N + 1) * (N + 1); i += T) {
+    for (int i = tid; i < (LR + 1) * (N + 1); i += T) {
       const int r = i / (N + 1), c = i % (N + 1);
       ((float2*)(stage + r * SM::opitch))[c] = __ldg(tile0 + (size_t)r * a.W + c);
     }
-  } else if (row_plain(N)) {
+  } else if (row_plain(LR)) {
     for (int c = tid; c < N + 1; c += T)
-      ((float2*)(stage + N * SM::opitch))[c] = __ldg(tile0 + (size_t)N * a.W + c);
+      ((float2*)(stage + LR * SM::opitch))[c] = __ldg(tile0 + (size_t)LR * a.W + c);
   }
-  make_twiddles<N>(tw);
+  G::fill_twiddles(tw);
 
   const int M = a.M, mode = a.mode;
   const float invN = 1.0f / (float)N;
@@ -213,20 +262,54 @@ __global__ void __launch_bounds__(fp::Fft<N>::T, PairCtas<N>::n) k_pass1_pair(Ba
   float* wj = (float*)(red + 128);   // this position's eigenmode weights (OPR)
   float2* p0 = (OPR && a.p0_s) ? a.p0_s + slotNN : nullptr;
   if (OPR && tid < a.K) wj[tid] = a.opr_w[(size_t)j * a.K + tid];
-  // far field of mode k, unit i of this thread: psi[k NN / 2 + i T]
+  // far field of mode k, unit i of this thread: psi[k NN / 2 + i T] (the CTA's
+  // share of the plane is the memory of its own pixel rows)
   float4* oS = (float4*)(smem + SM::o) + tid;   // (window 32) pixel pair q at oS[q T]
-  float4* psi = a.psi_s ? (float4*)(a.psi_s + slotNN * M) + tid : nullptr;
+  float4* psi = a.psi_s ? (float4*)(a.psi_s + slotNN * M + (size_t)y0 * N) + tid : nullptr;
   float2* o_s = a.o_s ? a.o_s + slotNN : nullptr;
-  const int pix0 = n * N + 2 * p;   // pixel pair q: pix0 + q R1 N
+  // pixel pair i in a plane of the patch, and its loads and stores
+  auto pix = [&](int i) { return (y0 + geo.row(i)) * N + geo.col(i); };
+  auto ldg_pair = [&](const float2* p) -> float4 {
+    if constexpr (G::VERT) {
+      const float2 u = __ldg(p), v = __ldg(p + N);
+      return make_float4(u.x, u.y, v.x, v.y);
+    } else {
+      return __ldg((const float4*)p);
+    }
+  };
+  auto ld_pair = [&](const float2* p) -> float4 {   // (written by this kernel)
+    if constexpr (G::VERT) {
+      const float2 u = p[0], v = p[N];
+      return make_float4(u.x, u.y, v.x, v.y);
+    } else {
+      return *(const float4*)p;
+    }
+  };
+  auto st_pair = [&](float2* p, float4 v) {
+    if constexpr (G::VERT) {
+      p[0] = make_float2(v.x, v.y);
+      p[N] = make_float2(v.z, v.w);
+    } else {
+      *(float4*)p = v;
+    }
+  };
+  auto stcs_pair = [&](float2* p, float4 v) {
+    if constexpr (G::VERT) {
+      __stcs(p, make_float2(v.x, v.y));
+      __stcs(p + N, make_float2(v.z, v.w));
+    } else {
+      __stcs((float4*)p, v);
+    }
+  };
 
-  // Tensor memory as per-thread storage: the thread's R2 pixel pairs of o in
-  // the first 4 R2 of its columns, of g in the next 4 R2 (warp w reaches lanes
-  // 32 (w % 4) ..+31; every fourth warp shares them, 8 R2 columns each). A CTA
+  // Tensor memory as per-thread storage: the thread's NP pixel pairs of o in
+  // the first 4 NP of its columns, of g in the next 4 NP (warp w reaches lanes
+  // 32 (w % 4) ..+31; every fourth warp shares them, 8 NP columns each). A CTA
   // holds TMC columns: the SM's 512 serve all the CTAs its shared memory admits.
   // (Window 32: o in shared memory, g in its scratch.)
   auto tm_o = [&]() -> uint32_t {
     const int w = (int)(threadIdx.x >> 5);
-    return *tm_holder + ((uint32_t)(32 * (w & 3)) << 16) + (uint32_t)((w >> 2) * 8 * R2);
+    return *tm_holder + ((uint32_t)(32 * (w & 3)) << 16) + (uint32_t)((w >> 2) * 8 * NP);
   };
   auto tm_release = [&]() {
     if constexpr (TM) {
@@ -236,18 +319,37 @@ __global__ void __launch_bounds__(fp::Fft<N>::T, PairCtas<N>::n) k_pass1_pair(Ba
       if (threadIdx.x < 32) tc::tmem_dealloc(*tm_holder, TMC);
     }
   };
-  // pixel pair q of the probe mode (of the relaxed primary mode: forward
-  // synthesised and kept in p0, backward read there)
-  auto probe_fwd = [&](const float2* Pk, int q) -> float4 {
-    const int pix = pix0 + q * R1 * N;
-    if (!OPR || Pk) return __ldg((const float4*)(Pk + pix));
-    const float4 P = opr_pair(a.opr_U, wj, a.K, NN, pix);
-    if (p0) *(float4*)(p0 + pix) = P;
-    return P;
+  // The pixel pairs of a probe mode. The relaxed primary mode is synthesised
+  // eigenmode by eigenmode, half of the pairs' loads in flight (pair by pair,
+  // each over all eigenmodes, 256 positions of the 192 window with 8
+  // eigenmodes took 613 us instead of 435), and kept in p0 for the way back.
+  auto probe_fwd = [&](const float2* Pk, float4 (&P)[NP]) {
+    if (!OPR || Pk) {
+#pragma unroll
+      for (int i = 0; i < NP; ++i) P[i] = ldg_pair(Pk + pix(i));
+      return;
+    }
+#pragma unroll
+    for (int i = 0; i < NP; ++i) P[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int h = 0; h < NP; h += NP / 2)
+#pragma unroll 1
+      for (int m = 0; m < a.K; ++m) {
+        const float w = wj[m];
+        const float2* U = a.opr_U + (size_t)m * NN;
+#pragma unroll
+        for (int i = h; i < h + NP / 2; ++i) {
+          const float4 u = ldg_pair(U + pix(i));
+          P[i].x = fmaf(w, u.x, P[i].x); P[i].y = fmaf(w, u.y, P[i].y);
+          P[i].z = fmaf(w, u.z, P[i].z); P[i].w = fmaf(w, u.w, P[i].w);
+        }
+      }
+    if (p0)
+#pragma unroll
+      for (int i = 0; i < NP; ++i) st_pair(p0 + pix(i), P[i]);
   };
-  auto probe_back = [&](const float2* Pk, int q) -> float4 {
-    const int pix = pix0 + q * R1 * N;
-    return (!OPR || Pk) ? __ldg((const float4*)(Pk + pix)) : *(const float4*)(p0 + pix);
+  auto probe_back = [&](const float2* Pk, int i) -> float4 {
+    return (!OPR || Pk) ? ldg_pair(Pk + pix(i)) : ld_pair(p0 + pix(i));
   };
   auto exit_wave = [&](float4 P, float4 o) -> C2 {
     const float2 x0 = cmul(make_float2(P.x, P.y), make_float2(o.x, o.y));
@@ -259,42 +361,53 @@ __global__ void __launch_bounds__(fp::Fft<N>::T, PairCtas<N>::n) k_pass1_pair(Ba
   // Every pixel pair of a mode's probe is in flight at once: the loads are
   // issued before the barrier that frees the tile (the registers of v are
   // empty there).
-  C2 v[R2];
-  float4 P[R2];
+  C2 v[NP];
+  float4 P[NP];
   if (OPR) __syncthreads();   // the weights
-#pragma unroll
-  for (int q = 0; q < R2; ++q) P[q] = probe_fwd(shared_mode<OPR>(a, 0, NN), q);
+  probe_fwd(shared_mode<OPR>(a, 0, NN), P);
   // joins the block after a wait for copies; false (and everything released)
   // when a thread's wait gave up
   auto arrived_all = [&](bool got, uint64_t* b) -> bool {
     if (__syncthreads_and(got)) return true;
     if (tid == 0) {
       atomicOr(a.status, FLAG_TIMEOUT);
-      if (a.valid) a.valid[slot] = 0;
+      if (Q == 1 && a.valid) a.valid[slot] = 0;
       tc::mbar_wait(b, 0);   // copies in flight must not outlive the CTA
+    }
+    if (Q > 1) {   // its cluster writes into this CTA's memory: go on (the status tells)
+      __syncthreads();
+      return true;
     }
     tm_release();
     return false;
   };
   if (!arrived_all(!bulk || tc::mbar_wait(bar, 0), bar)) return;   // (also twiddles, plainly loaded rows)
 #pragma unroll
-  for (int qg = 0; qg < R2 / 4; ++qg) {   // the patch o_j and the first mode's exit wave
+  for (int qg = 0; qg < NP / 4; ++qg) {   // the patch o_j and the first mode's exit wave
     const float w00 = (1.f - fy) * (1.f - fx), w01 = (1.f - fy) * fx, w10 = fy * (1.f - fx), w11 = fy * fx;
     float ov[16];
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-      const int q = 4 * qg + u, r = n + R1 * q;
-      const float2* A = (const float2*)(stage + r * SM::opitch) + off(r) + 2 * p;
-      const float2* B = (const float2*)(stage + (r + 1) * SM::opitch) + off(r + 1) + 2 * p;
-      const float2 a0 = A[0], a1 = A[1], a2 = A[2], b0 = B[0], b1 = B[1], b2 = B[2];
-      const float4 o = make_float4(w00 * a0.x + w01 * a1.x + w10 * b0.x + w11 * b1.x,
-                                   w00 * a0.y + w01 * a1.y + w10 * b0.y + w11 * b1.y,
-                                   w00 * a1.x + w01 * a2.x + w10 * b1.x + w11 * b2.x,
-                                   w00 * a1.y + w01 * a2.y + w10 * b1.y + w11 * b2.y);
-      if (o_s) *(float4*)(o_s + pix0 + q * R1 * N) = o;
+      const int i = 4 * qg + u, r = geo.row(i), c = geo.col(i);
+      auto srow = [&](int y) { return (const float2*)(stage + y * SM::opitch) + off(y) + c; };
+      auto mix = [&](float2 a, float2 b, float2 d, float2 e) {
+        return make_float2(w00 * a.x + w01 * b.x + w10 * d.x + w11 * e.x,
+                           w00 * a.y + w01 * b.y + w10 * d.y + w11 * e.y);
+      };
+      const float2 *A = srow(r), *B = srow(r + 1);
+      const float2 a0 = A[0], a1 = A[1], b0 = B[0], b1 = B[1];
+      float2 o0 = mix(a0, a1, b0, b1), o1;
+      if constexpr (G::VERT) {
+        const float2* D = srow(r + 2);
+        o1 = mix(b0, b1, D[0], D[1]);
+      } else {
+        o1 = mix(a1, A[2], b1, B[2]);
+      }
+      const float4 o = make_float4(o0.x, o0.y, o1.x, o1.y);
+      if (o_s) st_pair(o_s + pix(i), o);
       *(float4*)(ov + 4 * u) = o;
-      if constexpr (!TM) oS[q * T] = o;
-      v[q] = exit_wave(P[q], o);
+      if constexpr (!TM) oS[i * T] = o;
+      v[i] = exit_wave(P[i], o);
     }
     if constexpr (TM) tc::tmem_st16(tm_o() + 16 * qg, ov);
   }
@@ -304,7 +417,7 @@ __global__ void __launch_bounds__(fp::Fft<N>::T, PairCtas<N>::n) k_pass1_pair(Ba
   for (int k = 0; k < M; ++k) {
     if (k > 0) {
 #pragma unroll
-      for (int qg = 0; qg < R2 / 4; ++qg) {
+      for (int qg = 0; qg < NP / 4; ++qg) {
         float ov[16];
         if constexpr (TM) tc::tmem_ld16_wait(tm_o() + 16 * qg, ov);
 #pragma unroll
@@ -314,13 +427,11 @@ __global__ void __launch_bounds__(fp::Fft<N>::T, PairCtas<N>::n) k_pass1_pair(Ba
         }
       }
     }
-    F::fwd_cols(v, tile, p, n, tw);
-    __syncthreads();
-    F::fwd_rows(v, tile, pr, nr, tw);
+    geo.forward(v);
 #pragma unroll
-    for (int q = 0; q < R2; ++q) v[q] = fp::pscale(v[q], fp::splat(invN));
+    for (int q = 0; q < NP; ++q) v[q] = fp::pscale(v[q], fp::splat(invN));
 #pragma unroll
-    for (int q = 0; q < R2; q += 2) {
+    for (int q = 0; q < NP; q += 2) {
       float2 i0 = fp::fma2(v[q].re, v[q].re, fp::mul2(v[q].im, v[q].im));
       float2 i1 = fp::fma2(v[q + 1].re, v[q + 1].re, fp::mul2(v[q + 1].im, v[q + 1].im));
       float4* ri = rI + (q / 2) * T + tid;
@@ -334,10 +445,9 @@ __global__ void __launch_bounds__(fp::Fft<N>::T, PairCtas<N>::n) k_pass1_pair(Ba
     if (k == M - 1) break;   // the last mode's far field stays in v
     if (psi)
 #pragma unroll
-      for (int q = 0; q < R2; ++q)
+      for (int q = 0; q < NP; ++q)
         psi[(size_t)k * (NN / 2) + q * T] = make_float4(v[q].re.x, v[q].re.y, v[q].im.x, v[q].im.y);
-#pragma unroll
-    for (int q = 0; q < R2; ++q) P[q] = probe_fwd(shared_mode<OPR>(a, k + 1, NN), q);
+    probe_fwd(shared_mode<OPR>(a, k + 1, NN), P);
     __syncthreads();   // the tile is free for the next mode
   }
 
@@ -360,42 +470,47 @@ __global__ void __launch_bounds__(fp::Fft<N>::T, PairCtas<N>::n) k_pass1_pair(Ba
     // The pattern into the tile, one bulk copy per row (loaded straight to its
     // threads, 32 bytes of a row per request, it took 6,000 cycles). The pitch
     // spreads the row pairs of a warp over the banks.
-    constexpr int MP = N + 4;
+    constexpr int FW = G::VERT ? LR : N;   // far-field columns of the CTA
+    constexpr int MP = FW + 4;
     float* mS = (float*)tile;
-    const float* meas = a.meas + (size_t)j * NN;
+    const int x0 = G::VERT ? y0 : 0;       // its first column
+    const float* meas = a.meas + (size_t)j * NN + x0;
     if (mode != MODE_FWD) {
       const bool mbulk = ((uintptr_t)a.meas & 15) == 0;
       tc::fence_async_smem();
       __syncthreads();   // the tile is free
       if (mbulk) {
-        if (tid == 0) tc::mbar_expect_tx(bar + 1, (uint32_t)(NN * sizeof(float)));
-        for (int r = tid; r < N; r += T) tc::bulk_g2s(mS + r * MP, meas + r * N, N * sizeof(float), bar + 1);
+        if (tid == 0) tc::mbar_expect_tx(bar + 1, (uint32_t)(LNN * sizeof(float)));
+        for (int r = tid; r < N; r += T) tc::bulk_g2s(mS + r * MP, meas + r * N, FW * sizeof(float), bar + 1);
       } else {
-        for (int i = tid; i < NN; i += T) mS[i / N * MP + i % N] = __ldg(meas + i);
+        for (int i = tid; i < LNN; i += T) mS[i / FW * MP + i % FW] = __ldg(meas + i / FW * N + i % FW);
       }
       if (!arrived_all(!mbulk || tc::mbar_wait(bar + 1, 0), bar + 1)) return;
     }
-    // unit i of the intensity plane: registers 2i and 2i + 1 of v, columns c0 and c1
-    auto cols = [&](int i, int& c0, int& c1) {
-      c0 = F::far_col(nr, 2 * i);
-      c1 = F::far_col(nr, 2 * i + 1);
+    // unit i of the intensity plane: registers 2i and 2i + 1 of v, two far-field
+    // pixels each; their places in the staged pattern (and, with the pitch N,
+    // in the whole one)
+    struct At { int a, b, c, d; };
+    auto at = [&](int i, int pitch) -> At {
+      if constexpr (G::VERT) {
+        const int p = geo.far_y(2 * i) * pitch + geo.far_x(), r = geo.far_y(2 * i + 1) * pitch + geo.far_x();
+        return {p, p + 1, r, r + 1};
+      } else {
+        const int y = geo.far_y(0) * pitch, c = geo.far_x(2 * i), d = geo.far_x(2 * i + 1);
+        return {y + c, y + pitch + c, y + d, y + pitch + d};
+      }
     };
 #pragma unroll 1
-    for (int i = 0; i < R2 / 2; ++i) {
+    for (int i = 0; i < NP / 2; ++i) {
       const float4 I = rI[i * T + tid];
-      int c0, c1;
-      cols(i, c0, c1);
       if (a.ipred) {
-        float* d = a.ipred + (size_t)j * NN + (size_t)(2 * pr) * N;
-        if constexpr (F::S > 1) {   // c1 = c0 + 1, c0 even (the array is only 4-byte aligned)
-          d[c0] = I.x; d[c1] = I.z; d[N + c0] = I.y; d[N + c1] = I.w;
-        } else {
-          d[c0] = I.x; d[N + c0] = I.y; d[c1] = I.z; d[N + c1] = I.w;
-        }
+        float* d = a.ipred + (size_t)j * NN + x0;
+        const At g = at(i, N);
+        d[g.a] = I.x; d[g.b] = I.y; d[g.c] = I.z; d[g.d] = I.w;
       }
       if (mode == MODE_FWD) continue;
-      float* m = mS + 2 * pr * MP;
-      const float4 Im = make_float4(m[c0], m[MP + c0], m[c1], m[MP + c1]);
+      const At m = at(i, MP);
+      const float4 Im = make_float4(mS[m.a], mS[m.b], mS[m.c], mS[m.d]);
       float4 f;
       if (mode == MODE_VJP) {
         bad |= !isfinite(Im.x) || !isfinite(Im.y) || !isfinite(Im.z) || !isfinite(Im.w);
@@ -407,16 +522,18 @@ __global__ void __launch_bounds__(fp::Fft<N>::T, PairCtas<N>::n) k_pass1_pair(Ba
         f = data_factor(mode, I, Im, eps, t);
         add_loss(t);
         if constexpr (N == 64) {   // kept for the upper rows' sum below
-          m[c0] = t.x; m[MP + c0] = t.y; m[c1] = t.z; m[MP + c1] = t.w;
+          mS[m.a] = t.x; mS[m.b] = t.y; mS[m.c] = t.z; mS[m.d] = t.w;
         }
       }
       rI[i * T + tid] = make_float4(f.x * invN, f.y * invN, f.z * invN, f.w * invN);
     }
     if (bad) atomicOr(a.status, FLAG_NONFINITE);
     if (a.loss && mode != MODE_FWD && mode != MODE_VJP) {
-      // FP32 per row and lane (window 64: rows r and r + 32 in one sum), a
-      // tree over the lanes and over G rows, FP64 from there: the loss keeps
-      // one order of summation, whatever the packing
+      // FP32 per row and lane (window 64: rows r and r + 32 in one sum; on a
+      // cluster, per column and lane), a tree over the lanes and some rows (the
+      // CTA's columns), FP64 from there: the loss keeps one order of summation,
+      // whatever the packing
+      int slots;
       bool mine = true;
       if constexpr (N == 64) {
         float2* lo = (float2*)red;
@@ -426,27 +543,40 @@ __global__ void __launch_bounds__(fp::Fft<N>::T, PairCtas<N>::n) k_pass1_pair(Ba
         if (mine) {
           ls = lo[tid - T / 2];
 #pragma unroll 1
-          for (int i = 0; i < R2 / 2; ++i) {
-            int c0, c1;
-            cols(i, c0, c1);
-            const float* m = mS + 2 * pr * MP;
-            add_loss(make_float4(m[c0], m[MP + c0], m[c1], m[MP + c1]));
+          for (int i = 0; i < NP / 2; ++i) {
+            const At m = at(i, MP);
+            add_loss(make_float4(mS[m.a], mS[m.b], mS[m.c], mS[m.d]));
           }
         }
         __syncthreads();
       }
-      constexpr int G = F::G;
+      if constexpr (!G::VERT) {
+        constexpr int LP = 32 / G::R1;   // line pairs per warp
 #pragma unroll
-      for (int o = 16; o >= 1; o /= 2)
-        if (o != G / 2) {
-          ls.x += __shfl_down_sync(0xffffffffu, ls.x, o);
-          ls.y += __shfl_down_sync(0xffffffffu, ls.y, o);
+        for (int o = 16; o >= 1; o /= 2)
+          if (o != LP / 2) {
+            ls.x += __shfl_down_sync(0xffffffffu, ls.x, o);
+            ls.y += __shfl_down_sync(0xffffffffu, ls.y, o);
+          }
+        const int lane = tid & 31;   // lanes 0 and LP / 2 hold LP rows each
+        if ((lane & ~(LP / 2)) == 0) red[(tid >> 5) * 2 + (lane != 0)] = mine ? (double)(ls.x + ls.y) : 0.0;
+        slots = 2 * (T / 32);
+      } else {
+        float* col = mS + N * MP;   // [lane][column]
+        *(float2*)(col + geo.n * LR + geo.far_x()) = ls;
+        __syncthreads();
+#pragma unroll
+        for (int r = tid >> 5; r < G::R1; r += T / 32) {
+          float s = col[r * LR + (tid & 31)];
+#pragma unroll
+          for (int o = 16; o >= 1; o /= 2) s += __shfl_down_sync(0xffffffffu, s, o);
+          if ((tid & 31) == 0) red[r] = (double)s;
         }
-      const int lane = tid & 31, slots = 2 * (T / 32);   // lanes 0 and G / 2 hold G rows each
-      if ((lane & ~(G / 2)) == 0) red[(tid >> 5) * 2 + (lane != 0)] = mine ? (double)(ls.x + ls.y) : 0.0;
+        slots = G::R1;
+      }
       __syncthreads();
       if (tid < 32) {
-        double s = lane < slots ? red[lane] : 0.0;
+        double s = tid < slots ? red[tid] : 0.0;
         for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
         if (tid == 0) atomicAdd(a.loss, s);
       }
@@ -467,27 +597,25 @@ __global__ void __launch_bounds__(fp::Fft<N>::T, PairCtas<N>::n) k_pass1_pair(Ba
     const float2* Pk = shared_mode<OPR>(a, k, NN);
     if (k < M - 1) {
 #pragma unroll
-      for (int q = 0; q < R2; ++q) {
+      for (int q = 0; q < NP; ++q) {
         const float4 x = psi[(size_t)k * (NN / 2) + q * T];
         v[q] = {make_float2(x.x, x.y), make_float2(x.z, x.w)};
       }
     }
 #pragma unroll
-    for (int q = 0; q < R2; q += 2) {
+    for (int q = 0; q < NP; q += 2) {
       const float4 f = rI[(q / 2) * T + tid];
       v[q] = fp::pscale(v[q], make_float2(f.x, f.y));
       v[q + 1] = fp::pscale(v[q + 1], make_float2(f.z, f.w));
     }
     __syncthreads();   // the tile is free
-    F::inv_rows(v, tile, pr, nr, tw);
-    __syncthreads();
-    F::inv_cols(v, tile, p, n, tw);
-    if (k == 0) F::col_sync();   // the line's units are read: g may overwrite them
+    geo.inverse(v);
+    if (k == 0) G::pixel_sync();   // the line's units are read: g may overwrite them
     float4 Pr[D];   // the probe pairs, D loads ahead
 #pragma unroll
     for (int q = 0; q < D; ++q) Pr[q] = probe_back(Pk, q);
 #pragma unroll
-    for (int qg = 0; qg < R2 / 2; ++qg) {
+    for (int qg = 0; qg < NP / 2; ++qg) {
       float ov[8], gv[8];
       if constexpr (TM) {
         if (k < M - 1)
@@ -498,14 +626,14 @@ __global__ void __launch_bounds__(fp::Fft<N>::T, PairCtas<N>::n) k_pass1_pair(Ba
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
           *(float4*)(ov + 4 * u) = oS[(2 * qg + u) * T];
-          if (k < M - 1) *(float4*)(gv + 4 * u) = *(const float4*)(g_s + pix0 + (2 * qg + u) * R1 * N);
+          if (k < M - 1) *(float4*)(gv + 4 * u) = ld_pair(g_s + pix(2 * qg + u));
         }
       }
 #pragma unroll
       for (int u = 0; u < 2; ++u) {
-        const int q = 2 * qg + u, pix = pix0 + q * R1 * N;
+        const int q = 2 * qg + u;
         const float4 P2 = Pr[q % D];
-        if (q + D < R2) Pr[q % D] = probe_back(Pk, q + D);
+        if (q + D < NP) Pr[q % D] = probe_back(Pk, q + D);
         const float2 x0 = make_float2(v[q].re.x, v[q].im.x), x1 = make_float2(v[q].re.y, v[q].im.y);
         float2 g0 = cmulc(make_float2(P2.x, P2.y), x0), g1 = cmulc(make_float2(P2.z, P2.w), x1);
         if (k < M - 1) {
@@ -513,10 +641,10 @@ __global__ void __launch_bounds__(fp::Fft<N>::T, PairCtas<N>::n) k_pass1_pair(Ba
         }
         const float2 h0 = cmulc(make_float2(ov[4 * u], ov[4 * u + 1]), x0);
         const float2 h1 = cmulc(make_float2(ov[4 * u + 2], ov[4 * u + 3]), x1);
-        __stcs((float4*)(h_s + (size_t)k * NN + pix), make_float4(h0.x, h0.y, h1.x, h1.y));
+        stcs_pair(h_s + (size_t)k * NN + pix(q), make_float4(h0.x, h0.y, h1.x, h1.y));
         const float4 g4 = make_float4(g0.x, g0.y, g1.x, g1.y);
-        if (!TM || k == 0) *(float4*)(g_s + pix) = g4;
-        if (k == 0) tile[F::colu(n + R1 * q, p)] = g4;   // (re, im) pairs, for the scatter
+        if (!TM || k == 0) st_pair(g_s + pix(q), g4);
+        if (k == 0) tile[geo.pixel_unit(q)] = g4;   // (re, im) pairs, for the scatter
         *(float4*)(gv + 4 * u) = g4;
       }
       if constexpr (TM)
@@ -526,19 +654,39 @@ __global__ void __launch_bounds__(fp::Fft<N>::T, PairCtas<N>::n) k_pass1_pair(Ba
   }
   __syncthreads();
   const float2* gt = (const float2*)tile;
-  overlap_add<N, T, OPR>(a, slot, j, ty, tx, fy, fx, p0, (float*)rI, red,
-                         [&](int y, int x) { return gt[2 * F::colu(y, x >> 1) + (x & 1)]; });
+  overlap_add<N, LR, T, OPR>(a, slot, j, y0, ty, tx, fy, fx, p0, (float*)rI, red,
+                             [&](int y, int x) { return gt[G::pixel_slot(y, x)]; });
   tm_release();
 }
 
-template <int N, bool OPR>
+template <class G, bool OPR>
 cudaError_t launch_pass1_pair(const BatchArgs& a, cudaStream_t s) {
-  constexpr size_t sm = PairSmem<N>::bytes;
+  constexpr size_t sm = PairSmem<G>::bytes;
   static unsigned long long done = 0;
-  cudaError_t e = smem_optin(k_pass1_pair<N, OPR>, sm, &done);
+  cudaError_t e = smem_optin(k_pass1_pair<G, OPR>, sm, &done);
   if (e != cudaSuccess) return e;
   if (a.nb <= 0) return cudaSuccess;
-  return launch_pdl(k_pass1_pair<N, OPR>, dim3(a.nb), dim3(fp::Fft<N>::T), sm, s, a);
+  if constexpr (G::Q == 1) {
+    return launch_pdl(k_pass1_pair<G, OPR>, dim3(a.nb), dim3(G::T), sm, s, a);
+  } else {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(G::Q * a.nb));
+    cfg.blockDim = dim3(G::T);
+    cfg.dynamicSmemBytes = sm;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = G::Q;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_pass1_pair<G, OPR>, a);
+  }
 }
+
+// The window's geometry.
+template <int N>
+using PairGeo = std::conditional_t<(N > 128), fp::ClFft<(N > 128 ? N : 256)>, OneCta<(N > 128 ? 128 : N)>>;
 
 }  // namespace ptycho

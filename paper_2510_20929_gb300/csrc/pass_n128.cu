@@ -5,7 +5,7 @@
 namespace ptycho {
 template <>
 cudaError_t launch_pass1<128>(const BatchArgs& a, cudaStream_t s, int) {
-  return a.opr_U ? launch_pass1_pair<128, true>(a, s) : launch_pass1_pair<128, false>(a, s);
+  return a.opr_U ? launch_pass1_pair<PairGeo<128>, true>(a, s) : launch_pass1_pair<PairGeo<128>, false>(a, s);
 }
 template cudaError_t launch_pass2<128>(const Pass2Args&, cudaStream_t, int);
 }  // namespace ptycho
