@@ -33,10 +33,9 @@ template <int DIR> struct PDft<3, DIR> {
     const float2 s3 = splat(DIR * 0.86602540378443865f), mh = splat(-0.5f);
     const C2 t1 = padd(v[1], v[2]), t2 = psub(v[1], v[2]);
     const C2 m = {fma2(mh, t1.re, v[0].re), fma2(mh, t1.im, v[0].im)};
-    const C2 r = {mul2(neg2(s3), t2.im), mul2(s3, t2.re)};
     v[0] = padd(v[0], t1);
-    v[1] = padd(m, r);
-    v[2] = psub(m, r);
+    v[1] = {fma2(neg2(s3), t2.im, m.re), fma2(s3, t2.re, m.im)};
+    v[2] = {fma2(s3, t2.im, m.re), fma2(neg2(s3), t2.re, m.im)};
   }
 };
 

@@ -65,7 +65,10 @@ __device__ __forceinline__ C2 pmul(C2 a, float c, float s) {
   const float2 cc = splat(c), ss = splat(s);
   return {fma2(a.re, cc, neg2(mul2(a.im, ss))), fma2(a.re, ss, mul2(a.im, cc))};
 }
-// a * conj(t), with a twiddle per line
+// a * t and a * conj(t), with a twiddle per line
+__device__ __forceinline__ C2 pmul(C2 a, C2 t) {
+  return {fma2(a.re, t.re, neg2(mul2(a.im, t.im))), fma2(a.re, t.im, mul2(a.im, t.re))};
+}
 __device__ __forceinline__ C2 pmulc(C2 a, C2 t) {
   return {fma2(a.re, t.re, mul2(a.im, t.im)), fma2(a.im, t.re, neg2(mul2(a.re, t.im)))};
 }
@@ -165,13 +168,10 @@ __device__ __forceinline__ void pair_twiddles(C2 (&t)[R2], const float2* tw, int
     const float2 a = tw[n * (R2 + 1) + k], b = tw[(n + 1) * (R2 + 1) + k];
     t[k] = {make_float2(a.x, b.x), make_float2(a.y, b.y)};
   }
-  auto mul = [](C2 a, C2 b) -> C2 {
-    return {fma2(a.re, b.re, neg2(mul2(a.im, b.im))), fma2(a.re, b.im, mul2(a.im, b.re))};
-  };
 #pragma unroll
   for (int k = 5; k < R2; ++k) {
     const int a = k & ~3, b = k & 3;
-    t[k] = b == 0 ? mul(t[a - 4], t[4]) : mul(t[a], t[b]);
+    t[k] = b == 0 ? pmul(t[a - 4], t[4]) : pmul(t[a], t[b]);
   }
 }
 
@@ -179,6 +179,11 @@ __device__ __forceinline__ void pair_twiddles(C2 (&t)[R2], const float2* tw, int
 // quarter warp covers 8 consecutive line pairs of one lane index n; by rows 8
 // line pairs (R1 = 4), or 4 line pairs of two n that differ in bit 0 (R1 = 8).
 template <int N> struct Cfg;
+template <> struct Cfg<16> {
+  static constexpr int R1 = 4, R2 = 4;
+  __host__ __device__ static constexpr int rsw(int rp, int c) { return (rp & 7) ^ ((c >> 3) & 1); }
+  __host__ __device__ static constexpr int csw(int r, int) { return (r >> 1) & 7; }
+};
 template <> struct Cfg<32> {
   static constexpr int R1 = 4, R2 = 8;
   __host__ __device__ static constexpr int rsw(int rp, int c) { return (rp & 7) ^ ((c >> 3) & 1); }

@@ -77,6 +77,7 @@ struct OneCta {
 // memory (over a third of the SM's) keeps a third from fitting, so no CTA of
 // a cluster can wait for tensor memory that another waiting cluster holds.
 template <class G> struct PairCtas;
+template <> struct PairCtas<OneCta<16>> { static constexpr int n = 16; };
 template <> struct PairCtas<OneCta<32>> { static constexpr int n = 8; };
 template <> struct PairCtas<OneCta<64>> { static constexpr int n = 3; };
 template <> struct PairCtas<OneCta<128>> { static constexpr int n = 1; };
@@ -95,8 +96,8 @@ struct PairSmem {
   // the staged object tile: LR + 1 rows of up to N + 2 pixels, over the tile and
   // the intensity plane (free before the first transform). The pitch is 64
   // bytes off a multiple of 128: the rows of a half-warp's lanes alternate
-  // between the two halves of the banks.
-  static constexpr int opitch = N * 8 + 64;
+  // between the two halves of the banks (window 16: what fits).
+  static constexpr int opitch = N == 16 ? 160 : N * 8 + 64;
   static_assert((G::LR + 1) * opitch <= LNN * 12, "the object tile fits");
   static_assert(G::Q == 1 || 3 * (bytes + 1024) > 228 * 1024, "no third CTA (its tensor memory would not fit)");
 };
@@ -175,6 +176,315 @@ __device__ __forceinline__ float4 data_factor(int mode, float4 I, float4 Im, flo
   return make_float4(w * (rho[0].x - 1.f), w * (rho[0].y - 1.f), w * (rho[1].x - 1.f), w * (rho[1].y - 1.f));
 }
 
+// A thread's pixel pair at p in a plane of the patch: loads (read-only data, and
+// data this kernel writes) and stores.
+template <class G>
+__device__ __forceinline__ float4 ldg_pair(const float2* p) {
+  if constexpr (G::VERT) {
+    const float2 u = __ldg(p), v = __ldg(p + G::N);
+    return make_float4(u.x, u.y, v.x, v.y);
+  } else {
+    return __ldg((const float4*)p);
+  }
+}
+template <class G>
+__device__ __forceinline__ float4 ld_pair(const float2* p) {
+  if constexpr (G::VERT) {
+    const float2 u = p[0], v = p[G::N];
+    return make_float4(u.x, u.y, v.x, v.y);
+  } else {
+    return *(const float4*)p;
+  }
+}
+template <class G>
+__device__ __forceinline__ void st_pair(float2* p, float4 v) {
+  if constexpr (G::VERT) {
+    p[0] = make_float2(v.x, v.y);
+    p[G::N] = make_float2(v.z, v.w);
+  } else {
+    *(float4*)p = v;
+  }
+}
+template <class G>
+__device__ __forceinline__ void stcs_pair(float2* p, float4 v) {
+  if constexpr (G::VERT) {
+    __stcs(p, make_float2(v.x, v.y));
+    __stcs(p + G::N, make_float2(v.z, v.w));
+  } else {
+    __stcs((float4*)p, v);
+  }
+}
+// The packed pair of a pixel pair, and its product with one.
+__device__ __forceinline__ fp::C2 pack_pair(float2 a, float2 b) { return {make_float2(a.x, b.x), make_float2(a.y, b.y)}; }
+__device__ __forceinline__ fp::C2 exit_wave(float4 P, float4 o) {
+  return pack_pair(cmul(make_float2(P.x, P.y), make_float2(o.x, o.y)),
+                   cmul(make_float2(P.z, P.w), make_float2(o.z, o.w)));
+}
+
+// Runs use(i, load(i)) for the NP pixel pairs with D loads ahead of their use
+// (the wave of a thread fills half of its registers, so the loads of a whole
+// plane do not fit beside it).
+template <int NP, int D, class Load, class Use>
+__device__ __forceinline__ void ahead(Load&& load, Use&& use) {
+  decltype(load(0)) r[D];
+#pragma unroll
+  for (int i = 0; i < D; ++i) r[i] = load(i);
+#pragma unroll
+  for (int i = 0; i < NP; ++i) {
+    const auto x = r[i % D];
+    if (i + D < NP) r[i % D] = load(i + D);
+    use(i, x);
+  }
+}
+
+// The CTA's rows of the (N + 1)^2 object tile, staged in shared memory by one
+// bulk copy per row, from the row's start rounded down to 16 bytes (row r then
+// begins at pixel off(r)); rows of an unaligned object, and the one row whose
+// copy would end past the plane, by plain loads.
+template <class G>
+struct ObjStage {
+  static constexpr int N = G::N, LR = G::LR, T = G::T, PITCH = PairSmem<G>::opitch;
+  unsigned char* stage;
+  uint64_t* bar;
+  const float2* tile0;   // first pixel of the CTA's rows in the plane
+  int W;
+  bool bulk, end;        // bulk copies; the last row ends the plane
+  // plane: H x W pixels, `base` the (16-byte aligned, for bulk copies) array it lies in
+  __device__ __forceinline__ ObjStage(void* smem, uint64_t* bar_, const void* base, const float2* plane, int H, int W_,
+                                      int y, int x)
+      : stage((unsigned char*)smem), bar(bar_), tile0(plane + (size_t)y * W_ + x), W(W_), bulk(((uintptr_t)base & 15) == 0),
+        end((size_t)(y + LR) * W_ + x + N + 2 > (size_t)H * W_) {}
+  __device__ __forceinline__ int off(int r) const {
+    return bulk ? (int)(((uintptr_t)tile0 >> 3) + (uintptr_t)r * W) & 1 : 0;
+  }
+  __device__ __forceinline__ bool row_plain(int r) const { return !bulk || (r == LR && end && off(r) == 0); }
+  // one thread, before any copy completes; then the whole CTA
+  __device__ __forceinline__ void expect() const {
+    if (bulk) tc::mbar_expect_tx(bar, (uint32_t)((row_plain(LR) ? LR : LR + 1) * (N + 2) * sizeof(float2)));
+  }
+  __device__ __forceinline__ void copy() const {
+    for (int r = threadIdx.x; r < LR + 1; r += T)
+      if (!row_plain(r))
+        tc::bulk_g2s(stage + r * PITCH, tile0 + (size_t)r * W - off(r), (N + 2) * sizeof(float2), bar);
+    if (!bulk) {
+      for (int i = threadIdx.x; i < (LR + 1) * (N + 1); i += T) {
+        const int r = i / (N + 1), c = i % (N + 1);
+        ((float2*)(stage + r * PITCH))[c] = __ldg(tile0 + (size_t)r * W + c);
+      }
+    } else if (row_plain(LR)) {
+      for (int c = threadIdx.x; c < N + 1; c += T) ((float2*)(stage + LR * PITCH))[c] = __ldg(tile0 + (size_t)LR * W + c);
+    }
+  }
+  __device__ __forceinline__ bool wait(uint32_t parity) const { return !bulk || tc::mbar_wait(bar, parity); }
+  // the bilinear patch at a pixel pair (staged rows and joined threads)
+  __device__ __forceinline__ float4 patch(int r, int c, float fy, float fx) const {
+    const float w00 = (1.f - fy) * (1.f - fx), w01 = (1.f - fy) * fx, w10 = fy * (1.f - fx), w11 = fy * fx;
+    auto srow = [&](int y) { return (const float2*)(stage + y * PITCH) + off(y) + c; };
+    auto mix = [&](float2 a, float2 b, float2 d, float2 e) {
+      return make_float2(w00 * a.x + w01 * b.x + w10 * d.x + w11 * e.x, w00 * a.y + w01 * b.y + w10 * d.y + w11 * e.y);
+    };
+    const float2 *A = srow(r), *B = srow(r + 1);
+    const float2 a0 = A[0], a1 = A[1], b0 = B[0], b1 = B[1];
+    const float2 o0 = mix(a0, a1, b0, b1);
+    float2 o1;
+    if constexpr (G::VERT) {
+      const float2* D = srow(r + 2);
+      o1 = mix(b0, b1, D[0], D[1]);
+    } else {
+      o1 = mix(a1, A[2], b1, B[2]);
+    }
+    return make_float4(o0.x, o0.y, o1.x, o1.y);
+  }
+};
+
+// The far field v (scaled to the unitary transform) into the intensity plane.
+template <class G>
+__device__ __forceinline__ void add_intensity(const fp::C2 (&v)[G::NP], float4* rI, bool first) {
+#pragma unroll
+  for (int i = 0; i < G::NP; i += 2) {
+    float2 i0 = fp::fma2(v[i].re, v[i].re, fp::mul2(v[i].im, v[i].im));
+    float2 i1 = fp::fma2(v[i + 1].re, v[i + 1].re, fp::mul2(v[i + 1].im, v[i + 1].im));
+    float4* ri = rI + (i / 2) * G::T + threadIdx.x;
+    if (!first) {
+      const float4 s = *ri;
+      i0 = fp::add2(make_float2(s.x, s.y), i0);
+      i1 = fp::add2(make_float2(s.z, s.w), i1);
+    }
+    *ri = make_float4(i0.x, i0.y, i1.x, i1.y);
+  }
+}
+// v times the factors of the intensity plane.
+template <class G>
+__device__ __forceinline__ void mul_factor(fp::C2 (&v)[G::NP], const float4* rI) {
+#pragma unroll
+  for (int i = 0; i < G::NP; i += 2) {
+    const float4 f = rI[(i / 2) * G::T + threadIdx.x];
+    v[i] = fp::pscale(v[i], make_float2(f.x, f.y));
+    v[i + 1] = fp::pscale(v[i + 1], make_float2(f.z, f.w));
+  }
+}
+// A thread's far field in its scratch plane: unit i at plane[i T].
+template <class G>
+__device__ __forceinline__ void put_far(const fp::C2 (&v)[G::NP], float4* plane) {
+#pragma unroll
+  for (int i = 0; i < G::NP; ++i) plane[i * G::T] = make_float4(v[i].re.x, v[i].re.y, v[i].im.x, v[i].im.y);
+}
+template <class G>
+__device__ __forceinline__ void get_far(fp::C2 (&v)[G::NP], const float4* plane) {
+#pragma unroll
+  for (int i = 0; i < G::NP; ++i) {
+    const float4 x = plane[i * G::T];
+    v[i] = {make_float2(x.x, x.y), make_float2(x.z, x.w)};
+  }
+}
+
+// The data term of the CTA's far-field pixels: the intensity plane rI becomes
+// the plane of factors, `ipred` (when set) receives the intensities, `loss` the
+// loss. The tile must be free; `arrived(got, bar)` joins the block after the
+// wait for the pattern and says whether to go on. A rolled loop over the units
+// of the plane: unrolled over the far field's registers it would be most of the
+// kernel's code, and ran at the speed of instruction fetches.
+template <class G, bool CHAIN, class Arrived>
+__device__ __forceinline__ bool data_term(const G& geo, float4* rI, double* red, uint64_t* bar,
+                                          const float* __restrict__ meas_all, int j, float* ipred, int mode, float eps,
+                                          double* loss, int* status, Arrived&& arrived_all) {
+  constexpr int N = G::N, T = G::T, NP = G::NP, NN = N * N, LR = G::LR, LNN = LR * N;
+  const int tid = threadIdx.x, y0 = LR * geo.q;
+  const float invN = 1.0f / (float)N;
+  float4* tile = geo.tile;
+  float2 ls = make_float2(0.f, 0.f);   // rows 2pr and 2pr + 1
+  bool bad = false;
+  const bool sq = mode == MODE_LSQML_GAUSS || mode == MODE_GRAD_GAUSS;
+  auto add_loss = [&](float4 t) {
+    if (sq)
+      ls = fp::fma2(make_float2(t.z, t.w), make_float2(t.z, t.w),
+                    fp::fma2(make_float2(t.x, t.y), make_float2(t.x, t.y), ls));
+    else
+      ls = fp::add2(fp::add2(ls, make_float2(t.x, t.y)), make_float2(t.z, t.w));
+  };
+  // The pattern into the tile, one bulk copy per row (loaded straight to its
+  // threads, 32 bytes of a row per request, it took 6,000 cycles). The pitch
+  // spreads the row pairs of a warp over the banks.
+  constexpr int FW = G::VERT ? LR : N;   // far-field columns of the CTA
+  constexpr int MP = FW + 4;
+  float* mS = (float*)tile;
+  const int x0 = G::VERT ? y0 : 0;       // its first column
+  const float* meas = meas_all + (size_t)j * NN + x0;
+  if (mode != MODE_FWD) {
+    const bool mbulk = ((uintptr_t)meas_all & 15) == 0;
+    tc::fence_async_smem();
+    __syncthreads();   // the tile is free
+    if (mbulk) {
+      if (tid == 0) tc::mbar_expect_tx(bar, (uint32_t)(LNN * sizeof(float)));
+      for (int r = tid; r < N; r += T) tc::bulk_g2s(mS + r * MP, meas + r * N, FW * sizeof(float), bar);
+    } else {
+      for (int i = tid; i < LNN; i += T) mS[i / FW * MP + i % FW] = __ldg(meas + i / FW * N + i % FW);
+    }
+    if (!arrived_all(!mbulk || tc::mbar_wait(bar, 0), bar)) return false;
+  }
+  // unit i of the intensity plane: registers 2i and 2i + 1 of v, two far-field
+  // pixels each; their places in the staged pattern (and, with the pitch N,
+  // in the whole one)
+  struct At { int a, b, c, d; };
+  auto at = [&](int i, int pitch) -> At {
+    if constexpr (G::VERT) {
+      const int p = geo.far_y(2 * i) * pitch + geo.far_x(), r = geo.far_y(2 * i + 1) * pitch + geo.far_x();
+      return {p, p + 1, r, r + 1};
+    } else {
+      const int y = geo.far_y(0) * pitch, c = geo.far_x(2 * i), d = geo.far_x(2 * i + 1);
+      return {y + c, y + pitch + c, y + d, y + pitch + d};
+    }
+  };
+#pragma unroll 1
+  for (int i = 0; i < NP / 2; ++i) {
+    const float4 I = rI[i * T + tid];
+    if (ipred) {
+      float* d = ipred + (size_t)j * NN + x0;
+      const At g = at(i, N);
+      d[g.a] = I.x; d[g.b] = I.y; d[g.c] = I.z; d[g.d] = I.w;
+    }
+    if (mode == MODE_FWD) continue;
+    const At m = at(i, MP);
+    const float4 Im = make_float4(mS[m.a], mS[m.b], mS[m.c], mS[m.d]);
+    float4 f;
+    if (mode == MODE_VJP) {
+      bad |= !isfinite(Im.x) || !isfinite(Im.y) || !isfinite(Im.z) || !isfinite(Im.w);
+      f = make_float4(2.f * Im.x, 2.f * Im.y, 2.f * Im.z, 2.f * Im.w);
+    } else {
+      auto off = [](float x) { return !(x >= 0.f) || !isfinite(x); };
+      bad |= off(Im.x) || off(Im.y) || off(Im.z) || off(Im.w);
+      float4 t;
+      f = data_factor(mode, I, Im, eps, t);
+      add_loss(t);
+      if constexpr (CHAIN) {   // kept for the upper rows' sum below
+        mS[m.a] = t.x; mS[m.b] = t.y; mS[m.c] = t.z; mS[m.d] = t.w;
+      }
+    }
+    rI[i * T + tid] = make_float4(f.x * invN, f.y * invN, f.z * invN, f.w * invN);
+  }
+  if (bad) atomicOr(status, FLAG_NONFINITE);
+  if (loss && mode != MODE_FWD && mode != MODE_VJP) {
+    // FP32 per row and lane (CHAIN: rows r and r + N / 2 in one sum; on a
+    // cluster, per column and lane), a tree over the lanes and some rows (the
+    // CTA's columns), FP64 from there: the loss keeps one order of summation,
+    // whatever the packing
+    int slots;
+    bool mine = true;
+    if constexpr (CHAIN) {
+      float2* lo = (float2*)(mS + N * MP);
+      static_assert(N * MP * 4 + T / 2 * 8 <= LNN * 8, "room beside the pattern");
+      mine = tid >= T / 2;
+      if (!mine) lo[tid] = ls;
+      __syncthreads();
+      if (mine) {
+        ls = lo[tid - T / 2];
+#pragma unroll 1
+        for (int i = 0; i < NP / 2; ++i) {
+          const At m = at(i, MP);
+          add_loss(make_float4(mS[m.a], mS[m.b], mS[m.c], mS[m.d]));
+        }
+      }
+      __syncthreads();
+    }
+    if constexpr (!G::VERT) {
+      constexpr int LP = 32 / G::R1;   // line pairs per warp
+      auto down = [](float x, int o) { return x + __shfl_down_sync(0xffffffffu, x, o); };
+      float sum;
+      if constexpr (N == 16) {   // rows first, then lanes
+        ls = make_float2(down(down(ls.x, 2), 1), down(down(ls.y, 2), 1));
+        sum = down(down(ls.x + ls.y, 16), 8);
+      } else {
+#pragma unroll
+        for (int o = 16; o >= 1; o /= 2)
+          if (o != LP / 2) ls = make_float2(down(ls.x, o), down(ls.y, o));
+        sum = ls.x + ls.y;
+      }
+      const int lane = tid & 31;   // lanes 0 and LP / 2 hold LP rows each
+      if ((lane & ~(LP / 2)) == 0) red[(tid >> 5) * 2 + (lane != 0)] = mine ? (double)sum : 0.0;
+      slots = 2 * (T / 32);
+    } else {
+      float* col = mS + N * MP;   // [lane][column]
+      *(float2*)(col + geo.n * LR + geo.far_x()) = ls;
+      __syncthreads();
+#pragma unroll
+      for (int r = tid >> 5; r < G::R1; r += T / 32) {
+        float s = col[r * LR + (tid & 31)];
+#pragma unroll
+        for (int o = 16; o >= 1; o /= 2) s += __shfl_down_sync(0xffffffffu, s, o);
+        if ((tid & 31) == 0) red[r] = (double)s;
+      }
+      slots = G::R1;
+    }
+    __syncthreads();
+    if (tid < 32) {
+      double s = tid < slots ? red[tid] : 0.0;
+      for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+      if (tid == 0) atomicAdd(loss, s);
+    }
+  }
+  return true;
+}
+
 template <class G, bool OPR>
 __global__ void __launch_bounds__(G::T, PairCtas<G>::n) k_pass1_pair(BatchArgs a) {
   using SM = PairSmem<G>;
@@ -211,24 +521,13 @@ __global__ void __launch_bounds__(G::T, PairCtas<G>::n) k_pass1_pair(BatchArgs a
   // transforms: fetch them into L2 meanwhile (they may live in host memory)
   if (first && a.meas && a.mode != MODE_FWD)
     prefetch_l2_bulk(a.meas + (size_t)j * NN, (uint32_t)(NN * sizeof(float)));
-  // The CTA's rows of the (N + 1)^2 object tile come into shared memory by one bulk copy per
-  // row, from the row's start rounded down to 16 bytes (row r then begins at
-  // pixel off(r)); rows of an unaligned object, and the one row whose copy
-  // would end past the object, by plain loads.
-  unsigned char* stage = (unsigned char*)tile;
   uint64_t* bar = (uint64_t*)(red + 252);
-  const float2* tile0 = a.obj + (size_t)(ty + y0) * a.W + tx;
-  const bool bulk = ((uintptr_t)a.obj & 15) == 0;
-  auto off = [&](int r) -> int { return bulk ? (int)(((uintptr_t)tile0 >> 3) + (uintptr_t)r * a.W) & 1 : 0; };
-  auto row_plain = [&](int r) {
-    return !bulk || (off(r) == 0 && (size_t)(ty + y0 + r) * a.W + tx + N + 2 > (size_t)a.H * a.W);
-  };
+  const ObjStage<G> stage(tile, bar, a.obj, a.obj, a.H, a.W, ty + y0, tx);
   if (tid == 0) {
     tc::mbar_init(bar, 1);
     tc::mbar_init(bar + 1, 1);
     tc::fence_mbar_init();
-    const int last = row_plain(LR) ? LR : LR + 1;   // only the tile's last row can end the object
-    if (bulk) tc::mbar_expect_tx(bar, (uint32_t)(last * (N + 2) * sizeof(float2)));
+    stage.expect();
   }
   constexpr bool TM = N >= 64;
   constexpr int TMN = T / 128 * 8 * NP, TMC = TMN == 192 ? 256 : TMN, TG = 4 * NP;   // columns of the CTA; g's offset
@@ -242,18 +541,7 @@ __global__ void __launch_bounds__(G::T, PairCtas<G>::n) k_pass1_pair(BatchArgs a
   }
   __syncthreads();   // the barrier's state, the tensor-memory address
   if constexpr (TM) tc::fence_after_sync();
-  for (int r = tid; r < LR + 1; r += T)
-    if (!row_plain(r))
-      tc::bulk_g2s(stage + r * SM::opitch, tile0 + (size_t)r * a.W - off(r), (N + 2) * sizeof(float2), bar);
-  if (!bulk) {
-    for (int i = tid; i < (LR + 1) * (N + 1); i += T) {
-      const int r = i / (N + 1), c = i % (N + 1);
-      ((float2*)(stage + r * SM::opitch))[c] = __ldg(tile0 + (size_t)r * a.W + c);
-    }
-  } else if (row_plain(LR)) {
-    for (int c = tid; c < N + 1; c += T)
-      ((float2*)(stage + LR * SM::opitch))[c] = __ldg(tile0 + (size_t)LR * a.W + c);
-  }
+  stage.copy();
   G::fill_twiddles(tw);
 
   const int M = a.M, mode = a.mode;
@@ -267,40 +555,7 @@ __global__ void __launch_bounds__(G::T, PairCtas<G>::n) k_pass1_pair(BatchArgs a
   float4* oS = (float4*)(smem + SM::o) + tid;   // (window 32) pixel pair q at oS[q T]
   float4* psi = a.psi_s ? (float4*)(a.psi_s + slotNN * M + (size_t)y0 * N) + tid : nullptr;
   float2* o_s = a.o_s ? a.o_s + slotNN : nullptr;
-  // pixel pair i in a plane of the patch, and its loads and stores
-  auto pix = [&](int i) { return (y0 + geo.row(i)) * N + geo.col(i); };
-  auto ldg_pair = [&](const float2* p) -> float4 {
-    if constexpr (G::VERT) {
-      const float2 u = __ldg(p), v = __ldg(p + N);
-      return make_float4(u.x, u.y, v.x, v.y);
-    } else {
-      return __ldg((const float4*)p);
-    }
-  };
-  auto ld_pair = [&](const float2* p) -> float4 {   // (written by this kernel)
-    if constexpr (G::VERT) {
-      const float2 u = p[0], v = p[N];
-      return make_float4(u.x, u.y, v.x, v.y);
-    } else {
-      return *(const float4*)p;
-    }
-  };
-  auto st_pair = [&](float2* p, float4 v) {
-    if constexpr (G::VERT) {
-      p[0] = make_float2(v.x, v.y);
-      p[N] = make_float2(v.z, v.w);
-    } else {
-      *(float4*)p = v;
-    }
-  };
-  auto stcs_pair = [&](float2* p, float4 v) {
-    if constexpr (G::VERT) {
-      __stcs(p, make_float2(v.x, v.y));
-      __stcs(p + N, make_float2(v.z, v.w));
-    } else {
-      __stcs((float4*)p, v);
-    }
-  };
+  auto pix = [&](int i) { return (y0 + geo.row(i)) * N + geo.col(i); };   // pixel pair i in a plane
 
   // Tensor memory as per-thread storage: the thread's NP pixel pairs of o in
   // the first 4 NP of its columns, of g in the next 4 NP (warp w reaches lanes
@@ -326,7 +581,7 @@ __global__ void __launch_bounds__(G::T, PairCtas<G>::n) k_pass1_pair(BatchArgs a
   auto probe_fwd = [&](const float2* Pk, float4 (&P)[NP]) {
     if (!OPR || Pk) {
 #pragma unroll
-      for (int i = 0; i < NP; ++i) P[i] = ldg_pair(Pk + pix(i));
+      for (int i = 0; i < NP; ++i) P[i] = ldg_pair<G>(Pk + pix(i));
       return;
     }
 #pragma unroll
@@ -339,22 +594,17 @@ __global__ void __launch_bounds__(G::T, PairCtas<G>::n) k_pass1_pair(BatchArgs a
         const float2* U = a.opr_U + (size_t)m * NN;
 #pragma unroll
         for (int i = h; i < h + NP / 2; ++i) {
-          const float4 u = ldg_pair(U + pix(i));
+          const float4 u = ldg_pair<G>(U + pix(i));
           P[i].x = fmaf(w, u.x, P[i].x); P[i].y = fmaf(w, u.y, P[i].y);
           P[i].z = fmaf(w, u.z, P[i].z); P[i].w = fmaf(w, u.w, P[i].w);
         }
       }
     if (p0)
 #pragma unroll
-      for (int i = 0; i < NP; ++i) st_pair(p0 + pix(i), P[i]);
+      for (int i = 0; i < NP; ++i) st_pair<G>(p0 + pix(i), P[i]);
   };
   auto probe_back = [&](const float2* Pk, int i) -> float4 {
-    return (!OPR || Pk) ? ldg_pair(Pk + pix(i)) : ld_pair(p0 + pix(i));
-  };
-  auto exit_wave = [&](float4 P, float4 o) -> C2 {
-    const float2 x0 = cmul(make_float2(P.x, P.y), make_float2(o.x, o.y));
-    const float2 x1 = cmul(make_float2(P.z, P.w), make_float2(o.z, o.w));
-    return {make_float2(x0.x, x1.x), make_float2(x0.y, x1.y)};
+    return (!OPR || Pk) ? ldg_pair<G>(Pk + pix(i)) : ld_pair<G>(p0 + pix(i));
   };
 
   // ---- forward model: I_j = sum_k |F(P_k o_j)|^2 -------------------------------
@@ -381,30 +631,15 @@ __global__ void __launch_bounds__(G::T, PairCtas<G>::n) k_pass1_pair(BatchArgs a
     tm_release();
     return false;
   };
-  if (!arrived_all(!bulk || tc::mbar_wait(bar, 0), bar)) return;   // (also twiddles, plainly loaded rows)
+  if (!arrived_all(stage.wait(0), bar)) return;   // (also twiddles, plainly loaded rows)
 #pragma unroll
   for (int qg = 0; qg < NP / 4; ++qg) {   // the patch o_j and the first mode's exit wave
-    const float w00 = (1.f - fy) * (1.f - fx), w01 = (1.f - fy) * fx, w10 = fy * (1.f - fx), w11 = fy * fx;
     float ov[16];
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
-      const int i = 4 * qg + u, r = geo.row(i), c = geo.col(i);
-      auto srow = [&](int y) { return (const float2*)(stage + y * SM::opitch) + off(y) + c; };
-      auto mix = [&](float2 a, float2 b, float2 d, float2 e) {
-        return make_float2(w00 * a.x + w01 * b.x + w10 * d.x + w11 * e.x,
-                           w00 * a.y + w01 * b.y + w10 * d.y + w11 * e.y);
-      };
-      const float2 *A = srow(r), *B = srow(r + 1);
-      const float2 a0 = A[0], a1 = A[1], b0 = B[0], b1 = B[1];
-      float2 o0 = mix(a0, a1, b0, b1), o1;
-      if constexpr (G::VERT) {
-        const float2* D = srow(r + 2);
-        o1 = mix(b0, b1, D[0], D[1]);
-      } else {
-        o1 = mix(a1, A[2], b1, B[2]);
-      }
-      const float4 o = make_float4(o0.x, o0.y, o1.x, o1.y);
-      if (o_s) st_pair(o_s + pix(i), o);
+      const int i = 4 * qg + u;
+      const float4 o = stage.patch(geo.row(i), geo.col(i), fy, fx);
+      if (o_s) st_pair<G>(o_s + pix(i), o);
       *(float4*)(ov + 4 * u) = o;
       if constexpr (!TM) oS[i * T] = o;
       v[i] = exit_wave(P[i], o);
@@ -430,161 +665,19 @@ __global__ void __launch_bounds__(G::T, PairCtas<G>::n) k_pass1_pair(BatchArgs a
     geo.forward(v);
 #pragma unroll
     for (int q = 0; q < NP; ++q) v[q] = fp::pscale(v[q], fp::splat(invN));
-#pragma unroll
-    for (int q = 0; q < NP; q += 2) {
-      float2 i0 = fp::fma2(v[q].re, v[q].re, fp::mul2(v[q].im, v[q].im));
-      float2 i1 = fp::fma2(v[q + 1].re, v[q + 1].re, fp::mul2(v[q + 1].im, v[q + 1].im));
-      float4* ri = rI + (q / 2) * T + tid;
-      if (k > 0) {
-        const float4 s = *ri;
-        i0 = fp::add2(make_float2(s.x, s.y), i0);
-        i1 = fp::add2(make_float2(s.z, s.w), i1);
-      }
-      *ri = make_float4(i0.x, i0.y, i1.x, i1.y);
-    }
+    add_intensity<G>(v, rI, k == 0);
     if (k == M - 1) break;   // the last mode's far field stays in v
-    if (psi)
-#pragma unroll
-      for (int q = 0; q < NP; ++q)
-        psi[(size_t)k * (NN / 2) + q * T] = make_float4(v[q].re.x, v[q].re.y, v[q].im.x, v[q].im.y);
+    if (psi) put_far<G>(v, psi + (size_t)k * (NN / 2));
     probe_fwd(shared_mode<OPR>(a, k + 1, NN), P);
     __syncthreads();   // the tile is free for the next mode
   }
 
   // ---- data term: loss and the far-field factor, on the thread's own pixels ------
-  // (a rolled loop over the units of the intensity plane: unrolled over v it
-  // would be most of the kernel's code, and ran at the speed of instruction
-  // fetches)
-  {
-    const float eps = a.eps;
-    float2 ls = make_float2(0.f, 0.f);   // rows 2pr and 2pr + 1
-    bool bad = false;
-    const bool sq = mode == MODE_LSQML_GAUSS || mode == MODE_GRAD_GAUSS;
-    auto add_loss = [&](float4 t) {
-      if (sq)
-        ls = fp::fma2(make_float2(t.z, t.w), make_float2(t.z, t.w),
-                      fp::fma2(make_float2(t.x, t.y), make_float2(t.x, t.y), ls));
-      else
-        ls = fp::add2(fp::add2(ls, make_float2(t.x, t.y)), make_float2(t.z, t.w));
-    };
-    // The pattern into the tile, one bulk copy per row (loaded straight to its
-    // threads, 32 bytes of a row per request, it took 6,000 cycles). The pitch
-    // spreads the row pairs of a warp over the banks.
-    constexpr int FW = G::VERT ? LR : N;   // far-field columns of the CTA
-    constexpr int MP = FW + 4;
-    float* mS = (float*)tile;
-    const int x0 = G::VERT ? y0 : 0;       // its first column
-    const float* meas = a.meas + (size_t)j * NN + x0;
-    if (mode != MODE_FWD) {
-      const bool mbulk = ((uintptr_t)a.meas & 15) == 0;
-      tc::fence_async_smem();
-      __syncthreads();   // the tile is free
-      if (mbulk) {
-        if (tid == 0) tc::mbar_expect_tx(bar + 1, (uint32_t)(LNN * sizeof(float)));
-        for (int r = tid; r < N; r += T) tc::bulk_g2s(mS + r * MP, meas + r * N, FW * sizeof(float), bar + 1);
-      } else {
-        for (int i = tid; i < LNN; i += T) mS[i / FW * MP + i % FW] = __ldg(meas + i / FW * N + i % FW);
-      }
-      if (!arrived_all(!mbulk || tc::mbar_wait(bar + 1, 0), bar + 1)) return;
-    }
-    // unit i of the intensity plane: registers 2i and 2i + 1 of v, two far-field
-    // pixels each; their places in the staged pattern (and, with the pitch N,
-    // in the whole one)
-    struct At { int a, b, c, d; };
-    auto at = [&](int i, int pitch) -> At {
-      if constexpr (G::VERT) {
-        const int p = geo.far_y(2 * i) * pitch + geo.far_x(), r = geo.far_y(2 * i + 1) * pitch + geo.far_x();
-        return {p, p + 1, r, r + 1};
-      } else {
-        const int y = geo.far_y(0) * pitch, c = geo.far_x(2 * i), d = geo.far_x(2 * i + 1);
-        return {y + c, y + pitch + c, y + d, y + pitch + d};
-      }
-    };
-#pragma unroll 1
-    for (int i = 0; i < NP / 2; ++i) {
-      const float4 I = rI[i * T + tid];
-      if (a.ipred) {
-        float* d = a.ipred + (size_t)j * NN + x0;
-        const At g = at(i, N);
-        d[g.a] = I.x; d[g.b] = I.y; d[g.c] = I.z; d[g.d] = I.w;
-      }
-      if (mode == MODE_FWD) continue;
-      const At m = at(i, MP);
-      const float4 Im = make_float4(mS[m.a], mS[m.b], mS[m.c], mS[m.d]);
-      float4 f;
-      if (mode == MODE_VJP) {
-        bad |= !isfinite(Im.x) || !isfinite(Im.y) || !isfinite(Im.z) || !isfinite(Im.w);
-        f = make_float4(2.f * Im.x, 2.f * Im.y, 2.f * Im.z, 2.f * Im.w);
-      } else {
-        auto off = [](float x) { return !(x >= 0.f) || !isfinite(x); };
-        bad |= off(Im.x) || off(Im.y) || off(Im.z) || off(Im.w);
-        float4 t;
-        f = data_factor(mode, I, Im, eps, t);
-        add_loss(t);
-        if constexpr (N == 64) {   // kept for the upper rows' sum below
-          mS[m.a] = t.x; mS[m.b] = t.y; mS[m.c] = t.z; mS[m.d] = t.w;
-        }
-      }
-      rI[i * T + tid] = make_float4(f.x * invN, f.y * invN, f.z * invN, f.w * invN);
-    }
-    if (bad) atomicOr(a.status, FLAG_NONFINITE);
-    if (a.loss && mode != MODE_FWD && mode != MODE_VJP) {
-      // FP32 per row and lane (window 64: rows r and r + 32 in one sum; on a
-      // cluster, per column and lane), a tree over the lanes and some rows (the
-      // CTA's columns), FP64 from there: the loss keeps one order of summation,
-      // whatever the packing
-      int slots;
-      bool mine = true;
-      if constexpr (N == 64) {
-        float2* lo = (float2*)red;
-        mine = tid >= T / 2;
-        if (!mine) lo[tid] = ls;
-        __syncthreads();
-        if (mine) {
-          ls = lo[tid - T / 2];
-#pragma unroll 1
-          for (int i = 0; i < NP / 2; ++i) {
-            const At m = at(i, MP);
-            add_loss(make_float4(mS[m.a], mS[m.b], mS[m.c], mS[m.d]));
-          }
-        }
-        __syncthreads();
-      }
-      if constexpr (!G::VERT) {
-        constexpr int LP = 32 / G::R1;   // line pairs per warp
-#pragma unroll
-        for (int o = 16; o >= 1; o /= 2)
-          if (o != LP / 2) {
-            ls.x += __shfl_down_sync(0xffffffffu, ls.x, o);
-            ls.y += __shfl_down_sync(0xffffffffu, ls.y, o);
-          }
-        const int lane = tid & 31;   // lanes 0 and LP / 2 hold LP rows each
-        if ((lane & ~(LP / 2)) == 0) red[(tid >> 5) * 2 + (lane != 0)] = mine ? (double)(ls.x + ls.y) : 0.0;
-        slots = 2 * (T / 32);
-      } else {
-        float* col = mS + N * MP;   // [lane][column]
-        *(float2*)(col + geo.n * LR + geo.far_x()) = ls;
-        __syncthreads();
-#pragma unroll
-        for (int r = tid >> 5; r < G::R1; r += T / 32) {
-          float s = col[r * LR + (tid & 31)];
-#pragma unroll
-          for (int o = 16; o >= 1; o /= 2) s += __shfl_down_sync(0xffffffffu, s, o);
-          if ((tid & 31) == 0) red[r] = (double)s;
-        }
-        slots = G::R1;
-      }
-      __syncthreads();
-      if (tid < 32) {
-        double s = tid < slots ? red[tid] : 0.0;
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-        if (tid == 0) atomicAdd(a.loss, s);
-      }
-    }
-    if (mode == MODE_FWD || a.loss_only) {
-      tm_release();
-      return;
-    }
+  if (!data_term<G, N == 64>(geo, rI, red, bar + 1, a.meas, j, a.ipred, mode, a.eps, a.loss, a.status, arrived_all))
+    return;
+  if (mode == MODE_FWD || a.loss_only) {
+    tm_release();
+    return;
   }
 
   // ---- back-propagation: chi_k = F^-1[fac Psi_k], g = sum_k conj(P_k) chi_k, h_k ----
@@ -595,19 +688,8 @@ __global__ void __launch_bounds__(G::T, PairCtas<G>::n) k_pass1_pair(BatchArgs a
 #pragma unroll 1
   for (int k = M - 1; k >= 0; --k) {
     const float2* Pk = shared_mode<OPR>(a, k, NN);
-    if (k < M - 1) {
-#pragma unroll
-      for (int q = 0; q < NP; ++q) {
-        const float4 x = psi[(size_t)k * (NN / 2) + q * T];
-        v[q] = {make_float2(x.x, x.y), make_float2(x.z, x.w)};
-      }
-    }
-#pragma unroll
-    for (int q = 0; q < NP; q += 2) {
-      const float4 f = rI[(q / 2) * T + tid];
-      v[q] = fp::pscale(v[q], make_float2(f.x, f.y));
-      v[q + 1] = fp::pscale(v[q + 1], make_float2(f.z, f.w));
-    }
+    if (k < M - 1) get_far<G>(v, psi + (size_t)k * (NN / 2));
+    mul_factor<G>(v, rI);
     __syncthreads();   // the tile is free
     geo.inverse(v);
     if (k == 0) G::pixel_sync();   // the line's units are read: g may overwrite them
@@ -626,7 +708,7 @@ __global__ void __launch_bounds__(G::T, PairCtas<G>::n) k_pass1_pair(BatchArgs a
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
           *(float4*)(ov + 4 * u) = oS[(2 * qg + u) * T];
-          if (k < M - 1) *(float4*)(gv + 4 * u) = ld_pair(g_s + pix(2 * qg + u));
+          if (k < M - 1) *(float4*)(gv + 4 * u) = ld_pair<G>(g_s + pix(2 * qg + u));
         }
       }
 #pragma unroll
@@ -641,9 +723,9 @@ __global__ void __launch_bounds__(G::T, PairCtas<G>::n) k_pass1_pair(BatchArgs a
         }
         const float2 h0 = cmulc(make_float2(ov[4 * u], ov[4 * u + 1]), x0);
         const float2 h1 = cmulc(make_float2(ov[4 * u + 2], ov[4 * u + 3]), x1);
-        stcs_pair(h_s + (size_t)k * NN + pix(q), make_float4(h0.x, h0.y, h1.x, h1.y));
+        stcs_pair<G>(h_s + (size_t)k * NN + pix(q), make_float4(h0.x, h0.y, h1.x, h1.y));
         const float4 g4 = make_float4(g0.x, g0.y, g1.x, g1.y);
-        if (!TM || k == 0) st_pair(g_s + pix(q), g4);
+        if (!TM || k == 0) st_pair<G>(g_s + pix(q), g4);
         if (k == 0) tile[geo.pixel_unit(q)] = g4;   // (re, im) pairs, for the scatter
         *(float4*)(gv + 4 * u) = g4;
       }

@@ -1,7 +1,6 @@
 // Multislice entry points (Pty-Chi Sec. 1 and Sec. 2.1: multislice modelling):
 // the angular-spectrum propagator, the forward model and the adjoint of the
-// multislice per-position pass (kernels_ms.cuh; kernels_ms_cluster.cuh for the
-// 192 and 256 windows).
+// multislice per-position pass (kernels_ms.cuh).
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -21,8 +20,9 @@ namespace ptycho {
 // H[ky][kx] = exp(i 2 pi dz (sqrt(1/lambda^2 - |f|^2) - 1/lambda)) on the FFT
 // grid f = k / (N pixel) (k = 0..N/2-1, -N/2..-1), evanescent frequencies 0;
 // the bracket is evaluated as -|f|^2 / (sqrt(1/lambda^2 - |f|^2) + 1/lambda)
-// in FP64 so that the large constant 1/lambda cancels exactly.
-__global__ void k_asm_propagator(int N, double pixel, double wavelength, double dz, float2* Hf) {
+// in FP64 so that the large constant 1/lambda cancels exactly. Stored
+// [ky][kx], or [kx][ky] (`transposed`) for the windows whose threads run along ky.
+__global__ void k_asm_propagator(int N, double pixel, double wavelength, double dz, bool transposed, float2* Hf) {
   const int NN = N * N;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < NN; i += gridDim.x * blockDim.x) {
     const int ky = i / N, kx = i % N;
@@ -36,7 +36,7 @@ __global__ void k_asm_propagator(int N, double pixel, double wavelength, double 
       sincos(ph, &sn, &cs);
       h = make_float2((float)cs, (float)sn);
     }
-    Hf[i] = h;
+    Hf[transposed ? kx * N + ky : i] = h;
   }
 }
 
@@ -345,7 +345,7 @@ MsLayout ms_setup(const ptycho_dims& d, const ptycho_multislice& ms, int batch, 
   a.valid = (int*)(b + L.valid);
   a.status = &((WsHeader*)ws)->status;
   k_asm_propagator<<<grid_for((size_t)d.N * d.N, 256, sm_count()), 256, 0, s>>>(d.N, ms.pixel_size, ms.wavelength, ms.dz,
-                                                                          (float2*)(b + L.Hf));
+                                                                          d.N > 128, (float2*)(b + L.Hf));
   *err = cudaGetLastError();
   return L;
 }
