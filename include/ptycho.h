@@ -122,11 +122,10 @@ typedef struct {
  *   [0] the per-position pass: window 16: CTA sizes default / alternative; the
  *       others have one (window 128 accepts 0, 1 and 2, windows 32 and 64 accept
  *       0 and 1 for it);
- *   [1] the step-size pass: one kernel per position (0), or the partial sums
- *       spread over 8 chunks of every position, then a
- *       per-position solve and update (1), or (windows <= 128) a cluster of 4
- *       CTAs per position adding their partial sums over distributed shared
- *       memory, at 4 (2) or 3 (3) CTAs per SM;
+ *   [1] the step-size pass: one CTA per position or two launches that walk over
+ *       the positions, by the size of the minibatch (0), the two launches (1),
+ *       or (windows <= 128) a cluster of 4 CTAs per position adding their
+ *       partial sums over distributed shared memory, at 4 (2) or 3 (3) CTAs per SM;
  *   [2] the probe reduction: 16 (0), 8 (1) or 32 (2) positions in flight per
  *       thread, or the minibatch split into 4 ranges summed by 4 threads of
  *       a block with 8 positions in flight each (3). */

@@ -126,14 +126,16 @@ __global__ void k_probe_reduce(int NN, int k0, int Mc, int Ms, int nb, const flo
 
 // dP_k = dPacc_k / (Dp + delta_p max(Dp)); Cp = sum_k conj(P_k) dP_k; Sdp = sum_k |dP_k|^2.
 // The loads of up to KB modes are issued together (one L2 round trip per KB
-// modes instead of one per mode); the sums run over k in order.
+// modes instead of one per mode); the sums run over k in order. Also zeroes
+// the minibatch's step-size sums (nzero doubles).
 constexpr int kModeChunk = 8;
 __global__ void k_norm_probe(int NN, int M, const float2* __restrict__ dPacc, const float* __restrict__ Dp,
                              const float2* __restrict__ probe, float delta_p, int update_probe,
                              const BatchScalars* sc, float2* __restrict__ dP, float2* __restrict__ Cp,
-                             float* __restrict__ Sdp) {
+                             float* __restrict__ Sdp, double* __restrict__ zero, int nzero) {
   constexpr int KB = kModeChunk;
   wait_prior_grid();
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nzero; i += gridDim.x * blockDim.x) zero[i] = 0.0;
   const float damp = delta_p * __uint_as_float(sc->max_dp);
   for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < NN; p += gridDim.x * blockDim.x) {
     float2 c = make_float2(0.f, 0.f);
@@ -330,7 +332,7 @@ Layout make_layout(const ptycho_dims& d, int B, int K, bool epoch_object) {
     L.gram = take((size_t)B * (OPR_KMAX * (OPR_KMAX + 1) / 2 + OPR_KMAX) * sizeof(double));   // weight-step sums
   }
   L.possum = take((size_t)B * 5 * sizeof(double));
-  L.p2part = take((size_t)B * P2_CHUNKS * 5 * sizeof(double));
+  L.p2part = take((size_t)B * 5 * sizeof(double));
   L.dOe = epoch_object ? take(HW * sizeof(float2)) : 0;
   L.dft = 0;
   switch (d.N) {
@@ -446,8 +448,8 @@ struct TuneKey {
   }
 };
 // v[0]: the per-position pass (candidates: pass1_variants(N)), v[1]: the
-// step-size pass (candidates: pass2_variants(N): single kernel, split, cluster
-// at 4 or 3 CTAs per SM), v[2]: the probe reduction (positions
+// step-size pass (candidates: pass2_variants(N): by the minibatch, two launches,
+// cluster at 4 or 3 CTAs per SM), v[2]: the probe reduction (positions
 // in flight per thread: 16, 8, 32, or 8 in each of 4 threads splitting the
 // batch); ms[i][c]: candidate c's mean time.
 struct TuneEntry {
@@ -542,10 +544,10 @@ int grid_for(size_t n, int threads, int cap) {
 
 cudaError_t norm_probe(int NN, int M, const float2* dPacc, const float* Dp, const float2* probe, float delta_p,
                        int update_probe, const BatchScalars* sc, float2* dP, float2* Cp, float* Sdp,
-                       cudaStream_t s) {
+                       cudaStream_t s, double* zero, int nzero) {
   return timed(K_NORM_PROBE, s, [&] {
     return launch_pdl(k_norm_probe, dim3(grid_for(NN, 128, 2 * sm_count())), dim3(128), 0, s, NN, M, dPacc, Dp, probe, delta_p,
-                      update_probe, sc, dP, Cp, Sdp);
+                      update_probe, sc, dP, Cp, Sdp, zero, nzero);
   });
 }
 
@@ -667,7 +669,8 @@ static ptycho_status autotune(const ptycho_dims& d, float2* obj, float2* probe, 
                           o.update_probe ? w.Dp : nullptr, w.acc, HW, sc, s, 0, v);
     });
   t->v[2] = best(t->ms[2], kReduceVariants);
-  if (norm_probe(NN, M, w.dPacc, w.Dp, probe, (float)o.delta_p, o.update_probe, sc, w.dP, w.Cp, w.Sdp, s) !=
+  if (norm_probe(NN, M, w.dPacc, w.Dp, probe, (float)o.delta_p, o.update_probe, sc, w.dP, w.Cp, w.Sdp, s,
+                 w.p2part, nb * 5) !=
       cudaSuccess)
     return PTYCHO_ERR_CUDA;
   t->v[1] = 0;
@@ -759,7 +762,7 @@ ptycho_status run_epoch(const ptycho_dims& d, float2* obj, float2* probe, float*
       return PTYCHO_ERR_CUDA;
     if (tiles && tile_illum_max(d, nb, b0, pos, order, w.valid, w.acc, sc, s) != cudaSuccess) return PTYCHO_ERR_CUDA;
     if ((e = norm_probe(NN, M, w.dPacc, w.Dp, probe, (float)o.delta_p, o.update_probe, sc, w.dP, w.Cp, w.Sdp,
-                        s)) != cudaSuccess)
+                        s, w.p2part, nb * 5)) != cudaSuccess)
       return PTYCHO_ERR_CUDA;
     Pass2Args q;
     memset(&q, 0, sizeof(q));

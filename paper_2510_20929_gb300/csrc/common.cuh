@@ -105,13 +105,8 @@ struct Pass2Args {
   const float* opr_w;   // [J, K]
   int K;
   const float2* p0_s;   // [B, N, N] primary mode of each slot
-  // Split form (k_pass2_sums + k_pass2_update): partial sums of the five
-  // step-size terms per slot and chunk, FP64 [B, P2_CHUNKS, 5]; null selects
-  // the single-kernel form.
-  double* part;
+  double* part;         // [B, 5] sums of the step-size system, zero before the pass
 };
-
-constexpr int P2_CHUNKS = 8;   // chunks of a position's pixels and h planes in the split step-size pass
 
 // Arguments of the multislice per-position pass (kernels_ms.cuh).
 // Incident wave of slice s (1..S-1) of mode k in the slot's scratch: kept per
@@ -189,17 +184,6 @@ __device__ __forceinline__ float4 opr_pair(const float2* __restrict__ V, const f
     const float4 u = __ldg((const float4*)(V + (size_t)m * NN + p));
     const float w = wj[m];
     s.x = fmaf(w, u.x, s.x); s.y = fmaf(w, u.y, s.y); s.z = fmaf(w, u.z, s.z); s.w = fmaf(w, u.w, s.w);
-  }
-  return s;
-}
-
-// sum_m wj[m] V_m at one pixel.
-__device__ __forceinline__ float2 opr_pixel(const float2* __restrict__ V, const float* wj, int K, int NN, int p) {
-  float2 s = make_float2(0.f, 0.f);
-#pragma unroll 4
-  for (int m = 0; m < K; ++m) {
-    const float2 u = __ldg(V + (size_t)m * NN + p);
-    s.x = fmaf(wj[m], u.x, s.x); s.y = fmaf(wj[m], u.y, s.y);
   }
   return s;
 }

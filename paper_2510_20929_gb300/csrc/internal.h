@@ -14,7 +14,7 @@ struct Layout {
   size_t hdr, acc, psi, o, g, h, dPacc, Dp, dP, Sp, Cp, Sdp, valid;
   size_t p0, dUacc, Du, dU, gram;   // orthogonal probe relaxation (K > 0) only
   size_t possum;                     // position-correction sums [B, 5] (FP64)
-  size_t p2part;                     // partial step-size sums [B, P2_CHUNKS, 5] (FP64)
+  size_t p2part;                     // step-size sums [B, 5] (FP64)
   size_t dOe;                        // epoch object accumulator [H, W] (object_per_epoch) or 0
   size_t dft;                        // DFT-matrix chunks of the split-BF16 DFT-GEMM (N <= 128) or 0
   size_t total;
@@ -80,7 +80,7 @@ cudaError_t probe_reduce(int NN, int k0, int Mc, int Ms, int nb, const float2* h
                          BatchScalars* sc, cudaStream_t s, int o_stride = 0, int variant = kReduceDefault);
 cudaError_t norm_probe(int NN, int M, const float2* dPacc, const float* Dp, const float2* probe, float delta_p,
                        int update_probe, const BatchScalars* sc, float2* dP, float2* Cp, float* Sdp,
-                       cudaStream_t s);
+                       cudaStream_t s, double* zero = nullptr, int nzero = 0);
 cudaError_t probe_update(int NN, int M, float2* probe, const float2* dP, float* Sp, int update_probe,
                          const BatchScalars* sc, BatchScalars* sc_next, cudaStream_t s, float4* clear = nullptr,
                          size_t nclear = 0);

@@ -14,9 +14,7 @@
 //   object-frame accumulators (the LSQML preconditioner) with vector atomics,
 //   or, in gradient mode, S_j^T of the object gradient and the position
 //   gradient through the bilinear weights.
-// k_pass2: one CTA per position: the five reductions of the per-position
-//   least-squares step (LSQML's self-adaptive step sizes, Sec. 2.2), the
-//   FP64 2x2 solve, and the alpha-weighted object scatter.
+// The step-size pass is in pass2.cuh.
 #pragma once
 #include <cooperative_groups.h>
 #include "common.cuh"
@@ -509,9 +507,6 @@ __global__ void __launch_bounds__(T, 1) k_pass1(BatchArgs a) {
 }
 
 
-// CTA sizes of the step-size pass (default, alternative).
-constexpr int PASS2_T = 512;
-
 // Bilinear sample of dO_hat = dO_acc / (illum + damp) at the patch pixel whose
 // four corners start at q (the quotient is taken per corner, then interpolated).
 __device__ __forceinline__ float2 dohat(const float4* q, int W, float w00, float w01, float w10, float w11,
@@ -522,489 +517,6 @@ __device__ __forceinline__ float2 dohat(const float4* q, int W, float w00, float
   return make_float2(q00.x * i00 + q01.x * i01 + q10.x * i10 + q11.x * i11,
                      q00.y * i00 + q01.y * i01 + q10.y * i10 + q11.y * i11);
 }
-
-template <int N, int T, bool OPR>
-__global__ void __launch_bounds__(T, 1024 / T) k_pass2(Pass2Args a) {
-  constexpr int NN = N * N;
-  wait_prior_grid();
-  __shared__ double red[32 * 5];
-  __shared__ double alpha_sh;
-  const int slot = blockIdx.x, tid = threadIdx.x;
-  if (!a.valid[slot]) return;
-  const int e = a.b0 + slot;
-  const int j = a.order ? a.order[e] : e;
-  int ty, tx;
-  float fy, fx;
-  tile_of(a.pos[2 * j], a.pos[2 * j + 1], N, a.H, a.W, ty, tx, fy, fx);
-  const float w00 = (1.f - fy) * (1.f - fx), w01 = (1.f - fy) * fx, w10 = fy * (1.f - fx), w11 = fy * fx;
-  const float damp = a.delta_o * __uint_as_float(a.sc->max_illum);
-  const size_t slotNN = (size_t)slot * NN;
-  const int M = a.M;
-  const float2* g_s = a.g_s + slotNN;
-  const float2* o_s = a.o_s + slotNN;
-  const float2* h_s = a.h_s + slotNN * M;
-  // OPR: the primary mode P_j0 and its direction sum_m w_jm dU_m differ per
-  // position; Sp, Cp, Sdp and dP then hold the shared modes only
-  constexpr bool opr = OPR;
-  __shared__ float wsh[OPR_KMAX];
-  if (opr) {
-    if (tid < a.K) wsh[tid] = a.opr_w[(size_t)j * a.K + tid];
-    __syncthreads();
-  }
-  const float2* p0 = opr ? a.p0_s + slotNN : nullptr;
-
-  float A11 = 0.f, A12 = 0.f, A22 = 0.f, b1 = 0.f, b2 = 0.f;
-  {
-    // two adjacent pixels per iteration: 16-byte loads of g, o and Cp, and the
-    // six accumulator corners the pair shares (half the trips of this
-    // latency-bound loop); with OPR also the pair's primary mode, its
-    // direction sum_m w_jm dU_m (K 16-byte loads) and h_j0
-#pragma unroll 1
-    for (int p = 2 * tid; p < NN; p += 2 * T) {
-      const int r = p / N, c = p % N;
-      const float4 g2 = __ldg((const float4*)(g_s + p));   // kept in L2: the update reads g again
-      const float4 o2 = __ldcs((const float4*)(o_s + p));
-      float2 d0 = make_float2(0.f, 0.f), d1 = d0;
-      if (a.update_object) {
-        const float4* q = a.acc + (size_t)(ty + r) * a.W + (tx + c);
-        const float4 qa = __ldg(q), qb = __ldg(q + 1), qc = __ldg(q + 2);
-        const float4 qd = __ldg(q + a.W), qe = __ldg(q + a.W + 1), qf = __ldg(q + a.W + 2);
-        const float ia = 1.f / (qa.z + damp), ib = 1.f / (qb.z + damp), ic = 1.f / (qc.z + damp);
-        const float id = 1.f / (qd.z + damp), ie = 1.f / (qe.z + damp), iF = 1.f / (qf.z + damp);
-        // dO_hat at the pixel: each corner's quotient, then the bilinear weights
-        d0 = make_float2(w00 * ia * qa.x + w01 * ib * qb.x + w10 * id * qd.x + w11 * ie * qe.x,
-                         w00 * ia * qa.y + w01 * ib * qb.y + w10 * id * qd.y + w11 * ie * qe.y);
-        d1 = make_float2(w00 * ib * qb.x + w01 * ic * qc.x + w10 * ie * qe.x + w11 * iF * qf.x,
-                         w00 * ib * qb.y + w01 * ic * qc.y + w10 * ie * qe.y + w11 * iF * qf.y);
-      }
-      float2 sp = __ldg((const float2*)(a.Sp + p)), sdp = __ldg((const float2*)(a.Sdp + p));
-      float4 cp = __ldg((const float4*)(a.Cp + p));
-      if constexpr (OPR) {
-        const float4 P2 = *(const float4*)(p0 + p);
-        const float2 Pa = make_float2(P2.x, P2.y), Pb = make_float2(P2.z, P2.w);
-        sp.x += cabs2(Pa);
-        sp.y += cabs2(Pb);
-        if (a.update_probe) {
-          const float4 D2 = opr_pair(a.opr_dU, wsh, a.K, NN, p);
-          const float2 ea = make_float2(D2.x, D2.y), eb = make_float2(D2.z, D2.w);
-          const float2 ca = cmulc(Pa, ea), cb = cmulc(Pb, eb);
-          cp = make_float4(cp.x + ca.x, cp.y + ca.y, cp.z + cb.x, cp.w + cb.y);
-          sdp.x += cabs2(ea);
-          sdp.y += cabs2(eb);
-          const float4 h2 = __ldcs((const float4*)(h_s + p));
-          b2 += ea.x * h2.x + ea.y * h2.y + eb.x * h2.z + eb.y * h2.w;   // Re(conj(dP_j0) h_j0)
-        }
-      }
-      const float2 g0 = make_float2(g2.x, g2.y), g1 = make_float2(g2.z, g2.w);
-      const float2 o0 = make_float2(o2.x, o2.y), o1 = make_float2(o2.z, o2.w);
-      A11 += cabs2(d0) * sp.x + cabs2(d1) * sp.y;
-      const float2 od0 = cmulc(d0, o0), od1 = cmulc(d1, o1);   // conj(d) o
-      A12 += od0.x * cp.x - od0.y * cp.y + od1.x * cp.z - od1.y * cp.w;   // Re(conj(d) o Cp)
-      A22 += cabs2(o0) * sdp.x + cabs2(o1) * sdp.y;
-      b1 += d0.x * g0.x + d0.y * g0.y + d1.x * g1.x + d1.y * g1.y;       // Re(conj(d) g)
-    }
-  }
-  if (a.update_probe) {
-    // b2 = Re sum_k <dP_k, h_k> over the shared modes: their planes are
-    // contiguous, two pixels per 16-byte load
-    const float4* h4 = (const float4*)(h_s + (opr ? NN : 0));
-    const float4* d4 = (const float4*)a.dP;
-    const int Q = (opr ? M - 1 : M) * NN / 2;
-    int q = tid;
-    for (; q + 3 * T < Q; q += 4 * T) {      // four independent 16-byte streams per thread
-      float4 dp[4], h[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        dp[u] = __ldg(d4 + q + u * T);
-        h[u] = __ldcs(h4 + q + u * T);
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) b2 += dp[u].x * h[u].x + dp[u].y * h[u].y + dp[u].z * h[u].z + dp[u].w * h[u].w;
-    }
-    for (; q < Q; q += T) {
-      const float4 dp = __ldg(d4 + q);
-      const float4 h = __ldcs(h4 + q);
-      b2 += dp.x * h.x + dp.y * h.y + dp.z * h.z + dp.w * h.w;   // Re(conj(dP_k) h_k)
-    }
-  }
-  double v[5] = {A11, A12, A22, b1, b2};
-  block_sum<5>(v, red);
-  if (tid == 0) {
-    const double a11 = v[0], a12 = v[1], a22 = v[2], r1 = v[3], r2 = v[4];
-    const double tr = 0.5 * (a11 + a22);
-    const double d11 = a11 + a.lam * tr, d22 = a22 + a.lam * tr;
-    const double det = d11 * d22 - a12 * a12;
-    double aO, aP;
-    if (det > 0.0) {
-      aO = (d22 * r1 - a12 * r2) / det;
-      aP = (d11 * r2 - a12 * r1) / det;
-    } else {
-      aO = d11 > 0.0 ? r1 / d11 : 0.0;
-      aP = d22 > 0.0 ? r2 / d22 : 0.0;
-    }
-    alpha_sh = aO;
-    if (a.alpha_out) {
-      a.alpha_out[2 * j] = aO;
-      a.alpha_out[2 * j + 1] = aP;
-    }
-    atomicAdd(&a.sc->sum_alpha_p, aP);
-    atomicAdd(&a.sc->count, 1);
-  }
-  __syncthreads();
-  if (!a.update_object) return;
-  // O += alpha_O S_j^T g / (illum + delta_O): each object pixel of the (N+1)^2 tile
-  // gathers its four patch neighbours and is divided by its own preconditioner
-  const float aO = (float)alpha_sh;
-  const float c00 = aO * w00, c01 = aO * w01, c10 = aO * w10, c11 = aO * w11;
-  constexpr int N1 = N + 1;
-  if (((uintptr_t)a.obj & 15) == 0 && (a.W & 1) == 0) {
-    // pairs of object pixels at even object columns, one 16-byte vector atomic
-    // each (half the atomic operations); per tile row N/2 pairs and one single
-    // pixel (the first when tx is odd, else the last)
-    constexpr int PR = N / 2 + 1;
-    const int odd = tx & 1;
-    auto gat = [&](int y, int x) {
-      return (y >= 0 && y < N && x >= 0 && x < N) ? g_s[y * N + x] : make_float2(0.f, 0.f);
-    };
-    for (int i = tid; i < N1 * PR; i += T) {
-      const int y = i / PR, k = i % PR;
-      const size_t row = (size_t)(ty + y) * a.W + tx;
-      if (k < N / 2) {
-        const int x = 2 * k + odd;   // pixels x, x + 1 of the tile row
-        const float2 gA = gat(y, x - 1), gB = gat(y, x), gC = gat(y, x + 1);
-        const float2 hA = gat(y - 1, x - 1), hB = gat(y - 1, x), hC = gat(y - 1, x + 1);
-        const float2 s0 = make_float2(c00 * gB.x + c01 * gA.x + c10 * hB.x + c11 * hA.x,
-                                      c00 * gB.y + c01 * gA.y + c10 * hB.y + c11 * hA.y);
-        const float2 s1 = make_float2(c00 * gC.x + c01 * gB.x + c10 * hC.x + c11 * hB.x,
-                                      c00 * gC.y + c01 * gB.y + c10 * hC.y + c11 * hB.y);
-        const float i0 = 1.f / (__ldg(&a.acc[row + x].z) + damp);
-        const float i1 = 1.f / (__ldg(&a.acc[row + x + 1].z) + damp);
-        atomicAdd((float4*)(a.obj + row + x), make_float4(s0.x * i0, s0.y * i0, s1.x * i1, s1.y * i1));
-      } else {
-        const int x = odd ? 0 : N;
-        const float2 gA = gat(y, x - 1), gB = gat(y, x), hA = gat(y - 1, x - 1), hB = gat(y - 1, x);
-        const float2 s0 = make_float2(c00 * gB.x + c01 * gA.x + c10 * hB.x + c11 * hA.x,
-                                      c00 * gB.y + c01 * gA.y + c10 * hB.y + c11 * hA.y);
-        const float i0 = 1.f / (__ldg(&a.acc[row + x].z) + damp);
-        atomicAdd(a.obj + row + x, make_float2(s0.x * i0, s0.y * i0));
-      }
-    }
-    return;
-  }
-  // each object pixel of the (N+1)^2 tile gathers its four patch neighbours
-  // (independent outputs keep many global loads in flight)
-  for (int q = tid; q < N1 * N1; q += T) {
-    const int y = q / N1, x = q % N1;
-    float2 sacc = make_float2(0.f, 0.f);
-    if (y < N && x < N) { const float2 g = g_s[y * N + x]; sacc.x += c00 * g.x; sacc.y += c00 * g.y; }
-    if (y < N && x > 0) { const float2 g = g_s[y * N + x - 1]; sacc.x += c01 * g.x; sacc.y += c01 * g.y; }
-    if (y > 0 && x < N) { const float2 g = g_s[(y - 1) * N + x]; sacc.x += c10 * g.x; sacc.y += c10 * g.y; }
-    if (y > 0 && x > 0) { const float2 g = g_s[(y - 1) * N + x - 1]; sacc.x += c11 * g.x; sacc.y += c11 * g.y; }
-    const size_t oi = (size_t)(ty + y) * a.W + (tx + x);
-    const float inv = 1.f / (__ldg(&a.acc[oi].z) + damp);
-    atomicAdd(a.obj + oi, make_float2(sacc.x * inv, sacc.y * inv));
-  }
-}
-
-// Split form of the step-size pass. The five sums of a position are
-// independent over its pixels and its h planes, so k_pass2_sums spreads them
-// over P2_CHUNKS CTAs per position (every CTA a pure stream of 16-byte loads,
-// many CTAs per SM); each writes its FP64 partials without atomics, and
-// k_pass2_update adds a position's partials in chunk order (the result does
-// not depend on scheduling), solves the 2x2 system and scatters the object
-// update.
-constexpr int PASS2S_T = 256, PASS2U_T = 512;
-
-template <int N, bool OPR>
-__global__ void __launch_bounds__(PASS2S_T, 3) k_pass2_sums(Pass2Args a) {
-  constexpr int NN = N * N, T = PASS2S_T, C = P2_CHUNKS;
-  static_assert(NN % (2 * C) == 0, "chunks of pixel pairs");
-  wait_prior_grid();
-  __shared__ double red[32 * 5];
-  __shared__ float wsh[OPR_KMAX];
-  const int chunk = blockIdx.x, slot = blockIdx.y, tid = threadIdx.x;
-  double* out = a.part + ((size_t)slot * C + chunk) * 5;
-  if (!a.valid[slot]) {
-    if (tid < 5) out[tid] = 0.0;
-    return;
-  }
-  const int e = a.b0 + slot;
-  const int j = a.order ? a.order[e] : e;
-  int ty, tx;
-  float fy, fx;
-  tile_of(a.pos[2 * j], a.pos[2 * j + 1], N, a.H, a.W, ty, tx, fy, fx);
-  const float w00 = (1.f - fy) * (1.f - fx), w01 = (1.f - fy) * fx, w10 = fy * (1.f - fx), w11 = fy * fx;
-  const float damp = a.delta_o * __uint_as_float(a.sc->max_illum);
-  const size_t slotNN = (size_t)slot * NN;
-  const int M = a.M;
-  const float2* g_s = a.g_s + slotNN;
-  const float2* o_s = a.o_s + slotNN;
-  const float2* h_s = a.h_s + slotNN * M;
-  if (OPR) {
-    if (tid < a.K) wsh[tid] = a.opr_w[(size_t)j * a.K + tid];
-    __syncthreads();
-  }
-  const float2* p0 = OPR ? a.p0_s + slotNN : nullptr;
-
-  // pixels [p_lo, p_hi) of the patch
-  const int p_lo = chunk * (NN / C), p_hi = p_lo + NN / C;
-  float A11 = 0.f, A12 = 0.f, A22 = 0.f, b1 = 0.f, b2 = 0.f;
-#pragma unroll 1
-  for (int p = p_lo + tid; p < p_hi; p += T) {
-    const int r = p / N, c = p % N;
-    const float2 g = __ldcs(g_s + p);
-    const float2 o = __ldcs(o_s + p);
-    float2 d = make_float2(0.f, 0.f);
-    if (a.update_object) d = dohat(a.acc + (size_t)(ty + r) * a.W + (tx + c), a.W, w00, w01, w10, w11, damp);
-    float sp = __ldg(a.Sp + p), sdp = __ldg(a.Sdp + p);
-    float2 cp = __ldg(a.Cp + p);
-    if (OPR) {
-      const float2 P0 = p0[p];
-      sp += cabs2(P0);
-      if (a.update_probe) {
-        const float2 d0 = opr_pixel(a.opr_dU, wsh, a.K, NN, p);
-        cp = cadd(cp, cmulc(P0, d0));
-        sdp += cabs2(d0);
-        const float2 h0 = __ldcs(h_s + p);
-        b2 += d0.x * h0.x + d0.y * h0.y;     // Re(conj(dP_j0) h_j0)
-      }
-    }
-    A11 += cabs2(d) * sp;
-    const float2 od = cmulc(d, o);           // conj(d) o
-    A12 += od.x * cp.x - od.y * cp.y;        // Re(conj(d) o Cp)
-    A22 += cabs2(o) * sdp;
-    b1 += d.x * g.x + d.y * g.y;             // Re(conj(d) g)
-  }
-  if (a.update_probe) {
-    // b2 over this chunk of the shared modes' h planes (contiguous pixel pairs)
-    const float4* h4 = (const float4*)(h_s + (OPR ? NN : 0));
-    const float4* d4 = (const float4*)a.dP;
-    const int Q = (OPR ? M - 1 : M) * NN / 2;
-    const int q_lo = (int)((long long)Q * chunk / C), q_hi = (int)((long long)Q * (chunk + 1) / C);
-    int q = q_lo + tid;
-    for (; q + 3 * T < q_hi; q += 4 * T) {      // four independent 16-byte streams per thread
-      float4 dp[4], h[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        dp[u] = __ldg(d4 + q + u * T);
-        h[u] = __ldcs(h4 + q + u * T);
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) b2 += dp[u].x * h[u].x + dp[u].y * h[u].y + dp[u].z * h[u].z + dp[u].w * h[u].w;
-    }
-    for (; q < q_hi; q += T) {
-      const float4 dp = __ldg(d4 + q);
-      const float4 h = __ldcs(h4 + q);
-      b2 += dp.x * h.x + dp.y * h.y + dp.z * h.z + dp.w * h.w;   // Re(conj(dP_k) h_k)
-    }
-  }
-  double v[5] = {A11, A12, A22, b1, b2};
-  block_sum<5>(v, red);
-  if (tid == 0)
-#pragma unroll
-    for (int i = 0; i < 5; ++i) out[i] = v[i];
-}
-
-template <int N>
-__global__ void __launch_bounds__(PASS2U_T, 2) k_pass2_update(Pass2Args a) {
-  constexpr int T = PASS2U_T, C = P2_CHUNKS;
-  wait_prior_grid();
-  __shared__ double alpha_sh;
-  const int slot = blockIdx.x, tid = threadIdx.x;
-  if (!a.valid[slot]) return;
-  const int e = a.b0 + slot;
-  const int j = a.order ? a.order[e] : e;
-  if (tid == 0) {
-    const double* pp = a.part + (size_t)slot * C * 5;
-    double v[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-    for (int c = 0; c < C; ++c)
-#pragma unroll
-      for (int i = 0; i < 5; ++i) v[i] += pp[c * 5 + i];
-    const double a11 = v[0], a12 = v[1], a22 = v[2], r1 = v[3], r2 = v[4];
-    const double tr = 0.5 * (a11 + a22);
-    const double d11 = a11 + a.lam * tr, d22 = a22 + a.lam * tr;
-    const double det = d11 * d22 - a12 * a12;
-    double aO, aP;
-    if (det > 0.0) {
-      aO = (d22 * r1 - a12 * r2) / det;
-      aP = (d11 * r2 - a12 * r1) / det;
-    } else {
-      aO = d11 > 0.0 ? r1 / d11 : 0.0;
-      aP = d22 > 0.0 ? r2 / d22 : 0.0;
-    }
-    alpha_sh = aO;
-    if (a.alpha_out) {
-      a.alpha_out[2 * j] = aO;
-      a.alpha_out[2 * j + 1] = aP;
-    }
-    atomicAdd(&a.sc->sum_alpha_p, aP);
-    atomicAdd(&a.sc->count, 1);
-  }
-  __syncthreads();
-  if (!a.update_object) return;
-  int ty, tx;
-  float fy, fx;
-  tile_of(a.pos[2 * j], a.pos[2 * j + 1], N, a.H, a.W, ty, tx, fy, fx);
-  const float damp = a.delta_o * __uint_as_float(a.sc->max_illum);
-  const float2* g_s = a.g_s + (size_t)slot * N * N;
-  const float aO = (float)alpha_sh;
-  const float c00 = aO * (1.f - fy) * (1.f - fx), c01 = aO * (1.f - fy) * fx;
-  const float c10 = aO * fy * (1.f - fx), c11 = aO * fy * fx;
-  constexpr int N1 = N + 1;
-  // O += alpha_O S_j^T g / (illum + delta_O): each object pixel of the (N+1)^2
-  // tile gathers its four patch neighbours, divided by its own preconditioner
-  for (int q = tid; q < N1 * N1; q += T) {
-    const int y = q / N1, x = q % N1;
-    float2 sacc = make_float2(0.f, 0.f);
-    if (y < N && x < N) { const float2 g = g_s[y * N + x]; sacc.x += c00 * g.x; sacc.y += c00 * g.y; }
-    if (y < N && x > 0) { const float2 g = g_s[y * N + x - 1]; sacc.x += c01 * g.x; sacc.y += c01 * g.y; }
-    if (y > 0 && x < N) { const float2 g = g_s[(y - 1) * N + x]; sacc.x += c10 * g.x; sacc.y += c10 * g.y; }
-    if (y > 0 && x > 0) { const float2 g = g_s[(y - 1) * N + x - 1]; sacc.x += c11 * g.x; sacc.y += c11 * g.y; }
-    const size_t oi = (size_t)(ty + y) * a.W + (tx + x);
-    const float inv = 1.f / (__ldg(&a.acc[oi].z) + damp);
-    atomicAdd(a.obj + oi, make_float2(sacc.x * inv, sacc.y * inv));
-  }
-}
-
-// Cluster form of the step-size pass (N <= 128): the PASS2C_C CTAs of a
-// cluster share one position. CTA q reduces rows [q N/C, (q+1) N/C) of the
-// patch and chunk q of the h planes and keeps its rows of g in shared memory;
-// the C partial sums meet over distributed shared memory and are added in
-// rank order, so every CTA holds the same FP64 totals and solves the 2x2
-// system itself; then CTA q scatters the object update of its band of the
-// (N+1)^2 tile (rows q N/C .. (q+1) N/C - 1, the last band also row N) from
-// its own rows of g and, for its first row, the row above from L2. Against
-// one CTA per position: four times the CTAs (the minibatch no longer leaves
-// some SMs with one position and others with two), the serial solve of one
-// cluster overlaps the streams of the others, and g is read once.
-constexpr int PASS2C_T = 256, PASS2C_C = 4;
-
-template <int N, int MINB>
-__global__ void __cluster_dims__(PASS2C_C, 1, 1) __launch_bounds__(PASS2C_T, MINB) k_pass2_cluster(Pass2Args a) {
-  constexpr int NN = N * N, T = PASS2C_T, C = PASS2C_C, RB = N / C, N1 = N + 1;
-  static_assert(N % C == 0 && N <= 128, "bands of whole rows, g band in static shared memory");
-  wait_prior_grid();
-  cg::cluster_group cluster = cg::this_cluster();
-  __shared__ double red[32 * 5];
-  __shared__ double part[5];
-  __shared__ double alpha_sh;
-  __shared__ __align__(16) float2 gsh[RB * N];
-  const int q = (int)cluster.block_rank();
-  const int slot = blockIdx.x / C, tid = threadIdx.x;
-  if (!a.valid[slot]) return;   // the same decision in every CTA of the cluster
-  const int e = a.b0 + slot;
-  const int j = a.order ? a.order[e] : e;
-  int ty, tx;
-  float fy, fx;
-  tile_of(a.pos[2 * j], a.pos[2 * j + 1], N, a.H, a.W, ty, tx, fy, fx);
-  const float w00 = (1.f - fy) * (1.f - fx), w01 = (1.f - fy) * fx, w10 = fy * (1.f - fx), w11 = fy * fx;
-  const float damp = a.delta_o * __uint_as_float(a.sc->max_illum);
-  const size_t slotNN = (size_t)slot * NN;
-  const int M = a.M;
-  const float2* g_s = a.g_s + slotNN;
-  const float2* o_s = a.o_s + slotNN;
-  const float2* h_s = a.h_s + slotNN * M;
-
-  const int p_lo = q * RB * N;
-  float A11 = 0.f, A12 = 0.f, A22 = 0.f, b1 = 0.f, b2 = 0.f;
-#pragma unroll 1
-  for (int i = tid; i < RB * N; i += T) {
-    const int p = p_lo + i, r = p / N, c = p % N;
-    const float2 g = __ldcs(g_s + p);
-    const float2 o = __ldcs(o_s + p);
-    gsh[i] = g;
-    float2 d = make_float2(0.f, 0.f);
-    if (a.update_object) d = dohat(a.acc + (size_t)(ty + r) * a.W + (tx + c), a.W, w00, w01, w10, w11, damp);
-    const float sp = __ldg(a.Sp + p), sdp = __ldg(a.Sdp + p);
-    const float2 cp = __ldg(a.Cp + p);
-    A11 += cabs2(d) * sp;
-    const float2 od = cmulc(d, o);           // conj(d) o
-    A12 += od.x * cp.x - od.y * cp.y;        // Re(conj(d) o Cp)
-    A22 += cabs2(o) * sdp;
-    b1 += d.x * g.x + d.y * g.y;             // Re(conj(d) g)
-  }
-  if (a.update_probe) {
-    // b2 over chunk q of the h planes (contiguous pixel pairs)
-    const float4* h4 = (const float4*)h_s;
-    const float4* d4 = (const float4*)a.dP;
-    const int Q = M * NN / 2;
-    const int q_lo = (int)((long long)Q * q / C), q_hi = (int)((long long)Q * (q + 1) / C);
-    int k = q_lo + tid;
-    for (; k + 3 * T < q_hi; k += 4 * T) {   // four independent 16-byte streams per thread
-      float4 dp[4], h[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        dp[u] = __ldg(d4 + k + u * T);
-        h[u] = __ldcs(h4 + k + u * T);
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) b2 += dp[u].x * h[u].x + dp[u].y * h[u].y + dp[u].z * h[u].z + dp[u].w * h[u].w;
-    }
-    for (; k < q_hi; k += T) {
-      const float4 dp = __ldg(d4 + k);
-      const float4 h = __ldcs(h4 + k);
-      b2 += dp.x * h.x + dp.y * h.y + dp.z * h.z + dp.w * h.w;   // Re(conj(dP_k) h_k)
-    }
-  }
-  double v[5] = {A11, A12, A22, b1, b2};
-  block_sum<5>(v, red);
-  if (tid == 0)
-#pragma unroll
-    for (int i = 0; i < 5; ++i) part[i] = v[i];
-  cluster.sync();   // every CTA's partials (and its g band) are written
-  if (tid == 0) {
-    double t[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-#pragma unroll
-    for (int r = 0; r < C; ++r) {
-      const double* pr = cluster.map_shared_rank(part, r);
-#pragma unroll
-      for (int i = 0; i < 5; ++i) t[i] += pr[i];
-    }
-    const double a11 = t[0], a12 = t[1], a22 = t[2], r1 = t[3], r2 = t[4];
-    const double tr = 0.5 * (a11 + a22);
-    const double d11 = a11 + a.lam * tr, d22 = a22 + a.lam * tr;
-    const double det = d11 * d22 - a12 * a12;
-    double aO, aP;
-    if (det > 0.0) {
-      aO = (d22 * r1 - a12 * r2) / det;
-      aP = (d11 * r2 - a12 * r1) / det;
-    } else {
-      aO = d11 > 0.0 ? r1 / d11 : 0.0;
-      aP = d22 > 0.0 ? r2 / d22 : 0.0;
-    }
-    alpha_sh = aO;
-    if (q == 0) {
-      if (a.alpha_out) {
-        a.alpha_out[2 * j] = aO;
-        a.alpha_out[2 * j + 1] = aP;
-      }
-      atomicAdd(&a.sc->sum_alpha_p, aP);
-      atomicAdd(&a.sc->count, 1);
-    }
-  }
-  cluster.sync();   // no CTA leaves while another reads its partials; alpha_sh is visible
-  if (!a.update_object) return;
-  const float aO = (float)alpha_sh;
-  const float c00 = aO * w00, c01 = aO * w01, c10 = aO * w10, c11 = aO * w11;
-  const int y0 = q * RB, y1 = y0 + RB + (q == C - 1 ? 1 : 0);
-  // g at patch row yy (y0 - 1 <= yy < y0 + RB): the band from shared memory, the row above from L2
-  auto gat = [&](int yy, int xx) { return yy >= y0 ? gsh[(yy - y0) * N + xx] : __ldg(g_s + yy * N + xx); };
-  for (int i = tid; i < (y1 - y0) * N1; i += T) {
-    const int y = y0 + i / N1, x = i % N1;
-    float2 sacc = make_float2(0.f, 0.f);
-    if (y < N && x < N) { const float2 g = gat(y, x); sacc.x += c00 * g.x; sacc.y += c00 * g.y; }
-    if (y < N && x > 0) { const float2 g = gat(y, x - 1); sacc.x += c01 * g.x; sacc.y += c01 * g.y; }
-    if (y > 0 && x < N) { const float2 g = gat(y - 1, x); sacc.x += c10 * g.x; sacc.y += c10 * g.y; }
-    if (y > 0 && x > 0) { const float2 g = gat(y - 1, x - 1); sacc.x += c11 * g.x; sacc.y += c11 * g.y; }
-    const size_t oi = (size_t)(ty + y) * a.W + (tx + x);
-    const float inv = 1.f / (__ldg(&a.acc[oi].z) + damp);
-    atomicAdd(a.obj + oi, make_float2(sacc.x * inv, sacc.y * inv));
-  }
-}
-
-}  // namespace ptycho
-
-namespace ptycho {
 
 // Opts a kernel into more than 48 KB of dynamic shared memory, once per device
 // (so that no attribute call happens while a stream is being captured).
@@ -1037,29 +549,6 @@ cudaError_t launch_pass1(const BatchArgs& a, cudaStream_t s, int variant) {
   if (a.opr_U) return launch_pass1_t<N, Threads<N>::T, true>(a, s);
   return variant == 1 ? launch_pass1_t<N, Threads<N>::ALT, false>(a, s)
                       : launch_pass1_t<N, Threads<N>::T, false>(a, s);
-}
-
-// variant 0: the single-kernel form of PASS2_T threads, 1: the split form
-// (when the partials buffer is given), 2 and 3: the cluster form at four and
-// three CTAs per SM (64 and 80 registers; N <= 128, not OPR)
-template <int N>
-cudaError_t launch_pass2(const Pass2Args& a, cudaStream_t s, int variant) {
-  if (a.nb <= 0) return cudaSuccess;
-  if constexpr (N <= 128) {
-    if (variant == 2 && !a.opr_dU)
-      return launch_pdl(k_pass2_cluster<N, 4>, dim3(PASS2C_C * a.nb), dim3(PASS2C_T), 0, s, a);
-    if (variant == 3 && !a.opr_dU)
-      return launch_pdl(k_pass2_cluster<N, 3>, dim3(PASS2C_C * a.nb), dim3(PASS2C_T), 0, s, a);
-  }
-  if (a.part && variant == 1) {
-    cudaError_t e = a.opr_dU
-        ? launch_pdl(k_pass2_sums<N, true>, dim3(P2_CHUNKS, a.nb), dim3(PASS2S_T), 0, s, a)
-        : launch_pdl(k_pass2_sums<N, false>, dim3(P2_CHUNKS, a.nb), dim3(PASS2S_T), 0, s, a);
-    if (e != cudaSuccess) return e;
-    return launch_pdl(k_pass2_update<N>, dim3(a.nb), dim3(PASS2U_T), 0, s, a);
-  }
-  if (a.opr_dU) return launch_pdl(k_pass2<N, PASS2_T, true>, dim3(a.nb), dim3(PASS2_T), 0, s, a);
-  return launch_pdl(k_pass2<N, PASS2_T, false>, dim3(a.nb), dim3(PASS2_T), 0, s, a);
 }
 
 }  // namespace ptycho

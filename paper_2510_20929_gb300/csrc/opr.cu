@@ -425,7 +425,7 @@ ptycho_status run_epoch_opr(const ptycho_dims& d, const ptycho_opr_opts& r, floa
       if (cudaGetLastError() != cudaSuccess) return PTYCHO_ERR_CUDA;
     }
     if (norm_probe(NN, M - 1, w.dPacc, w.Dp, P_rest, (float)o.delta_p, o.update_probe, sc, w.dP, w.Cp, w.Sdp,
-                   s) != cudaSuccess)
+                   s, w.p2part, nb * 5) != cudaSuccess)
       return PTYCHO_ERR_CUDA;
     k_norm_opr<<<grid_for(KNN, 256, 2 * sm_count()), 256, 0, s>>>(KNN, w.dUacc, w.Du, o.update_probe, (float)o.delta_p,
                                                              sc, w.dU);

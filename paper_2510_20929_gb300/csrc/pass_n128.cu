@@ -1,6 +1,7 @@
 // Per-position kernels instantiated for the 128 x 128 window.
 #include "kernels_pair.cuh"
 #include "launch.h"
+#include "pass2.cuh"
 
 namespace ptycho {
 template <>

@@ -1,6 +1,7 @@
 // Per-position kernels instantiated for the 16 x 16 window.
 #include "kernels.cuh"
 #include "launch.h"
+#include "pass2.cuh"
 
 namespace ptycho {
 template cudaError_t launch_pass1<16>(const BatchArgs&, cudaStream_t, int);

@@ -1,6 +1,7 @@
 // Per-position kernels instantiated for the 192 x 192 window.
 #include "kernels_pair.cuh"
 #include "launch.h"
+#include "pass2.cuh"
 
 namespace ptycho {
 template <>

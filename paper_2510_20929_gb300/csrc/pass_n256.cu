@@ -1,6 +1,7 @@
 // Per-position kernels instantiated for the 256 x 256 window.
 #include "kernels_pair.cuh"
 #include "launch.h"
+#include "pass2.cuh"
 
 namespace ptycho {
 template <>

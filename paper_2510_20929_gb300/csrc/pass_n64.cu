@@ -1,6 +1,7 @@
 // Per-position kernels instantiated for the 64 x 64 window.
 #include "kernels_pair.cuh"
 #include "launch.h"
+#include "pass2.cuh"
 
 namespace ptycho {
 template <>
