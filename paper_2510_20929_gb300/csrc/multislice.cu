@@ -13,7 +13,7 @@
 #include "internal.h"
 #include "launch.h"
 #include "profile.h"
-#include "kernels.cuh"
+#include "pass2.cuh"
 
 namespace ptycho {
 
@@ -169,75 +169,90 @@ __global__ void k_ms_illum_max(size_t HW, const float4* __restrict__ acc, unsign
   if (threadIdx.x == 0) atomicMax(smax + blockIdx.y, __float_as_uint(m));
 }
 
-// One CTA per (position, slice): the slice's preconditioned direction at the
-// position, d_s = S_j(dO_acc_s / (illum_s + delta_O,s)) (bilinear, the
-// quotient taken per corner), into scratch for the tangent pass, and the
-// right-hand-side term Re<d_s, g_s>; the slice-0 CTA adds the probe's
-// Re sum_k <dP_k, h_k>.
+// One CTA per 32 rows of a (position, slice): the slice's preconditioned
+// direction at the position, d_s = S_j(dO_acc_s / (illum_s + delta_O,s))
+// (bilinear, the quotient taken per corner), into scratch for the tangent pass,
+// and the right-hand-side term Re<d_s, g_s>; the CTAs of slice s add the
+// probe's Re <dP_k, h_k> of the modes k = s, s + S, .. over their rows. A thread
+// takes two adjacent pixels at a time, which share two of their six
+// accumulator corners, with 16-byte loads and stores. The partial sums meet in
+// FP64 (dsum, zero on entry).
+// Bound by the latency of the loads; one CTA per (position, slice) reading
+// pixel by pixel left a third of the GPU idle in its last wave:
+// MSFIG
 template <int N>
-__global__ void __launch_bounds__(512, 1) k_ms_dir(MsPass2Args a) {
-  constexpr int NN = N * N, T = 512;
+__global__ void __launch_bounds__(UPD_T, 4) k_ms_dir(MsPass2Args a) {
+  constexpr int NN = N * N, T = UPD_T, PAIRS = Bands<N>::ROWS * N / 2;
+  wait_prior_grid();
   __shared__ double red[32 * 2];
-  const int slot = blockIdx.x, s = blockIdx.y, tid = threadIdx.x, S = a.S;
-  double* out = a.dsum + ((size_t)slot * S + s) * 2;
-  if (!a.valid[slot]) {
-    if (tid < 2) out[tid] = 0.0;
-    return;
-  }
+  const int slot = blockIdx.x / Bands<N>::NUM, band = blockIdx.x % Bands<N>::NUM;
+  const int s = blockIdx.y, tid = threadIdx.x, S = a.S;
+  if (!a.valid[slot]) return;
   const int e = a.b0 + slot;
   const int j = a.order ? a.order[e] : e;
   int ty, tx;
   float fy, fx;
   tile_of(a.pos[2 * j], a.pos[2 * j + 1], N, a.H, a.W, ty, tx, fy, fx);
   const float w00 = (1.f - fy) * (1.f - fx), w01 = (1.f - fy) * fx, w10 = fy * (1.f - fx), w11 = fy * fx;
-  const size_t HW = (size_t)a.H * a.W;
-  const float4* acc = a.acc + s * HW;
+  const float4* acc = a.acc + (size_t)s * a.H * a.W;
   const float damp = a.delta_o * __uint_as_float(a.smax[s]);
-  const float2* g_s = a.go_s + ((size_t)slot * S + s) * NN;
-  float2* d_s = a.d_s + ((size_t)slot * S + s) * NN;
+  const size_t base = ((size_t)slot * S + s) * NN;
+  const int p0 = band * PAIRS * 2;   // the band's first pixel
   float b1 = 0.f, b2 = 0.f;
-#pragma unroll 1
-  for (int p = tid; p < NN; p += T) {
-    const int r = p / N, c = p % N;
-    float2 d = make_float2(0.f, 0.f);
-    if (a.update_object) d = dohat(acc + (size_t)(ty + r) * a.W + (tx + c), a.W, w00, w01, w10, w11, damp);
-    d_s[p] = d;
-    const float2 g = __ldcs(g_s + p);
-    b1 += d.x * g.x + d.y * g.y;             // Re(conj(d) g)
-  }
-  if (s == 0 && a.update_probe) {
-    const float4* h4 = (const float4*)(a.h_s + (size_t)slot * a.M * NN);
-    const float4* d4 = (const float4*)a.dP;
-    const int Qp = a.M * NN / 2;
-    for (int q = tid; q < Qp; q += T) {
-      const float4 dp = __ldg(d4 + q);
-      const float4 h = __ldcs(h4 + q);
-      b2 += dp.x * h.x + dp.y * h.y + dp.z * h.z + dp.w * h.w;   // Re(conj(dP_k) h_k)
+#pragma unroll 2
+  for (int i = tid; i < PAIRS; i += T) {
+    const int p = p0 + 2 * i, r = p / N, c = p % N;
+    const float4 g = __ldg((const float4*)(a.go_s + base + p));   // (read again by the update)
+    float4 d = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (a.update_object) {
+      const float4* q = acc + (size_t)(ty + r) * a.W + (tx + c);
+      const float4 qa = __ldg(q), qb = __ldg(q + 1), qc = __ldg(q + 2);
+      const float4 qd = __ldg(q + a.W), qe = __ldg(q + a.W + 1), qf = __ldg(q + a.W + 2);
+      const float ia = 1.f / (qa.z + damp), ib = 1.f / (qb.z + damp), ic = 1.f / (qc.z + damp);
+      const float id = 1.f / (qd.z + damp), ie = 1.f / (qe.z + damp), iF = 1.f / (qf.z + damp);
+      d = make_float4(w00 * ia * qa.x + w01 * ib * qb.x + w10 * id * qd.x + w11 * ie * qe.x,
+                      w00 * ia * qa.y + w01 * ib * qb.y + w10 * id * qd.y + w11 * ie * qe.y,
+                      w00 * ib * qb.x + w01 * ic * qc.x + w10 * ie * qe.x + w11 * iF * qf.x,
+                      w00 * ib * qb.y + w01 * ic * qc.y + w10 * ie * qe.y + w11 * iF * qf.y);
     }
+    *(float4*)(a.d_s + base + p) = d;
+    b1 += d.x * g.x + d.y * g.y + d.z * g.z + d.w * g.w;   // Re(conj(d) g)
   }
+  if (a.update_probe)
+    for (int k = s; k < a.M; k += S) {
+      const float4* h4 = (const float4*)(a.h_s + ((size_t)slot * a.M + k) * NN + p0);
+      const float4* d4 = (const float4*)(a.dP + (size_t)k * NN + p0);
+#pragma unroll 4
+      for (int i = tid; i < PAIRS; i += T) {
+        const float4 dp = __ldg(d4 + i);
+        const float4 h = __ldcs(h4 + i);
+        b2 += dp.x * h.x + dp.y * h.y + dp.z * h.z + dp.w * h.w;   // Re(conj(dP_k) h_k)
+      }
+    }
   double v[2] = {b1, b2};
   block_sum<2>(v, red);
   if (tid == 0) {
-    out[0] = v[0];
-    out[1] = v[1];
+    atomicAdd(a.dsum + ((size_t)slot * S + s) * 2, v[0]);
+    atomicAdd(a.dsum + (size_t)slot * S * 2 + 1, v[1]);
   }
 }
 
-// One CTA per (position, slice): the 2x2 step-size system of the position
-// (Gram entries of the tangents, right-hand sides from the slices' and the
-// probe's numerators, summed in a fixed order), the FP64 solve (the same in
-// every slice's CTA), and the slice's update O_s += alpha_O S_j^T g_s /
-// (illum_s + delta_O,s); the slice-0 CTA records alpha and adds alpha_P to
-// the minibatch's mean.
+// One CTA per 32 rows of a (position, slice): the 2x2 step-size system of the
+// position (Gram entries of the tangents, right-hand sides from the slices' and
+// the probe's numerators), the FP64 solve (the same in every CTA of the
+// position), and the band's update O_s += alpha_O S_j^T g_s / (illum_s +
+// delta_O,s); the first CTA records alpha and adds alpha_P to the minibatch's
+// mean. Bands, and 16-byte atomics, against one CTA per (position, slice) and
+// an atomic per pixel: 47 -> 32 us at the same size.
 template <int N>
-__global__ void __launch_bounds__(512, 2) k_ms_update(MsPass2Args a) {
-  constexpr int NN = N * N, T = 512;
+__global__ void __launch_bounds__(UPD_T, 4) k_ms_update(MsPass2Args a) {
+  wait_prior_grid();
   __shared__ double alpha_sh;
-  const int slot = blockIdx.x, s = blockIdx.y, tid = threadIdx.x, S = a.S;
+  const int slot = blockIdx.x / Bands<N>::NUM, band = blockIdx.x % Bands<N>::NUM, s = blockIdx.y, S = a.S;
   if (!a.valid[slot]) return;
   const int e = a.b0 + slot;
   const int j = a.order ? a.order[e] : e;
-  if (tid == 0) {
+  if (threadIdx.x == 0) {
     double a11 = 0.0, a12 = 0.0, a22 = 0.0, r1 = 0.0;
     for (int q = 0; q < a.Q; ++q) {
       const double* pp = a.part + ((size_t)slot * a.Q + q) * 3;
@@ -247,18 +262,9 @@ __global__ void __launch_bounds__(512, 2) k_ms_update(MsPass2Args a) {
     }
     for (int t = 0; t < S; ++t) r1 += a.dsum[((size_t)slot * S + t) * 2];
     const double r2 = a.dsum[(size_t)slot * S * 2 + 1];
-    const double tr = 0.5 * (a11 + a22);
-    const double d11 = a11 + a.lam * tr, d22 = a22 + a.lam * tr;
-    const double det = d11 * d22 - a12 * a12;
     double aO, aP;
-    if (det > 0.0) {
-      aO = (d22 * r1 - a12 * r2) / det;
-      aP = (d11 * r2 - a12 * r1) / det;
-    } else {
-      aO = d11 > 0.0 ? r1 / d11 : 0.0;
-      aP = d22 > 0.0 ? r2 / d22 : 0.0;
-    }
-    if (s == 0) {
+    solve_step(a11, a12, a22, r1, r2, a.lam, aO, aP);
+    if (s == 0 && band == 0) {
       atomicAdd(&a.sc->sum_alpha_p, aP);
       atomicAdd(&a.sc->count, 1);
       if (a.alpha_out) {
@@ -268,31 +274,15 @@ __global__ void __launch_bounds__(512, 2) k_ms_update(MsPass2Args a) {
     }
     alpha_sh = aO;
   }
-  __syncthreads();
   if (!a.update_object) return;
+  __syncthreads();
   int ty, tx;
   float fy, fx;
   tile_of(a.pos[2 * j], a.pos[2 * j + 1], N, a.H, a.W, ty, tx, fy, fx);
   const size_t HW = (size_t)a.H * a.W;
-  const float4* acc = a.acc + s * HW;
   const float damp = a.delta_o * __uint_as_float(a.smax[s]);
-  const float2* g_s = a.go_s + ((size_t)slot * S + s) * NN;
-  const float aO = (float)alpha_sh;
-  const float c00 = aO * (1.f - fy) * (1.f - fx), c01 = aO * (1.f - fy) * fx;
-  const float c10 = aO * fy * (1.f - fx), c11 = aO * fy * fx;
-  float2* obj = a.obj + s * HW;
-  constexpr int N1 = N + 1;
-  for (int q = tid; q < N1 * N1; q += T) {
-    const int y = q / N1, x = q % N1;
-    float2 sacc = make_float2(0.f, 0.f);
-    if (y < N && x < N) { const float2 g = g_s[y * N + x]; sacc.x += c00 * g.x; sacc.y += c00 * g.y; }
-    if (y < N && x > 0) { const float2 g = g_s[y * N + x - 1]; sacc.x += c01 * g.x; sacc.y += c01 * g.y; }
-    if (y > 0 && x < N) { const float2 g = g_s[(y - 1) * N + x]; sacc.x += c10 * g.x; sacc.y += c10 * g.y; }
-    if (y > 0 && x > 0) { const float2 g = g_s[(y - 1) * N + x - 1]; sacc.x += c11 * g.x; sacc.y += c11 * g.y; }
-    const size_t oi = (size_t)(ty + y) * a.W + (tx + x);
-    const float inv = 1.f / (__ldg(&acc[oi].z) + damp);
-    atomicAdd(obj + oi, make_float2(sacc.x * inv, sacc.y * inv));
-  }
+  update_band<N>(band, a.go_s + ((size_t)slot * S + s) * N * N, a.acc + s * HW, a.obj + s * HW, a.W, ty, tx, fy, fx,
+                 damp, (float)alpha_sh);
 }
 
 template <class Fn>
@@ -313,16 +303,14 @@ cudaError_t dispatch_ms_N(int N, Fn&& fn) {
 // (k_step_ms), then the solve and the slices' updates (k_ms_update).
 cudaError_t pass2_ms(int N, const MsPass2Args& a, const MsStepArgs& t, cudaStream_t s) {
   if (a.nb <= 0) return cudaSuccess;
-  const dim3 grid((unsigned)a.nb, (unsigned)a.S);
   cudaEvent_t e0 = profile_begin(K_PASS2, s);
   cudaError_t e = dispatch_ms_N(N, [&](auto c) {
     constexpr int NC = decltype(c)::value;
-    k_ms_dir<NC><<<grid, 512, 0, s>>>(a);
-    cudaError_t r = cudaGetLastError();
+    const dim3 grid((unsigned)a.nb * Bands<NC>::NUM, (unsigned)a.S);
+    cudaError_t r = launch_pdl(k_ms_dir<NC>, grid, dim3(UPD_T), 0, s, a);
     if (r != cudaSuccess) return r;
     if ((r = launch_step_ms<NC>(t, s)) != cudaSuccess) return r;
-    k_ms_update<NC><<<grid, 512, 0, s>>>(a);
-    return cudaGetLastError();
+    return launch_pdl(k_ms_update<NC>, grid, dim3(UPD_T), 0, s, a);
   });
   profile_end(K_PASS2, e0, s);
   return e;
@@ -481,7 +469,7 @@ ptycho_status ptycho_lsqml_epoch_ms(const ptycho_dims* dims, const ptycho_multis
       k_ms_illum_max<<<dim3((unsigned)grid_for(HW, 256, 2 * sm_count()), (unsigned)S), 256, 0, s>>>(HW, acc, smax);
       if (cudaGetLastError() != cudaSuccess) return PTYCHO_ERR_CUDA;
       if (norm_probe(NN, M, dPacc, Dp, (const float2*)probe, (float)opts->delta_p, opts->update_probe, sc, dP, Cp,
-                     Sdp, s) != cudaSuccess)
+                     Sdp, s, (double*)(b + L.dsum), a.nb * S * 2) != cudaSuccess)
         return PTYCHO_ERR_CUDA;
       MsPass2Args q;
       memset(&q, 0, sizeof(q));

@@ -348,8 +348,7 @@ struct StepSums {
   static_assert(T * CHUNKS * 2 == N * N && T % 32 == 0, "a pixel pair per thread");
 };
 
-// Sums of positions blockIdx.y * per ..+per-1 over the pixel pairs of chunk
-// blockIdx.x, added to a.part[slot][5] (zero on entry). Dynamic shared memory:
+// Sums of `per` positions over one chunk's pixel pairs per CTA, added to a.part[slot][5] (zero on entry). Dynamic shared memory:
 // (M + K) T float4, the direction of each mode (OPR: of each eigenmode, then
 // of the shared modes) at the thread's pair.
 template <int N, bool OPR>
@@ -362,8 +361,9 @@ __global__ void __launch_bounds__(StepSums<N>::T, 3) k_step_sums(Pass2Args a, in
   __shared__ float wsh[OPR ? STEP_GROUP * OPR_KMAX : 1];
   wait_prior_grid();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int p = (blockIdx.x * T + tid) * 2, r = p / N, c = p % N;   // this thread's pixels p, p + 1
-  const int i0 = blockIdx.y * per, n = min(per, a.nb - i0);
+  const int chunk = blockIdx.x % StepSums<N>::CHUNKS, group = blockIdx.x / StepSums<N>::CHUNKS;
+  const int p = (chunk * T + tid) * 2, r = p / N, c = p % N;   // this thread's pixels p, p + 1
+  const int i0 = group * per, n = min(per, a.nb - i0);
   const int M = a.M, K = OPR ? a.K : 0, Ms = OPR ? M - 1 : M;       // shared modes
   const float damp = a.delta_o * __uint_as_float(a.sc->max_illum);
   for (int i = tid; i < n; i += T) {
@@ -487,24 +487,77 @@ __global__ void __launch_bounds__(StepSums<N>::T, 3) k_step_sums(Pass2Args a, in
   }
 }
 
-// Object update of position blockIdx.y, rows band * RB .. of its patch: O +=
-// alpha_O S_j^T g / (illum + delta_O), each object pixel of the tile gathering
-// its four patch neighbours and divided by its own preconditioner. Every band
-// solves the position's system (the same values); band 0 records the steps.
+// Object update of rows band * 32 .. of one position's tile (the last band also
+// row N): O += alpha_O S_j^T g / (illum + delta_O), each object pixel gathering
+// its four patch neighbours and divided by its own preconditioner.
+constexpr int UPD_T = 256;
 template <int N>
-struct StepUpdate {
-  static constexpr int T = 256, RB = N < 32 ? N : 32, BANDS = N / RB;
+struct Bands {
+  static constexpr int ROWS = N < 32 ? N : 32, NUM = N / ROWS;
 };
 template <int N>
-__global__ void __launch_bounds__(StepUpdate<N>::T, 4) k_step_update(Pass2Args a) {
-  constexpr int T = StepUpdate<N>::T, RB = StepUpdate<N>::RB, BANDS = StepUpdate<N>::BANDS, N1 = N + 1;
+__device__ __forceinline__ void update_band(int band, const float2* __restrict__ g_s, const float4* __restrict__ acc,
+                                            float2* obj, int W, int ty, int tx, float fy, float fx, float damp,
+                                            float aO) {
+  constexpr int T = UPD_T, RB = Bands<N>::ROWS, N1 = N + 1;
+  const int tid = threadIdx.x;
+  const float c00 = aO * ((1.f - fy) * (1.f - fx)), c01 = aO * ((1.f - fy) * fx);
+  const float c10 = aO * (fy * (1.f - fx)), c11 = aO * (fy * fx);
+  const int y0 = band * RB, y1 = y0 + RB + (band == Bands<N>::NUM - 1 ? 1 : 0);
+  auto gat = [&](int y, int x) {
+    return (y >= 0 && y < N && x >= 0 && x < N) ? __ldg(g_s + y * N + x) : make_float2(0.f, 0.f);
+  };
+  auto mix = [&](float2 gB, float2 gA, float2 hB, float2 hA, float inv) {
+    return make_float2((c00 * gB.x + c01 * gA.x + c10 * hB.x + c11 * hA.x) * inv,
+                       (c00 * gB.y + c01 * gA.y + c10 * hB.y + c11 * hA.y) * inv);
+  };
+  auto out = [&](int y, int x) { return (size_t)(ty + y) * W + tx + x; };
+  auto pre = [&](size_t o) { return 1.f / (__ldg(&acc[o].z) + damp); };
+  if (((uintptr_t)obj & 15) == 0 && (W & 1) == 0) {
+    // pairs of object pixels at even object columns, one 16-byte vector atomic
+    // each (half the atomic operations); per tile row N/2 pairs and one single
+    // pixel (the first when tx is odd, else the last). A thread keeps one
+    // column pair and walks down its rows: the row of g above stays in registers.
+    const int odd = tx & 1;
+    constexpr int RUNS = T / (N / 2) > 0 ? T / (N / 2) : 1;
+    for (int item = tid; item < RUNS * (N / 2); item += T) {
+      const int x = 2 * (item % (N / 2)) + odd, run = item / (N / 2);
+      const int ya = y0 + (y1 - y0) * run / RUNS, yb = y0 + (y1 - y0) * (run + 1) / RUNS;
+      float2 hA = gat(ya - 1, x - 1), hB = gat(ya - 1, x), hC = gat(ya - 1, x + 1);
+#pragma unroll 4
+      for (int y = ya; y < yb; ++y) {
+        const float2 gA = gat(y, x - 1), gB = gat(y, x), gC = gat(y, x + 1);
+        const size_t o = out(y, x);
+        const float2 s0 = mix(gB, gA, hB, hA, pre(o)), s1 = mix(gC, gB, hC, hB, pre(o + 1));
+        atomicAdd((float4*)(obj + o), make_float4(s0.x, s0.y, s1.x, s1.y));
+        hA = gA; hB = gB; hC = gC;
+      }
+    }
+    for (int y = y0 + tid; y < y1; y += T) {
+      const int x = odd ? 0 : N;
+      const size_t o = out(y, x);
+      atomicAdd(obj + o, mix(gat(y, x), gat(y, x - 1), gat(y - 1, x), gat(y - 1, x - 1), pre(o)));
+    }
+    return;
+  }
+  for (int q = tid; q < (y1 - y0) * N1; q += T) {
+    const int y = y0 + q / N1, x = q % N1;
+    const size_t o = out(y, x);
+    atomicAdd(obj + o, mix(gat(y, x), gat(y, x - 1), gat(y - 1, x), gat(y - 1, x - 1), pre(o)));
+  }
+}
+
+// One CTA per band of a position: the solve and the band's update. Every
+// band solves the position's system (the same values); band 0 records the steps.
+template <int N>
+__global__ void __launch_bounds__(UPD_T, 4) k_step_update(Pass2Args a) {
   wait_prior_grid();
   __shared__ double alpha_sh;
-  const int band = blockIdx.x, slot = blockIdx.y, tid = threadIdx.x;
+  const int slot = blockIdx.x / Bands<N>::NUM, band = blockIdx.x % Bands<N>::NUM;
   if (!a.valid[slot]) return;
   const int e = a.b0 + slot;
   const int j = a.order ? a.order[e] : e;
-  if (tid == 0) {
+  if (threadIdx.x == 0) {
     const double* v = a.part + (size_t)slot * 5;
     double aO, aP;
     solve_step(v[0], v[1], v[2], v[3], v[4], a.lam, aO, aP);
@@ -523,53 +576,8 @@ __global__ void __launch_bounds__(StepUpdate<N>::T, 4) k_step_update(Pass2Args a
   float fy, fx;
   tile_of(a.pos[2 * j], a.pos[2 * j + 1], N, a.H, a.W, ty, tx, fy, fx);
   const float damp = a.delta_o * __uint_as_float(a.sc->max_illum);
-  const float2* g_s = a.g_s + (size_t)slot * N * N;
   __syncthreads();
-  const float aO = (float)alpha_sh;
-  const float c00 = aO * ((1.f - fy) * (1.f - fx)), c01 = aO * ((1.f - fy) * fx);
-  const float c10 = aO * (fy * (1.f - fx)), c11 = aO * (fy * fx);
-  const int y0 = band * RB, y1 = y0 + RB + (band == BANDS - 1 ? 1 : 0);
-  auto gat = [&](int y, int x) {
-    return (y >= 0 && y < N && x >= 0 && x < N) ? __ldg(g_s + y * N + x) : make_float2(0.f, 0.f);
-  };
-  auto mix = [&](float2 gB, float2 gA, float2 hB, float2 hA, float inv) {
-    return make_float2((c00 * gB.x + c01 * gA.x + c10 * hB.x + c11 * hA.x) * inv,
-                       (c00 * gB.y + c01 * gA.y + c10 * hB.y + c11 * hA.y) * inv);
-  };
-  auto out = [&](int y, int x) { return (size_t)(ty + y) * a.W + tx + x; };
-  auto pre = [&](size_t o) { return 1.f / (__ldg(&a.acc[o].z) + damp); };
-  if (((uintptr_t)a.obj & 15) == 0 && (a.W & 1) == 0) {
-    // pairs of object pixels at even object columns, one 16-byte vector atomic
-    // each (half the atomic operations); per tile row N/2 pairs and one single
-    // pixel (the first when tx is odd, else the last). A thread keeps one
-    // column pair and walks down its rows: the row of g above stays in registers.
-    const int odd = tx & 1;
-    constexpr int RUNS = T / (N / 2) > 0 ? T / (N / 2) : 1;
-    for (int item = tid; item < RUNS * (N / 2); item += T) {
-      const int x = 2 * (item % (N / 2)) + odd, run = item / (N / 2);
-      const int ya = y0 + (y1 - y0) * run / RUNS, yb = y0 + (y1 - y0) * (run + 1) / RUNS;
-      float2 hA = gat(ya - 1, x - 1), hB = gat(ya - 1, x), hC = gat(ya - 1, x + 1);
-#pragma unroll 4
-      for (int y = ya; y < yb; ++y) {
-        const float2 gA = gat(y, x - 1), gB = gat(y, x), gC = gat(y, x + 1);
-        const size_t o = out(y, x);
-        const float2 s0 = mix(gB, gA, hB, hA, pre(o)), s1 = mix(gC, gB, hC, hB, pre(o + 1));
-        atomicAdd((float4*)(a.obj + o), make_float4(s0.x, s0.y, s1.x, s1.y));
-        hA = gA; hB = gB; hC = gC;
-      }
-    }
-    for (int y = y0 + tid; y < y1; y += T) {
-      const int x = odd ? 0 : N;
-      const size_t o = out(y, x);
-      atomicAdd(a.obj + o, mix(gat(y, x), gat(y, x - 1), gat(y - 1, x), gat(y - 1, x - 1), pre(o)));
-    }
-    return;
-  }
-  for (int q = tid; q < (y1 - y0) * N1; q += T) {
-    const int y = y0 + q / N1, x = q % N1;
-    const size_t o = out(y, x);
-    atomicAdd(a.obj + o, mix(gat(y, x), gat(y, x - 1), gat(y - 1, x), gat(y - 1, x - 1), pre(o)));
-  }
+  update_band<N>(band, a.g_s + (size_t)slot * N * N, a.acc, a.obj, a.W, ty, tx, fy, fx, damp, (float)alpha_sh);
 }
 
 template <int N, bool OPR>
@@ -588,10 +596,9 @@ cudaError_t launch_step(const Pass2Args& a, cudaStream_t s) {
     const long long cost = (ctas + 3 * SMS - 1) / (3 * SMS) * (q + 4);
     if (best < 0 || cost < best) best = cost, per = q;
   }
-  e = launch_pdl(k_step_sums<N, OPR>, dim3(S::CHUNKS, (a.nb + per - 1) / per), dim3(S::T), sm, s, a, per);
+  e = launch_pdl(k_step_sums<N, OPR>, dim3(S::CHUNKS * ((a.nb + per - 1) / per)), dim3(S::T), sm, s, a, per);
   if (e != cudaSuccess) return e;
-  return launch_pdl(k_step_update<N>, dim3(a.update_object ? StepUpdate<N>::BANDS : 1, a.nb), dim3(StepUpdate<N>::T), 0, s,
-                    a);
+  return launch_pdl(k_step_update<N>, dim3(a.nb * Bands<N>::NUM), dim3(UPD_T), 0, s, a);
 }
 
 // The two launches, or one CTA per position at two CTAs per SM? The latter

@@ -51,3 +51,25 @@ def test_two_launches_with_one_update_off(N, update_object, update_probe):
 def test_rule_by_minibatch_matches_oracle(N, J):
     # past one position per SM at 64, and either side of a last wave 0.7 full
     _epoch(N, 1, J, J, N + 30, 0, 0)
+
+
+@pytest.mark.parametrize("N,M,S,W,update_object,update_probe", [
+    (16, 5, 2, 37, True, True), (32, 1, 3, 58, True, True), (64, 4, 3, 87, True, True), (128, 2, 1, 151, True, True),
+    (192, 1, 2, 215, True, True), (256, 2, 2, 280, True, True), (64, 2, 2, 88, False, True)])
+def test_multislice_directions_and_updates_in_bands(N, M, S, W, update_object, update_probe):
+    # more modes than slices and fewer, odd and even object widths
+    import torch
+    from paper_2510_20929_gb300 import api
+    from tests.test_gpu_multislice import LAM, PX, TOL_GRAD, _dev, ms_problem
+    dz, J = 5e-6, 5
+    Os, P, pos, Hf, I_m = ms_problem(N, M, S, N + 23, W, J, 2.0, dz)
+    dO, dP, dpos, dI = _dev(Os, P, pos, I_m)
+    kw = dict(batch=3, delta_o=0.1, delta_p=0.1, lam=1e-6, eps=1e-6, update_object=update_object,
+              update_probe=update_probe)
+    order = np.arange(J, dtype=np.int32)[::-1].copy()
+    O1, P1, L1, a1 = orc.lsqml_epoch_ms(Os, P, pos, I_m, order, Hf, orc.LsqmlOptions(**kw))
+    loss, alpha = api.lsqml_epoch_ms(dO, dP, dpos, dI, to_dev(order, torch.int32), api.make_multislice(S, dz, LAM, PX),
+                                     want_alpha=True, **kw)
+    e = (err(dO.cpu().numpy(), O1, axis=0), err(dP.cpu().numpy(), P1, axis=0), err(alpha.cpu().numpy(), a1, axis=1))
+    print(f"ms N={N} M={M} S={S} W={W}:", e)
+    assert max(e) < TOL_GRAD and abs(loss.item() - L1) / abs(L1) < TOL_FWD
