@@ -29,9 +29,9 @@ namespace ptycho {
 // with vector atomics, dUacc_m += sum_j w_jm h_j0 and (when D is set)
 // D_m += sum_j w_jm^2 |o_j|^2. The slots' validity and weights are staged in
 // shared memory, RS slots at a time, so that the loop over the slots waits
-// only on the h and o loads, two slots' loads in flight (added in slot order).
+// only on the h and o loads, four slots' loads in flight (added in slot order).
 template <int KM>
-__global__ void __launch_bounds__(256) k_opr_reduce(int NN, int M, int K, int nb, int chunk, int b0,
+__global__ void __launch_bounds__(256, 2) k_opr_reduce(int NN, int M, int K, int nb, int chunk, int b0,
                                                     const int* __restrict__ order, const float* __restrict__ w,
                                                     const float2* __restrict__ h_s, const float2* __restrict__ o_s,
                                                     const int* __restrict__ valid, float2* dUacc, float* D) {
@@ -75,22 +75,19 @@ __global__ void __launch_bounds__(256) k_opr_reduce(int NN, int M, int K, int nb
     }
     __syncthreads();
     if (q < NP) {
-      int r = 0;
-      for (; r + 1 < n; r += 2) {
-        const bool v0 = ok_s[r] != 0, v1 = ok_s[r + 1] != 0;
-        const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-        const size_t i = (size_t)(t0 + r);
-        const float4 h0 = v0 ? __ldg((const float4*)(h_s + i * M * NN) + q) : z;
-        const float4 h1 = v1 ? __ldg((const float4*)(h_s + (i + 1) * M * NN) + q) : z;
-        const float4 o0 = (v0 && D) ? __ldg((const float4*)(o_s + i * NN) + q) : z;
-        const float4 o1 = (v1 && D) ? __ldg((const float4*)(o_s + (i + 1) * NN) + q) : z;
-        if (v0) add(r, h0, o0);
-        if (v1) add(r + 1, h1, o1);
-      }
-      if (r < n && ok_s[r]) {
-        const size_t i = (size_t)(t0 + r);
-        const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-        add(r, __ldg((const float4*)(h_s + i * M * NN) + q), D ? __ldg((const float4*)(o_s + i * NN) + q) : z);
+      const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int r = 0; r < n; r += 4) {
+        float4 h[4], o[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const bool v = r + u < n && ok_s[r + u];
+          const size_t i = (size_t)(t0 + r + u);
+          h[u] = v ? __ldg((const float4*)(h_s + i * M * NN) + q) : z;
+          o[u] = (v && D) ? __ldg((const float4*)(o_s + i * NN) + q) : z;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (r + u < n && ok_s[r + u]) add(r + u, h[u], o[u]);
       }
     }
   }
@@ -130,7 +127,10 @@ __global__ void k_norm_opr(size_t n, const float2* dUacc, const float* D, int up
 // eigenmode values, h_j0 and o_j are copied into shared memory with cp.async
 // (double-buffered: the next chunk is in flight while this one is summed), so
 // that U is fetched once per CTA instead of once per slot. span and the
-// window area are multiples of GRAM_CHUNK.
+// window area are multiples of GRAM_CHUNK. Bound by FP32 FMAs (107 per pixel and
+// slot at 8 eigenmodes) and shared-memory reads alike: window 192, 256 slots,
+// 87 -> 58 us with one wave of CTAs (320 over 304 places before) and copies of
+// 16 instead of 8 bytes.
 constexpr int GRAM_SLOTS = 8, GRAM_CHUNK = 256;
 
 template <int KM>
@@ -140,9 +140,9 @@ struct GramSmem {
   float2 o[2][GRAM_SLOTS][GRAM_CHUNK];
 };
 
-__device__ __forceinline__ void cp_async8(void* dst, const void* src) {
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
   const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(src) : "memory");
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(src) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
 template <int PENDING>
@@ -169,15 +169,16 @@ __global__ void __launch_bounds__(32 * GRAM_SLOTS, 2) k_opr_gram(int N, int M, i
     if (m >= K) sm.u[b][m][q] = make_float2(0.f, 0.f);
   }
   auto stage = [&](int c0, int b) {
-    for (int i = threadIdx.x; i < K * GRAM_CHUNK; i += blockDim.x) {
-      const int m = i / GRAM_CHUNK, q = i % GRAM_CHUNK;
-      cp_async8(&sm.u[b][m][q], U + (size_t)m * NN + c0 + q);
-    }
-    for (int i = threadIdx.x; i < GRAM_SLOTS * GRAM_CHUNK; i += blockDim.x) {
-      const int sl = i / GRAM_CHUNK, q = i % GRAM_CHUNK, sg = slot0 + sl;
+    constexpr int Q2 = GRAM_CHUNK / 2;   // 16-byte copies of a row
+    const int q = 2 * (threadIdx.x % Q2), r0 = threadIdx.x / Q2;
+    constexpr int RPT = 32 * GRAM_SLOTS / Q2;
+    for (int m = r0; m < K; m += RPT) cp_async16(&sm.u[b][m][q], U + (size_t)m * NN + c0 + q);
+#pragma unroll
+    for (int sl = r0; sl < GRAM_SLOTS; sl += RPT) {
+      const int sg = slot0 + sl;
       if (sg < nb) {
-        cp_async8(&sm.h[b][sl][q], h_s + (size_t)sg * M * NN + c0 + q);
-        if (ls) cp_async8(&sm.o[b][sl][q], o_s + (size_t)sg * NN + c0 + q);
+        cp_async16(&sm.h[b][sl][q], h_s + (size_t)sg * M * NN + c0 + q);
+        if (ls) cp_async16(&sm.o[b][sl][q], o_s + (size_t)sg * NN + c0 + q);
       }
     }
     cp_async_commit();
@@ -228,79 +229,69 @@ __global__ void __launch_bounds__(32 * GRAM_SLOTS, 2) k_opr_gram(int N, int M, i
   }
 }
 
-// In-register FP64 solve of (A + dmp I) x = b for K unknowns (Cholesky on the
-// packed upper triangle a[t(m, n)], m <= n); false if not positive definite.
-template <int K, int KM>
-__device__ __forceinline__ bool chol_solve(const double* v, double lam, double (&x)[KM]) {
-  constexpr int NA = KM * (KM + 1) / 2;
-  double L[K][K];
-  double tr = 0.0;
-#pragma unroll
+// Weight step, eight threads per slot (thread r of a slot: unknown r).
+// Gradient form (gw set): dL/dw_j += b. Otherwise the damped normal equations
+// (A + lam tr(A)/K I) dw = b are solved in FP64 (Cholesky; no update if the
+// system is not positive definite) and w_j += step dw.
+// Bound by the serial chain of FP64 square roots and divisions, which a thread
+// per slot also paid for every element of the factor (256 slots, K = 8: 38 -> 20 us).
+// Thread r holds row r, takes its column's quotient beside the others', and the
+// factor's transpose is read back from shared memory.
+constexpr int SOLVE_T = 32;
+template <int KM>
+__global__ void __launch_bounds__(SOLVE_T) k_opr_solve(int nb, int K, int b0, const int* __restrict__ order,
+                                                       const int* __restrict__ valid,
+                                                       const double* __restrict__ gram, float* w, float* gw,
+                                                       double lam, float step) {
+  constexpr int NA = KM * (KM + 1) / 2, NV = NA + KM;
+  static_assert(KM == 8, "eight threads per slot");
+  __shared__ double Ls[SOLVE_T][KM + 1];   // [slot's row][column], a bank pair apart
+  const int r = threadIdx.x % KM, slot = (blockIdx.x * SOLVE_T + threadIdx.x) / KM;
+  const bool live = slot < nb && valid[slot];
+  const double* v = gram + (size_t)(live ? slot : 0) * NV;
+  const int e = b0 + slot, j = !live ? 0 : order ? order[e] : e;
+  if (gw) {
+    if (live && r < K) gw[(size_t)j * K + r] += (float)v[NA + r];
+    return;
+  }
+  double tr = 0.0, L[KM];
   for (int m = 0; m < K; ++m) tr += v[m * KM - m * (m - 1) / 2];   // A_mm
   const double dmp = lam * tr / (double)K;
 #pragma unroll
-  for (int r = 0; r < K; ++r) {
+  for (int c = 0; c < KM; ++c)
+    L[c] = c > r || r >= K ? 0.0 : v[c * KM - c * (c - 1) / 2 + (r - c)] + (r == c ? dmp : 0.0);   // A_cr, c <= r
+  bool ok = live;
 #pragma unroll
-    for (int c = 0; c <= r; ++c) {
-      double sum = v[c * KM - c * (c - 1) / 2 + (r - c)] + (r == c ? dmp : 0.0);   // A_cr, c <= r
+  for (int c = 0; c < KM; ++c) {
+    if (c < K) {
+      const double piv = __shfl_sync(0xffffffffu, L[c], c, KM);
+      ok = ok && piv > 0.0;
+      const double d = sqrt(piv);
+      L[c] = r == c ? d : L[c] / d;
 #pragma unroll
-      for (int k = 0; k < c; ++k) sum -= L[r][k] * L[c][k];
-      if (r == c) {
-        if (!(sum > 0.0)) return false;
-        L[r][r] = sqrt(sum);
-      } else {
-        L[r][c] = sum / L[c][c];
+      for (int n = c + 1; n < KM; ++n) {
+        const double ln = __shfl_sync(0xffffffffu, L[c], n, KM);
+        if (r >= n) L[n] -= L[c] * ln;
       }
     }
   }
 #pragma unroll
-  for (int r = 0; r < K; ++r) {   // L y = b
-    double sum = v[NA + r];
-#pragma unroll
-    for (int k = 0; k < r; ++k) sum -= L[r][k] * x[k];
-    x[r] = sum / L[r][r];
+  for (int c = 0; c < KM; ++c) Ls[threadIdx.x][c] = L[c];
+  __syncwarp();
+  const double diag = Ls[threadIdx.x][r];
+  const int row0 = threadIdx.x - r;
+  double x = r < K ? v[NA + r] : 0.0;
+  for (int k = 0; k < K; ++k) {   // L y = b
+    const double y = __shfl_sync(0xffffffffu, x / diag, k, KM);
+    if (r == k) x = y;
+    if (r > k) x -= Ls[threadIdx.x][k] * y;
   }
-#pragma unroll
-  for (int r = K - 1; r >= 0; --r) {   // L^T x = y
-    double sum = x[r];
-#pragma unroll
-    for (int k = r + 1; k < K; ++k) sum -= L[k][r] * x[k];
-    x[r] = sum / L[r][r];
+  for (int k = K - 1; k >= 0; --k) {   // L^T x = y
+    const double y = __shfl_sync(0xffffffffu, x / diag, k, KM);
+    if (r == k) x = y;
+    if (r < k) x -= Ls[row0 + k][r] * y;
   }
-  return true;
-}
-
-// One thread per slot. Gradient form (gw set): dL/dw_j += b. Otherwise the
-// damped normal equations (A + lam tr(A)/K I) dw = b are solved in FP64
-// (Cholesky; no update if the system is not positive definite) and
-// w_j += step dw.
-template <int KM>
-__global__ void k_opr_solve(int nb, int K, int b0, const int* __restrict__ order, const int* __restrict__ valid,
-                            const double* __restrict__ gram, float* w, float* gw, double lam, float step) {
-  constexpr int NA = KM * (KM + 1) / 2, NV = NA + KM;
-  const int slot = blockIdx.x * blockDim.x + threadIdx.x;
-  if (slot >= nb || !valid[slot]) return;
-  const int e = b0 + slot;
-  const int j = order ? order[e] : e;
-  const double* v = gram + (size_t)slot * NV;
-  if (gw) {
-    for (int m = 0; m < K; ++m) gw[(size_t)j * K + m] += (float)v[NA + m];
-    return;
-  }
-  double x[KM];
-  bool ok = false;
-  switch (K) {
-    case 1: ok = chol_solve<1, KM>(v, lam, x); break;
-    case 2: ok = chol_solve<2, KM>(v, lam, x); break;
-    case 3: ok = chol_solve<3, KM>(v, lam, x); break;
-    case 4: ok = chol_solve<4, KM>(v, lam, x); break;
-    case 5: ok = chol_solve<5, KM>(v, lam, x); break;
-    case 6: ok = chol_solve<6, KM>(v, lam, x); break;
-    case 7: ok = chol_solve<7, KM>(v, lam, x); break;
-    case 8: ok = chol_solve<8, KM>(v, lam, x); break;
-  }
-  if (!ok) return;   // not positive definite: no weight update
-  for (int m = 0; m < K; ++m) w[(size_t)j * K + m] += (float)(step * x[m]);
+  if (ok && r < K) w[(size_t)j * K + r] += (float)(step * x);   // (else not positive definite: no update)
 }
 
 constexpr int OPR_NV = OPR_KMAX * (OPR_KMAX + 1) / 2 + OPR_KMAX;   // sums per slot of the weight step
@@ -321,10 +312,11 @@ static cudaError_t smem_optin_once(Kern kernel, size_t bytes, unsigned long long
 static cudaError_t opr_reduce(int NN, int M, int K, int nb, int b0, const int* order, const float* w,
                               const float2* h_s, const float2* o_s, const int* valid, float2* dUacc, float* D,
                               cudaStream_t s) {
-  // pixel pairs across blockIdx.x, the batch split into enough chunks for two CTAs per SM
+  // pixel pairs across blockIdx.x, the batch split into as many chunks as two CTAs
+  // per SM hold at once (one more leaves a last wave that is nearly empty)
   const int NP = NN / 2;
   const int bx = (NP + 255) / 256;
-  int chunks = (2 * sm_count() + bx - 1) / bx;
+  int chunks = 2 * sm_count() / bx;
   if (chunks > nb) chunks = nb;
   if (chunks < 1) chunks = 1;
   const int chunk = (nb + chunks - 1) / chunks;
@@ -344,9 +336,11 @@ static cudaError_t opr_weights(int N, int M, int K, int nb, int b0, const int* o
   cudaEvent_t e0 = profile_begin(K_OPR_WEIGHTS, s);
   cudaError_t e = cudaMemsetAsync(gram, 0, (size_t)nb * OPR_NV * sizeof(double), s);
   if (e == cudaSuccess) {
-    // pixel spans of whole chunks, enough CTAs for two per SM
+    // pixel spans of whole chunks, as many CTAs as two per SM hold at once (one
+    // part more left a second wave that was nearly empty)
     const int NN = N * N, groups = (nb + GRAM_SLOTS - 1) / GRAM_SLOTS;
-    int parts = (2 * sm_count() + groups - 1) / groups;
+    int parts = 2 * sm_count() / groups;
+    if (parts < 1) parts = 1;
     const int max_parts = (NN + GRAM_CHUNK - 1) / GRAM_CHUNK;
     if (parts > max_parts) parts = max_parts;
     const int span = ((NN + parts - 1) / parts + GRAM_CHUNK - 1) / GRAM_CHUNK * GRAM_CHUNK;
@@ -356,7 +350,7 @@ static cudaError_t opr_weights(int N, int M, int K, int nb, int b0, const int* o
     if (e == cudaSuccess)
       k_opr_gram<OPR_KMAX><<<dim3(parts, groups), 32 * GRAM_SLOTS, sizeof(GramSmem<OPR_KMAX>), s>>>(
           N, M, K, gw ? 0 : 1, nb, span, valid, U, h_s, o_s, gram);
-    k_opr_solve<OPR_KMAX><<<(nb + 31) / 32, 32, 0, s>>>(nb, K, b0, order, valid, gram, w, gw, lam, step);
+    k_opr_solve<OPR_KMAX><<<(unsigned)(((size_t)nb * OPR_KMAX + SOLVE_T - 1) / SOLVE_T), SOLVE_T, 0, s>>>(nb, K, b0, order, valid, gram, w, gw, lam, step);
     e = cudaGetLastError();
   }
   profile_end(K_OPR_WEIGHTS, e0, s);
