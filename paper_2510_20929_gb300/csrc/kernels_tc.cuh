@@ -27,14 +27,15 @@
 // scaled and transformed back, and chi_jk = F^-1[(rho - 1) Psi_jk] overwrites
 // the scratch for the overlap-add part of the pass.
 //
-// Warp roles: eight producer warps write the B operand of every K step (a
+// Warp roles: eight producer warps (sixteen at N = 128, taking the K steps in
+// turn) write the B operand of every K step (a
 // 16-wide K slice of four BF16 planes) into a ring of shared-memory slots;
 // one MMA warp streams the DFT-matrix chunks and issues the MMAs as slices
 // land; one TMA warp stages the exit waves and the measured intensities from
 // global memory into a second ring with tiled tensor copies (128-byte
 // swizzle). Pass-1 slices come from the staged exit waves, from the last
 // forward far field still in TMEM (the first inverse transform) or from the
-// far fields in L2 (the other inverse transforms); pass-2 slices from the
+// far fields, staged again (the other inverse transforms); pass-2 slices from the
 // pass-1 accumulator in TMEM. Pass 1 accumulates in TMEM buffer A, pass 2 in
 // buffer B, so an image's pass-2 result drains while the next image's pass 1
 // runs.
@@ -49,12 +50,14 @@ namespace ptycho {
 template <int N>
 struct FarTc {
   static_assert(N == 32 || N == 64 || N == 128, "DFT-GEMM windows");
-  static constexpr int PW = 8;                    // producer warps: TMEM lane quarter w % 4, column set w / 4
+  static constexpr int G = N == 128 ? 2 : 1;      // groups of producer warps, slices s % G each
+  static constexpr int PW = 8 * G;                // producer warps: TMEM lane quarter w % 4, slice half (w / 4) % 2,
+                                                  // group w / 8
   static constexpr int T = 32 * (PW + 2);         // and the MMA warp (PW) and the TMA warp (PW + 1)
-  static constexpr int HALF = N / 2;              // columns per producer thread: 16 s + 8 (w / 4) + [0, 8)
+  static constexpr int COLS_T = N / 2 / G;        // columns per producer thread: 16 s + 8 ((w / 4) % 2) + [0, 8)
   static constexpr int NCH = N / 16;              // K steps of one pass (= DFT chunks)
   static constexpr int NSF = 4;                   // ring slots of DFT chunks
-  static constexpr int NSB = 6;                   // ring slots of B slices
+  static constexpr int NSB = 4;                   // ring slots of B slices
   static constexpr int NSS = 4;                   // ring slots of staged tiles
   static constexpr int MT = 128;                  // MMA tile rows (DFT rows beyond N are zero)
   static constexpr uint32_t APLANE = MT * 16 * 2;            // one 128 x 16 BF16 plane of a chunk
@@ -67,10 +70,14 @@ struct FarTc {
   static constexpr size_t fring = 0;
   static constexpr size_t sring = fring + (size_t)NSF * CHUNK;   // 1024-byte aligned (swizzled tiles)
   static constexpr size_t bring = sring + (size_t)NSS * SSLOT;
-  static constexpr size_t bars = bring + (size_t)NSB * SLICE;
-  static constexpr int NBAR = 2 * NSF + 2 * NSB + 2 * NSS + 3;   // F, B and staging rings, p1, p2, drained
+  static constexpr uint32_t WTILE = 32 * 64;                 // a producer warp's 32 rows x 8 complex columns
+  static constexpr size_t wtile = bring + (size_t)NSB * SLICE;
+  static constexpr size_t bars = wtile + (size_t)PW * WTILE;
+  static constexpr int NBAR = 2 * NSF + 2 * NSB + 2 * NSS + 4 + PW;   // F, B and staging rings, p1, p2, drained, stored,
+                                                                      // and a hand-over per producer warp
   static constexpr size_t misc = bars + 8 * (size_t)NBAR;
-  static constexpr size_t bytes = misc + 16 + 1024;             // + alignment of the base to 1024 bytes
+  static constexpr size_t mail = misc + 16;                     // running loss of each pair of producer warps
+  static constexpr size_t bytes = mail + 8 * 32 * 4 + 1024;   // + alignment of the base to 1024 bytes
   static constexpr uint32_t COLS = 4 * N;                    // buffer A [0, 2N), buffer B [2N, 4N)
   static constexpr size_t dft_bytes = (size_t)NCH * CHUNK;
   static_assert(bytes <= 232448, "shared memory per CTA");
@@ -191,9 +198,12 @@ __global__ void __launch_bounds__(512, 1) k_exit_tma(BatchArgs a, const __grid_c
 __device__ __forceinline__ uint16_t bf16_bits(float v) { return __bfloat16_as_ushort(__float2bfloat16_rn(v)); }
 __device__ __forceinline__ float bf16_value(uint16_t b) { return __bfloat162float(__ushort_as_bfloat16(b)); }
 // x = hi + lo to within 2^-16 |x| (BF16 keeps 8 significant bits)
-__device__ __forceinline__ void split_bf16(float v, uint16_t& hi, uint16_t& lo) {
-  hi = bf16_bits(v);
-  lo = bf16_bits(v - bf16_value(hi));
+// Two values as their hi and lo BF16 parts, packed (x in the low half).
+__device__ __forceinline__ void split2_bf16(float x, float y, uint32_t& hi, uint32_t& lo) {
+  const __nv_bfloat162 h = __floats2bfloat162_rn(x, y);
+  hi = *(const uint32_t*)&h;
+  const __nv_bfloat162 l = __floats2bfloat162_rn(x - __uint_as_float(hi << 16), y - __uint_as_float(hi & 0xffff0000u));
+  lo = *(const uint32_t*)&l;
 }
 
 // The DFT matrix of one pass as NCH chunks (one per 16-wide K slice), each the
@@ -233,15 +243,8 @@ __device__ __forceinline__ void put8(unsigned char* slice, int row, int h, const
   uint32_t rh[4], rl[4], ih[4], il[4];
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
-    uint16_t a0, b0, a1, b1;
-    split_bf16(re[2 * q], a0, b0);
-    split_bf16(re[2 * q + 1], a1, b1);
-    rh[q] = (uint32_t)a0 | ((uint32_t)a1 << 16);
-    rl[q] = (uint32_t)b0 | ((uint32_t)b1 << 16);
-    split_bf16(im[2 * q], a0, b0);
-    split_bf16(im[2 * q + 1], a1, b1);
-    ih[q] = (uint32_t)a0 | ((uint32_t)a1 << 16);
-    il[q] = (uint32_t)b0 | ((uint32_t)b1 << 16);
+    split2_bf16(re[2 * q], re[2 * q + 1], rh[q], rl[q]);
+    split2_bf16(im[2 * q], im[2 * q + 1], ih[q], il[q]);
   }
   unsigned char* p = slice + (size_t)(row / 8) * C::BSBO + h * 128 + (row % 8) * 16;
   *(uint4*)p = make_uint4(rh[0], rh[1], rh[2], rh[3]);
@@ -277,7 +280,7 @@ template <int N>
 __global__ void __launch_bounds__(FarTc<N>::T, 1)
     k_far_tc(FarArgs a, const __grid_constant__ TmaDesc tm_psi, const __grid_constant__ TmaDesc tm_meas) {
   using C = FarTc<N>;
-  constexpr int NN = N * N, HALF = C::HALF, NCH = C::NCH, NSB = C::NSB, NSS = C::NSS;
+  constexpr int NN = N * N, G = C::G, NU = C::NCH / G, NCH = C::NCH, NSB = C::NSB, NSS = C::NSS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   wait_prior_grid();
   unsigned char* smem = smem_raw + ((1024u - (tc::smem_u32(smem_raw) & 1023u)) & 1023u);
@@ -293,6 +296,8 @@ __global__ void __launch_bounds__(FarTc<N>::T, 1)
   uint64_t* p1done = emptyS + NSS;
   uint64_t* p2done = p1done + 1;
   uint64_t* drained = p2done + 1;
+  uint64_t* stored = drained + 1;
+  uint64_t* handed = stored + 1;
   uint32_t* holder = (uint32_t*)(smem + C::misc);
   volatile int* abort_s = (volatile int*)(holder + 1);
 
@@ -303,7 +308,7 @@ __global__ void __launch_bounds__(FarTc<N>::T, 1)
       tc::mbar_init(&emptyF[s], 1);
     }
     for (int s = 0; s < NSB; ++s) {
-      tc::mbar_init(&fullB[s], C::PW);
+      tc::mbar_init(&fullB[s], 8);
       tc::mbar_init(&emptyB[s], 1);
     }
     for (int s = 0; s < NSS; ++s) {
@@ -313,6 +318,8 @@ __global__ void __launch_bounds__(FarTc<N>::T, 1)
     tc::mbar_init(p1done, 1);
     tc::mbar_init(p2done, 1);
     tc::mbar_init(drained, C::PW);
+    tc::mbar_init(stored, C::PW);
+    for (int w = 0; w < C::PW; ++w) tc::mbar_init(&handed[w], 1);
     *abort_s = 0;
     tc::fence_mbar_init();
   }
@@ -427,10 +434,12 @@ __global__ void __launch_bounds__(FarTc<N>::T, 1)
   } else if (warp == C::PW + 1) {
     // ================================ TMA warp ====================================
     // Stages, in the order the producers consume them, the exit waves of the
-    // forward transforms (N x 32-float tiles, 16 complex columns each) and
-    // the measured intensities of the data term (N x 32-float tiles).
+    // forward transforms (N x 32-float tiles, 16 complex columns each), the
+    // measured intensities of the data term (N x 32-float tiles) and, once the
+    // producers have stored them, the far fields of the inverse transforms but
+    // the first.
     if (lane == 0) {
-      uint32_t ps = 0;
+      uint32_t ps = 0, np = 0;
       bool ok = true;
       auto stage = [&](const TmaDesc* map, int x, int z) {
         const int sl = (int)(ps % NSS);
@@ -449,6 +458,11 @@ __global__ void __launch_bounds__(FarTc<N>::T, 1)
           for (int s = 0; s < NCH && ok; ++s) stage(&tm_psi, 32 * s, slot * a.M + k);
         if (backward)
           for (int b = 0; b < (NCH + 1) / 2 && ok; ++b) stage(&tm_meas, 32 * b, j);
+        if (backward && a.M > 1 && ok) {
+          if (!tc::mbar_wait(stored, np++ & 1)) ok = false;
+          for (int k = a.M - 2; k >= 0 && ok; --k)
+            for (int s = 0; s < NCH && ok; ++s) stage(&tm_psi, 32 * s, slot * a.M + k);
+        }
       }
       if (!ok) *abort_s = 1;
       // tiles still in flight land before the CTA exits (the last fill of each slot)
@@ -460,15 +474,19 @@ __global__ void __launch_bounds__(FarTc<N>::T, 1)
     }
   } else {
     // ============================= producer warps =================================
-    const int q4 = warp & 3, h = warp >> 2;
+    // At window 128 the slices of even and odd K steps come from eight warps
+    // each: a slice's chain (load, split, store, publish) is long, and eight
+    // warps in a row left the tensor cores waiting for it. (At 32 and 64, where a
+    // pass has two and four slices, eight warps are faster.)
+    const int q4 = warp & 3, h = (warp >> 2) & 1, g = warp >> 3;
     const int row = 32 * q4 + lane;           // TMEM lane = operand row
     const bool act = row < N;                  // warp-uniform
     const uint32_t lrow = (uint32_t)(32 * q4) << 16;
     const float invN = 1.0f / (float)N;
-    uint32_t pb = 0, ps = 0, n = 0, nd = 0;
-    float acc[HALF];                           // I, then the far-field factor, of columns 16 s + 8 h + [0, 8)
+    uint32_t pb = g, ps = 0, n = 0, nd = 0, nh = 0;
+    float acc[C::COLS_T];                      // I, then the far-field factor, of columns 16 (G u + g) + 8 h + [0, 8)
 #pragma unroll
-    for (int i = 0; i < HALF; ++i) acc[i] = 0.f;
+    for (int i = 0; i < C::COLS_T; ++i) acc[i] = 0.f;
     bool alive = true;
 
     // takes B slot pb (waiting for it to be free), fills it, publishes it
@@ -483,7 +501,7 @@ __global__ void __launch_bounds__(FarTc<N>::T, 1)
       tc::fence_before_sync();
       __syncwarp();
       if (lane == 0) tc::mbar_arrive(&fullB[sb]);
-      ++pb;
+      pb += G;
     };
     // waits for staged tile ps; returns it (null if a wait gave up)
     auto staged = [&]() -> const unsigned char* {
@@ -499,128 +517,111 @@ __global__ void __launch_bounds__(FarTc<N>::T, 1)
       if (lane == 0) tc::mbar_arrive(&emptyS[(int)(ps % NSS)]);
       ++ps;
     };
-    // pass-1 slices of a forward transform from the staged exit wave
+    // passes over a staged tile of the other warps' slices
+    auto skip_staged = [&]() {
+      staged();
+      if (alive) release_staged();
+    };
+    // pass-1 slice G u + g from staged tile G u + g (of G) of an exit wave, or
+    // (SCALE) of a far field, times the factors
+    auto produce_slice = [&](int u, auto scale) {
+      if (G == 2 && g == 1) skip_staged();
+      if (!alive) return;
+      const unsigned char* tile = staged();
+      if (!alive) return;
+      float4 v[4];
+      if (act) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) v[i] = staged_chunk(tile, row, 4 * h + i);
+      }
+      publish([&](unsigned char* slice) {
+        float re[8], im[8];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const float f0 = scale(u, 2 * i), f1 = scale(u, 2 * i + 1);
+          re[2 * i] = v[i].x * f0; im[2 * i] = v[i].y * f0;
+          re[2 * i + 1] = v[i].z * f1; im[2 * i + 1] = v[i].w * f1;
+        }
+        put8<N>(slice, row, h, re, im);
+      });
+      if (!alive) return;
+      release_staged();
+      if (G == 2 && g == 0) skip_staged();
+    };
     auto produce_staged = [&]() {
 #pragma unroll 1
-      for (int s = 0; s < NCH; ++s) {
-        const unsigned char* tile = staged();
-        if (!alive) break;
-        float4 v[4];
-        if (act) {
-#pragma unroll
-          for (int i = 0; i < 4; ++i) v[i] = staged_chunk(tile, row, 4 * h + i);
-        }
-        publish([&](unsigned char* slice) {
-          float re[8], im[8];
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            re[2 * i] = v[i].x; im[2 * i] = v[i].y; re[2 * i + 1] = v[i].z; im[2 * i + 1] = v[i].w;
-          }
-          put8<N>(slice, row, h, re, im);
-        });
-        if (!alive) break;
-        release_staged();
-      }
+      for (int u = 0; u < NU && alive; ++u) produce_slice(u, [](int, int) { return 1.f; });
     };
-    // pass-1 slices of an inverse transform from a far field in global memory
-    // (just written by this CTA, so in L2), times the factors
-    auto produce_global = [&](const float2* src) {
-      constexpr int G = 2;   // slices of loads in flight
+    auto produce_scaled = [&]() {
 #pragma unroll
-      for (int s0 = 0; s0 < NCH; s0 += G) {
-        if (!alive) break;
-        float4 v[G][4];
-        if (act) {
-#pragma unroll
-          for (int g = 0; g < G; ++g) {
-            const float4* p4 = (const float4*)(src + (size_t)row * N + 16 * (s0 + g) + 8 * h);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) v[g][i] = __ldcg(p4 + i);
-          }
-        }
-#pragma unroll
-        for (int g = 0; g < G; ++g) {
-          if (!alive) break;
-          publish([&](unsigned char* slice) {
-            float re[8], im[8];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              re[2 * i] = v[g][i].x; im[2 * i] = v[g][i].y; re[2 * i + 1] = v[g][i].z; im[2 * i + 1] = v[g][i].w;
-            }
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              re[i] *= acc[8 * (s0 + g) + i];
-              im[i] *= acc[8 * (s0 + g) + i];
-            }
-            put8<N>(slice, row, h, re, im);
-          });
-        }
-      }
+      for (int u = 0; u < NU; ++u)
+        if (alive) produce_slice(u, [&](int v, int i) { return acc[8 * v + i]; });
     };
     // slices from an accumulator in TMEM: pass-2 slices from buffer A, or
     // (SCALE) the first inverse transform's pass-1 slices from the last forward
     // far field in buffer B, times 1/N and the factors
-    auto produce_tmem = [&](uint32_t buf, bool scale) {
-      constexpr int G = NCH < 2 ? NCH : 2;   // slices per TMEM round trip
-      if (scale) {
+    auto tmem_slice = [&](uint32_t buf, int u, auto scale) {
+      float re[8], im[8];
+      if (act) {
+        const uint32_t col = 16 * (G * u + g) + 8 * h;
+        tc::tmem_ld8(buf + lrow + col, re);
+        tc::tmem_ld8(buf + lrow + N + col, im);
+        tc::tmem_wait_ld();
 #pragma unroll
-        for (int s = 0; s < NCH; ++s) {
-          if (!alive) break;
-          float re[8], im[8];
-          if (act) {
-            tc::tmem_ld8(buf + lrow + 16 * s + 8 * h, re);
-            tc::tmem_ld8(buf + lrow + N + 16 * s + 8 * h, im);
-            tc::tmem_wait_ld();
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              const float f = acc[8 * s + i] * invN;
-              re[i] *= f;
-              im[i] *= f;
-            }
-          }
-          publish([&](unsigned char* slice) { put8<N>(slice, row, h, re, im); });
+        for (int i = 0; i < 8; ++i) {
+          const float f = scale(u, i);
+          re[i] *= f;
+          im[i] *= f;
         }
-        return;
       }
+      publish([&](unsigned char* slice) { put8<N>(slice, row, h, re, im); });
+    };
+    auto produce_tmem = [&]() {   // (rolled: straight-line code runs at the rate of its fetch)
 #pragma unroll 1
-      for (int s0 = 0; s0 < NCH; s0 += G) {
-        if (!alive) break;
-        float re[G][8], im[G][8];
-        if (act) {
+      for (int u = 0; u < NU && alive; ++u) tmem_slice(bufA, u, [](int, int) { return 1.f; });
+    };
+    auto produce_tmem_scaled = [&]() {
 #pragma unroll
-          for (int g = 0; g < G; ++g) {
-            tc::tmem_ld8(buf + lrow + 16 * (s0 + g) + 8 * h, re[g]);
-            tc::tmem_ld8(buf + lrow + N + 16 * (s0 + g) + 8 * h, im[g]);
-          }
-          tc::tmem_wait_ld();
-        }
-#pragma unroll
-        for (int g = 0; g < G; ++g) {
-          if (!alive) break;
-          publish([&](unsigned char* slice) { put8<N>(slice, row, h, re[g], im[g]); });
-        }
-      }
+      for (int u = 0; u < NU; ++u)
+        if (alive) tmem_slice(bufB, u, [&](int v, int i) { return acc[8 * v + i] * invN; });
+    };
+    // 16-byte chunk c (of 4) of row r of the warp's tile; rows of 64 bytes,
+    // chunks permuted so that rows and columns of it are free of bank conflicts
+    auto wtile_chunk = [&](int r, int c) -> float4* {
+      return (float4*)(smem + C::wtile + warp * C::WTILE + r * 64 + ((c ^ ((r >> 1) & 3)) << 4));
     };
     // the pass-2 accumulator (buffer B) times `scale` to global memory (unless
     // dst is null); with `accumulate` its squared modulus is stored into
-    // (first) or added to acc
+    // (first) or added to acc. A thread owns a row of the accumulator: stored
+    // from there a warp's store touches 32 lines, 16 bytes each, and the rate of
+    // these requests bound the kernel; turned through the warp's tile it touches
+    // eight rows, 64 bytes each.
     auto drain = [&](float2* dst, bool accumulate, bool first, float scale) {
       if (act) {
 #pragma unroll
-        for (int s = 0; s < NCH; ++s) {
+        for (int u = 0; u < NU; ++u) {
+          const int col = 16 * (G * u + g) + 8 * h;
           float re[8], im[8];
-          tc::tmem_ld8(bufB + lrow + 16 * s + 8 * h, re);
-          tc::tmem_ld8(bufB + lrow + N + 16 * s + 8 * h, im);
+          tc::tmem_ld8(bufB + lrow + col, re);
+          tc::tmem_ld8(bufB + lrow + N + col, im);
           tc::tmem_wait_ld();
-          float4* d4 = dst ? (float4*)(dst + (size_t)row * N + 16 * s + 8 * h) : nullptr;
+          if (dst) __syncwarp();   // the previous slice has left the warp's tile
 #pragma unroll
           for (int i = 0; i < 8; i += 2) {
             const float x0 = re[i] * scale, y0 = im[i] * scale, x1 = re[i + 1] * scale, y1 = im[i + 1] * scale;
-            if (d4) d4[i / 2] = make_float4(x0, y0, x1, y1);
+            if (dst) *wtile_chunk(lane, i / 2) = make_float4(x0, y0, x1, y1);
             if (accumulate) {
               const float a0 = fmaf(x0, x0, y0 * y0), a1 = fmaf(x1, x1, y1 * y1);
-              acc[8 * s + i] = first ? a0 : acc[8 * s + i] + a0;
-              acc[8 * s + i + 1] = first ? a1 : acc[8 * s + i + 1] + a1;
+              acc[8 * u + i] = first ? a0 : acc[8 * u + i] + a0;
+              acc[8 * u + i + 1] = first ? a1 : acc[8 * u + i + 1] + a1;
+            }
+          }
+          if (dst) {
+            __syncwarp();
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+              const int r = 8 * t + lane / 4;
+              *(float4*)(dst + (size_t)(32 * q4 + r) * N + col + 2 * (lane % 4)) = *wtile_chunk(r, lane % 4);
             }
           }
         }
@@ -633,65 +634,94 @@ __global__ void __launch_bounds__(FarTc<N>::T, 1)
     };
     // the data term of position j from the intensities in acc: loss, ipred, and
     // the far-field factor (times 1/N for the unnormalised inverse) into acc;
-    // the measured values come from the staged tiles (none in the forward mode)
+    // the measured values come from the staged tiles (none in the forward mode).
+    // The loss of a row's columns is one running FP32 sum in column order of the
+    // half: the two warps that share the half hand it over after every slice.
     auto data_term = [&](int j) {
       float lsum = 0.f;
       bool bad = false;
-      float* ip = (a.ipred && act) ? a.ipred + (size_t)j * NN + (size_t)row * N + 8 * h : nullptr;
+      const bool sums = backward && a.mode != MODE_VJP;
+      float* mail = (float*)(smem + C::mail) + 32 * (warp & 7) + lane;
+      float* ip = (a.ipred && act) ? a.ipred + (size_t)j * NN + (size_t)(32 * q4) * N + 8 * h : nullptr;
+      const bool vec = ((uintptr_t)a.ipred & 15) == 0;
 #pragma unroll
-      for (int b = 0; b < (NCH + 1) / 2; ++b) {
-        float mv[2][8];
-        if (backward) {
+      for (int u = 0; u < NU; ++u) {
+        const int s = G * u + g, half = s & 1;
+        float mv[8];
+        if (backward) {   // (a tile holds the columns of two slices)
           const unsigned char* tile = staged();
           if (!alive) break;
           if (act) {
+            const float4 m0 = staged_chunk(tile, row, 4 * half + 2 * h);
+            const float4 m1 = staged_chunk(tile, row, 4 * half + 2 * h + 1);
+            mv[0] = m0.x; mv[1] = m0.y; mv[2] = m0.z; mv[3] = m0.w;
+            mv[4] = m1.x; mv[5] = m1.y; mv[6] = m1.z; mv[7] = m1.w;
+          }
+          if (G == 2 || half == 1) release_staged();
+        }
+        if (ip) {   // 16 rows x 32 bytes per store, through the warp's tile
+          __syncwarp();
 #pragma unroll
-            for (int g = 0; g < 2; ++g) {
-              const float4 m0 = staged_chunk(tile, row, 4 * g + 2 * h), m1 = staged_chunk(tile, row, 4 * g + 2 * h + 1);
-              mv[g][0] = m0.x; mv[g][1] = m0.y; mv[g][2] = m0.z; mv[g][3] = m0.w;
-              mv[g][4] = m1.x; mv[g][5] = m1.y; mv[g][6] = m1.z; mv[g][7] = m1.w;
+          for (int i = 0; i < 2; ++i)
+            *wtile_chunk(lane, i) = make_float4(acc[8 * u + 4 * i], acc[8 * u + 4 * i + 1], acc[8 * u + 4 * i + 2],
+                                                acc[8 * u + 4 * i + 3]);
+          __syncwarp();
+#pragma unroll
+          for (int t = 0; t < 2; ++t) {
+            const int r = 16 * t + lane / 2;
+            const float4 v = *wtile_chunk(r, lane & 1);
+            float* d = ip + (size_t)r * N + 16 * s + 4 * (lane & 1);
+            if (vec) {
+              *(float4*)d = v;
+            } else {
+              d[0] = v.x; d[1] = v.y; d[2] = v.z; d[3] = v.w;
             }
           }
-          release_staged();
+        }
+        if (!backward) continue;
+        if (G == 2 && sums && s > 0) {   // the other warp's sum up to the slice before
+          if (!role_wait(&handed[warp ^ 8], nh & 1, abort_s)) {
+            alive = false;
+            break;
+          }
+          ++nh;
+          lsum = *mail;
         }
         if (act) {
 #pragma unroll
-          for (int g = 0; g < 2; ++g) {
-            const int s = 2 * b + g;
-            if (s >= NCH) break;
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              const int c = 16 * s + i, ai = 8 * s + i;
-              const float I = acc[ai];
-              if (ip) ip[c] = I;
-              if (!backward) continue;
-              const float Im = mv[g][i];
-              float fac;
-              if (a.mode == MODE_VJP) {
-                bad |= !isfinite(Im);
-                fac = 2.f * Im;
+          for (int i = 0; i < 8; ++i) {
+            const int ai = 8 * u + i;
+            const float I = acc[ai], Im = mv[i];
+            float fac;
+            if (a.mode == MODE_VJP) {
+              bad |= !isfinite(Im);
+              fac = 2.f * Im;
+            } else {
+              bad |= !(Im >= 0.f) || !isfinite(Im);
+              const float Ie = I + a.eps;
+              if (a.mode == MODE_LSQML_GAUSS || a.mode == MODE_GRAD_GAUSS) {
+                const float sIe = sqrtf(Ie), sIm = sqrtf(Im);
+                const float dd = sIe - sIm;
+                lsum = fmaf(dd, dd, lsum);
+                const float rho = sIm / sIe;
+                fac = (a.mode == MODE_LSQML_GAUSS) ? rho - 1.f : 2.f * (1.f - rho);
               } else {
-                bad |= !(Im >= 0.f) || !isfinite(Im);
-                const float Ie = I + a.eps;
-                if (a.mode == MODE_LSQML_GAUSS || a.mode == MODE_GRAD_GAUSS) {
-                  const float sIe = sqrtf(Ie), sIm = sqrtf(Im);
-                  const float dd = sIe - sIm;
-                  lsum = fmaf(dd, dd, lsum);
-                  const float rho = sIm / sIe;
-                  fac = (a.mode == MODE_LSQML_GAUSS) ? rho - 1.f : 2.f * (1.f - rho);
-                } else {
-                  lsum += I - Im * logf(Ie);
-                  const float qq = Im / Ie;
-                  fac = (a.mode == MODE_LSQML_POISSON) ? 0.5f * (qq - 1.f) : 2.f * (1.f - qq);
-                }
+                lsum += I - Im * logf(Ie);
+                const float qq = Im / Ie;
+                fac = (a.mode == MODE_LSQML_POISSON) ? 0.5f * (qq - 1.f) : 2.f * (1.f - qq);
               }
-              acc[ai] = fac * invN;
             }
+            acc[ai] = fac * invN;
           }
+        }
+        if (G == 2 && sums && s < NCH - 1) {
+          *mail = lsum;
+          __syncwarp();
+          if (lane == 0) tc::mbar_arrive(&handed[warp]);
         }
       }
       if (bad) atomicOr(a.status, FLAG_NONFINITE);
-      if (a.loss && backward && a.mode != MODE_VJP) {
+      if (a.loss && sums && g == G - 1) {
         double v = (double)lsum;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
@@ -701,7 +731,7 @@ __global__ void __launch_bounds__(FarTc<N>::T, 1)
 
     // the previous image, drained once the next image's pass-1 slices are out
     float2* prev_dst = nullptr;
-    bool have_prev = false, prev_fwd = false, prev_first = false, prev_last_fwd = false;
+    bool have_prev = false, prev_fwd = false, prev_first = false, prev_last_fwd = false, prev_before_last = false;
     int prev_j = -1;
     auto drain_prev = [&]() {
       if (!role_wait(p2done, (uint32_t)(nd & 1), abort_s)) {
@@ -714,6 +744,11 @@ __global__ void __launch_bounds__(FarTc<N>::T, 1)
       drain(prev_fwd && !backward ? nullptr : prev_dst, prev_fwd, prev_first, prev_fwd ? invN : 1.f);
       arrive_drained();
       ++nd;
+      if (backward && prev_before_last) {   // every far field that is read again has been stored
+        asm volatile("fence.proxy.async;\n" ::: "memory");   // (the copies that read them are asynchronous)
+        __syncwarp();
+        if (lane == 0) tc::mbar_arrive(stored);
+      }
       if (prev_fwd && prev_last_fwd && !backward) data_term(prev_j);
       have_prev = false;
     };
@@ -741,11 +776,11 @@ __global__ void __launch_bounds__(FarTc<N>::T, 1)
           drain(nullptr, true, a.M == 1, invN);
           ++nd;
           data_term(j);
-          if (alive) produce_tmem(bufB, true);
+          if (alive) produce_tmem_scaled();
           arrive_drained();
           have_prev = false;
         } else {
-          produce_global(io);
+          produce_scaled();
           if (have_prev && alive) drain_prev();
         }
         if (!alive) break;
@@ -754,12 +789,13 @@ __global__ void __launch_bounds__(FarTc<N>::T, 1)
           break;
         }
         tc::fence_after_sync();
-        produce_tmem(bufA, false);
+        produce_tmem();
         prev_dst = io;
         have_prev = true;
         prev_fwd = fwd;
         prev_first = fwd && k == 0;
         prev_last_fwd = fwd && k == a.M - 1;
+        prev_before_last = fwd && k == a.M - 2;
         prev_j = j;
       }
     }
