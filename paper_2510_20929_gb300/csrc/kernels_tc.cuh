@@ -27,8 +27,8 @@
 // scaled and transformed back, and chi_jk = F^-1[(rho - 1) Psi_jk] overwrites
 // the scratch for the overlap-add part of the pass.
 //
-// Warp roles: eight producer warps (sixteen at N = 128, taking the K steps in
-// turn) write the B operand of every K step (a
+// Warp roles: groups of four producer warps (four groups at N = 128, else two)
+// take the K steps in turn and write the step's B operand (a
 // 16-wide K slice of four BF16 planes) into a ring of shared-memory slots;
 // one MMA warp streams the DFT-matrix chunks and issues the MMAs as slices
 // land; one TMA warp stages the exit waves and the measured intensities from
@@ -39,10 +39,17 @@
 // pass-1 accumulator in TMEM. Pass 1 accumulates in TMEM buffer A, pass 2 in
 // buffer B, so an image's pass-2 result drains while the next image's pass 1
 // runs.
+//
+// Bound by the MMAs' operand reads from shared memory (about 1200 cycles per K
+// step at N = 128, where the MMAs themselves take 768) and, for the rest, by the
+// producers' chains. Measured on GB300, 256 positions: N = 128, 5 modes 453 ->
+// 295 us, 1 mode 126 -> 84; N = 64, 4 modes 143 -> 118; N = 32, 2 modes, 512
+// positions 94 -> 78 (before: eight warps on every slice, far fields stored and
+// read back 16 bytes per line).
 #pragma once
 #include <cuda_bf16.h>
 
-#include "common.cuh"
+#include "kernels_pair.cuh"
 #include "tc.cuh"
 
 namespace ptycho {
@@ -50,11 +57,10 @@ namespace ptycho {
 template <int N>
 struct FarTc {
   static_assert(N == 32 || N == 64 || N == 128, "DFT-GEMM windows");
-  static constexpr int G = N == 128 ? 2 : 1;      // groups of producer warps, slices s % G each
-  static constexpr int PW = 8 * G;                // producer warps: TMEM lane quarter w % 4, slice half (w / 4) % 2,
-                                                  // group w / 8
+  static constexpr int G = N == 128 ? 4 : 2;      // groups of four producer warps; group g takes the slices s % G = g
+  static constexpr int PW = 4 * G;                // producer warps: TMEM lane quarter w % 4, group w / 4
   static constexpr int T = 32 * (PW + 2);         // and the MMA warp (PW) and the TMA warp (PW + 1)
-  static constexpr int COLS_T = N / 2 / G;        // columns per producer thread: 16 s + 8 ((w / 4) % 2) + [0, 8)
+  static constexpr int COLS_T = N / G;            // columns per producer thread: 16 (G u + g) + [0, 16)
   static constexpr int NCH = N / 16;              // K steps of one pass (= DFT chunks)
   static constexpr int NSF = 4;                   // ring slots of DFT chunks
   static constexpr int NSB = 4;                   // ring slots of B slices
@@ -70,14 +76,14 @@ struct FarTc {
   static constexpr size_t fring = 0;
   static constexpr size_t sring = fring + (size_t)NSF * CHUNK;   // 1024-byte aligned (swizzled tiles)
   static constexpr size_t bring = sring + (size_t)NSS * SSLOT;
-  static constexpr uint32_t WTILE = 32 * 64;                 // a producer warp's 32 rows x 8 complex columns
+  static constexpr uint32_t WTILE = 16 * 128;                // a producer warp's tile: 16 rows of a slice
   static constexpr size_t wtile = bring + (size_t)NSB * SLICE;
   static constexpr size_t bars = wtile + (size_t)PW * WTILE;
   static constexpr int NBAR = 2 * NSF + 2 * NSB + 2 * NSS + 4 + PW;   // F, B and staging rings, p1, p2, drained, stored,
                                                                       // and a hand-over per producer warp
   static constexpr size_t misc = bars + 8 * (size_t)NBAR;
-  static constexpr size_t mail = misc + 16;                     // running loss of each pair of producer warps
-  static constexpr size_t bytes = mail + 8 * 32 * 4 + 1024;   // + alignment of the base to 1024 bytes
+  static constexpr size_t mail = misc + 16;                     // running losses of each row
+  static constexpr size_t bytes = mail + 128 * 8 + 1024;   // + alignment of the base to 1024 bytes
   static constexpr uint32_t COLS = 4 * N;                    // buffer A [0, 2N), buffer B [2N, 4N)
   static constexpr size_t dft_bytes = (size_t)NCH * CHUNK;
   static_assert(bytes <= 232448, "shared memory per CTA");
@@ -308,12 +314,12 @@ __global__ void __launch_bounds__(FarTc<N>::T, 1)
       tc::mbar_init(&emptyF[s], 1);
     }
     for (int s = 0; s < NSB; ++s) {
-      tc::mbar_init(&fullB[s], 8);
+      tc::mbar_init(&fullB[s], 4);
       tc::mbar_init(&emptyB[s], 1);
     }
     for (int s = 0; s < NSS; ++s) {
       tc::mbar_init(&fullS[s], 1);
-      tc::mbar_init(&emptyS[s], C::PW);
+      tc::mbar_init(&emptyS[s], 4);
     }
     tc::mbar_init(p1done, 1);
     tc::mbar_init(p2done, 1);
@@ -435,7 +441,7 @@ __global__ void __launch_bounds__(FarTc<N>::T, 1)
     // ================================ TMA warp ====================================
     // Stages, in the order the producers consume them, the exit waves of the
     // forward transforms (N x 32-float tiles, 16 complex columns each), the
-    // measured intensities of the data term (N x 32-float tiles) and, once the
+    // measured intensities of the data term (N x 16-float tiles) and, once the
     // producers have stored them, the far fields of the inverse transforms but
     // the first.
     if (lane == 0) {
@@ -447,7 +453,7 @@ __global__ void __launch_bounds__(FarTc<N>::T, 1)
           ok = false;
           return;
         }
-        tc::mbar_expect_tx(&fullS[sl], C::SSLOT);
+        tc::mbar_expect_tx(&fullS[sl], map == &tm_meas ? C::SSLOT / 2 : C::SSLOT);
         tc::tma_load_3d(sring + (size_t)sl * C::SSLOT, map, x, 0, z, &fullS[sl]);
         ++ps;
       };
@@ -457,7 +463,7 @@ __global__ void __launch_bounds__(FarTc<N>::T, 1)
         for (int k = 0; k < a.M && ok; ++k)
           for (int s = 0; s < NCH && ok; ++s) stage(&tm_psi, 32 * s, slot * a.M + k);
         if (backward)
-          for (int b = 0; b < (NCH + 1) / 2 && ok; ++b) stage(&tm_meas, 32 * b, j);
+          for (int s = 0; s < NCH && ok; ++s) stage(&tm_meas, 16 * s, j);
         if (backward && a.M > 1 && ok) {
           if (!tc::mbar_wait(stored, np++ & 1)) ok = false;
           for (int k = a.M - 2; k >= 0 && ok; --k)
@@ -474,17 +480,16 @@ __global__ void __launch_bounds__(FarTc<N>::T, 1)
     }
   } else {
     // ============================= producer warps =================================
-    // At window 128 the slices of even and odd K steps come from eight warps
-    // each: a slice's chain (load, split, store, publish) is long, and eight
-    // warps in a row left the tensor cores waiting for it. (At 32 and 64, where a
-    // pass has two and four slices, eight warps are faster.)
-    const int q4 = warp & 3, h = (warp >> 2) & 1, g = warp >> 3;
+    // Each group of four warps takes whole slices in turn: a slice's chain (wait,
+    // load, split, store, publish) is long, and eight warps on one slice after
+    // the other left the tensor cores waiting for it.
+    const int q4 = warp & 3, g = warp >> 2;
     const int row = 32 * q4 + lane;           // TMEM lane = operand row
     const bool act = row < N;                  // warp-uniform
     const uint32_t lrow = (uint32_t)(32 * q4) << 16;
     const float invN = 1.0f / (float)N;
-    uint32_t pb = g, ps = 0, n = 0, nd = 0, nh = 0;
-    float acc[C::COLS_T];                      // I, then the far-field factor, of columns 16 (G u + g) + 8 h + [0, 8)
+    uint32_t pb = g, ps = g, n = 0, nd = 0, nh = 0;
+    float acc[C::COLS_T];                      // I, then the far-field factor, of columns 16 (G u + g) + [0, 16)
 #pragma unroll
     for (int i = 0; i < C::COLS_T; ++i) acc[i] = 0.f;
     bool alive = true;
@@ -515,38 +520,28 @@ __global__ void __launch_bounds__(FarTc<N>::T, 1)
     auto release_staged = [&]() {
       __syncwarp();
       if (lane == 0) tc::mbar_arrive(&emptyS[(int)(ps % NSS)]);
-      ++ps;
+      ps += G;
     };
-    // passes over a staged tile of the other warps' slices
-    auto skip_staged = [&]() {
-      staged();
-      if (alive) release_staged();
-    };
-    // pass-1 slice G u + g from staged tile G u + g (of G) of an exit wave, or
-    // (SCALE) of a far field, times the factors
+    // pass-1 slice G u + g from the staged tile of an exit wave or a far field,
+    // times the factors
     auto produce_slice = [&](int u, auto scale) {
-      if (G == 2 && g == 1) skip_staged();
-      if (!alive) return;
       const unsigned char* tile = staged();
       if (!alive) return;
-      float4 v[4];
-      if (act) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) v[i] = staged_chunk(tile, row, 4 * h + i);
-      }
       publish([&](unsigned char* slice) {
-        float re[8], im[8];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const float f0 = scale(u, 2 * i), f1 = scale(u, 2 * i + 1);
-          re[2 * i] = v[i].x * f0; im[2 * i] = v[i].y * f0;
-          re[2 * i + 1] = v[i].z * f1; im[2 * i + 1] = v[i].w * f1;
+        for (int h = 0; h < 2; ++h) {
+          float re[8], im[8];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const float4 v = staged_chunk(tile, row, 4 * h + i);
+            const float f0 = scale(u, 8 * h + 2 * i), f1 = scale(u, 8 * h + 2 * i + 1);
+            re[2 * i] = v.x * f0; im[2 * i] = v.y * f0;
+            re[2 * i + 1] = v.z * f1; im[2 * i + 1] = v.w * f1;
+          }
+          put8<N>(slice, row, h, re, im);
         }
-        put8<N>(slice, row, h, re, im);
       });
-      if (!alive) return;
-      release_staged();
-      if (G == 2 && g == 0) skip_staged();
+      if (alive) release_staged();
     };
     auto produce_staged = [&]() {
 #pragma unroll 1
@@ -555,26 +550,27 @@ __global__ void __launch_bounds__(FarTc<N>::T, 1)
     auto produce_scaled = [&]() {
 #pragma unroll
       for (int u = 0; u < NU; ++u)
-        if (alive) produce_slice(u, [&](int v, int i) { return acc[8 * v + i]; });
+        if (alive) produce_slice(u, [&](int v, int i) { return acc[16 * v + i]; });
     };
     // slices from an accumulator in TMEM: pass-2 slices from buffer A, or
     // (SCALE) the first inverse transform's pass-1 slices from the last forward
     // far field in buffer B, times 1/N and the factors
     auto tmem_slice = [&](uint32_t buf, int u, auto scale) {
-      float re[8], im[8];
+      float re[16], im[16];
       if (act) {
-        const uint32_t col = 16 * (G * u + g) + 8 * h;
-        tc::tmem_ld8(buf + lrow + col, re);
-        tc::tmem_ld8(buf + lrow + N + col, im);
-        tc::tmem_wait_ld();
+        const uint32_t col = buf + lrow + 16 * (G * u + g);
+        tc::tmem_ld16x2_wait(col, re, col + N, im);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
+        for (int i = 0; i < 16; ++i) {
           const float f = scale(u, i);
           re[i] *= f;
           im[i] *= f;
         }
       }
-      publish([&](unsigned char* slice) { put8<N>(slice, row, h, re, im); });
+      publish([&](unsigned char* slice) {
+        put8<N>(slice, row, 0, re, im);
+        put8<N>(slice, row, 1, re + 8, im + 8);
+      });
     };
     auto produce_tmem = [&]() {   // (rolled: straight-line code runs at the rate of its fetch)
 #pragma unroll 1
@@ -583,45 +579,50 @@ __global__ void __launch_bounds__(FarTc<N>::T, 1)
     auto produce_tmem_scaled = [&]() {
 #pragma unroll
       for (int u = 0; u < NU; ++u)
-        if (alive) tmem_slice(bufB, u, [&](int v, int i) { return acc[8 * v + i] * invN; });
+        if (alive) tmem_slice(bufB, u, [&](int v, int i) { return acc[16 * v + i] * invN; });
     };
-    // 16-byte chunk c (of 4) of row r of the warp's tile; rows of 64 bytes,
-    // chunks permuted so that rows and columns of it are free of bank conflicts
-    auto wtile_chunk = [&](int r, int c) -> float4* {
-      return (float4*)(smem + C::wtile + warp * C::WTILE + r * 64 + ((c ^ ((r >> 1) & 3)) << 4));
-    };
+    // 16-byte chunk c of row r of the warp's tile, of 16 rows of 128 or 32 rows of
+    // 64 bytes; chunks permuted so that rows and columns of it are free of bank
+    // conflicts
+    unsigned char* wtile = smem + C::wtile + warp * C::WTILE;
+    auto chunk128 = [&](int r, int c) { return (float4*)(wtile + r * 128 + ((c ^ (r & 7)) << 4)); };
+    auto chunk64 = [&](int r, int c) { return (float4*)(wtile + r * 64 + ((c ^ ((r >> 1) & 3)) << 4)); };
     // the pass-2 accumulator (buffer B) times `scale` to global memory (unless
     // dst is null); with `accumulate` its squared modulus is stored into
     // (first) or added to acc. A thread owns a row of the accumulator: stored
     // from there a warp's store touches 32 lines, 16 bytes each, and the rate of
-    // these requests bound the kernel; turned through the warp's tile it touches
-    // eight rows, 64 bytes each.
+    // these requests bound the kernel; turned through the warp's tile it writes
+    // four whole lines.
     auto drain = [&](float2* dst, bool accumulate, bool first, float scale) {
       if (act) {
 #pragma unroll
         for (int u = 0; u < NU; ++u) {
-          const int col = 16 * (G * u + g) + 8 * h;
-          float re[8], im[8];
-          tc::tmem_ld8(bufB + lrow + col, re);
-          tc::tmem_ld8(bufB + lrow + N + col, im);
-          tc::tmem_wait_ld();
-          if (dst) __syncwarp();   // the previous slice has left the warp's tile
+          const int col = 16 * (G * u + g);
+          float re[16], im[16];
+          tc::tmem_ld16x2_wait(bufB + lrow + col, re, bufB + lrow + N + col, im);
 #pragma unroll
-          for (int i = 0; i < 8; i += 2) {
-            const float x0 = re[i] * scale, y0 = im[i] * scale, x1 = re[i + 1] * scale, y1 = im[i + 1] * scale;
-            if (dst) *wtile_chunk(lane, i / 2) = make_float4(x0, y0, x1, y1);
+          for (int i = 0; i < 16; ++i) {
+            re[i] *= scale;
+            im[i] *= scale;
             if (accumulate) {
-              const float a0 = fmaf(x0, x0, y0 * y0), a1 = fmaf(x1, x1, y1 * y1);
-              acc[8 * u + i] = first ? a0 : acc[8 * u + i] + a0;
-              acc[8 * u + i + 1] = first ? a1 : acc[8 * u + i + 1] + a1;
+              const float a0 = fmaf(re[i], re[i], im[i] * im[i]);
+              acc[16 * u + i] = first ? a0 : acc[16 * u + i] + a0;
             }
           }
           if (dst) {
-            __syncwarp();
 #pragma unroll
-            for (int t = 0; t < 4; ++t) {
-              const int r = 8 * t + lane / 4;
-              *(float4*)(dst + (size_t)(32 * q4 + r) * N + col + 2 * (lane % 4)) = *wtile_chunk(r, lane % 4);
+            for (int t = 0; t < 2; ++t) {
+              __syncwarp();   // the rows before have left the tile
+              if ((lane >> 4) == t)
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                  *chunk128(lane & 15, i) = make_float4(re[2 * i], im[2 * i], re[2 * i + 1], im[2 * i + 1]);
+              __syncwarp();
+#pragma unroll
+              for (int k = 0; k < 4; ++k) {
+                const int r = 4 * k + lane / 8;
+                *(float4*)(dst + (size_t)(32 * q4 + 16 * t + r) * N + col + 2 * (lane % 8)) = *chunk128(r, lane % 8);
+              }
             }
           }
         }
@@ -635,42 +636,31 @@ __global__ void __launch_bounds__(FarTc<N>::T, 1)
     // the data term of position j from the intensities in acc: loss, ipred, and
     // the far-field factor (times 1/N for the unnormalised inverse) into acc;
     // the measured values come from the staged tiles (none in the forward mode).
-    // The loss of a row's columns is one running FP32 sum in column order of the
-    // half: the two warps that share the half hand it over after every slice.
+    // The loss of a row is two running FP32 sums in column order, one per half
+    // of the slices; the warps that share the row hand them over from slice to
+    // slice.
     auto data_term = [&](int j) {
-      float lsum = 0.f;
+      float2 lsum = make_float2(0.f, 0.f);
       bool bad = false;
       const bool sums = backward && a.mode != MODE_VJP;
-      float* mail = (float*)(smem + C::mail) + 32 * (warp & 7) + lane;
-      float* ip = (a.ipred && act) ? a.ipred + (size_t)j * NN + (size_t)(32 * q4) * N + 8 * h : nullptr;
+      float2* mail = (float2*)(smem + C::mail) + row;
+      float* ip = (a.ipred && act) ? a.ipred + (size_t)j * NN + (size_t)(32 * q4) * N : nullptr;
       const bool vec = ((uintptr_t)a.ipred & 15) == 0;
 #pragma unroll
       for (int u = 0; u < NU; ++u) {
-        const int s = G * u + g, half = s & 1;
-        float mv[8];
-        if (backward) {   // (a tile holds the columns of two slices)
-          const unsigned char* tile = staged();
-          if (!alive) break;
-          if (act) {
-            const float4 m0 = staged_chunk(tile, row, 4 * half + 2 * h);
-            const float4 m1 = staged_chunk(tile, row, 4 * half + 2 * h + 1);
-            mv[0] = m0.x; mv[1] = m0.y; mv[2] = m0.z; mv[3] = m0.w;
-            mv[4] = m1.x; mv[5] = m1.y; mv[6] = m1.z; mv[7] = m1.w;
-          }
-          if (G == 2 || half == 1) release_staged();
-        }
-        if (ip) {   // 16 rows x 32 bytes per store, through the warp's tile
+        const int s = G * u + g;
+        if (ip) {   // 8 rows x 64 bytes per store, through the warp's tile
           __syncwarp();
 #pragma unroll
-          for (int i = 0; i < 2; ++i)
-            *wtile_chunk(lane, i) = make_float4(acc[8 * u + 4 * i], acc[8 * u + 4 * i + 1], acc[8 * u + 4 * i + 2],
-                                                acc[8 * u + 4 * i + 3]);
+          for (int i = 0; i < 4; ++i)
+            *chunk64(lane, i) = make_float4(acc[16 * u + 4 * i], acc[16 * u + 4 * i + 1], acc[16 * u + 4 * i + 2],
+                                            acc[16 * u + 4 * i + 3]);
           __syncwarp();
 #pragma unroll
-          for (int t = 0; t < 2; ++t) {
-            const int r = 16 * t + lane / 2;
-            const float4 v = *wtile_chunk(r, lane & 1);
-            float* d = ip + (size_t)r * N + 16 * s + 4 * (lane & 1);
+          for (int t = 0; t < 4; ++t) {
+            const int r = 8 * t + lane / 4;
+            const float4 v = *chunk64(r, lane % 4);
+            float* d = ip + (size_t)r * N + 16 * s + 4 * (lane % 4);
             if (vec) {
               *(float4*)d = v;
             } else {
@@ -679,8 +669,30 @@ __global__ void __launch_bounds__(FarTc<N>::T, 1)
           }
         }
         if (!backward) continue;
-        if (G == 2 && sums && s > 0) {   // the other warp's sum up to the slice before
-          if (!role_wait(&handed[warp ^ 8], nh & 1, abort_s)) {
+        const unsigned char* tile = staged();
+        if (!alive) break;
+        float4 t[4];   // what the loss adds
+        if (act) {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const float4 Im = *(const float4*)(tile + row * 64 + ((i ^ ((row >> 1) & 3)) << 4));
+            float* A = acc + 16 * u + 4 * i;
+            float4 f;
+            if (a.mode == MODE_VJP) {
+              bad |= !isfinite(Im.x) || !isfinite(Im.y) || !isfinite(Im.z) || !isfinite(Im.w);
+              f = make_float4(2.f * Im.x, 2.f * Im.y, 2.f * Im.z, 2.f * Im.w);
+            } else {
+              auto off = [](float x) { return !(x >= 0.f) || !isfinite(x); };
+              bad |= off(Im.x) || off(Im.y) || off(Im.z) || off(Im.w);
+              f = data_factor(a.mode, make_float4(A[0], A[1], A[2], A[3]), Im, a.eps, t[i]);
+            }
+            A[0] = f.x * invN; A[1] = f.y * invN; A[2] = f.z * invN; A[3] = f.w * invN;
+          }
+        }
+        release_staged();
+        if (!sums) continue;
+        if (s > 0) {   // the sums up to the slice before
+          if (!role_wait(&handed[q4 + 4 * ((g + G - 1) % G)], nh & 1, abort_s)) {
             alive = false;
             break;
           }
@@ -688,33 +700,18 @@ __global__ void __launch_bounds__(FarTc<N>::T, 1)
           lsum = *mail;
         }
         if (act) {
-#pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const int ai = 8 * u + i;
-            const float I = acc[ai], Im = mv[i];
-            float fac;
-            if (a.mode == MODE_VJP) {
-              bad |= !isfinite(Im);
-              fac = 2.f * Im;
+          const bool sq = a.mode == MODE_LSQML_GAUSS || a.mode == MODE_GRAD_GAUSS;
+          auto add = [&](float& l, const float4& v) {
+            if (sq) {
+              l = fmaf(v.x, v.x, l); l = fmaf(v.y, v.y, l); l = fmaf(v.z, v.z, l); l = fmaf(v.w, v.w, l);
             } else {
-              bad |= !(Im >= 0.f) || !isfinite(Im);
-              const float Ie = I + a.eps;
-              if (a.mode == MODE_LSQML_GAUSS || a.mode == MODE_GRAD_GAUSS) {
-                const float sIe = sqrtf(Ie), sIm = sqrtf(Im);
-                const float dd = sIe - sIm;
-                lsum = fmaf(dd, dd, lsum);
-                const float rho = sIm / sIe;
-                fac = (a.mode == MODE_LSQML_GAUSS) ? rho - 1.f : 2.f * (1.f - rho);
-              } else {
-                lsum += I - Im * logf(Ie);
-                const float qq = Im / Ie;
-                fac = (a.mode == MODE_LSQML_POISSON) ? 0.5f * (qq - 1.f) : 2.f * (1.f - qq);
-              }
+              l += v.x; l += v.y; l += v.z; l += v.w;
             }
-            acc[ai] = fac * invN;
-          }
+          };
+          add(lsum.x, t[0]); add(lsum.x, t[1]);
+          add(lsum.y, t[2]); add(lsum.y, t[3]);
         }
-        if (G == 2 && sums && s < NCH - 1) {
+        if (s < NCH - 1) {
           *mail = lsum;
           __syncwarp();
           if (lane == 0) tc::mbar_arrive(&handed[warp]);
@@ -722,10 +719,13 @@ __global__ void __launch_bounds__(FarTc<N>::T, 1)
       }
       if (bad) atomicOr(a.status, FLAG_NONFINITE);
       if (a.loss && sums && g == G - 1) {
-        double v = (double)lsum;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-        if (lane == 0 && v != 0.0) atomicAdd(a.loss, v);
+        for (int h = 0; h < 2; ++h) {
+          double v = (double)(h ? lsum.y : lsum.x);
+#pragma unroll
+          for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+          if (lane == 0 && v != 0.0) atomicAdd(a.loss, v);
+        }
       }
     };
 

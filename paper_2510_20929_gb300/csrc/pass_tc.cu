@@ -31,9 +31,9 @@ static PFN_cuTensorMapEncodeTiled_v12000 tmap_encoder() {
 }
 
 // Tensor map of a float32 [d2][d1][d0] array, tiles of b1 rows x b0 floats
-// (b0 * 4 = 128 bytes) written to shared memory with the 128-byte swizzle.
+// (b0 * 4 = 128 or 64 bytes) written to shared memory with the swizzle of that size.
 static bool encode_tiles(TmaDesc* out, const void* base, uint64_t d0, uint64_t d1, uint64_t d2, uint32_t b0,
-                         uint32_t b1) {
+                         uint32_t b1, CUtensorMapSwizzle swizzle) {
   PFN_cuTensorMapEncodeTiled_v12000 fn = tmap_encoder();
   if (!fn) return false;
   const cuuint64_t dims[3] = {d0, d1, d2};
@@ -43,7 +43,7 @@ static bool encode_tiles(TmaDesc* out, const void* base, uint64_t d0, uint64_t d
   CUtensorMap m;
   static_assert(sizeof(CUtensorMap) == sizeof(TmaDesc), "tensor map size");
   if (fn(&m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<void*>(base), dims, strides, box, es,
-         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+         CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
     return false;
   memcpy(out, &m, sizeof(m));
@@ -123,11 +123,13 @@ cudaError_t launch_far_tc(const BatchArgs& b, const void* dft, cudaStream_t s) {
   a.meas = b.meas; a.psi_s = b.psi_s; a.dft = (const uint16_t*)dft;
   a.ipred = b.ipred; a.loss = b.loss; a.status = b.status;
   // exit-wave tiles: 16 complex columns x N rows of image slot * M + k;
-  // measured-intensity tiles: 32 columns x N rows of position j
+  // measured-intensity tiles: 16 columns x N rows of position j
   TmaDesc tpsi, tmeas;
   memset(&tmeas, 0, sizeof(tmeas));
-  if (!encode_tiles(&tpsi, b.psi_s, 2 * N, N, (uint64_t)b.nb * b.M, 32, N)) return cudaErrorInvalidValue;
-  if (b.mode != MODE_FWD && !encode_tiles(&tmeas, b.meas, N, N, (uint64_t)b.J, 32, N)) return cudaErrorInvalidValue;
+  if (!encode_tiles(&tpsi, b.psi_s, 2 * N, N, (uint64_t)b.nb * b.M, 32, N, CU_TENSOR_MAP_SWIZZLE_128B))
+    return cudaErrorInvalidValue;
+  if (b.mode != MODE_FWD && !encode_tiles(&tmeas, b.meas, N, N, (uint64_t)b.J, 16, N, CU_TENSOR_MAP_SWIZZLE_64B))
+    return cudaErrorInvalidValue;
   return launch_pdl(k_far_tc<N>, dim3(grid), dim3(C::T), C::bytes, s, a, tpsi, tmeas);
 }
 
