@@ -233,10 +233,11 @@ __global__ void __launch_bounds__(32 * GRAM_SLOTS, 2) k_opr_gram(int N, int M, i
 // Gradient form (gw set): dL/dw_j += b. Otherwise the damped normal equations
 // (A + lam tr(A)/K I) dw = b are solved in FP64 (Cholesky; no update if the
 // system is not positive definite) and w_j += step dw.
-// Bound by the serial chain of FP64 square roots and divisions, which a thread
-// per slot also paid for every element of the factor (256 slots, K = 8: 38 -> 20 us).
-// Thread r holds row r, takes its column's quotient beside the others', and the
-// factor's transpose is read back from shared memory.
+// Bound by the serial chain of FP64 functions: one reciprocal square root per
+// column, where a thread per slot took a square root per column and a division
+// per element (256 slots, K = 8: 38 -> 9 us). Thread r holds row r and takes its
+// column's product beside the others'; the factor's transpose is read back from
+// shared memory.
 constexpr int SOLVE_T = 32;
 template <int KM>
 __global__ void __launch_bounds__(SOLVE_T) k_opr_solve(int nb, int K, int b0, const int* __restrict__ order,
@@ -255,19 +256,22 @@ __global__ void __launch_bounds__(SOLVE_T) k_opr_solve(int nb, int K, int b0, co
     return;
   }
   double tr = 0.0, L[KM];
-  for (int m = 0; m < K; ++m) tr += v[m * KM - m * (m - 1) / 2];   // A_mm
+#pragma unroll
+  for (int m = 0; m < KM; ++m) tr += m < K ? v[m * KM - m * (m - 1) / 2] : 0.0;   // A_mm
   const double dmp = lam * tr / (double)K;
 #pragma unroll
   for (int c = 0; c < KM; ++c)
     L[c] = c > r || r >= K ? 0.0 : v[c * KM - c * (c - 1) / 2 + (r - c)] + (r == c ? dmp : 0.0);   // A_cr, c <= r
   bool ok = live;
+  double inv = 0.0;   // 1 / L_rr
 #pragma unroll
   for (int c = 0; c < KM; ++c) {
     if (c < K) {
       const double piv = __shfl_sync(0xffffffffu, L[c], c, KM);
       ok = ok && piv > 0.0;
-      const double d = sqrt(piv);
-      L[c] = r == c ? d : L[c] / d;
+      const double y = rsqrt(piv);   // (one function per column; the rest of the solve multiplies)
+      L[c] *= y;
+      if (r == c) inv = y;
 #pragma unroll
       for (int n = c + 1; n < KM; ++n) {
         const double ln = __shfl_sync(0xffffffffu, L[c], n, KM);
@@ -278,16 +282,15 @@ __global__ void __launch_bounds__(SOLVE_T) k_opr_solve(int nb, int K, int b0, co
 #pragma unroll
   for (int c = 0; c < KM; ++c) Ls[threadIdx.x][c] = L[c];
   __syncwarp();
-  const double diag = Ls[threadIdx.x][r];
   const int row0 = threadIdx.x - r;
   double x = r < K ? v[NA + r] : 0.0;
   for (int k = 0; k < K; ++k) {   // L y = b
-    const double y = __shfl_sync(0xffffffffu, x / diag, k, KM);
+    const double y = __shfl_sync(0xffffffffu, x * inv, k, KM);
     if (r == k) x = y;
     if (r > k) x -= Ls[threadIdx.x][k] * y;
   }
   for (int k = K - 1; k >= 0; --k) {   // L^T x = y
-    const double y = __shfl_sync(0xffffffffu, x / diag, k, KM);
+    const double y = __shfl_sync(0xffffffffu, x * inv, k, KM);
     if (r == k) x = y;
     if (r < k) x -= Ls[row0 + k][r] * y;
   }
