@@ -1,8 +1,9 @@
 // Per-scan-position kernels of the LSQML hot path (templated on the window N).
 //
-// k_pass1: one CTA per position of a minibatch (window 16, and the parts
-//   around the tensor-core far field; kernels_pair.cuh holds the whole pass of
-//   the windows 32 to 128). For every incoherent probe mode k it extracts the sub-pixel object patch o_j = S_j(O) (bilinear),
+// k_pass1: one CTA per position of a minibatch at window 16 (kernels_pair.cuh
+//   holds the windows from 32 on; its line pairs leave 16 too few threads:
+//   measured equal or slower, with a relaxed probe 12 -> 16 us per 256
+//   positions). For every incoherent probe mode k it extracts the sub-pixel object patch o_j = S_j(O) (bilinear),
 //   forms the exit wave psi_jk = P_k o_j (Pty-Chi Sec. 2.1, the psi = p o of
 //   Eq. 2), propagates it with the unitary 2-D FFT and accumulates the
 //   incoherent intensity I_j = sum_k |Psi_jk|^2 (Eq. 4's forward model). It
@@ -23,14 +24,10 @@
 namespace ptycho {
 namespace cg = cooperative_groups;
 
-// CTA sizes of k_pass1 (the full count of line slots N*R1 at windows 16, 32
-// and 128): the default, and at window 16 the alternative the autotuner may
-// pick (half of it, two lines per thread).
+// CTA sizes of k_pass1 (a thread per line slot N*R1): the default, and the
+// alternative the autotuner may pick (half of it, two lines per thread).
 template <int N> struct Threads;
 template <> struct Threads<16> { static constexpr int T = 64, ALT = 32; };
-template <> struct Threads<32> { static constexpr int T = 128; };
-template <> struct Threads<64> { static constexpr int T = 256; };
-template <> struct Threads<128> { static constexpr int T = 1024; };
 
 template <int N>
 struct Pass1Smem {
@@ -230,13 +227,7 @@ __device__ __forceinline__ void overlap_add(const BatchArgs& a, int slot, int j,
 
 // OPR: the primary probe mode is synthesised per position (a separate
 // instantiation, so that the shared-probe kernel carries none of it).
-// PART 0 is the whole pass. With the far field evaluated elsewhere (the
-// tensor-core DFT-GEMM stage, k_far_tc) it runs in two parts around it:
-// PART 1 writes the exit waves psi_jk to the far-field scratch (and the
-// patches, the relaxed primary mode and the slot flags) and stops; PART 2
-// reads chi_jk from the scratch and does the rest (g, h, the overlap-add, the
-// position sums).
-template <int N, int T, bool OPR, int PART>
+template <int N, int T, bool OPR>
 __global__ void __launch_bounds__(T, 1) k_pass1(BatchArgs a) {
   using F = Fft2<N>;
   using SM = Pass1Smem<N>;
@@ -266,9 +257,9 @@ __global__ void __launch_bounds__(T, 1) k_pass1(BatchArgs a) {
   if (tid == 0 && a.valid) a.valid[slot] = 1;
   // the measured intensities are first read by the data term, after the forward
   // transforms: fetch them into L2 meanwhile (they may live in host memory)
-  if (PART == 0 && tid == 0 && a.meas && a.mode != MODE_FWD)
+  if (tid == 0 && a.meas && a.mode != MODE_FWD)
     prefetch_l2_bulk(a.meas + (size_t)j * N * N, (uint32_t)(N * N * sizeof(float)));
-  if (PART == 0) make_twiddles<N>(tw);
+  make_twiddles<N>(tw);
 
   const int M = a.M;
   const float invN = 1.0f / (float)N;
@@ -284,7 +275,7 @@ __global__ void __launch_bounds__(T, 1) k_pass1(BatchArgs a) {
 
   // ---- forward model: I_j = sum_k |F(P_k o_j)|^2 -------------------------------
 #pragma unroll 1
-  for (int k = 0; k < (PART == 2 ? 0 : M); ++k) {
+  for (int k = 0; k < M; ++k) {
     const float2* Pk = shared_mode<OPR>(a, k, NN);
     // psi_k = P_k o_j into the tile, two adjacent pixels per thread and iteration
     const NatPairs<N, T> np;
@@ -308,17 +299,13 @@ __global__ void __launch_bounds__(T, 1) k_pass1(BatchArgs a) {
         if (p0) *(float4*)(p0 + p) = P2;
       }
       const float2 x0 = cmul(make_float2(P2.x, P2.y), o0), x1 = cmul(make_float2(P2.z, P2.w), o1);
-      if constexpr (PART == 1)
-        *(float4*)(psi_s + (size_t)k * NN + p) = make_float4(x0.x, x0.y, x1.x, x1.y);
-      else
-        store_pair(tile, np.phys(q), x0, x1);
+      store_pair(tile, np.phys(q), x0, x1);
     }
-    if constexpr (PART == 1) continue;
     __syncthreads();
     // the last mode's far field stays in the tile (each row in its own line's
     // storage, free once the row transform is done): the first inverse
     // transform reads it there instead of from the scratch
-    const bool keep = (PART == 0) && k == M - 1 && a.mode != MODE_FWD && !a.loss_only;
+    const bool keep = k == M - 1 && a.mode != MODE_FWD && !a.loss_only;
     fft2_forward<N, T>(tile, tw, [&](int row, float2 (&v)[R2]) {
 #pragma unroll
       for (int m = 0; m < R2; ++m) v[m] = cscale(v[m], invN);
@@ -355,75 +342,72 @@ __global__ void __launch_bounds__(T, 1) k_pass1(BatchArgs a) {
     __syncthreads();
   }
 
-  if constexpr (PART == 1) return;
   const int mode = a.mode;
   // ---- data term: loss and the far-field factor (same thread owns each pixel) ----
-  if constexpr (PART == 0) {
-    const float eps = a.eps;
-    const float* meas = a.meas + (size_t)j * NN;
-    float lsum = 0.f;
-    bool bad = false;
-    {
-      constexpr int L = T / R1, ITER = N / L;
-      const int gid = F::line_slot();
+  const float eps = a.eps;
+  const float* meas = a.meas + (size_t)j * NN;
+  float lsum = 0.f;
+  bool bad = false;
+  {
+    constexpr int L = T / R1, ITER = N / L;
+    const int gid = F::line_slot();
 #pragma unroll 1
-      for (int it = 0; it < ITER; ++it) {
-        const int row = gid + it * L;
-        // the row's measured intensities, all loads issued before any use
-        // (registers 2q, 2q+1 are adjacent columns when S = 2: 8-byte loads)
-        float Imv[R2];
-        if (mode != MODE_FWD) {
-          if constexpr (F::S == 2) {
+    for (int it = 0; it < ITER; ++it) {
+      const int row = gid + it * L;
+      // the row's measured intensities, all loads issued before any use
+      // (registers 2q, 2q+1 are adjacent columns when S = 2: 8-byte loads)
+      float Imv[R2];
+      if (mode != MODE_FWD) {
+        if constexpr (F::S == 2) {
 #pragma unroll
-            for (int q = 0; q < R2 / 2; ++q) {
-              const float2 t = __ldg((const float2*)(meas + row * N + F::out_index(n, 2 * q)));
-              Imv[2 * q] = t.x;
-              Imv[2 * q + 1] = t.y;
-            }
-          } else {
-#pragma unroll
-            for (int m = 0; m < R2; ++m) Imv[m] = __ldg(meas + row * N + F::out_index(n, m));
+          for (int q = 0; q < R2 / 2; ++q) {
+            const float2 t = __ldg((const float2*)(meas + row * N + F::out_index(n, 2 * q)));
+            Imv[2 * q] = t.x;
+            Imv[2 * q + 1] = t.y;
           }
-        }
+        } else {
 #pragma unroll
-        for (int m = 0; m < R2; ++m) {
-          const int col = F::out_index(n, m);
-          const int pix = row * N + col;
-          const float I = rI[row * RP + col];
-          if (a.ipred) a.ipred[(size_t)j * NN + pix] = I;
-          if (mode == MODE_FWD) continue;
-          const float Im = Imv[m];
-          float fac;
-          if (mode == MODE_VJP) {
-            bad |= !isfinite(Im);
-            fac = 2.f * Im;
-          } else {
-            bad |= !(Im >= 0.f) || !isfinite(Im);
-            const float Ie = I + eps;
-            if (mode == MODE_LSQML_GAUSS || mode == MODE_GRAD_GAUSS) {
-              const float sIe = sqrtf(Ie), sIm = sqrtf(Im);
-              const float d = sIe - sIm;
-              lsum = fmaf(d, d, lsum);
-              const float rho = sIm / sIe;
-              fac = (mode == MODE_LSQML_GAUSS) ? rho - 1.f : 2.f * (1.f - rho);
-            } else {
-              lsum += I - Im * logf(Ie);
-              const float q = Im / Ie;
-              fac = (mode == MODE_LSQML_POISSON) ? 0.5f * (q - 1.f) : 2.f * (1.f - q);
-            }
-          }
-          rI[row * RP + col] = fac * invN;
+          for (int m = 0; m < R2; ++m) Imv[m] = __ldg(meas + row * N + F::out_index(n, m));
         }
       }
+#pragma unroll
+      for (int m = 0; m < R2; ++m) {
+        const int col = F::out_index(n, m);
+        const int pix = row * N + col;
+        const float I = rI[row * RP + col];
+        if (a.ipred) a.ipred[(size_t)j * NN + pix] = I;
+        if (mode == MODE_FWD) continue;
+        const float Im = Imv[m];
+        float fac;
+        if (mode == MODE_VJP) {
+          bad |= !isfinite(Im);
+          fac = 2.f * Im;
+        } else {
+          bad |= !(Im >= 0.f) || !isfinite(Im);
+          const float Ie = I + eps;
+          if (mode == MODE_LSQML_GAUSS || mode == MODE_GRAD_GAUSS) {
+            const float sIe = sqrtf(Ie), sIm = sqrtf(Im);
+            const float d = sIe - sIm;
+            lsum = fmaf(d, d, lsum);
+            const float rho = sIm / sIe;
+            fac = (mode == MODE_LSQML_GAUSS) ? rho - 1.f : 2.f * (1.f - rho);
+          } else {
+            lsum += I - Im * logf(Ie);
+            const float q = Im / Ie;
+            fac = (mode == MODE_LSQML_POISSON) ? 0.5f * (q - 1.f) : 2.f * (1.f - q);
+          }
+        }
+        rI[row * RP + col] = fac * invN;
+      }
     }
-    if (bad) atomicOr(a.status, FLAG_NONFINITE);
-    if (a.loss && mode != MODE_FWD && mode != MODE_VJP) {
-      double v[1] = {(double)lsum};
-      block_sum<1>(v, red);
-      if (tid == 0) atomicAdd(a.loss, v[0]);
-    }
-    if (mode == MODE_FWD || a.loss_only) return;
   }
+  if (bad) atomicOr(a.status, FLAG_NONFINITE);
+  if (a.loss && mode != MODE_FWD && mode != MODE_VJP) {
+    double v[1] = {(double)lsum};
+    block_sum<1>(v, red);
+    if (tid == 0) atomicAdd(a.loss, v[0]);
+  }
+  if (mode == MODE_FWD || a.loss_only) return;
 
   // ---- back-propagation: chi_k = F^-1[fac Psi_k], g = sum_k conj(P_k) chi_k, h_k ----
   // The modes run last to first: the far fields written last are read first,
@@ -433,54 +417,46 @@ __global__ void __launch_bounds__(T, 1) k_pass1(BatchArgs a) {
 #pragma unroll 1
   for (int k = M - 1; k >= 0; --k) {
     const float2* Pk = shared_mode<OPR>(a, k, NN);
-    if constexpr (PART == 0) {
-      __syncthreads();
-      fft2_inverse<N, T>(
-          tile, tw,
-          [&](int row, float2 (&v)[R2]) {
-            if (k == M - 1) {   // the last mode's far field was kept in the tile
-              F::template load_out<true>(v, tile, row, n);
-              __syncwarp();     // every lane of the line has read before the exchange writes
-            } else if constexpr (F::S == 2) {
+    __syncthreads();
+    fft2_inverse<N, T>(
+        tile, tw,
+        [&](int row, float2 (&v)[R2]) {
+          if (k == M - 1) {   // the last mode's far field was kept in the tile
+            F::template load_out<true>(v, tile, row, n);
+            __syncwarp();     // every lane of the line has read before the exchange writes
+          } else if constexpr (F::S == 2) {
 #pragma unroll
-              for (int q = 0; q < R2 / 2; ++q) {
-                const float4 X = *(const float4*)(psi_s + (size_t)k * NN + row * N + F::out_index(n, 2 * q));
-                v[2 * q] = make_float2(X.x, X.y);
-                v[2 * q + 1] = make_float2(X.z, X.w);
-              }
-            } else {
-#pragma unroll
-              for (int m = 0; m < R2; ++m) v[m] = psi_s[(size_t)k * NN + row * N + F::out_index(n, m)];
+            for (int q = 0; q < R2 / 2; ++q) {
+              const float4 X = *(const float4*)(psi_s + (size_t)k * NN + row * N + F::out_index(n, 2 * q));
+              v[2 * q] = make_float2(X.x, X.y);
+              v[2 * q + 1] = make_float2(X.z, X.w);
             }
-            if constexpr (F::S == 2) {
+          } else {
 #pragma unroll
-              for (int q = 0; q < R2 / 2; ++q) {
-                const float2 f = *(const float2*)(rI + row * RP + F::out_index(n, 2 * q));
-                v[2 * q] = cscale(v[2 * q], f.x);
-                v[2 * q + 1] = cscale(v[2 * q + 1], f.y);
-              }
-            } else {
+            for (int m = 0; m < R2; ++m) v[m] = psi_s[(size_t)k * NN + row * N + F::out_index(n, m)];
+          }
+          if constexpr (F::S == 2) {
 #pragma unroll
-              for (int m = 0; m < R2; ++m) v[m] = cscale(v[m], rI[row * RP + F::out_index(n, m)]);
+            for (int q = 0; q < R2 / 2; ++q) {
+              const float2 f = *(const float2*)(rI + row * RP + F::out_index(n, 2 * q));
+              v[2 * q] = cscale(v[2 * q], f.x);
+              v[2 * q + 1] = cscale(v[2 * q + 1], f.y);
             }
-          },
-          [&](int col, float2 (&v)[R2]) { F::template store_in<false>(v, tile, col, n); });
-      __syncthreads();
-    }
-    // chi_k (natural layout) is in the tile, or in PART 2 in the scratch:
+          } else {
+#pragma unroll
+            for (int m = 0; m < R2; ++m) v[m] = cscale(v[m], rI[row * RP + F::out_index(n, m)]);
+          }
+        },
+        [&](int col, float2 (&v)[R2]) { F::template store_in<false>(v, tile, col, n); });
+    __syncthreads();
+    // chi_k (natural layout) is in the tile:
     // g += conj(P_k) chi_k, h_k = conj(o) chi_k
     const NatPairs<N, T> np;
 #pragma unroll 2
     for (int q = 0; q < NatPairs<N, T>::STEPS; ++q) {
       const int p = np.pix(q);
       float2 x0, x1;
-      if constexpr (PART == 2) {
-        const float4 c = *(const float4*)(psi_s + (size_t)k * NN + p);
-        x0 = make_float2(c.x, c.y);
-        x1 = make_float2(c.z, c.w);
-      } else {
-        load_pair(tile, np.phys(q), x0, x1);
-      }
+      load_pair(tile, np.phys(q), x0, x1);
       const float4 P2 = (!OPR || Pk) ? __ldg((const float4*)(Pk + p)) : *(const float4*)(p0 + p);
       const float4 o2 = *(const float4*)(o_s + p);
       const float2 g0 = cmulc(make_float2(P2.x, P2.y), x0), g1 = cmulc(make_float2(P2.z, P2.w), x1);
@@ -532,14 +508,14 @@ cudaError_t smem_optin(K kernel, size_t bytes, unsigned long long* done_mask) {
   return e;
 }
 
-template <int N, int T, bool OPR, int PART = 0>
+template <int N, int T, bool OPR>
 cudaError_t launch_pass1_t(const BatchArgs& a, cudaStream_t s) {
   constexpr size_t sm = Pass1Smem<N>::bytes;
   static unsigned long long done = 0;
-  cudaError_t e = smem_optin(k_pass1<N, T, OPR, PART>, sm, &done);
+  cudaError_t e = smem_optin(k_pass1<N, T, OPR>, sm, &done);
   if (e != cudaSuccess) return e;
   if (a.nb <= 0) return cudaSuccess;
-  return launch_pdl(k_pass1<N, T, OPR, PART>, dim3(a.nb), dim3(T), sm, s, a);
+  return launch_pdl(k_pass1<N, T, OPR>, dim3(a.nb), dim3(T), sm, s, a);
 }
 
 // variant 0: default CTA size, 1: the alternative (the relaxed-probe form has

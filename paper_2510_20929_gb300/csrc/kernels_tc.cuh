@@ -16,9 +16,7 @@
 // products on separate re/im planes, the sign of the Fi terms chosen by the
 // instruction descriptor's negate-A bit.
 //
-// k_exit_tma (below) writes the exit waves psi_jk of a minibatch to the
-// scratch from object tiles staged by tensor copies (objects of odd width go
-// through the first part of the per-position pass instead).
+// k_exit (below) writes the exit waves psi_jk of a minibatch to the scratch.
 //
 // k_far_tc: per minibatch position (persistent CTAs): the exit waves psi_jk
 // are transformed mode by mode; the far fields overwrite them in the scratch and their intensities
@@ -111,94 +109,104 @@ struct FarArgs {
   int* status;
 };
 
-// Exit waves of the split-BF16 form: per position the object tile (rows
-// ty..ty+N, columns xs..xs+N+1 with xs = tx rounded down to an even column,
-// so that the copy starts on a 16-byte boundary) lands in shared memory with
-// one tiled tensor copy; the bilinear patch o_j = S_j(O) (Sec. 2.1, the same
-// weights and expression as the per-position pass) is interpolated from it,
-// and o_j and psi_jk = P_k o_j of every mode go to the scratch.
+// Exit waves of the split-BF16 form, one CTA per 32 rows of a position: the
+// bilinear patch o_j = S_j(O) (Sec. 2.1) and psi_jk = P_k o_j of every mode go to
+// the scratch, a pixel pair per thread. Bound by the stores (M + 1 planes of a
+// position, 29 us at window 128, 5 modes, 256 positions: 42 us; with one CTA per
+// position and its object tile staged by a tensor copy 56 us).
+constexpr int BAND_T = 256;
 template <int N>
-struct ExitTma {
-  static constexpr int T = 512;
-  static constexpr int TW = N + 2, TH = N + 1;   // staged tile: TH rows of TW complex values
-  static constexpr uint32_t TILE_BYTES = (uint32_t)TW * TH * 8;
-  static constexpr size_t tile = 0;
-  static constexpr size_t bar = ((size_t)TILE_BYTES + 127) / 128 * 128;
-  static constexpr size_t wsh = bar + 16;        // eigenmode weights of the position (OPR)
-  static constexpr size_t bytes = wsh + 4 * 8 + 128;   // + alignment of the base to 128 bytes
-  static_assert(TW <= 256 && TH <= 256, "tensor-copy box dimensions");
-  static_assert((TW * 8) % 16 == 0, "tensor-copy box rows are multiples of 16 bytes");
-  static_assert(bytes <= 232448, "shared memory per CTA");
+struct DftBands {
+  static constexpr int ROWS = 32, NUM = N / ROWS, PAIRS = ROWS * N / 2, PP = PAIRS / BAND_T;
+  static constexpr size_t bytes = (size_t)ROWS * N * 12;   // g and the probe intensity of a band
+  static_assert(PP * BAND_T == PAIRS, "whole pairs per thread");
 };
-
-template <int N, bool OPR>
-__global__ void __launch_bounds__(512, 1) k_exit_tma(BatchArgs a, const __grid_constant__ TmaDesc tm_obj) {
-  using C = ExitTma<N>;
-  constexpr int NN = N * N, T = C::T;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
+template <int N>
+__global__ void __launch_bounds__(BAND_T, 4) k_exit(BatchArgs a) {
+  using C = DftBands<N>;
+  constexpr int NN = N * N;
   wait_prior_grid();
-  unsigned char* smem = smem_raw + ((128u - (tc::smem_u32(smem_raw) & 127u)) & 127u);
-  const float2* tile = (const float2*)(smem + C::tile);
-  uint64_t* bar = (uint64_t*)(smem + C::bar);
-  float* wj = (float*)(smem + C::wsh);
-  const int slot = blockIdx.x, tid = threadIdx.x;
-  const int e = a.b0 + slot;
-  const int j = a.order ? a.order[e] : e;
+  const int slot = blockIdx.x / C::NUM, p0 = (blockIdx.x % C::NUM) * C::PAIRS * 2, tid = threadIdx.x;
+  const int e = a.b0 + slot, j = a.order ? a.order[e] : e;
   int ty = 0, tx = 0;
   float fy = 0.f, fx = 0.f;
-  bool ok = (j >= 0 && j < a.J);
-  if (ok) ok = tile_of(a.pos[2 * j], a.pos[2 * j + 1], N, a.H, a.W, ty, tx, fy, fx);
-  if (!ok) {
-    if (tid == 0) {
-      atomicOr(a.status, FLAG_BOUNDS);
-      if (a.valid) a.valid[slot] = 0;
-    }
-    return;
+  const bool ok = j >= 0 && j < a.J && tile_of(a.pos[2 * j], a.pos[2 * j + 1], N, a.H, a.W, ty, tx, fy, fx);
+  if (tid == 0 && p0 == 0) {
+    if (!ok) atomicOr(a.status, FLAG_BOUNDS);
+    if (a.valid) a.valid[slot] = ok;
   }
-  const int xs = tx & ~1, d = tx - xs;
-  if (tid == 0) {
-    if (a.valid) a.valid[slot] = 1;
-    tc::mbar_init(bar, 1);
-    tc::fence_mbar_init();
-    tc::mbar_expect_tx(bar, C::TILE_BYTES);
-    tc::tma_load_2d(smem + C::tile, &tm_obj, xs, ty, bar);
-  }
-  if (OPR && tid < a.K) wj[tid] = a.opr_w[(size_t)j * a.K + tid];
-  __syncthreads();
-  if (!__syncthreads_and(tc::mbar_wait(bar, 0))) {
-    if (tid == 0) atomicOr(a.status, FLAG_TIMEOUT);
-    return;
-  }
-  const int M = a.M;
-  const size_t slotNN = (size_t)slot * NN;
-  float2* o_s = a.o_s ? a.o_s + slotNN : nullptr;
-  float2* psi = a.psi_s + slotNN * M;
-  float2* p0 = (OPR && a.p0_s) ? a.p0_s + slotNN : nullptr;
-  const float w00 = (1.f - fy) * (1.f - fx), w01 = (1.f - fy) * fx, w10 = fy * (1.f - fx), w11 = fy * fx;
+  if (!ok) return;
+  float2* psi = a.psi_s + (size_t)slot * a.M * NN;
 #pragma unroll 2
-  for (int q = tid; q < NN / 2; q += T) {   // pixel pairs (r, c), (r, c + 1)
-    const int p = 2 * q, r = p / N, c = p % N;
-    const float2* t0 = tile + r * C::TW + c + d;
-    const float2* t1 = t0 + C::TW;
-    const float2 a0 = t0[0], a1 = t0[1], a2 = t0[2], b0 = t1[0], b1 = t1[1], b2 = t1[2];
-    const float2 o0 = make_float2(w00 * a0.x + w01 * a1.x + w10 * b0.x + w11 * b1.x,
-                                  w00 * a0.y + w01 * a1.y + w10 * b0.y + w11 * b1.y);
-    const float2 o1 = make_float2(w00 * a1.x + w01 * a2.x + w10 * b1.x + w11 * b2.x,
-                                  w00 * a1.y + w01 * a2.y + w10 * b1.y + w11 * b2.y);
-    if (o_s) *(float4*)(o_s + p) = make_float4(o0.x, o0.y, o1.x, o1.y);
-    for (int k = 0; k < M; ++k) {
-      const float2* Pk = shared_mode<OPR>(a, k, NN);
-      float4 P2;
-      if (!OPR || Pk) {
-        P2 = __ldg((const float4*)(Pk + p));
-      } else {   // relaxed primary mode of this position
-        P2 = opr_pair(a.opr_U, wj, a.K, NN, p);
-        if (p0) *(float4*)(p0 + p) = P2;
-      }
+  for (int i = 0; i < C::PP; ++i) {
+    const int p = p0 + 2 * (i * BAND_T + tid);
+    float2 o0, o1;
+    bilinear2(a.obj, a.W, ty + p / N, tx + p % N, fy, fx, o0, o1);
+    if (a.o_s) *(float4*)(a.o_s + (size_t)slot * NN + p) = make_float4(o0.x, o0.y, o1.x, o1.y);
+    for (int k = 0; k < a.M; ++k) {
+      const float4 P2 = __ldg((const float4*)(a.probe + (size_t)k * NN + p));
       const float2 x0 = cmul(make_float2(P2.x, P2.y), o0), x1 = cmul(make_float2(P2.z, P2.w), o1);
       *(float4*)(psi + (size_t)k * NN + p) = make_float4(x0.x, x0.y, x1.x, x1.y);
     }
   }
+}
+
+// The pass after the far field, one CTA per 32 rows of a position: g += conj(P_k)
+// chi_k (in registers over the modes, last mode first as the FP32 pass) and
+// h_k = conj(o) chi_k, then the overlap-add and the position sums of the band.
+// Bound by DRAM (2 M + 3 planes of a position, about 59 us at window 128, 5
+// modes, 256 positions): 95 us there; one CTA of 1024 threads per position, g in
+// global memory between the modes, took 155 us.
+template <int N>
+__global__ void __launch_bounds__(BAND_T, 3) k_overlap(BatchArgs a) {
+  using C = DftBands<N>;
+  constexpr int NN = N * N, U = C::PP < 4 ? C::PP : 4;   // pairs in flight
+  extern __shared__ __align__(16) float2 gS[];           // the band of g, then of the probe intensity
+  __shared__ double red[32 * 5];
+  wait_prior_grid();
+  const int slot = blockIdx.x / C::NUM, y0 = (blockIdx.x % C::NUM) * C::ROWS, tid = threadIdx.x;
+  const int e = a.b0 + slot, j = a.order ? a.order[e] : e;
+  int ty = 0, tx = 0;
+  float fy = 0.f, fx = 0.f;
+  if (!(j >= 0 && j < a.J) || !tile_of(a.pos[2 * j], a.pos[2 * j + 1], N, a.H, a.W, ty, tx, fy, fx)) return;   // (flagged)
+  const size_t base = (size_t)slot * NN;
+  const int M = a.M;
+#pragma unroll 1
+  for (int i0 = 0; i0 < C::PP; i0 += U) {
+    const int l = 2 * (i0 * BAND_T + tid), p = y0 * N + l;   // in the band, in the patch
+    float4 o[U], g[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      o[u] = *(const float4*)(a.o_s + base + p + 2 * u * BAND_T);
+      g[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+#pragma unroll 1
+    for (int k = M - 1; k >= 0; --k) {
+      const size_t at = (base * M + (size_t)k * NN) + p;
+      float4 c[U], P[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        c[u] = __ldcs((const float4*)(a.psi_s + at + 2 * u * BAND_T));
+        P[u] = __ldg((const float4*)(a.probe + (size_t)k * NN + p + 2 * u * BAND_T));
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const float2 x0 = make_float2(c[u].x, c[u].y), x1 = make_float2(c[u].z, c[u].w);
+        const float2 g0 = cmulc(make_float2(P[u].x, P[u].y), x0), g1 = cmulc(make_float2(P[u].z, P[u].w), x1);
+        g[u] = k == M - 1 ? make_float4(g0.x, g0.y, g1.x, g1.y)
+                          : make_float4(g0.x + g[u].x, g0.y + g[u].y, g1.x + g[u].z, g1.y + g[u].w);
+        const float2 h0 = cmulc(make_float2(o[u].x, o[u].y), x0), h1 = cmulc(make_float2(o[u].z, o[u].w), x1);
+        __stcs((float4*)(a.h_s + at + 2 * u * BAND_T), make_float4(h0.x, h0.y, h1.x, h1.y));
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      *(float4*)(a.g_s + base + p + 2 * u * BAND_T) = g[u];
+      *(float4*)(gS + l + 2 * u * BAND_T) = g[u];
+    }
+  }
+  overlap_add<N, C::ROWS, BAND_T, false>(a, slot, j, y0, ty, tx, fy, fx, nullptr, (float*)(gS + C::ROWS * N), red,
+                                         [&](int y, int x) { return gS[y * N + x]; });
 }
 
 __device__ __forceinline__ uint16_t bf16_bits(float v) { return __bfloat16_as_ushort(__float2bfloat16_rn(v)); }
