@@ -982,6 +982,7 @@ ptycho_status ptycho_adjoint_ex(const ptycho_dims* dims, int32_t precision, cons
     a.eps = (float)eps;
     a.psi_s = w.psi; a.o_s = w.o; a.g_s = w.g; a.h_s = w.h; a.valid = w.valid;
     a.gobj = (float2*)g_object; a.gpos = g_pos; a.loss = loss; a.status = &w.hdr->status;
+    if (tc && g_pos) a.gsum = w.possum;   // (that form splits a position into bands)
     a.loss_only = loss_only ? 1 : 0;
     if ((tc ? pass1_dft(dims->N, a, w.dft, s) : pass1(dims->N, a, s)) != cudaSuccess) return PTYCHO_ERR_CUDA;
     if (loss_only) continue;

@@ -218,8 +218,23 @@ __device__ __forceinline__ void overlap_add(const BatchArgs& a, int slot, int j,
       double v[2] = {(double)gy, (double)gx};
       block_sum<2>(v, red);
       if (tid == 0) {
-        atomicAdd(a.gpos + 2 * j, (float)v[0]);
-        atomicAdd(a.gpos + 2 * j + 1, (float)v[1]);
+        bool last = true;
+        if (N > LR && a.gsum) {   // the CTAs' shares meet in FP64; the last to arrive rounds the sums, once
+          double* sum = a.gsum + (size_t)slot * 5;
+          atomicAdd(sum, v[0]);
+          atomicAdd(sum + 1, v[1]);
+          __threadfence();
+          last = atomicAdd((int*)(sum + 2), 1) == N / LR - 1;
+          __threadfence();
+          if (last) {
+            v[0] = __ldcg(sum);
+            v[1] = __ldcg(sum + 1);
+          }
+        }
+        if (last) {
+          atomicAdd(a.gpos + 2 * j, (float)v[0]);
+          atomicAdd(a.gpos + 2 * j + 1, (float)v[1]);
+        }
       }
     }
   }

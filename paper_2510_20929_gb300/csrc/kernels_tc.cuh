@@ -134,6 +134,8 @@ __global__ void __launch_bounds__(BAND_T, 4) k_exit(BatchArgs a) {
   if (tid == 0 && p0 == 0) {
     if (!ok) atomicOr(a.status, FLAG_BOUNDS);
     if (a.valid) a.valid[slot] = ok;
+    if (a.gsum)
+      for (int q = 0; q < 3; ++q) a.gsum[(size_t)slot * 5 + q] = 0.0;
   }
   if (!ok) return;
   float2* psi = a.psi_s + (size_t)slot * a.M * NN;
@@ -153,7 +155,8 @@ __global__ void __launch_bounds__(BAND_T, 4) k_exit(BatchArgs a) {
 
 // The pass after the far field, one CTA per 32 rows of a position: g += conj(P_k)
 // chi_k (in registers over the modes, last mode first as the FP32 pass) and
-// h_k = conj(o) chi_k, then the overlap-add and the position sums of the band.
+// h_k = conj(o) chi_k, then the overlap-add and the position sums of the band
+// (a position's gradient is summed over its bands in FP64 and rounded once).
 // Bound by DRAM (2 M + 3 planes of a position, about 59 us at window 128, 5
 // modes, 256 positions): 95 us there; one CTA of 1024 threads per position, g in
 // global memory between the modes, took 155 us.
