@@ -75,10 +75,7 @@ struct BatchArgs {
   // Position correction (LSQML): per slot the sums A11, A12, A22, b1, b2 of
   // the least-squares shift, FP64, accumulated with atomics (or null).
   double* possum;      // [B, 5]
-  // Position gradient of a form that splits a position over several CTAs: per
-  // slot the two FP64 sums and the count of CTAs that added theirs, zero before
-  // the overlap-add (null: each CTA adds its own share to gpos).
-  double* gsum;        // [B, 5]
+  double* gsum;        // [B, 2] FP64 sums of the position gradient (split-BF16 form, with gpos)
   // Gradient modes: evaluate the forward model and the data term (loss) only,
   // without the back-propagation.
   int loss_only;

@@ -141,8 +141,9 @@ __device__ __forceinline__ void bilinear_scatter(float fy, float fx, Load&& load
 // probe intensity are scattered into the object frame, then the position
 // gradient or the sums of the position step are reduced. The CTA holds rows
 // y0 .. y0 + LR - 1 of the patch (getg's y counts from y0). `spS` is LR * N
-// floats of shared memory that are free on entry.
-template <int N, int LR, int T, bool OPR, class Get>
+// floats of shared memory that are free on entry. FP64_SUMS: the position
+// gradient goes to a.gsum.
+template <int N, int LR, int T, bool OPR, bool FP64_SUMS = false, class Get>
 __device__ __forceinline__ void overlap_add(const BatchArgs& a, int slot, int j, int y0, int ty, int tx, float fy,
                                             float fx, const float2* p0, float* spS, double* red, Get&& getg) {
   constexpr int LNN = LR * N;
@@ -218,20 +219,10 @@ __device__ __forceinline__ void overlap_add(const BatchArgs& a, int slot, int j,
       double v[2] = {(double)gy, (double)gx};
       block_sum<2>(v, red);
       if (tid == 0) {
-        bool last = true;
-        if (N > LR && a.gsum) {   // the CTAs' shares meet in FP64; the last to arrive rounds the sums, once
-          double* sum = a.gsum + (size_t)slot * 5;
-          atomicAdd(sum, v[0]);
-          atomicAdd(sum + 1, v[1]);
-          __threadfence();
-          last = atomicAdd((int*)(sum + 2), 1) == N / LR - 1;
-          __threadfence();
-          if (last) {
-            v[0] = __ldcg(sum);
-            v[1] = __ldcg(sum + 1);
-          }
-        }
-        if (last) {
+        if constexpr (FP64_SUMS) {
+          atomicAdd(a.gsum + 2 * slot, v[0]);
+          atomicAdd(a.gsum + 2 * slot + 1, v[1]);
+        } else {
           atomicAdd(a.gpos + 2 * j, (float)v[0]);
           atomicAdd(a.gpos + 2 * j + 1, (float)v[1]);
         }

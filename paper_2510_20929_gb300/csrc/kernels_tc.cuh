@@ -134,8 +134,7 @@ __global__ void __launch_bounds__(BAND_T, 4) k_exit(BatchArgs a) {
   if (tid == 0 && p0 == 0) {
     if (!ok) atomicOr(a.status, FLAG_BOUNDS);
     if (a.valid) a.valid[slot] = ok;
-    if (a.gsum)
-      for (int q = 0; q < 3; ++q) a.gsum[(size_t)slot * 5 + q] = 0.0;
+    if (a.gsum) a.gsum[2 * slot] = a.gsum[2 * slot + 1] = 0.0;
   }
   if (!ok) return;
   float2* psi = a.psi_s + (size_t)slot * a.M * NN;
@@ -155,8 +154,10 @@ __global__ void __launch_bounds__(BAND_T, 4) k_exit(BatchArgs a) {
 
 // The pass after the far field, one CTA per 32 rows of a position: g += conj(P_k)
 // chi_k (in registers over the modes, last mode first as the FP32 pass) and
-// h_k = conj(o) chi_k, then the overlap-add and the position sums of the band
-// (a position's gradient is summed over its bands in FP64 and rounded once).
+// h_k = conj(o) chi_k, then the overlap-add and the position sums of the band. The
+// bands of a position add their shares of its gradient in FP64; k_gpos rounds
+// the sum, once. (With the last band to arrive doing that, behind a fence that
+// waits for the band's scatter, this kernel took 105 us instead of 95.)
 // Bound by DRAM (2 M + 3 planes of a position, about 59 us at window 128, 5
 // modes, 256 positions): 95 us there; one CTA of 1024 threads per position, g in
 // global memory between the modes, took 155 us.
@@ -208,8 +209,17 @@ __global__ void __launch_bounds__(BAND_T, 3) k_overlap(BatchArgs a) {
       *(float4*)(gS + l + 2 * u * BAND_T) = g[u];
     }
   }
-  overlap_add<N, C::ROWS, BAND_T, false>(a, slot, j, y0, ty, tx, fy, fx, nullptr, (float*)(gS + C::ROWS * N), red,
-                                         [&](int y, int x) { return gS[y * N + x]; });
+  overlap_add<N, C::ROWS, BAND_T, false, true>(a, slot, j, y0, ty, tx, fy, fx, nullptr, (float*)(gS + C::ROWS * N), red,
+                                               [&](int y, int x) { return gS[y * N + x]; });
+}
+
+// gpos += the position gradient's FP64 sums of the valid slots.
+__global__ void __launch_bounds__(BAND_T) k_gpos(BatchArgs a) {
+  wait_prior_grid();
+  const int i = blockIdx.x * BAND_T + threadIdx.x, slot = i / 2;
+  if (slot >= a.nb || !a.valid[slot]) return;
+  const int e = a.b0 + slot, j = a.order ? a.order[e] : e;
+  atomicAdd(a.gpos + 2 * j + i % 2, (float)a.gsum[i]);
 }
 
 __device__ __forceinline__ uint16_t bf16_bits(float v) { return __bfloat16_as_ushort(__float2bfloat16_rn(v)); }

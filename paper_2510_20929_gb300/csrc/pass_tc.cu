@@ -73,7 +73,8 @@ cudaError_t launch_pass1_part(const BatchArgs& a, cudaStream_t s, int part) {
   static unsigned long long done = 0;
   cudaError_t e = smem_optin(k_overlap<N>, C::bytes, &done);
   if (e != cudaSuccess) return e;
-  return launch_pdl(k_overlap<N>, grid, dim3(BAND_T), C::bytes, s, a);
+  if ((e = launch_pdl(k_overlap<N>, grid, dim3(BAND_T), C::bytes, s, a)) != cudaSuccess || !a.gpos) return e;
+  return launch_pdl(k_gpos, dim3((unsigned)((2 * a.nb + BAND_T - 1) / BAND_T)), dim3(BAND_T), 0, s, a);
 }
 
 // Persistent: as many CTAs as fit at once (one per SM at N = 128), at most one per position.
