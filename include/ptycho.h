@@ -474,6 +474,21 @@ ptycho_status ptycho_status_read(void* ws, void* stream);
  * size at least). */
 ptycho_status ptycho_selftest_wait_timeout(void* ws, size_t ws_bytes, void* stream);
 
+/* Diagnostic of the copy waits of the FP32 per-position passes: the gradients of
+ * the amplitude loss (eps = 1 count, one chunk of J positions; ms NULL for a
+ * plain object) as if the wait for every position's object tile (copy = 1) or
+ * measured pattern (copy = 2) had given up, on the windows 192 and 256 in one
+ * CTA of the position's cluster. Such positions add nothing to g_object and
+ * g_probe, and the next ptycho_status_read() returns PTYCHO_ERR_TIMEOUT (the
+ * loss is not to be used then). The passes of small windows that read object and
+ * pattern with plain loads have no such wait, and the call is an ordinary one.
+ * Workspace as for ptycho_adjoint or ptycho_adjoint_ms with batch = J; other
+ * values of `copy` and J < 1 are PTYCHO_ERR_ARG. */
+ptycho_status ptycho_selftest_copy_timeout(const ptycho_dims* dims, const ptycho_multislice* ms, int32_t copy,
+                                           const float* object, const float* probe, const float* pos,
+                                           const float* meas, float* g_object, float* g_probe, double* loss,
+                                           void* ws, size_t ws_bytes, void* stream);
+
 /* Static description of a status code. */
 const char* ptycho_status_string(ptycho_status status);
 

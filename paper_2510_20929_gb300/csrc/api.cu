@@ -948,10 +948,10 @@ ptycho_status ptycho_forward(const ptycho_dims* dims, const float* object, const
   return ptycho_forward_ex(dims, PTYCHO_PRECISION_FP32, 1, object, probe, pos, I_pred, ws, ws_bytes, stream);
 }
 
-ptycho_status ptycho_adjoint_ex(const ptycho_dims* dims, int32_t precision, const float* object, const float* probe,
-                                const float* pos, const float* meas, int32_t noise, double eps, int32_t batch,
-                                float* g_object, float* g_probe, float* g_pos, double* loss, void* ws,
-                                size_t ws_bytes, void* stream) {
+static ptycho_status adjoint(const ptycho_dims* dims, int32_t precision, const float* object, const float* probe,
+                             const float* pos, const float* meas, int32_t noise, double eps, int32_t batch,
+                             float* g_object, float* g_probe, float* g_pos, double* loss, void* ws, size_t ws_bytes,
+                             void* stream, int give_up) {
   ptycho_status st = check_dims(dims);
   if (st != PTYCHO_OK) return st;
   if ((st = check_precision(dims->N, precision, meas)) != PTYCHO_OK) return st;
@@ -984,6 +984,7 @@ ptycho_status ptycho_adjoint_ex(const ptycho_dims* dims, int32_t precision, cons
     a.gobj = (float2*)g_object; a.gpos = g_pos; a.loss = loss; a.status = &w.hdr->status;
     if (tc && g_pos) a.gsum = w.possum;   // (that form splits a position into bands)
     a.loss_only = loss_only ? 1 : 0;
+    a.give_up = give_up;
     if ((tc ? pass1_dft(dims->N, a, w.dft, s) : pass1(dims->N, a, s)) != cudaSuccess) return PTYCHO_ERR_CUDA;
     if (loss_only) continue;
     if (probe_reduce(NN, 0, dims->M, dims->M, nb, w.h, w.o, w.valid, (float2*)g_probe, 1, nullptr, nullptr, 0,
@@ -991,6 +992,25 @@ ptycho_status ptycho_adjoint_ex(const ptycho_dims* dims, int32_t precision, cons
       return PTYCHO_ERR_CUDA;
   }
   return PTYCHO_OK;
+}
+
+ptycho_status ptycho_adjoint_ex(const ptycho_dims* dims, int32_t precision, const float* object, const float* probe,
+                                const float* pos, const float* meas, int32_t noise, double eps, int32_t batch,
+                                float* g_object, float* g_probe, float* g_pos, double* loss, void* ws,
+                                size_t ws_bytes, void* stream) {
+  return adjoint(dims, precision, object, probe, pos, meas, noise, eps, batch, g_object, g_probe, g_pos, loss, ws,
+                 ws_bytes, stream, 0);
+}
+
+ptycho_status ptycho_selftest_copy_timeout(const ptycho_dims* dims, const ptycho_multislice* ms, int32_t copy,
+                                           const float* object, const float* probe, const float* pos,
+                                           const float* meas, float* g_object, float* g_probe, double* loss, void* ws,
+                                           size_t ws_bytes, void* stream) {
+  if ((copy != 1 && copy != 2) || !dims || dims->J < 1) return PTYCHO_ERR_ARG;
+  return ms ? adjoint_ms(dims, ms, object, probe, pos, meas, PTYCHO_NOISE_GAUSSIAN, 1.0, dims->J, g_object, g_probe,
+                         nullptr, loss, ws, ws_bytes, stream, copy)
+            : adjoint(dims, PTYCHO_PRECISION_FP32, object, probe, pos, meas, PTYCHO_NOISE_GAUSSIAN, 1.0, dims->J,
+                      g_object, g_probe, nullptr, loss, ws, ws_bytes, stream, copy);
 }
 
 ptycho_status ptycho_adjoint(const ptycho_dims* dims, const float* object, const float* probe, const float* pos,

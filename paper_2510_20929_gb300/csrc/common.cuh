@@ -79,6 +79,7 @@ struct BatchArgs {
   // Gradient modes: evaluate the forward model and the data term (loss) only,
   // without the back-propagation.
   int loss_only;
+  int give_up;         // self-test: the wait for the object tile (1) or the measured pattern (2) gives up
 };
 
 struct Pass2Args {
@@ -145,6 +146,7 @@ struct MsArgs {
   float4* acc;          // [S, H, W] (dO_acc.re, dO_acc.im, illum, unused)
   float* w_s;           // [B, S - 1, N, N]
   const float* Sp;      // [N, N]
+  int give_up;          // as in BatchArgs
 };
 
 // Arguments of the multislice LSQML tangent pass (k_step_ms): per slot the

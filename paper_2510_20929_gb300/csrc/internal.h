@@ -111,6 +111,12 @@ ptycho_status run_epoch_opr(const ptycho_dims& d, const ptycho_opr_opts& r, floa
                             const ptycho_lsqml_opts& o, double* loss, double* alpha, void* ws, cudaStream_t s);
 ptycho_status check_opr_opts(const ptycho_opr_opts* r);
 
+// ptycho_adjoint_ms; `give_up`: see BatchArgs.
+ptycho_status adjoint_ms(const ptycho_dims* dims, const ptycho_multislice* ms, const float* object, const float* probe,
+                         const float* pos, const float* meas, int32_t noise, double eps, int32_t batch,
+                         float* g_object, float* g_probe, float* g_pos, double* loss, void* ws, size_t ws_bytes,
+                         void* stream, int give_up);
+
 // Byte-exact key of a captured launch sequence (dimensions, options, pointers).
 struct GraphKey {
   std::vector<unsigned char> bytes;

@@ -142,13 +142,17 @@ __device__ __forceinline__ void bilinear_scatter(float fy, float fx, Load&& load
 // gradient or the sums of the position step are reduced. The CTA holds rows
 // y0 .. y0 + LR - 1 of the patch (getg's y counts from y0). `spS` is LR * N
 // floats of shared memory that are free on entry. FP64_SUMS: the position
-// gradient goes to a.gsum.
+// gradient goes to a.gsum. On a cluster (the other callers with several CTAs per
+// position) a position marked invalid meanwhile is left out.
 template <int N, int LR, int T, bool OPR, bool FP64_SUMS = false, class Get>
 __device__ __forceinline__ void overlap_add(const BatchArgs& a, int slot, int j, int y0, int ty, int tx, float fy,
                                             float fx, const float2* p0, float* spS, double* red, Get&& getg) {
   constexpr int LNN = LR * N;
   const int tid = threadIdx.x, mode = a.mode, pb = y0 * N;
   const bool lsqml = (mode == MODE_LSQML_GAUSS || mode == MODE_LSQML_POISSON);
+  constexpr bool CLUSTER = N > LR && !FP64_SUMS;
+  int live = 1;
+  if constexpr (CLUSTER) live = *(const volatile int*)(a.valid + slot);
   // LSQML: the probe intensity sum_k |P_k|^2 of every pixel into shared memory
   // (the intensity/factor plane is free by now), so that the scatter's row walk
   // waits on shared memory rather than on L2
@@ -164,7 +168,11 @@ __device__ __forceinline__ void overlap_add(const BatchArgs& a, int slot, int j,
       *(float4*)(spS + p) = v;
     }
   }
-  __syncthreads();
+  if constexpr (CLUSTER) {
+    if (!__syncthreads_and(live)) return;
+  } else {
+    __syncthreads();
+  }
   if (lsqml) {
     bilinear_scatter<N, LR, T>(
         fy, fx,

@@ -102,17 +102,9 @@ __global__ void __launch_bounds__(G::T, PairCtas<G>::n) k_pass1_ms(MsArgs a) {
   }
   if (first && a.valid) a.valid[slot] = 1;
   ms_begin<G>(tw, bar);
-  // joins the block after a wait for copies; a wait that gave up is recorded
-  // and waited for once more (copies in flight must not outlive the CTA)
-  auto arrived = [&](bool got, uint64_t* b, uint32_t parity) {
-    if (!__syncthreads_and(got)) {
-      if (tid == 0) {
-        atomicOr(a.status, FLAG_TIMEOUT);
-        tc::mbar_wait(b, parity);
-      }
-      __syncthreads();
-    }
-    return true;
+  // joins the block after a wait for copies; false when a thread's wait gave up (see copy_arrived)
+  auto arrived = [&](bool got, uint64_t* b, uint32_t parity) -> bool {
+    return copy_arrived(geo, got, b, parity, a.status, a.valid + slot, (a.give_up >> (int)(b - bar)) & 1);
   };
 
   const int M = a.M, S = a.S, mode = a.mode;
@@ -130,13 +122,18 @@ __global__ void __launch_bounds__(G::T, PairCtas<G>::n) k_pass1_ms(MsArgs a) {
     return (float4*)(a.in_s + ms_inc_offset(a.recompute != 0, slotNN, M, S, k, s, NN) + (size_t)y0 * N) + tid;
   };
 
+  bool lost = false;   // a copy of this CTA's never arrived
   // ---- slice patches o^(s) = S_j(O^(s)) -------------------------------------------
 #pragma unroll 1
   for (int s = 0; s < S; ++s) {
     const ObjStage<G> stage(tile, bar, a.obj, a.obj + s * HW, a.H, a.W, ty + y0, tx);
     if (tid == 0) stage.expect();
     stage.copy();
-    arrived(stage.wait(s & 1), bar, s & 1);
+    if (!arrived(stage.wait(s & 1), bar, s & 1)) {
+      if (Q == 1) return;
+      lost = true;
+      break;
+    }
 #pragma unroll 4
     for (int i = 0; i < NP; ++i)
       st_pair<G>(o_s + (size_t)s * NN + pix(i), stage.patch(geo.row(i), geo.col(i), fy, fx));
@@ -187,9 +184,13 @@ __global__ void __launch_bounds__(G::T, PairCtas<G>::n) k_pass1_ms(MsArgs a) {
           __syncthreads();   // the tile is free
           continue;
         }
-        data_term<G, N == 64 || N == 128>(geo, rI, red, bar + 1, a.meas, j, a.ipred, mode, a.eps, a.loss, a.status,
-                                          [&](bool got, uint64_t* b) { return arrived(got, b, 0); });
+        if (!data_term<G, N == 64 || N == 128>(geo, rI, red, bar + 1, a.meas, j, a.ipred, mode, a.eps, a.loss,
+                                               a.status, [&](bool got, uint64_t* b) { return arrived(got, b, 0); })) {
+          if (Q == 1) return;
+          lost = true;
+        }
         if (!grad) return;
+        settle_lost<G>(a.valid + slot, lost);
         if (rec) {
           ph = REC;
           s = 0;
@@ -270,6 +271,9 @@ __global__ void __launch_bounds__(G::T, PairCtas<G>::n) k_pass1_ms(MsArgs a) {
     }
     __syncthreads();   // the tile is free
   }
+
+  if constexpr (Q > 1)
+    if (!__syncthreads_and(*(const volatile int*)(a.valid + slot))) return;   // given up by a CTA of the cluster
 
   // ---- per slice: scatter S_j^T of its gradient; position gradient over the slices ----
   const float2* gt = (const float2*)tile;

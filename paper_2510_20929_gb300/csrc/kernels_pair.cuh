@@ -70,6 +70,34 @@ struct OneCta {
   __device__ __forceinline__ static int pixel_slot(int y, int x) { return 2 * F::colu(y, x >> 1) + (x & 1); }
 };
 
+// What a CTA does about a copy whose wait gave up (`got` false in one of its
+// threads): the status records it, and after a second bounded wait (copies in
+// flight must not outlive the CTA) the position is dropped, with nothing of it
+// scattered and its slot marked invalid. A CTA of a cluster cannot leave before
+// the others, which write into its memory until the last transform, and goes on.
+// After the forward transforms, whose barriers put that after the mark of the
+// cluster's first CTA, it clears valid[slot] (settle_lost); after the inverse
+// ones, whose barriers make that visible, every CTA of the cluster reads it
+// before it scatters. The outputs of a forward model or of a loss alone are not
+// held back on a cluster.
+template <class G>
+__device__ __forceinline__ bool copy_arrived(const G& geo, bool got, uint64_t* bar, uint32_t parity, int* status,
+                                             int* valid, bool give_up) {
+  if (give_up) got = got && geo.q < G::Q - 1;   // (self-test: in one CTA)
+  if (__syncthreads_and(got)) return true;
+  if (threadIdx.x == 0) {
+    atomicOr(status, FLAG_TIMEOUT);
+    if (G::Q == 1 && valid) *valid = 0;
+    tc::mbar_wait(bar, parity);
+  }
+  __syncthreads();
+  return false;
+}
+template <class G>
+__device__ __forceinline__ void settle_lost(int* valid, bool lost) {
+  if (G::Q > 1 && threadIdx.x == 0 && lost) *(volatile int*)valid = 0;
+}
+
 // Launch shape: CTAs per SM (shared memory at the windows 128 and up; the
 // register budget, 80 and 128 a thread, at 64 and 32). On the cluster windows
 // two CTAs of different clusters share an SM: one computes while the other
@@ -615,23 +643,16 @@ __global__ void __launch_bounds__(G::T, PairCtas<G>::n) k_pass1_pair(BatchArgs a
   float4 P[NP];
   if (OPR) __syncthreads();   // the weights
   probe_fwd(shared_mode<OPR>(a, 0, NN), P);
-  // joins the block after a wait for copies; false (and everything released)
-  // when a thread's wait gave up
+  // joins the block after a wait for copies; false when a thread's wait gave up
+  // (everything is released then, but on a cluster: see copy_arrived)
   auto arrived_all = [&](bool got, uint64_t* b) -> bool {
-    if (__syncthreads_and(got)) return true;
-    if (tid == 0) {
-      atomicOr(a.status, FLAG_TIMEOUT);
-      if (Q == 1 && a.valid) a.valid[slot] = 0;
-      tc::mbar_wait(b, 0);   // copies in flight must not outlive the CTA
-    }
-    if (Q > 1) {   // its cluster writes into this CTA's memory: go on (the status tells)
-      __syncthreads();
+    if (copy_arrived(geo, got, b, 0, a.status, a.valid ? a.valid + slot : nullptr, (a.give_up >> (int)(b - bar)) & 1))
       return true;
-    }
-    tm_release();
+    if (Q == 1) tm_release();
     return false;
   };
-  if (!arrived_all(stage.wait(0), bar)) return;   // (also twiddles, plainly loaded rows)
+  bool lost = !arrived_all(stage.wait(0), bar);   // (also twiddles, plainly loaded rows)
+  if (lost && Q == 1) return;
 #pragma unroll
   for (int qg = 0; qg < NP / 4; ++qg) {   // the patch o_j and the first mode's exit wave
     float ov[16];
@@ -673,12 +694,15 @@ __global__ void __launch_bounds__(G::T, PairCtas<G>::n) k_pass1_pair(BatchArgs a
   }
 
   // ---- data term: loss and the far-field factor, on the thread's own pixels ------
-  if (!data_term<G, N == 64>(geo, rI, red, bar + 1, a.meas, j, a.ipred, mode, a.eps, a.loss, a.status, arrived_all))
-    return;
+  if (!data_term<G, N == 64>(geo, rI, red, bar + 1, a.meas, j, a.ipred, mode, a.eps, a.loss, a.status, arrived_all)) {
+    if (Q == 1) return;
+    lost = true;
+  }
   if (mode == MODE_FWD || a.loss_only) {
     tm_release();
     return;
   }
+  settle_lost<G>(a.valid + slot, lost);
 
   // ---- back-propagation: chi_k = F^-1[fac Psi_k], g = sum_k conj(P_k) chi_k, h_k ----
   // The modes run last to first: the far fields written last are read first,

@@ -339,6 +339,42 @@ MsLayout ms_setup(const ptycho_dims& d, const ptycho_multislice& ms, int batch, 
 }
 
 }  // namespace
+
+ptycho_status adjoint_ms(const ptycho_dims* dims, const ptycho_multislice* ms, const float* object, const float* probe,
+                         const float* pos, const float* meas, int32_t noise, double eps, int32_t batch,
+                         float* g_object, float* g_probe, float* g_pos, double* loss, void* ws, size_t ws_bytes,
+                         void* stream, int give_up) {
+  ptycho_status st = check_ms(dims, ms);
+  if (st != PTYCHO_OK) return st;
+  if (batch < 1 || !(eps >= 0.0)) return PTYCHO_ERR_ARG;
+  if (noise != PTYCHO_NOISE_GAUSSIAN && noise != PTYCHO_NOISE_POISSON && noise != PTYCHO_NOISE_VJP)
+    return PTYCHO_ERR_ARG;
+  if (!object || !probe || !g_object || !g_probe || (dims->J > 0 && (!pos || !meas))) return PTYCHO_ERR_ARG;
+  if ((st = check_ws(ws, ws_bytes, ms_layout(*dims, ms->S, batch, ms->recompute != 0).total)) != PTYCHO_OK)
+    return st;
+  if (dims->J == 0) return PTYCHO_OK;
+  cudaStream_t s = (cudaStream_t)stream;
+  MsArgs a;
+  cudaError_t e = cudaSuccess;
+  ms_setup(*dims, *ms, batch, ws, a, s, &e);
+  if (e != cudaSuccess) return PTYCHO_ERR_CUDA;
+  a.obj = (const float2*)object; a.probe = (const float2*)probe; a.pos = pos; a.meas = meas;
+  a.mode = noise == PTYCHO_NOISE_GAUSSIAN ? MODE_GRAD_GAUSS : noise == PTYCHO_NOISE_POISSON ? MODE_GRAD_POISSON
+                                                                                          : MODE_VJP;
+  a.eps = (float)eps;
+  a.gobj = (float2*)g_object; a.gpos = g_pos; a.loss = loss; a.give_up = give_up;
+  const int NN = dims->N * dims->N;
+  for (int b0 = 0; b0 < dims->J; b0 += batch) {
+    a.b0 = b0;
+    a.nb = (dims->J - b0 < batch) ? dims->J - b0 : batch;
+    if (pass1_ms(dims->N, a, s) != cudaSuccess) return PTYCHO_ERR_CUDA;
+    if (probe_reduce(NN, 0, dims->M, dims->M, a.nb, a.h_s, a.o_s, a.valid, (float2*)g_probe, 1, nullptr, nullptr, 0,
+                     nullptr, s) != cudaSuccess)
+      return PTYCHO_ERR_CUDA;
+  }
+  return PTYCHO_OK;
+}
+
 }  // namespace ptycho
 
 using namespace ptycho;
@@ -378,35 +414,8 @@ ptycho_status ptycho_adjoint_ms(const ptycho_dims* dims, const ptycho_multislice
                                 const float* probe, const float* pos, const float* meas, int32_t noise, double eps,
                                 int32_t batch, float* g_object, float* g_probe, float* g_pos, double* loss, void* ws,
                                 size_t ws_bytes, void* stream) {
-  ptycho_status st = check_ms(dims, ms);
-  if (st != PTYCHO_OK) return st;
-  if (batch < 1 || !(eps >= 0.0)) return PTYCHO_ERR_ARG;
-  if (noise != PTYCHO_NOISE_GAUSSIAN && noise != PTYCHO_NOISE_POISSON && noise != PTYCHO_NOISE_VJP)
-    return PTYCHO_ERR_ARG;
-  if (!object || !probe || !g_object || !g_probe || (dims->J > 0 && (!pos || !meas))) return PTYCHO_ERR_ARG;
-  if ((st = check_ws(ws, ws_bytes, ms_layout(*dims, ms->S, batch, ms->recompute != 0).total)) != PTYCHO_OK)
-    return st;
-  if (dims->J == 0) return PTYCHO_OK;
-  cudaStream_t s = (cudaStream_t)stream;
-  MsArgs a;
-  cudaError_t e = cudaSuccess;
-  ms_setup(*dims, *ms, batch, ws, a, s, &e);
-  if (e != cudaSuccess) return PTYCHO_ERR_CUDA;
-  a.obj = (const float2*)object; a.probe = (const float2*)probe; a.pos = pos; a.meas = meas;
-  a.mode = noise == PTYCHO_NOISE_GAUSSIAN ? MODE_GRAD_GAUSS : noise == PTYCHO_NOISE_POISSON ? MODE_GRAD_POISSON
-                                                                                          : MODE_VJP;
-  a.eps = (float)eps;
-  a.gobj = (float2*)g_object; a.gpos = g_pos; a.loss = loss;
-  const int NN = dims->N * dims->N;
-  for (int b0 = 0; b0 < dims->J; b0 += batch) {
-    a.b0 = b0;
-    a.nb = (dims->J - b0 < batch) ? dims->J - b0 : batch;
-    if (pass1_ms(dims->N, a, s) != cudaSuccess) return PTYCHO_ERR_CUDA;
-    if (probe_reduce(NN, 0, dims->M, dims->M, a.nb, a.h_s, a.o_s, a.valid, (float2*)g_probe, 1, nullptr, nullptr, 0,
-                     nullptr, s) != cudaSuccess)
-      return PTYCHO_ERR_CUDA;
-  }
-  return PTYCHO_OK;
+  return adjoint_ms(dims, ms, object, probe, pos, meas, noise, eps, batch, g_object, g_probe, g_pos, loss, ws, ws_bytes,
+                    stream, 0);
 }
 
 size_t ptycho_workspace_bytes_lsqml_ms(const ptycho_dims* dims, const ptycho_multislice* ms,
