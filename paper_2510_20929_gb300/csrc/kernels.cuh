@@ -200,6 +200,8 @@ __device__ __forceinline__ void overlap_add(const BatchArgs& a, int slot, int j,
   if (a.gpos || a.possum) {
     const bool ls = a.possum != nullptr;
     float gy = 0.f, gx = 0.f, a11 = 0.f, a12 = 0.f, a22 = 0.f;
+    // (four pixels' loads in flight: the small windows' few threads take many each)
+#pragma unroll 4
     for (int p = tid; p < LNN; p += T) {
       const int r = p / N, c = p % N;
       const float2* o = a.obj + (size_t)(ty + y0 + r) * a.W + (tx + c);

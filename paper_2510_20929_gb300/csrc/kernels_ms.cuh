@@ -314,6 +314,7 @@ __global__ void __launch_bounds__(G::T, PairCtas<G>::n) k_pass1_ms(MsArgs a) {
     }
     if (a.gpos) {
       const float2* Os = a.obj + s * HW;
+#pragma unroll 4
       for (int p = tid; p < LNN; p += T) {
         const int r = p / N, c = p % N;
         const float2* o = Os + (size_t)(ty + y0 + r) * a.W + (tx + c);
