@@ -1,9 +1,9 @@
 // Per-scan-position kernels of the LSQML hot path (templated on the window N).
 //
-// k_pass1: one CTA per position of a minibatch at window 16 (kernels_pair.cuh
-//   holds the windows from 32 on; its line pairs leave 16 too few threads:
-//   measured equal or slower, with a relaxed probe 12 -> 16 us per 256
-//   positions). For every incoherent probe mode k it extracts the sub-pixel object patch o_j = S_j(O) (bilinear),
+// k_pass1: one CTA per position of a minibatch at window 16, and at 32 while a
+//   launch has few positions per SM (kernels_pair.cuh holds the other windows; its
+//   line pairs leave 16 too few threads: measured equal or slower, with a relaxed
+//   probe 12 -> 16 us per 256 positions). For every incoherent probe mode k it extracts the sub-pixel object patch o_j = S_j(O) (bilinear),
 //   forms the exit wave psi_jk = P_k o_j (Pty-Chi Sec. 2.1, the psi = p o of
 //   Eq. 2), propagates it with the unitary 2-D FFT and accumulates the
 //   incoherent intensity I_j = sum_k |Psi_jk|^2 (Eq. 4's forward model). It
@@ -28,6 +28,7 @@ namespace cg = cooperative_groups;
 // alternative the autotuner may pick (half of it, two lines per thread).
 template <int N> struct Threads;
 template <> struct Threads<16> { static constexpr int T = 64, ALT = 32; };
+template <> struct Threads<32> { static constexpr int T = 128; };
 
 template <int N>
 struct Pass1Smem {

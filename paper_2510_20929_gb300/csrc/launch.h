@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 namespace ptycho {
+int sm_count();   // of the current device
 struct BatchArgs;
 struct Pass2Args;
 struct MsArgs;
