@@ -26,7 +26,9 @@
 // 6.26 ms; the LSQML pass at window 128 with 3 slices, 2 modes, 128 positions
 // 373 -> 289 us.
 #pragma once
+#include "kernels_ms_line.cuh"
 #include "kernels_pair.cuh"
+#include "launch.h"
 
 namespace ptycho {
 
@@ -448,17 +450,40 @@ static cudaError_t launch_ms(K kernel, const A& a, cudaStream_t s, unsigned long
   return cudaLaunchKernelEx(&cfg, kernel, a);
 }
 
+// One line of a transform per lane group (kernels_ms_line.cuh), or packed line
+// pairs? At 16 and 32 the packed form leaves a position 32 and 64 threads; while
+// a launch has few positions per SM, all that counts is how long one takes.
+// Measured on GB300, one line <- or -> packed, us per launch (slices x modes):
+//   window 16, forward 3x2: 8 positions 9 <- 13, 512: 13 <- 15, 1024: 15 <- 17, 2048: 26 -> 23
+//   window 16, gradients 3x2: 8: 18 <- 25, 400: 23 <- 27, 512: 26 <- 29, 1024: 36 -> 33
+//   window 16, LSQML (pass and tangents) 3x2: 8: 40 <- 48, 256: 51 <- 56, 400: 60 -> 58
+//   window 32, forward 3x2: 8: 15 <- 20, 256: 21 <- 23, 400: 39 -> 29
+//   window 32, gradients 3x2: 8: 36 <- 46, 152: 38 <- 46, 200: 51 -> 49
+//   window 32, LSQML 3x2: 8: 72 <- 82, 152: 78 <- 86, 200: 114 -> 90; 2x1: 8: 49 -> 48, 152: 60 -> 50
+enum class MsUse { FORWARD, GRADIENT, LSQML };
+inline bool ms_one_line(int N, int nb, int S, MsUse use) {
+  const int sms = sm_count();
+  if (N == 16) return nb <= (use == MsUse::FORWARD ? 6 : use == MsUse::GRADIENT ? 4 : 2) * sms;
+  if (N == 32) return use == MsUse::LSQML ? S > 2 && nb <= sms : nb <= (use == MsUse::FORWARD ? 2 : 1) * sms;
+  return false;
+}
+
 template <int N>
 cudaError_t launch_pass1_ms(const MsArgs& a, cudaStream_t s) {
+  const bool lsqml = a.mode == MODE_LSQML_GAUSS || a.mode == MODE_LSQML_POISSON;
+  if constexpr (N <= 32)
+    if (ms_one_line(N, a.nb, a.S, a.mode == MODE_FWD ? MsUse::FORWARD : lsqml ? MsUse::LSQML : MsUse::GRADIENT))
+      return launch_pass1_ms_line<N>(a, s);
   using G = PairGeo<N>;
   static unsigned long long done[2] = {0, 0};
-  return (a.mode == MODE_LSQML_GAUSS || a.mode == MODE_LSQML_POISSON)
-             ? launch_ms<G>(k_pass1_ms<G, true>, a, s, &done[1])
-             : launch_ms<G>(k_pass1_ms<G, false>, a, s, &done[0]);
+  return lsqml ? launch_ms<G>(k_pass1_ms<G, true>, a, s, &done[1])
+               : launch_ms<G>(k_pass1_ms<G, false>, a, s, &done[0]);
 }
 
 template <int N>
 cudaError_t launch_step_ms(const MsStepArgs& a, cudaStream_t s) {
+  if constexpr (N <= 32)   // (it reads the incident waves in the order the pass left them)
+    if (ms_one_line(N, a.nb, a.S, MsUse::LSQML)) return launch_step_ms_line<N>(a, s);
   using G = PairGeo<N>;
   static unsigned long long done = 0;
   return launch_ms<G>(k_step_ms<G>, a, s, &done);
