@@ -315,13 +315,23 @@ static cudaError_t smem_optin_once(Kern kernel, size_t bytes, unsigned long long
 static cudaError_t opr_reduce(int NN, int M, int K, int nb, int b0, const int* order, const float* w,
                               const float2* h_s, const float2* o_s, const int* valid, float2* dUacc, float* D,
                               cudaStream_t s) {
-  // pixel pairs across blockIdx.x, the batch split into as many chunks as two CTAs
-  // per SM hold at once (one more leaves a last wave that is nearly empty)
+  // pixel pairs across blockIdx.x, the batch in as many chunks as fill one to four
+  // waves of two CTAs per SM: the fewest slots one after another (4 more stand
+  // for a CTA's start and its atomics). One wave leaves a sixth of the places
+  // empty at window 256 with its 128 CTAs per chunk, 8 eigenmodes, 256 slots: 2
+  // chunks 73.5 us, 3 (a second wave nearly empty) 92.8, 7 (three waves) 68.0; 700
+  // slots: 183, 224, 161; 64 slots: 2 chunks 24.9, 7: 27.4.
   const int NP = NN / 2;
   const int bx = (NP + 255) / 256;
-  int chunks = 2 * sm_count() / bx;
-  if (chunks > nb) chunks = nb;
-  if (chunks < 1) chunks = 1;
+  int chunks = 1;
+  long long best = -1;
+  for (int waves = 1; waves <= 4; ++waves) {
+    int c = waves * 2 * sm_count() / bx;
+    if (c > nb) c = nb;
+    if (c < 1) c = 1;
+    const long long cost = (long long)waves * ((nb + c - 1) / c + 4);
+    if (best < 0 || cost < best) best = cost, chunks = c;
+  }
   const int chunk = (nb + chunks - 1) / chunks;
   chunks = (nb + chunk - 1) / chunk;
   cudaEvent_t e0 = profile_begin(K_OPR_REDUCE, s);
