@@ -121,7 +121,7 @@ typedef struct {
  * candidates (the "variants" below):
  *   [0] the per-position pass: window 16: CTA sizes default / alternative; the
  *       others have one (window 128 accepts 0, 1 and 2, windows 32 and 64 accept
- *       0 and 1 for it);
+ *       0 and 1 for it, and its time is reported for each);
  *   [1] the step-size pass: one CTA per position or two launches that walk over
  *       the positions, by the size of the minibatch (0), the two launches (1),
  *       or (windows <= 128) a cluster of 4 CTAs per position adding their

@@ -447,7 +447,7 @@ struct TuneKey {
     return dev == o.dev && N == o.N && M == o.M && H == o.H && W == o.W && B == o.B;
   }
 };
-// v[0]: the per-position pass (candidates: pass1_variants(N)), v[1]: the
+// v[0]: the per-position pass (candidates: pass1_forms(N)), v[1]: the
 // step-size pass (candidates: pass2_variants(N): by the minibatch, two launches,
 // cluster at 4 or 3 CTAs per SM), v[2]: the probe reduction (positions
 // in flight per thread: 16, 8, 32, or 8 in each of 4 threads splitting the
@@ -458,8 +458,10 @@ struct TuneEntry {
   float ms[PTYCHO_TUNE_KERNELS][PTYCHO_TUNE_MAX];
 };
 
-// (only window 16 has two that differ; the others' numbers stay accepted)
+// Numbers accepted for the per-position pass, and how many of them differ: only
+// window 16 has two CTA sizes. The others name one kernel, which is timed once.
 static int pass1_variants(int N) { return N == 128 ? 3 : (N <= 128 ? 2 : 1); }
+static int pass1_forms(int N) { return N == 16 ? 2 : 1; }
 static int pass2_variants(int N) { return N <= 128 ? 4 : 2; }
 static constexpr int kReduceVariants = 4;
 static std::mutex g_tune_mu;
@@ -657,8 +659,9 @@ static ptycho_status autotune(const ptycho_dims& d, float2* obj, float2* probe, 
       if (ms[c] < ms[b]) b = c;
     return b;
   };
-  const int n1 = pass1_variants(N);
+  const int n1 = pass1_forms(N);
   for (int v = 0; v < n1; ++v) t->ms[0][v] = time_launch(s, 3, [&] { return pass1(N, a, s, v); });
+  for (int v = n1; v < pass1_variants(N); ++v) t->ms[0][v] = t->ms[0][0];
   t->v[0] = best(t->ms[0], n1);
   // one clean pass 1 with the chosen variant feeds the other candidates
   if (cudaMemsetAsync(w.acc, 0, (size_t)HW * sizeof(float4), s) != cudaSuccess) return PTYCHO_ERR_CUDA;
