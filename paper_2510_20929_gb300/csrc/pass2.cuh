@@ -18,6 +18,7 @@
 // ahead and staged corners all measured the same).
 #pragma once
 #include "kernels.cuh"
+#include "launch.h"
 
 namespace ptycho {
 
@@ -339,7 +340,6 @@ __global__ void __cluster_dims__(PASS2C_C, 1, 1) __launch_bounds__(PASS2C_T, MIN
 }
 
 constexpr int STEP_T = 256, STEP_U = 4, STEP_GROUP = 96;   // threads, positions per tree, most positions per CTA
-constexpr int SMS = 152;   // of a GB300
 
 template <int N>
 struct StepSums {
@@ -589,11 +589,12 @@ cudaError_t launch_step(const Pass2Args& a, cudaStream_t s) {
   if (e != cudaSuccess) return e;
   // Positions per CTA: the fewest rounds of positions with 3 CTAs per SM at
   // work (4 more stand for a CTA's start), not a last wave that is nearly empty.
+  const long long places = 3 * sm_count();
   int per = STEP_U;
   long long best = -1;
   for (int q = STEP_U; q <= STEP_GROUP; q += STEP_U) {
     const long long ctas = (long long)S::CHUNKS * ((a.nb + q - 1) / q);
-    const long long cost = (ctas + 3 * SMS - 1) / (3 * SMS) * (q + 4);
+    const long long cost = (ctas + places - 1) / places * (q + 4);
     if (best < 0 || cost < best) best = cost, per = q;
   }
   e = launch_pdl(k_step_sums<N, OPR>, dim3(S::CHUNKS * ((a.nb + per - 1) / per)), dim3(S::T), sm, s, a, per);
@@ -618,8 +619,8 @@ cudaError_t launch_step(const Pass2Args& a, cudaStream_t s) {
 inline bool use_step(int N, int nb, bool opr) {
   if (N < 64) return false;
   if (opr && N >= 128) return true;
-  const int slots = 2 * SMS, waves = (nb + slots - 1) / slots;
-  if (N == 64 && nb <= SMS) return opr;
+  const int slots = 2 * sm_count(), waves = (nb + slots - 1) / slots;
+  if (N == 64 && nb <= sm_count()) return opr;
   return 10LL * nb < 7LL * slots * waves;
 }
 
