@@ -29,7 +29,8 @@ namespace fp {
 namespace cg = cooperative_groups;
 
 template <int DIR> struct PDft<3, DIR> {
-  template <class V> __device__ __forceinline__ static void run(V& v) {   // see Dft<3>
+  // X0 = v0 + (v1 + v2); X1,2 = v0 - (v1 + v2)/2 +- i DIR sin(2 pi / 3) (v1 - v2)
+  template <class V> __device__ __forceinline__ static void run(V& v) {
     const float2 s3 = splat(DIR * 0.86602540378443865f), mh = splat(-0.5f);
     const C2 t1 = padd(v[1], v[2]), t2 = psub(v[1], v[2]);
     const C2 m = {fma2(mh, t1.re, v[0].re), fma2(mh, t1.im, v[0].im)};
@@ -58,7 +59,7 @@ __device__ __forceinline__ C2 ptw24(C2 a) {
 }
 
 template <int DIR> struct PDft<24, DIR> {
-  // n = b + 3a, k = k1 + 8k2 (see Dft<24>)
+  // n = b + 3a, k = k1 + 8k2: X[k] = sum_b W3^(b k2) W24^(b k1) sum_a W8^(a k1) v[b + 3a]
   template <class V> __device__ __forceinline__ static void run(V& v) {
     C2 y[3][8];
 #pragma unroll
@@ -99,7 +100,6 @@ struct ClFft {
   static constexpr int NP = R2;         // pixel pairs per thread
   static constexpr bool VERT = true;    // a pixel pair is two rows of one column
   static_assert(R1 * R2 == N && S * R1 == R2 && 32 % R1 == 0, "line split; a line's lanes share a warp");
-  using Line = LineFft<R1, R2, false, void>;
   static constexpr int TW = R1 * (R2 + 1);
   __device__ __forceinline__ static void fill_twiddles(float2* tw) { make_line_twiddles<N, R1, R2>(tw); }
 
@@ -152,7 +152,7 @@ struct ClFft {
   template <int DIR>   // v[k] *= exp(DIR 2 pi i n k / N)
   __device__ __forceinline__ void twiddle(C2 (&v)[R2]) const {
     float2 t[R2];
-    Line::twiddles(t, tw, n);
+    LineTwiddles<R1, R2>::twiddles(t, tw, n);
 #pragma unroll
     for (int k = 1; k < R2; ++k)
       v[k] = DIR < 0 ? pmul(v[k], t[k].x, t[k].y) : pmulc(v[k], {splat(t[k].x), splat(t[k].y)});

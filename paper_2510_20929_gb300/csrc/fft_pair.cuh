@@ -129,7 +129,7 @@ template <int DIR> struct PDft<8, DIR> {
   }
 };
 template <int DIR> struct PDft<16, DIR> {
-  // n = b + 4a, k = k1 + 4k2 (see Dft<16>)
+  // n = b + 4a, k = k1 + 4k2: X[k] = sum_b W16^(b k1) W4^(b k2) sum_a W4^(a k1) v[b + 4a]
   template <class V> __device__ __forceinline__ static void run(V& v) {
     C2 y[4][4];
 #pragma unroll
@@ -205,7 +205,7 @@ struct Fft {
   using C = Cfg<N>;
   static constexpr int R1 = C::R1, R2 = C::R2, S = R2 / R1, G = 32 / R1, T = N / 2 * R1;
   static_assert(R1 * R2 == N && S * R1 == R2 && R1 % 2 == 0 && T % 32 == 0, "line split");
-  static_assert(R1 == Fft2<N>::R1 && R2 == Fft2<N>::R2, "the line transforms of fft.cuh");
+  static_assert(R1 == FftCfg<N>::R1 && R2 == FftCfg<N>::R2, "the line split of fft.cuh");
   static constexpr int UNITS = N * N / 2;   // 16-byte units of the tile
 
   // this thread's index within its line, and its line pair, by rows and by columns
@@ -245,7 +245,7 @@ struct Fft {
   // W^(n k), k = 1..R2-1: the first four from the table, the rest as products
   // (fft.cuh's); one lane index for both lines of the pack
   __device__ __forceinline__ static void twiddles(float2 (&t)[R2], const float2* tw, int n) {
-    Fft2<N>::twiddles(t, tw, n);
+    LineTwiddles<R1, R2>::twiddles(t, tw, n);
   }
   // Forward, first pass: columns. In: v[n2] = pixels (n + R1 n2, 2p), (.., 2p + 1).
   // Leaves the half-transformed tile in row units.
