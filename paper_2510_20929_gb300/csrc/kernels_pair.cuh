@@ -1,7 +1,8 @@
-// The per-position pass on the packed line-pair transforms: windows 32, 64 and
-// 128 in one CTA (fft_pair.cuh), 192 and 256 on a cluster of CTAs with 32 rows
-// each (fft_cluster.cuh). It computes what k_pass1 (kernels.cuh) describes;
-// what differs is where the data lives:
+// The per-position pass on the packed line-pair transforms: windows 32 (but for
+// launches of few positions, see pass_n32.cu), 64 and 128 in one CTA
+// (fft_pair.cuh), 192 and 256 on a cluster of CTAs with 32 rows each
+// (fft_cluster.cuh). It computes what k_pass1 (kernels.cuh) describes; what
+// differs is where the data lives:
 //   * every thread owns the same pixel pairs (two neighbours of one row, or, on
 //     a cluster, of one column) when a mode's exit wave is built and when its chi comes back, so
 //     psi_jk goes from the loads straight into the column transform's
@@ -18,14 +19,15 @@
 // wavefronts and issue slots), then the rate of L2 requests of the probe
 // loads, the far-field scratch and the h stores (about 2.8 cycles per 128-byte
 // request when all SMs stream), with one CTA of 512 threads filling an SM at
-// window 128, and on the cluster windows the waits for the cluster. Straight-line code that a CTA runs once costs instruction
-// fetches, so loops over a thread's pixels stay rolled where v is not indexed.
+// window 128, and on the cluster windows the waits for the cluster.
+// Straight-line code that a CTA runs once costs instruction fetches, so loops
+// over a thread's pixels stay rolled where v is not indexed.
 // Measured on GB300 against the one-line-per-lane-group passes it replaced (per
 // launch): window 256, 8 modes, 256 positions 2423 -> 1705 us, 1 mode 496 ->
-// 342; window 192, 4 modes 986 -> 673, 1 mode 406 -> 293; window 128, 5 modes, 256 positions 287 -> 249 us (1 mode: 101 -> 92,
-// 1024 positions 1002 -> 860); window 64, 4 modes, 256 positions 63 -> 51,
-// 1216 positions 227 -> 166, 1 mode, 16 positions 24.7 -> 20.7; window 32, 4
-// modes, 2000 positions 116 -> 72.
+// 342; window 192, 4 modes 986 -> 673, 1 mode 406 -> 293; window 128, 5 modes,
+// 256 positions 287 -> 249 us (1 mode: 101 -> 92, 1024 positions 1002 -> 860);
+// window 64, 4 modes, 256 positions 63 -> 51, 1216 positions 227 -> 166, 1 mode,
+// 16 positions 24.7 -> 20.7; window 32, 4 modes, 2000 positions 116 -> 72.
 #pragma once
 #include <type_traits>
 
@@ -134,9 +136,10 @@ struct PairSmem {
 // loss and returns the far-field factor. Square roots and quotients are
 // formed from rsqrtf with one residual correction each (Markstein, IBM J. Res.
 // Dev. 34, 1990: s += r y / 2 with the residual r = x - s^2 exact in one fused
-// multiply-add; q += r / d likewise), within the rounding of the correctly
-// rounded results: sqrtf and the division leave the straight code for a zero
-// operand, and most counts of a diffraction pattern are zero. Values outside
+// multiply-add; q += r / d likewise): sqrtf and the division leave the straight
+// code for a zero operand, and most counts of a diffraction pattern are zero. The
+// values were sqrtf's for every float in [1, 4) and the division's, for both
+// likelihoods, in all of 2^24 pairs of a count and an intensity. Values outside
 // 2^-96 .. 2^96 (zero counts aside) take the functions. `t` receives what the
 // loss adds per pixel: the difference of the amplitudes (added squared), or
 // the Poisson term; (x, z) and (y, w) are two rows.
@@ -606,6 +609,11 @@ __global__ void __launch_bounds__(G::T, PairCtas<G>::n) k_pass1_pair(BatchArgs a
   // eigenmode by eigenmode, half of the pairs' loads in flight (pair by pair,
   // each over all eigenmodes, 256 positions of the 192 window with 8
   // eigenmodes took 613 us instead of 435), and kept in p0 for the way back.
+  // The one call that is slower for it than with the unpacked pass is the
+  // forward model of a lone relaxed mode at window 256 (700 positions, 8
+  // eigenmodes 524 -> 600 us, 1: 448 -> 466): two eigenmodes in flight (629 us),
+  // quarters of the pairs with four (591, but 192 slower) and a prefetch of
+  // the next eigenmode into L1 (632) did not mend it.
   auto probe_fwd = [&](const float2* Pk, float4 (&P)[NP]) {
     if (!OPR || Pk) {
 #pragma unroll

@@ -348,9 +348,12 @@ struct StepSums {
   static_assert(T * CHUNKS * 2 == N * N && T % 32 == 0, "a pixel pair per thread");
 };
 
-// Sums of `per` positions over one chunk's pixel pairs per CTA, added to a.part[slot][5] (zero on entry). Dynamic shared memory:
-// (M + K) T float4, the direction of each mode (OPR: of each eigenmode, then
-// of the shared modes) at the thread's pair.
+// Sums of `per` positions over one chunk's pixel pairs per CTA, added to
+// a.part[slot][5] (zero on entry) by FP64 atomics: the last bits of a position's
+// sums, and so of its alpha, depend on the order in which the chunks finish (one
+// CTA per position adds in a fixed order). Dynamic shared memory: (M + K) T
+// float4, the direction of each mode (OPR: of each eigenmode, then of the shared
+// modes) at the thread's pair.
 template <int N, bool OPR>
 __global__ void __launch_bounds__(StepSums<N>::T, 3) k_step_sums(Pass2Args a, int per) {
   constexpr int NN = N * N, T = StepSums<N>::T, U = STEP_U, W = T / 32;
