@@ -201,8 +201,9 @@ __device__ __forceinline__ void overlap_add(const BatchArgs& a, int slot, int j,
   if (a.gpos || a.possum) {
     const bool ls = a.possum != nullptr;
     float gy = 0.f, gx = 0.f, a11 = 0.f, a12 = 0.f, a22 = 0.f;
-    // (four pixels' loads in flight: the small windows' few threads take many each)
-#pragma unroll 4
+    // four pixels' loads in flight: the smaller CTAs' threads take many each (512
+    // threads gain 1 % from four and lose as much when no sums are wanted)
+#pragma unroll (T < 512 ? 4 : 2)
     for (int p = tid; p < LNN; p += T) {
       const int r = p / N, c = p % N;
       const float2* o = a.obj + (size_t)(ty + y0 + r) * a.W + (tx + c);
